@@ -138,10 +138,9 @@ int dilbm_create(const dilbm_grid *grid, dilbm_lattice lattice, double tau,
  * 28-29).  Each step is one fused pull-stream + collide sweep over every node,
  * a per-particle FP64 force/torque reduction and a rigid-body update.
  * Asynchronous: returns once the work is queued; errors raised on the device
- * (UNSTABLE, OVERFLOW) surface at the next dilbm_sync().  Whole pairs of
- * steps replay a CUDA graph captured on the context's stream on first use
- * (not on the legacy default stream, not while timing, and not while the
- * caller is capturing that stream, where the launches are issued directly).
+ * (UNSTABLE, OVERFLOW) surface at the next dilbm_sync().  One cooperative
+ * launch runs many steps (about 2^27 node updates); with PS-LBM, while timing,
+ * and while the caller is capturing the context's stream, one step.
  */
 int dilbm_step(dilbm_ctx *ctx, long long nsteps);
 
@@ -225,8 +224,7 @@ int dilbm_force_mean_reset(dilbm_ctx *ctx);
  * one column against the fixed end densities, which the ends re-absorb.
  * Positions reported by dilbm_forces() are frame positions.  A checkpoint
  * (dilbm_get_populations, dilbm_forces' state) holds frame positions and
- * populations: keep the offset beside it.  One more kernel launch per step
- * while the frame is on.  Requires
+ * populations: keep the offset beside it.  Requires
  * nx x (bytes per stored population) <= 48 KiB.  Contexts with a moving
  * frame cannot join a batch.
  * Errors: INVALID_ARG (particle out of range, x_ref not finite, lattice too
@@ -293,9 +291,10 @@ void dilbm_destroy(dilbm_ctx *ctx);
 const char *dilbm_last_error(void);
 
 /*
- * Measurement: with timing on, CUDA events bracket every lattice-sweep launch
- * on the context's stream; dilbm_sweep_time() returns their summed duration
- * in milliseconds and the number of launches since timing was (re)enabled.
+ * Measurement: with timing on, each step is a launch of its own (the sweep,
+ * with the particle update running beside it), bracketed by CUDA events on
+ * the context's stream; dilbm_sweep_time() returns their summed duration in
+ * milliseconds and the number of launches since timing was (re)enabled.
  * dilbm_launch_count() is the number of kernels this context has launched.
  */
 int dilbm_set_timing(dilbm_ctx *ctx, int enable);
@@ -304,10 +303,9 @@ long long dilbm_launch_count(const dilbm_ctx *ctx);
 
 /*
  * Batches: many contexts advanced together (the same equations, Eqs. 13-19,
- * 22-24, 28-29, on every member).  One step of a batch is one sweep launch
- * over the concatenated row segments of all members and one particle launch
- * over all their particles, replayed from CUDA graphs captured at create;
- * every member's result is bit for bit the one dilbm_step gives it alone.
+ * 22-24, 28-29, on every member).  One launch runs several steps over the
+ * concatenated row segments and particles of all members (up to 84 members;
+ * larger batches take a launch per 84); every member's result is bit for bit the one dilbm_step gives it alone.
  *
  * dilbm_batch_create: members[0..n-1] (1 <= n <= 1024 distinct contexts, all
  *   with the same storage; they stay owned by the caller and must outlive the
@@ -321,8 +319,10 @@ long long dilbm_launch_count(const dilbm_ctx *ctx);
  * dilbm_batch_errors: wait; codes[k] (host, n ints) receives member k's error
  *   (DILBM_OK, UNSTABLE, TIMEOUT or OVERFLOW).  Returns CUDA on a CUDA error.
  * dilbm_batch_set_timing / dilbm_batch_sweep_time: CUDA events around every
- *   batched sweep launch (timing replaces graph replay by direct launches).
- * dilbm_batch_launch_count: kernels the batch has launched.
+ *   step, which is then a launch of its own.
+ * dilbm_batch_launch_count: the passes the batch has run: a sweep pass per
+ *   launch group and step, a particle pass per step, and the error gathers of
+ *   dilbm_batch_sync (a launch covers both passes of several steps).
  */
 typedef struct dilbm_batch dilbm_batch;
 int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilbm_batch **out);

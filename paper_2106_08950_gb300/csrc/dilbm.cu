@@ -49,8 +49,12 @@ struct dilbm_ctx {
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;
     Particles P{};
-    Bins bins[2]{};                   // tile bins by step parity
-    float4 *partial = nullptr;        // per tile, slot and row: force / torque partials
+    unsigned tag = 0;                 // step number, marks the step's force partials
+    int rot = 0;                      // which of the three tile-count arrays the next step reads
+    BinSet B{};                       // tile bins
+    float4 *partial = nullptr;        // per particle, tile of its list and row: force / torque partials
+    PartArgs *pa = nullptr;           // device: the particle update's arguments (push_part_args)
+    GridSync *sync = nullptr;         // device: the barrier of launches over several steps
     double *force = nullptr, *fcol = nullptr;
     double *fsum = nullptr;           // per particle: sum of (Fx, Fy, T) since the last reset
     long long fsum_steps = 0;
@@ -67,11 +71,9 @@ struct dilbm_ctx {
     size_t ev_used = 0;
     long long launches = 0;
     SweepShape shape{};               // launch shape of the step sweep (autotuned or default)
-    cudaGraphExec_t g_pair[2] = {nullptr, nullptr};   // two steps from parity 0 / 1, replayed by dilbm_step
     int track = -1;                   // moving frame: tracked particle, -1 when off
     double track_x = 0.0;             // its reference x
     long long *frame_off = nullptr;   // device: columns the frame has moved, allocated on first use
-    float *cover = nullptr;           // PS: per-particle covered-area tables (grown by upload_particles)
     // A strip of a lattice decomposed over ranks (dilbm_create_strip): L holds
     // rows [y0, y0 + L.ny) with halo rows across its cuts, Lg the whole
     // lattice (the particles' geometry), tile rows [ty_lo, ty_lo + L.nty).
@@ -178,11 +180,12 @@ unsigned long long footprint_of(int nx, int ny, size_t elem, int np) {
         (unsigned long long)((nx + TILE_W - 1) / TILE_W) * (unsigned long long)((ny + TILE_H - 1) / TILE_H);
     const unsigned long long npa = np > 0 ? (unsigned long long)np : 1ull;
     unsigned long long b = 2ull * (9ull * plane + 2ull * GUARD) * elem;           // populations A, B
-    b += 10ull * npa * sizeof(double) + 4ull * npa * sizeof(float) + npa * sizeof(int);   // particle state
+    b += 15ull * npa * sizeof(double) + 5ull * npa * sizeof(float) + npa * sizeof(int);   // particle state
     b += 6ull * npa * sizeof(double) + 2ull * npa * sizeof(double) + sizeof(int);         // force, fsum, fcol, err
-    b += ntiles * MAXC * TILE_H * sizeof(float4);                                         // partials
-    b += 2ull * (ntiles * sizeof(int) + ntiles * MAXC * sizeof(int) + ntiles * MAXC * NREC * sizeof(float4) +
-                 npa * MAXT * sizeof(int) + npa * sizeof(int));                           // bins, two parities
+    b += npa * MAXT * TILE_H * sizeof(float4);                                            // partials
+    b += 3ull * ntiles * sizeof(int) + 2ull * ntiles * MAXC * (sizeof(int2) + NREC * sizeof(float4)) +
+         2ull * npa * (MAXT + 2) * sizeof(int);                                           // bins
+    b += sizeof(PartArgs) + sizeof(GridSync);
     return b;
 }
 
@@ -200,52 +203,56 @@ int check_reach(double cut_d, const dilbm_particle *p, int np) {
     return DILBM_OK;
 }
 
-PartArgs particle_args(const dilbm_ctx *c, int cur, int integrate, int phase = 0) {
-    const int nxt = integrate ? cur ^ 1 : cur;
+PartArgs particle_args(const dilbm_ctx *c) {
     PartArgs a{};
     a.L = c->strip ? c->Lg : c->L;
     if (c->strip) {
         a.ty_lo = c->ty_lo;
         a.ty_hi = c->ty_lo + c->L.nty;
-        a.phase = phase;
         a.fpart = c->fpart;
     }
     a.ph = c->ph;
     a.P = c->P;
     a.bp = c->bp;
-    a.bin_in = c->bins[cur];
-    a.bin_out = c->bins[nxt];
+    a.B = c->B;
     a.partial = c->partial;
-    a.pin = cur;
-    a.pout = nxt;
-    a.integrate = integrate;
     a.force = c->force;
     a.fcol = c->fcol;
-    a.fsum = integrate ? c->fsum : nullptr;
+    a.fsum = c->fsum;
     a.err = c->err;
     a.track = c->track;
     a.track_x = c->track_x;
+    a.frame_off = c->frame_off;
     return a;
 }
 
-int launch_particles(dilbm_ctx *c, int integrate, int phase = 0) {
-    const int np = c->np;
-    particles_kernel<false><<<(np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, c->stream>>>(
-        particle_args(c, c->cur, integrate, phase), nullptr, BatchIndex{});
-    DILBM_CUDA(cudaGetLastError());
-    c->launches += 1;
-    if (c->method == DILBM_METHOD_PS && phase != 1) {
-        // the covered-area tables of the positions just written
-        const int pout = integrate ? c->cur ^ 1 : c->cur;
-        cover_kernel<<<np, dim3(COVER_BX, COVER_BY), 0, c->stream>>>(c->cover, c->P.x[pout], c->P.y[pout], c->P.r, np,
-                                                                     c->ph);
-        DILBM_CUDA(cudaGetLastError());
-        c->launches += 1;
-    }
+// The device copy that fused steps read, after anything in it has changed.
+int push_part_args(dilbm_ctx *c) {
+    const PartArgs a = particle_args(c);
+    DILBM_CUDA(cudaMemcpyAsync(c->pa, &a, sizeof(a), cudaMemcpyHostToDevice, c->stream));
     return DILBM_OK;
 }
 
-void drop_graphs(dilbm_ctx *c);
+// PS: the covered-area tables of position copy `pos`.
+int launch_cover(dilbm_ctx *c, int pos) {
+    cover_kernel<<<c->np, dim3(COVER_BX, COVER_BY), 0, c->stream>>>(c->B.cover, c->P.x[pos], c->P.y[pos], c->P.r, c->np,
+                                                                    c->ph);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
+    return DILBM_OK;
+}
+
+// The particle update as a launch of its own: an upload's binning
+// (integrate == 0), or a phase of a strip's step.
+int launch_particles(dilbm_ctx *c, int integrate, int phase = 0) {
+    particles_kernel<<<(c->np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, c->stream>>>(particle_args(c), c->cur,
+                                                                                              c->rot, integrate ? c->tag + 1 : c->tag,
+                                                                                              integrate, phase);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
+    if (c->method == DILBM_METHOD_PS && phase != 1) return launch_cover(c, integrate ? c->cur ^ 1 : c->cur);
+    return DILBM_OK;
+}
 
 // Rows of shared memory the moving frame's in-place column shift may use.
 constexpr size_t FRAME_ROW_BYTES = 48 * 1024;
@@ -286,15 +293,14 @@ int size_cover_tables(dilbm_ctx *c, const dilbm_particle *p, int np) {
     const int K = (int)std::ceil(rmax + c->ph.cut_d) + 1;
     if (K <= c->ph.ck) return DILBM_OK;
     const size_t S = 2 * (size_t)K + 1;
-    if (c->cover) {
+    float *grown = nullptr;
+    DILBM_CUDA(cudaMalloc(&grown, sizeof(float) * S * S * (size_t)np));
+    if (c->B.cover) {
         DILBM_CUDA(cudaStreamSynchronize(c->stream));
-        DILBM_CUDA(cudaFree(c->cover));
-        c->cover = nullptr;
+        DILBM_CUDA(cudaFree(c->B.cover));
     }
-    DILBM_CUDA(cudaMalloc(&c->cover, sizeof(float) * S * S * (size_t)np));
+    c->B.cover = grown;
     c->ph.ck = K;
-    c->bins[0].cover = c->bins[1].cover = c->cover;
-    drop_graphs(c);
     return DILBM_OK;
 }
 
@@ -302,10 +308,10 @@ int upload_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
     // every check before any state changes
     int rc = check_reach(c->ph.cut_d, p, np);
     if (rc) return rc;
-    const int wx = c->L.wrap_x, wy = c->L.wrap_y;
+    const int wx = c->L.wrap_x, wy = c->L.wrap_y, ck = c->ph.ck;
     set_wrap_flags(c, p, np);
-    if (c->L.wrap_x != wx || c->L.wrap_y != wy) drop_graphs(c);
     if ((rc = size_cover_tables(c, p, np))) return rc;
+    if ((c->L.wrap_x != wx || c->L.wrap_y != wy || c->ph.ck != ck) && (rc = push_part_args(c))) return rc;
     // pinned staging: x, y, then r, ux, uy, omega, theta, rho_s (one device
     // slice), as doubles, then fixed as ints; reused once the previous
     // upload's copies have read it
@@ -333,161 +339,127 @@ int upload_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
     DILBM_CUDA(cudaMemcpyAsync(c->P.r, h + 2 * np, sizeof(double) * 6 * np, cudaMemcpyHostToDevice, c->stream));
     DILBM_CUDA(cudaMemcpyAsync(c->P.fixed, fx, sizeof(int) * np, cudaMemcpyHostToDevice, c->stream));
     DILBM_CUDA(cudaEventRecord(c->up_done, c->stream));
-    DILBM_CUDA(cudaMemsetAsync(c->bins[cur].count, 0, sizeof(int) * c->ntiles, c->stream));
+    DILBM_CUDA(cudaMemsetAsync(c->B.count + (size_t)c->rot * c->ntiles, 0, sizeof(int) * c->ntiles, c->stream));
     return launch_particles(c, 0);
 }
 
 template <typename T>
-SweepArgs<T> sweep_args(const dilbm_ctx *c, int cur, const void *src, void *dst, bool clear, FieldsOut fo) {
+SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     SweepArgs<T> a{};
-    a.src = (const T *)src;
-    a.dst = (T *)dst;
+    a.buf[0] = (T *)c->buf[0];
+    a.buf[1] = (T *)c->buf[1];
     a.L = c->L;
     a.ph = c->ph;
-    a.B = c->np > 0 ? c->bins[cur] : Bins{};     // no particles: no bins to read
+    a.B = c->B;
     a.partial = c->partial;
-    a.clear = (clear && c->np > 0) ? c->bins[cur ^ 1].count : nullptr;
     a.err = c->err;
-    a.fo = fo;
+    a.pa = c->np > 0 ? c->pa : nullptr;
+    a.np = c->np;
+    a.cur = c->cur;
+    a.rot = c->rot;
+    a.tag = c->tag;
+    a.ntx_inv = ntx_inverse(c->L.ntx);
     return a;
-}
-
-// The FIELDS-mode sweep (dilbm_fields) in the default shape.
-template <typename T, bool EDGES, bool PS>
-cudaError_t launch_fields_sweep_m(dilbm_ctx *c, const void *src, FieldsOut fo) {
-    static int cache[64] = {};
-    constexpr size_t smem = sweep_smem_bytes<T>();
-    int per_sm = 1;
-    cudaError_t e = occupancy_of(sweep_kernel<T, MODE_FIELDS, EDGES, SWEEP_WARPS, PS>, SWEEP_WARPS, smem, cache, &per_sm);
-    if (e != cudaSuccess) return e;
-    const long long blocks = persistent_grid((long long)c->L.ny * c->L.ntx, SWEEP_WARPS, per_sm, c->num_sms, SweepShape{});
-    sweep_kernel<T, MODE_FIELDS, EDGES, SWEEP_WARPS, PS><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, c->stream>>>(
-        sweep_args<T>(c, c->cur, src, nullptr, false, fo));
-    return cudaGetLastError();
-}
-
-template <typename T, bool EDGES>
-cudaError_t launch_fields_sweep(dilbm_ctx *c, const void *src, FieldsOut fo) {
-    return c->method == DILBM_METHOD_PS ? launch_fields_sweep_m<T, EDGES, true>(c, src, fo)
-                                        : launch_fields_sweep_m<T, EDGES, false>(c, src, fo);
 }
 
 bool has_edges(const dilbm_ctx *c) { return !(c->L.per_x && c->L.per_y); }
 
-// The step sweep of the current parity in shape `sh` (query: occupancy only).
-cudaError_t step_sweep(dilbm_ctx *c, const SweepShape &sh, bool query = false, int *per_sm = nullptr) {
-    const void *src = c->buf[c->cur];
-    void *dst = c->buf[c->cur ^ 1];
-    const bool edges = has_edges(c);
-    if (c->method == DILBM_METHOD_PS) {       // the comparison method: default shape only
-        if (query) {
-            if (per_sm) *per_sm = 1;
-            return cudaSuccess;
-        }
-        switch (c->storage) {
-        case DILBM_FP32:
-            return launch_step_sweep_ps<float>(sweep_args<float>(c, c->cur, src, dst, true, FieldsOut{}), edges,
-                                               c->num_sms, c->stream);
-        case DILBM_FP16_DEV:
-            return launch_step_sweep_ps<__half>(sweep_args<__half>(c, c->cur, src, dst, true, FieldsOut{}), edges,
-                                                c->num_sms, c->stream);
-        default:
-            return launch_step_sweep_ps<__nv_bfloat16>(
-                sweep_args<__nv_bfloat16>(c, c->cur, src, dst, true, FieldsOut{}), edges, c->num_sms, c->stream);
-        }
-    }
-    switch (c->storage) {
-    case DILBM_FP32:
-        return launch_step_sweep<float>(sweep_args<float>(c, c->cur, src, dst, true, FieldsOut{}), edges, sh,
-                                        c->num_sms, c->stream, query, per_sm);
-    case DILBM_FP16_DEV:
-        return launch_step_sweep<__half>(sweep_args<__half>(c, c->cur, src, dst, true, FieldsOut{}), edges, sh,
-                                         c->num_sms, c->stream, query, per_sm);
-    default:
-        return launch_step_sweep<__nv_bfloat16>(sweep_args<__nv_bfloat16>(c, c->cur, src, dst, true, FieldsOut{}),
-                                                edges, sh, c->num_sms, c->stream, query, per_sm);
+template <typename F>
+cudaError_t by_storage(int storage, F f) {
+    switch (storage) {
+    case DILBM_FP32: return f(float{});
+    case DILBM_FP16_DEV: return f(__half{});
+    default: return f(__nv_bfloat16{});
     }
 }
 
-template <int MODE>
-int launch_sweep(dilbm_ctx *c, const void *src, void *dst, FieldsOut fo) {
-    cudaError_t e;
-    if (MODE == MODE_STEP) {
-        (void)src;
-        (void)dst;
-        e = step_sweep(c, c->shape);
-    } else {
-        const bool edges = has_edges(c);
-        switch (c->storage) {
-        case DILBM_FP32: e = edges ? launch_fields_sweep<float, true>(c, src, fo) : launch_fields_sweep<float, false>(c, src, fo); break;
-        case DILBM_FP16_DEV: e = edges ? launch_fields_sweep<__half, true>(c, src, fo) : launch_fields_sweep<__half, false>(c, src, fo); break;
-        default: e = edges ? launch_fields_sweep<__nv_bfloat16, true>(c, src, fo) : launch_fields_sweep<__nv_bfloat16, false>(c, src, fo); break;
-        }
-    }
+// `run.nsteps` fused steps in shape `sh` (per_sm: occupancy only).
+cudaError_t fused_steps(dilbm_ctx *c, const SweepShape &sh, const StepRun &run, int *per_sm = nullptr) {
+    return by_storage(c->storage, [&](auto t) {
+        using T = decltype(t);
+        return Launch<T>::steps(sweep_args<T>(c), particle_args(c), run, has_edges(c), c->method == DILBM_METHOD_PS, sh, c->num_sms,
+                                c->stream, per_sm);
+    });
+}
+
+int launch_fields(dilbm_ctx *c, const FieldsOut &fo) {
+    const cudaError_t e = by_storage(c->storage, [&](auto t) {
+        using T = decltype(t);
+        return Launch<T>::fields(sweep_args<T>(c), fo, has_edges(c), c->method == DILBM_METHOD_PS, c->num_sms, c->stream);
+    });
     if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
     c->launches += 1;
     return DILBM_OK;
 }
 
-int one_step(dilbm_ctx *c) {
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (c->timing) {
-        if (c->ev_used + 2 > c->ev.size()) {
-            for (int k = 0; k < 64; ++k) {
-                cudaEvent_t e;
-                DILBM_CUDA(cudaEventCreate(&e));
-                c->ev.push_back(e);
-            }
-        }
-        e0 = c->ev[c->ev_used];
-        e1 = c->ev[c->ev_used + 1];
-        c->ev_used += 2;
-        DILBM_CUDA(cudaEventRecord(e0, c->stream));
-    }
-    int rc = launch_sweep<MODE_STEP>(c, c->buf[c->cur], c->buf[c->cur ^ 1], FieldsOut{});
-    if (rc) return rc;
-    if (c->timing) DILBM_CUDA(cudaEventRecord(e1, c->stream));
-    if (c->np > 0 && (rc = launch_particles(c, 1))) return rc;
-    if (c->track >= 0 && (rc = launch_frame_shift(c))) return rc;
-    c->cur ^= 1;
-    c->fsum_steps += 1;
+int launch_strip_sweep(dilbm_ctx *c) {
+    const cudaError_t e = by_storage(c->storage, [&](auto t) {
+        using T = decltype(t);
+        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, c->num_sms, c->stream);
+    });
+    if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
+    c->launches += 1;
     return DILBM_OK;
 }
 
-void drop_graphs(dilbm_ctx *c) {
-    for (int p = 0; p < 2; ++p)
-        if (c->g_pair[p]) {
-            cudaGraphExecDestroy(c->g_pair[p]);
-            c->g_pair[p] = nullptr;
-        }
+// The state the next step starts from, k steps on.
+void advance(dilbm_ctx *c, int k) {
+    c->cur ^= k & 1;
+    c->rot = (c->rot + k) % 3;
+    c->tag += (unsigned)k;
+    c->fsum_steps += k;
 }
 
-// Two steps starting at parity p, captured into a graph on the context's
-// stream (nothing runs while capturing).
-int capture_pair(dilbm_ctx *c, int p) {
-    if (c->g_pair[p]) return DILBM_OK;
-    const int cur = c->cur;
-    const long long l0 = c->launches, f0 = c->fsum_steps;
-    c->cur = p;
-    cudaGraph_t g = nullptr;
-    DILBM_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = one_step(c);
-    if (rc == DILBM_OK) rc = one_step(c);
-    const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
-    c->cur = cur;
-    c->launches = l0;
-    c->fsum_steps = f0;
-    if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
+// k steps in one launch (k == 1: no barrier, and the PS tables and the moving
+// frame's shift as launches of their own).
+int launch_fused(dilbm_ctx *c, int k) {
+    const cudaError_t e = fused_steps(c, c->shape, StepRun{k, 0, c->sync, 0});
+    if (e != cudaSuccess) return cuda_fail(e, "step_kernel launch");
+    c->launches += 1;
+    int rc;
+    if (c->method == DILBM_METHOD_PS && c->np > 0 && (rc = launch_cover(c, c->cur ^ 1))) return rc;
+    if (k == 1 && c->track >= 0 && (rc = launch_frame_shift(c))) return rc;
+    advance(c, k);
+    return DILBM_OK;
+}
+
+// Steps one launch may run: about 2^27 node updates (two milliseconds at the
+// rates of large lattices), so that work on other streams never waits long
+// behind a launch that holds the SMs, and the gap between launches stays
+// below a thousandth of its time.
+int steps_per_launch(double nodes) {
+    const double k = 134217728.0 / nodes;
+    return k < 1.0 ? 1 : (k > 1024.0 ? 1024 : (int)k);
+}
+
+// A pair of events around a launch, for dilbm_sweep_time.
+int timing_pair(std::vector<cudaEvent_t> &ev, size_t &used, cudaEvent_t *e0, cudaEvent_t *e1) {
+    if (used + 2 > ev.size()) {
+        for (int k = 0; k < 64; ++k) {
+            cudaEvent_t e;
+            DILBM_CUDA(cudaEventCreate(&e));
+            ev.push_back(e);
+        }
     }
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-    const cudaError_t e2 = cudaGraphInstantiate(&c->g_pair[p], g, 0);
-    cudaGraphDestroy(g);
-    if (e2 != cudaSuccess) {
-        c->g_pair[p] = nullptr;
-        return cuda_fail(e2, "cudaGraphInstantiate");
-    }
+    *e0 = ev[used];
+    *e1 = ev[used + 1];
+    used += 2;
+    return DILBM_OK;
+}
+
+// One step, its launch bracketed by events.
+int timed_step(dilbm_ctx *c) {
+    cudaEvent_t e0, e1;
+    int rc = timing_pair(c->ev, c->ev_used, &e0, &e1);
+    if (rc) return rc;
+    DILBM_CUDA(cudaEventRecord(e0, c->stream));
+    const cudaError_t e = fused_steps(c, c->shape, StepRun{1, 0, c->sync, 0});
+    if (e != cudaSuccess) return cuda_fail(e, "step_kernel launch");
+    DILBM_CUDA(cudaEventRecord(e1, c->stream));
+    c->launches += 1;
+    if (c->method == DILBM_METHOD_PS && c->np > 0 && (rc = launch_cover(c, c->cur ^ 1))) return rc;
+    if (c->track >= 0 && (rc = launch_frame_shift(c))) return rc;
+    advance(c, 1);
     return DILBM_OK;
 }
 
@@ -625,6 +597,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     c->np = np;
     c->storage = g->storage;
     c->method = g->method;
+    if (c->method == DILBM_METHOD_PS) c->shape = PS_SHAPE;
     c->elem = g->storage == DILBM_FP32 ? 4 : 2;
     Lattice &L = c->L;
     L.nx = g->nx;
@@ -701,6 +674,9 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     bp.eps_w = g->wan_turek[2];
     bp.eps_w2 = g->wan_turek[3];
     bp.xi = g->wan_turek[4];
+    bp.xi_f = (float)bp.xi;
+    bp.len[0] = g->nx;
+    bp.len[1] = g->ny;
 
     auto bail = [&](int code) { dilbm_destroy(c); return code; };
     {
@@ -724,22 +700,25 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     const int npa = np > 0 ? np : 1;
     double *pd = nullptr;
     float *pf = nullptr;
-    if ((rc = dev_alloc(c, &pd, 10 * (size_t)npa)) || (rc = dev_alloc(c, &pf, 4 * (size_t)npa)) ||
+    if ((rc = dev_alloc(c, &pd, 15 * (size_t)npa)) || (rc = dev_alloc(c, &pf, 5 * (size_t)npa)) ||
         (rc = dev_alloc(c, &c->P.fixed, (size_t)npa)) || (rc = dev_alloc(c, &c->force, 3 * (size_t)npa)) ||
         (rc = dev_alloc(c, &c->fsum, 3 * (size_t)npa)) || (rc = dev_alloc(c, &c->fcol, 2 * (size_t)npa)) ||
         (rc = dev_alloc(c, &c->err, 1)) ||
-        (rc = dev_alloc(c, &c->partial, (size_t)c->ntiles * MAXC * TILE_H)))
+        (rc = dev_alloc(c, &c->partial, (size_t)npa * MAXT * TILE_H)) || (rc = dev_alloc(c, &c->pa, 1)) ||
+        (rc = dev_alloc(c, &c->sync, 1)))
         return bail(rc);
-    for (int b = 0; b < 2; ++b) {
-        Bins &B = c->bins[b];
-        if ((rc = dev_alloc(c, &B.count, (size_t)c->ntiles)) || (rc = dev_alloc(c, &B.ids, (size_t)c->ntiles * MAXC)) ||
-            (rc = dev_alloc(c, &B.rec, (size_t)c->ntiles * MAXC * NREC)) ||
-            (rc = dev_alloc(c, &B.pslot, (size_t)npa * MAXT)) || (rc = dev_alloc(c, &B.npslot, (size_t)npa)))
-            return bail(rc);
-    }
+    BinSet &B = c->B;
+    B.tiles = c->ntiles;
+    B.parts = npa;
+    if ((rc = dev_alloc(c, &B.count, 3 * (size_t)c->ntiles)) || (rc = dev_alloc(c, &B.ids, 2 * (size_t)c->ntiles * MAXC)) ||
+        (rc = dev_alloc(c, &B.rec, 2 * (size_t)c->ntiles * MAXC * NREC)) ||
+        (rc = dev_alloc(c, &B.pslot, 2 * (size_t)npa * MAXT)) || (rc = dev_alloc(c, &B.npslot, 2 * (size_t)npa)) ||
+        (rc = dev_alloc(c, &B.done, 2 * (size_t)npa)))
+        return bail(rc);
     c->P.x[0] = pd; c->P.x[1] = pd + npa; c->P.y[0] = pd + 2 * npa; c->P.y[1] = pd + 3 * npa;
     c->P.r = pd + 4 * npa; c->P.ux = pd + 5 * npa; c->P.uy = pd + 6 * npa; c->P.omega = pd + 7 * npa;
-    c->P.theta = pd + 8 * npa; c->P.rho_s = pd + 9 * npa;
+    c->P.theta = pd + 8 * npa; c->P.rho_s = pd + 9 * npa; c->P.im = pd + 10 * npa; c->P.iI = pd + 11 * npa;
+    c->P.wx = pd + 12 * npa; c->P.wy = pd + 13 * npa; c->P.reach = pd + 14 * npa; c->P.rf = pf + 4 * npa;
     c->P.xf[0] = pf; c->P.xf[1] = pf + npa; c->P.yf[0] = pf + 2 * npa; c->P.yf[1] = pf + 3 * npa;
     if (c->strip) {
         // exchange buffers: 9 plane rows each, GUARD readable elements around
@@ -762,8 +741,10 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         (e = cudaMemsetAsync(c->force, 0, sizeof(double) * 3 * npa, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->fsum, 0, sizeof(double) * 3 * npa, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->fcol, 0, sizeof(double) * 2 * npa, c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->bins[0].count, 0, sizeof(int) * c->ntiles, c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->bins[1].count, 0, sizeof(int) * c->ntiles, c->stream)) != cudaSuccess)
+        (e = cudaMemsetAsync(c->sync, 0, sizeof(GridSync), c->stream)) != cudaSuccess ||
+        // (no partial carries the tag of a step to come)
+        (e = cudaMemsetAsync(c->partial, 0xff, sizeof(float4) * MAXT * TILE_H * npa, c->stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * c->ntiles, c->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMemsetAsync"));
     // uniform initial state f^eq(rho_init, u0)
     const int blocks = 152 * 8;
@@ -788,7 +769,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         if ((e = cudaGetLastError()) != cudaSuccess) return bail(cuda_fail(e, "init_kernel"));
         c->launches += 1;
     }
-    if (np > 0 && (rc = upload_particles(c, particles, np))) return bail(rc);
+    if ((rc = push_part_args(c)) || (np > 0 && (rc = upload_particles(c, particles, np)))) return bail(rc);
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return bail(cuda_fail(e, "cudaStreamSynchronize"));
     *out = c;
     return DILBM_OK;
@@ -828,7 +809,7 @@ int dilbm_create_strip(const dilbm_grid *g, dilbm_lattice lattice, double tau, d
 int dilbm_strip_begin(dilbm_ctx *c) {
     const dilbm::TraceRange trace("dilbm_strip_begin");
     if (!c || !c->strip || c->strip_open) return fail(DILBM_ERR_INVALID_ARG, "not a strip, or a step already begun");
-    int rc = launch_sweep<MODE_STEP>(c, c->buf[c->cur], c->buf[c->cur ^ 1], FieldsOut{});
+    int rc = launch_strip_sweep(c);
     if (rc) return rc;
     if (c->np > 0 && (rc = launch_particles(c, 1, 1))) return rc;
     // this strip's first and last rows of every plane, for the neighbours
@@ -846,8 +827,7 @@ int dilbm_strip_end(dilbm_ctx *c) {
     if (!c || !c->strip || !c->strip_open) return fail(DILBM_ERR_INVALID_ARG, "not a strip, or no step begun");
     int rc;
     if (c->np > 0 && (rc = launch_particles(c, 1, 2))) return rc;
-    c->cur ^= 1;
-    c->fsum_steps += 1;
+    advance(c, 1);
     c->strip_open = false;
     return DILBM_OK;
 }
@@ -868,25 +848,20 @@ int dilbm_step(dilbm_ctx *c, long long nsteps) {
     const dilbm::TraceRange trace("dilbm_step");
     if (!c || nsteps < 0) return fail(DILBM_ERR_INVALID_ARG, "bad context or step count");
     if (c->strip) return fail(DILBM_ERR_INVALID_ARG, "a strip steps through dilbm_strip_begin / dilbm_strip_end");
-    // whole step pairs replay a captured graph (timing brackets every sweep
-    // launch with events instead; a stream the caller is capturing gets the
-    // launches themselves)
-    bool graphs = !c->timing && nsteps >= 2 && c->stream != nullptr && c->stream != cudaStreamLegacy;
-    if (graphs) {
+    // several steps per launch; one per launch where timing brackets each
+    // step, the PS tables follow each step (made by the particle warps, a
+    // table took 20 us and the step 283 us instead of 237), or the caller is
+    // capturing the stream
+    long long most = c->method == DILBM_METHOD_PS ? 1 : steps_per_launch((double)c->L.nx * c->L.ny);
+    if (most > 1 && nsteps > 1 && c->stream != nullptr && c->stream != cudaStreamLegacy) {
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        graphs = cudaStreamIsCapturing(c->stream, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) most = 1;
     }
-    long long t = 0;
-    if (graphs) {
-        int rc = capture_pair(c, c->cur);
+    for (long long t = 0; t < nsteps;) {
+        const int k = (int)std::min(most, nsteps - t);
+        const int rc = c->timing ? timed_step(c) : launch_fused(c, k);
         if (rc) return rc;
-        for (; t + 2 <= nsteps; t += 2) DILBM_CUDA(cudaGraphLaunch(c->g_pair[c->cur], c->stream));
-        c->launches += t * ((c->np > 0 ? (c->method == DILBM_METHOD_PS ? 3 : 2) : 1) + (c->track >= 0 ? 1 : 0));
-        c->fsum_steps += t;
-    }
-    for (; t < nsteps; ++t) {
-        int rc = one_step(c);
-        if (rc) return rc;
+        t += c->timing ? 1 : k;
     }
     return DILBM_OK;
 }
@@ -968,8 +943,7 @@ int dilbm_set_moving_frame(dilbm_ctx *c, int particle, double x_ref) {
     }
     c->track = particle;
     c->track_x = particle >= 0 ? x_ref : 0.0;
-    drop_graphs(c);
-    return DILBM_OK;
+    return push_part_args(c);
 }
 
 int dilbm_frame_offset(dilbm_ctx *c, long long *offset) {
@@ -1017,7 +991,7 @@ int dilbm_fields(dilbm_ctx *c, float *rho, float *ux, float *uy, float *phi, int
     FieldsOut fo{};
     if (on_device) {
         fo = FieldsOut{rho, ux, uy, phi};
-        return launch_sweep<MODE_FIELDS>(c, c->buf[c->cur], nullptr, fo);
+        return launch_fields(c, fo);
     }
     if (!c->fields) {
         void *q = nullptr;
@@ -1026,7 +1000,7 @@ int dilbm_fields(dilbm_ctx *c, float *rho, float *ux, float *uy, float *phi, int
         c->fields = (float *)q;
     }
     fo = FieldsOut{c->fields, c->fields + n, c->fields + 2 * n, c->fields + 3 * n};
-    int rc = launch_sweep<MODE_FIELDS>(c, c->buf[c->cur], nullptr, fo);
+    int rc = launch_fields(c, fo);
     if (rc) return rc;
     float *dst[4] = {rho, ux, uy, phi};
     for (int k = 0; k < 4; ++k)
@@ -1093,9 +1067,8 @@ int dilbm_set_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
 void dilbm_destroy(dilbm_ctx *c) {
     if (!c) return;
     cudaStreamSynchronize(c->stream);
-    drop_graphs(c);
     for (int k = 0; k < c->nowned; ++k) cudaFree(c->owned[k]);
-    if (c->cover) cudaFree(c->cover);
+    if (c->B.cover) cudaFree(c->B.cover);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     if (c->up_done) cudaEventDestroy(c->up_done);
     if (c->up_stage) cudaFreeHost(c->up_stage);
@@ -1137,26 +1110,22 @@ int dilbm_footprint(const dilbm_grid *g, int np, unsigned long long *bytes) {
 }  // extern "C"
 
 // ---------------------------------------------------------------- batches
-// Many lattices advanced together: one sweep launch over the concatenated row
-// segments of every member and one particle launch over all their particles
-// per step, replayed from CUDA graphs.
+// Many lattices advanced together: the fused steps over the concatenated row
+// segments and particles of every member, several steps per launch.
 struct dilbm_batch {
     std::vector<dilbm_ctx *> members;
-    std::vector<int> cur0;              // members' parity when the launches were captured
     int storage = DILBM_FP32;
-    long long done = 0;                 // batch steps since the capture
-    cudaStream_t stream = nullptr;      // private stream the graphs run on
+    cudaStream_t stream = nullptr;      // private stream the batch runs on
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     std::vector<cudaStream_t> member_streams;
-    std::vector<void *> sweep_params[2];   // BatchArgs<T> per launch group, per phase (host copies)
-    PartArgs *part_args[2] = {nullptr, nullptr};
-    int *part_start = nullptr;          // n + 1
+    std::vector<void *> groups;         // BatchArgs<T> per launch group (host)
+    std::vector<GridSync *> sync;       // and its barrier (device)
     int *const *err_ptrs = nullptr;     // device: every member's error word
     int *err_out = nullptr;             // device: their values, gathered for one copy
     std::vector<int> err_host;
     int nparts = 0;
+    double nodes = 0.0;
     SweepShape shape{};                 // launch shape of the batched sweep
-    cudaGraphExec_t g_pair = nullptr, g_single[2] = {nullptr, nullptr};
     bool timing = false;
     std::vector<cudaEvent_t> ev;
     size_t ev_used = 0;
@@ -1173,138 +1142,40 @@ __global__ void gather_errors_kernel(int *const *__restrict__ err, int n, int *_
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) out[k] = *err[k];
 }
 
-void free_sweep_params(dilbm_batch *b) {
-    for (int phase = 0; phase < 2; ++phase) {
-        for (void *q : b->sweep_params[phase]) std::free(q);
-        b->sweep_params[phase].clear();
-    }
-}
-
-// Host copies of the batched sweep's parameters: members in groups of at
-// most BATCH_LAUNCH_MAX, both phases (the second step of a pair runs every
-// member at the other parity).
+// The launch arguments from the members' present state: members in groups of
+// at most BATCH_LAUNCH_MAX.
 template <typename T>
-void build_sweep_params(dilbm_batch *b) {
-    free_sweep_params(b);
+void fill_groups(dilbm_batch *b) {
     const int n = (int)b->members.size();
-    for (int g0 = 0; g0 < n; g0 += BATCH_LAUNCH_MAX) {
-        const int gn = n - g0 < BATCH_LAUNCH_MAX ? n - g0 : BATCH_LAUNCH_MAX;
-        for (int phase = 0; phase < 2; ++phase) {
-            BatchArgs<T> *ba = static_cast<BatchArgs<T> *>(std::calloc(1, sizeof(BatchArgs<T>)));
-            ba->n = gn;
-            ba->item_start[0] = ba->tile_start[0] = 0;
-            for (int k = 0; k < gn; ++k) {
-                const dilbm_ctx *c = b->members[g0 + k];
-                const int cur = b->cur0[g0 + k] ^ phase;
-                ba->a[k] = sweep_args<T>(c, cur, c->buf[cur], c->buf[cur ^ 1], true, FieldsOut{});
-                ba->item_start[k + 1] = ba->item_start[k] + c->L.ny * c->L.ntx;
-                ba->tile_start[k + 1] = ba->tile_start[k] + c->L.ntx * c->L.nty;
-            }
-            b->sweep_params[phase].push_back(ba);
+    for (int g0 = 0, g = 0; g0 < n; g0 += BATCH_LAUNCH_MAX, ++g) {
+        BatchArgs<T> &ba = *static_cast<BatchArgs<T> *>(b->groups[g]);
+        ba.n = n - g0 < BATCH_LAUNCH_MAX ? n - g0 : BATCH_LAUNCH_MAX;
+        for (int k = 0; k < ba.n; ++k) {
+            const dilbm_ctx *c = b->members[g0 + k];
+            ba.a[k] = sweep_args<T>(c);
+            ba.item_start[k + 1] = ba.item_start[k] + c->L.ny * c->L.ntx;
+            ba.tile_start[k + 1] = ba.tile_start[k] + c->L.ntx * c->L.nty;
+            ba.part_start[k + 1] = ba.part_start[k] + c->np;
         }
     }
 }
 
-int upload_part_args(dilbm_batch *b) {
-    const size_t n = b->members.size();
-    for (int phase = 0; phase < 2; ++phase) {
-        std::vector<PartArgs> pa(n);
-        for (size_t k = 0; k < n; ++k) pa[k] = particle_args(b->members[k], b->cur0[k] ^ phase, 1);
-        DILBM_CUDA(cudaMemcpyAsync(b->part_args[phase], pa.data(), sizeof(PartArgs) * n, cudaMemcpyHostToDevice, b->stream));
-        DILBM_CUDA(cudaStreamSynchronize(b->stream));
-    }
-    return DILBM_OK;
+// `nsteps` fused steps of every group in shape `sh`.
+cudaError_t batch_groups(dilbm_batch *b, const SweepShape &sh, int nsteps, int dry) {
+    return by_storage(b->storage, [&](auto t) {
+        using T = decltype(t);
+        fill_groups<T>(b);
+        for (size_t g = 0; g < b->groups.size(); ++g) {
+            const cudaError_t e = Launch<T>::batch(*static_cast<const BatchArgs<T> *>(b->groups[g]),
+                                                   StepRun{nsteps, dry, b->sync[g], 0}, sh, b->members[0]->num_sms, b->stream);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
+    });
 }
 
-template <typename T>
-cudaError_t batch_sweep_groups(dilbm_batch *b, int phase, const SweepShape &sh) {
-    const int num_sms = b->members[0]->num_sms;
-    for (size_t g = 0; g < b->sweep_params[phase].size(); ++g) {
-        const BatchArgs<T> &ba = *static_cast<const BatchArgs<T> *>(b->sweep_params[phase][g]);
-        cudaError_t e = launch_batch_sweep<T>(ba, sh, num_sms, b->stream);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
-// Every launch group of the batched sweep at `phase` in shape `sh`.
-cudaError_t batch_sweep(dilbm_batch *b, int phase, const SweepShape &sh) {
-    if (b->storage == DILBM_FP32) return batch_sweep_groups<float>(b, phase, sh);
-    if (b->storage == DILBM_FP16_DEV) return batch_sweep_groups<__half>(b, phase, sh);
-    return batch_sweep_groups<__nv_bfloat16>(b, phase, sh);
-}
-
-// One batch step at `phase`: the sweep over every member, then the particles.
-int batch_phase(dilbm_batch *b, int phase) {
-    cudaEvent_t e0 = nullptr, e1 = nullptr;
-    if (b->timing) {
-        if (b->ev_used + 2 > b->ev.size())
-            for (int k = 0; k < 64; ++k) {
-                cudaEvent_t e;
-                DILBM_CUDA(cudaEventCreate(&e));
-                b->ev.push_back(e);
-            }
-        e0 = b->ev[b->ev_used];
-        e1 = b->ev[b->ev_used + 1];
-        b->ev_used += 2;
-        DILBM_CUDA(cudaEventRecord(e0, b->stream));
-    }
-    cudaError_t e = batch_sweep(b, phase, b->shape);
-    if (e != cudaSuccess) return cuda_fail(e, "batched sweep_kernel launch");
-    if (b->timing) DILBM_CUDA(cudaEventRecord(e1, b->stream));
-    b->launches += (long long)b->sweep_params[phase].size();
-    if (b->nparts > 0) {
-        BatchIndex pi{b->part_start, nullptr, (int)b->members.size()};
-        particles_kernel<true><<<(b->nparts + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, b->stream>>>(PartArgs{}, b->part_args[phase], pi);
-        DILBM_CUDA(cudaGetLastError());
-        b->launches += 1;
-    }
-    return DILBM_OK;
-}
-
-int capture(dilbm_batch *b, int first_phase, int nphases, cudaGraphExec_t *out) {
-    if (*out) {
-        cudaGraphExecDestroy(*out);
-        *out = nullptr;
-    }
-    cudaGraph_t g = nullptr;
-    const long long l0 = b->launches;
-    DILBM_CUDA(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-    int rc = DILBM_OK;
-    for (int k = 0; k < nphases && rc == DILBM_OK; ++k) rc = batch_phase(b, (first_phase + k) & 1);
-    cudaError_t e = cudaStreamEndCapture(b->stream, &g);
-    b->launches = l0;    // capturing launches nothing
-    if (rc) {
-        if (g) cudaGraphDestroy(g);
-        return rc;
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-    e = cudaGraphInstantiate(out, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-    return DILBM_OK;
-}
-
-// (Re)build every launch of the batch from the members' current parity:
-// sweep parameters, particle descriptors and the three graphs.
-int prepare_batch(dilbm_batch *b) {
-    for (size_t k = 0; k < b->members.size(); ++k) b->cur0[k] = b->members[k]->cur;
-    b->done = 0;
-    if (b->storage == DILBM_FP32) build_sweep_params<float>(b);
-    else if (b->storage == DILBM_FP16_DEV) build_sweep_params<__half>(b);
-    else build_sweep_params<__nv_bfloat16>(b);
-    int rc;
-    if ((rc = upload_part_args(b))) return rc;
-    if ((rc = capture(b, 0, 2, &b->g_pair)) || (rc = capture(b, 0, 1, &b->g_single[0])) ||
-        (rc = capture(b, 1, 1, &b->g_single[1])))
-        return rc;
-    return DILBM_OK;
-}
-
-// Kernels launched by one batch step (sweep groups + particles).
-int batch_launches_per_step(const dilbm_batch *b) {
-    return (int)b->sweep_params[0].size() + (b->nparts > 0 ? 1 : 0);
-}
+// Sweep and particle passes of one batch step.
+int batch_passes_per_step(const dilbm_batch *b) { return (int)b->groups.size() + (b->nparts > 0 ? 1 : 0); }
 
 }  // namespace
 
@@ -1331,7 +1202,6 @@ int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilb
     dilbm_batch *b = new dilbm_batch();
     auto bail = [&](int code) { dilbm_batch_destroy(b); return code; };
     b->members.assign(members, members + n);
-    b->cur0.resize(n);
     b->storage = members[0]->storage;
     cudaError_t e;
     if ((e = cudaStreamCreateWithFlags(&b->stream, cudaStreamNonBlocking)) != cudaSuccess ||
@@ -1343,16 +1213,21 @@ int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilb
         for (cudaStream_t s : b->member_streams) seen |= s == members[k]->stream;
         if (!seen) b->member_streams.push_back(members[k]->stream);
     }
-    // particles of each member, in one list
-    std::vector<int> ps(n + 1, 0);
-    for (int k = 0; k < n; ++k) ps[k + 1] = ps[k] + members[k]->np;
-    b->nparts = ps[n];
-    for (int phase = 0; phase < 2; ++phase)
-        if ((e = cudaMalloc((void **)&b->part_args[phase], sizeof(PartArgs) * n)) != cudaSuccess)
-            return bail(cuda_fail(e, "cudaMalloc batch descriptors"));
-    if ((e = cudaMalloc((void **)&b->part_start, sizeof(int) * (n + 1))) != cudaSuccess ||
-        (e = cudaMemcpy(b->part_start, ps.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice)) != cudaSuccess)
-        return bail(cuda_fail(e, "batch particle list"));
+    for (int k = 0; k < n; ++k) {
+        b->nparts += members[k]->np;
+        b->nodes += (double)members[k]->L.nx * members[k]->L.ny;
+    }
+    for (int g0 = 0; g0 < n; g0 += BATCH_LAUNCH_MAX) {
+        const size_t bytes = b->storage == DILBM_FP32 ? sizeof(BatchArgs<float>) : sizeof(BatchArgs<__half>);
+        void *ba = std::calloc(1, bytes);
+        if (!ba) return bail(fail(DILBM_ERR_OOM, "batch launch arguments"));
+        b->groups.push_back(ba);
+        GridSync *q = nullptr;
+        if ((e = cudaMalloc((void **)&q, sizeof(GridSync))) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc batch barrier"));
+        b->sync.push_back(q);
+        if ((e = cudaMemsetAsync(q, 0, sizeof(GridSync), b->stream)) != cudaSuccess)
+            return bail(cuda_fail(e, "cudaMemsetAsync"));
+    }
     {
         std::vector<int *> ep(n);
         for (int k = 0; k < n; ++k) ep[k] = members[k]->err;
@@ -1364,13 +1239,6 @@ int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilb
             return bail(cuda_fail(e, "batch error words"));
         b->err_host.assign(n, 0);
     }
-    // order after every member's queued work, then build the launches
-    for (cudaStream_t s : b->member_streams) {
-        if ((e = cudaEventRecord(b->ev_in, s)) != cudaSuccess || (e = cudaStreamWaitEvent(b->stream, b->ev_in, 0)) != cudaSuccess)
-            return bail(cuda_fail(e, "batch stream ordering"));
-    }
-    int rc;
-    if ((rc = prepare_batch(b))) return bail(rc);
     *out = b;
     return DILBM_OK;
 }
@@ -1380,37 +1248,23 @@ int dilbm_batch_step(dilbm_batch *b, long long nsteps) {
     if (!b || nsteps < 0) return fail(DILBM_ERR_INVALID_ARG, "bad batch or step count");
     if (nsteps == 0) return DILBM_OK;
     cudaError_t e;
-    // a member stepped on its own since the descriptors were built: rebuild
-    bool stale = false;
-    for (size_t k = 0; k < b->members.size(); ++k)
-        stale |= b->members[k]->cur != (b->cur0[k] ^ (int)(b->done & 1));
     for (cudaStream_t s : b->member_streams) {
         if ((e = cudaEventRecord(b->ev_in, s)) != cudaSuccess || (e = cudaStreamWaitEvent(b->stream, b->ev_in, 0)) != cudaSuccess)
             return cuda_fail(e, "batch stream ordering");
     }
-    int rc;
-    if (stale && (rc = prepare_batch(b))) return rc;
-    long long left = nsteps;
-    if (b->timing) {
-        for (; left > 0; --left, ++b->done)
-            if ((rc = batch_phase(b, (int)(b->done & 1)))) return rc;
-    } else {
-        if (b->done & 1) {                       // finish the pair in progress
-            DILBM_CUDA(cudaGraphLaunch(b->g_single[1], b->stream));
-            ++b->done;
-            --left;
+    const long long most = b->timing ? 1 : steps_per_launch(b->nodes);
+    for (long long t = 0; t < nsteps;) {
+        const int k = (int)std::min(most, nsteps - t);
+        cudaEvent_t e0 = nullptr, e1 = nullptr;
+        if (b->timing) {
+            if (int rc = timing_pair(b->ev, b->ev_used, &e0, &e1)) return rc;
+            DILBM_CUDA(cudaEventRecord(e0, b->stream));
         }
-        for (; left >= 2; left -= 2, b->done += 2) DILBM_CUDA(cudaGraphLaunch(b->g_pair, b->stream));
-        if (left == 1) {
-            DILBM_CUDA(cudaGraphLaunch(b->g_single[0], b->stream));
-            ++b->done;
-        }
-        b->launches += nsteps * batch_launches_per_step(b);
-    }
-    for (size_t k = 0; k < b->members.size(); ++k) {
-        dilbm_ctx *c = b->members[k];
-        c->cur = b->cur0[k] ^ (int)(b->done & 1);
-        c->fsum_steps += nsteps;
+        if ((e = batch_groups(b, b->shape, k, 0)) != cudaSuccess) return cuda_fail(e, "step_batch_kernel launch");
+        if (b->timing) DILBM_CUDA(cudaEventRecord(e1, b->stream));
+        b->launches += (long long)k * batch_passes_per_step(b);
+        for (dilbm_ctx *c : b->members) advance(c, k);
+        t += k;
     }
     // members' own streams see the batch's work before anything queued later
     DILBM_CUDA(cudaEventRecord(b->ev_out, b->stream));
@@ -1474,13 +1328,8 @@ long long dilbm_batch_launch_count(const dilbm_batch *b) { return b ? b->launche
 void dilbm_batch_destroy(dilbm_batch *b) {
     if (!b) return;
     if (b->stream) cudaStreamSynchronize(b->stream);
-    if (b->g_pair) cudaGraphExecDestroy(b->g_pair);
-    for (int k = 0; k < 2; ++k) {
-        if (b->g_single[k]) cudaGraphExecDestroy(b->g_single[k]);
-        cudaFree(b->part_args[k]);
-    }
-    free_sweep_params(b);
-    cudaFree(b->part_start);
+    for (void *q : b->groups) std::free(q);
+    for (GridSync *q : b->sync) cudaFree(q);
     cudaFree((void *)b->err_ptrs);
     cudaFree(b->err_out);
     for (cudaEvent_t e : b->ev) cudaEventDestroy(e);
@@ -1605,13 +1454,9 @@ extern "C" {
 int dilbm_set_shape(dilbm_ctx *c, int warps, int blocks_per_sm) {
     const SweepShape sh{warps, blocks_per_sm};
     if (!c || !shape_valid(sh)) return fail(DILBM_ERR_INVALID_ARG, "warps must be 2, 4 or 8 and blocks_per_sm >= 0");
-    if (c->method == DILBM_METHOD_PS && !same_shape(sh, SweepShape{}))
+    if (c->method == DILBM_METHOD_PS && !same_shape(sh, PS_SHAPE))
         return fail(DILBM_ERR_INVALID_ARG, "a PS-LBM context runs the sweep in the default shape (8 warps, 0)");
-    if (!same_shape(sh, c->shape)) {
-        DILBM_CUDA(cudaStreamSynchronize(c->stream));
-        drop_graphs(c);
-        c->shape = sh;
-    }
+    c->shape = sh;
     return DILBM_OK;
 }
 
@@ -1628,12 +1473,13 @@ int dilbm_autotune(dilbm_ctx *c, int reps, int *warps, int *blocks_per_sm) {
     if (!tuned(key, &best)) {
         std::vector<SweepShape> cands;
         std::vector<int> wps;
-        int rc = shape_candidates([&](const SweepShape &sh, int *per_sm) { return step_sweep(c, sh, true, per_sm); },
+        int rc = shape_candidates([&](const SweepShape &sh, int *per_sm) { return fused_steps(c, sh, StepRun{}, per_sm); },
                                   &cands, &wps);
         if (rc) return rc;
-        // each launch sweeps the current state into the other buffer: what
-        // the next step writes anyway
-        rc = time_shapes(c->stream, reps, cands, wps, [&](const SweepShape &sh) { return step_sweep(c, sh); }, &best);
+        // each launch sweeps the current state into the other buffer (what
+        // the next step writes anyway) and updates no particle
+        rc = time_shapes(c->stream, reps, cands, wps,
+                         [&](const SweepShape &sh) { return fused_steps(c, sh, StepRun{1, 1, c->sync, 0}); }, &best);
         c->launches += (long long)cands.size() * (reps + 1) * TUNE_ROUNDS;
         if (rc) return rc;
         remember(key, best);
@@ -1645,10 +1491,8 @@ int dilbm_autotune(dilbm_ctx *c, int reps, int *warps, int *blocks_per_sm) {
 int dilbm_batch_set_shape(dilbm_batch *b, int warps, int blocks_per_sm) {
     const SweepShape sh{warps, blocks_per_sm};
     if (!b || !shape_valid(sh)) return fail(DILBM_ERR_INVALID_ARG, "warps must be 2, 4 or 8 and blocks_per_sm >= 0");
-    if (same_shape(sh, b->shape)) return DILBM_OK;
-    DILBM_CUDA(cudaStreamSynchronize(b->stream));
     b->shape = sh;
-    return prepare_batch(b);     // re-capture the graphs in the new shape
+    return DILBM_OK;
 }
 
 int dilbm_batch_autotune(dilbm_batch *b, int reps, int *warps, int *blocks_per_sm) {
@@ -1661,30 +1505,23 @@ int dilbm_batch_autotune(dilbm_batch *b, int reps, int *warps, int *blocks_per_s
     SweepShape best = b->shape;
     if (!tuned(key, &best)) {
         cudaError_t e;
-        // order after the members' queued work; bring the launches up to date
+        // order after the members' queued work
         for (cudaStream_t s : b->member_streams)
             if ((e = cudaEventRecord(b->ev_in, s)) != cudaSuccess || (e = cudaStreamWaitEvent(b->stream, b->ev_in, 0)) != cudaSuccess)
                 return cuda_fail(e, "batch stream ordering");
-        bool stale = false;
-        for (size_t k = 0; k < b->members.size(); ++k)
-            stale |= b->members[k]->cur != (b->cur0[k] ^ (int)(b->done & 1));
-        int rc;
-        if (stale && (rc = prepare_batch(b))) return rc;
-        const int phase = (int)(b->done & 1);
         std::vector<SweepShape> cands;
         std::vector<int> wps;
-        rc = shape_candidates(
+        int rc = shape_candidates(
             [&](const SweepShape &sh, int *per_sm) {
-                switch (b->storage) {
-                case DILBM_FP32: return launch_batch_sweep<float>(*static_cast<const BatchArgs<float> *>(b->sweep_params[0][0]), sh, 1, b->stream, true, per_sm);
-                case DILBM_FP16_DEV: return launch_batch_sweep<__half>(*static_cast<const BatchArgs<__half> *>(b->sweep_params[0][0]), sh, 1, b->stream, true, per_sm);
-                default: return launch_batch_sweep<__nv_bfloat16>(*static_cast<const BatchArgs<__nv_bfloat16> *>(b->sweep_params[0][0]), sh, 1, b->stream, true, per_sm);
-                }
+                return by_storage(b->storage, [&](auto t) {
+                    using T = decltype(t);
+                    return Launch<T>::batch(*static_cast<const BatchArgs<T> *>(b->groups[0]), StepRun{}, sh, 1, b->stream, per_sm);
+                });
             },
             &cands, &wps);
         if (rc) return rc;
-        rc = time_shapes(b->stream, reps, cands, wps, [&](const SweepShape &sh) { return batch_sweep(b, phase, sh); }, &best);
-        b->launches += (long long)cands.size() * (reps + 1) * TUNE_ROUNDS * (long long)b->sweep_params[phase].size();
+        rc = time_shapes(b->stream, reps, cands, wps, [&](const SweepShape &sh) { return batch_groups(b, sh, 1, 1); }, &best);
+        b->launches += (long long)cands.size() * (reps + 1) * TUNE_ROUNDS * (long long)b->groups.size();
         if (rc) return rc;
         remember(key, best);
         if ((e = cudaEventRecord(b->ev_out, b->stream)) != cudaSuccess) return cuda_fail(e, "cudaEventRecord");

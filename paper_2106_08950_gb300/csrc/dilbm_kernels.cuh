@@ -1,16 +1,17 @@
 // Device code of the DI-LBM step on sm_103a.
 //
-// One time step (the paper's procedure, Sec. 2.3) is two kernels:
-//   sweep_kernel     -- every node: pull-stream, edge extrapolation, solid
-//                       fraction (Eq. 14), corrected velocity (Eq. 17),
-//                       collision with the force term (Eqs. 13, 15), and the
-//                       node's share of force/torque (Eqs. 18-19) summed per
-//                       row segment and nearby particle;
-//   particles_kernel -- one warp per particle: fixed-order FP64 sum of its
-//                       partials (Eqs. 18-19), Wan-Turek repulsion (Eqs.
-//                       28-29), Newton-Euler update (Eqs. 22-24), then binning
-//                       of the particle into the lattice tiles its phi tail
-//                       reaches, for the next sweep.
+// One time step (the paper's procedure, Sec. 2.3) is two kinds of work, which
+// run side by side in one launch over many steps (run_steps):
+//   the sweep     -- every node: pull-stream, edge extrapolation, solid
+//                    fraction (Eq. 14), corrected velocity (Eq. 17),
+//                    collision with the force term (Eqs. 13, 15), and the
+//                    node's share of force/torque (Eqs. 18-19) summed per
+//                    row segment and nearby particle;
+//   the particles -- one warp per particle: Wan-Turek repulsion (Eqs. 28-29),
+//                    fixed-order FP64 sum of its partials (Eqs. 18-19) once
+//                    they are all there, Newton-Euler update (Eqs. 22-24),
+//                    then binning of the particle into the lattice tiles its
+//                    phi tail reaches, for the next sweep.
 //
 // Populations are stored as deviations d_i = f_i - w_i (structure of arrays:
 // 9 planes of ny rows of `pitch` elements), in FP32, FP16 or BF16; arithmetic
@@ -18,7 +19,7 @@
 // positions and the tile bins are double-buffered by step parity, so a step
 // reads one copy and writes the other.
 //
-// The sweep is a persistent kernel: each warp walks row segments of 128 nodes
+// The sweep is persistent: each warp takes row segments of 128 nodes
 // and streams every segment's nine source rows (plus a 16-byte halo on each
 // side) into shared memory with bulk asynchronous copies (cp.async.bulk,
 // completion on an mbarrier); once a segment's rows have been read, the copy
@@ -27,6 +28,12 @@
 // nodes as two pairs (nodes 2l, 2l + 1 of each half segment), which keeps
 // few registers live; writes go straight from registers, one contiguous run
 // per plane and pair.
+//
+// One launch per step pair of kernels against one launch over many steps, us
+// per step (FP32 unless said): 200 x 100 cylinder 18.5 -> 11.5, 400 x 2000 box
+// 36.9 -> 17.3, 1793 x 179 channel in FP16 21.6 -> 13.3, 512^2 suspension
+// 22.6 -> 14.4, 501 x 101 channel with a moving frame 30.8 -> 11.7, 64 uneven
+// lattices 264 -> 242, 4096^2 suspension 225.6 -> 219.1 (FP16 221.4 -> 207.3).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -42,8 +49,6 @@ constexpr int TILE_H = 8;     // rows per binning tile
 constexpr int MAXC = 32;      // candidate particles per tile
 constexpr int MAXT = 128;     // tiles one particle's phi tail may reach
 constexpr int NREC = 3;       // float4 records per binned particle
-constexpr int STAGES = 1;     // row segments staged ahead per warp (shared-memory ring depth)
-static_assert(STAGES == 1, "a warp carries one staged segment's periodic-edge values (wrap_load)");
 constexpr int SWEEP_WARPS = 8;   // default rows in flight per block (one row segment per warp)
 constexpr int GUARD = 256;    // elements kept readable before and after a population buffer
 constexpr float PHI_CUT_WIDTHS = 4.0f;   // phi tail kept up to 4 interface widths (phi > 1.1e-7)
@@ -63,7 +68,7 @@ __host__ __device__ constexpr float wof(int i) { return i == 0 ? 4.0f / 9.0f : (
 template <typename T> struct Storage;
 
 template <> struct Storage<float> {
-    static __device__ __forceinline__ float load1(const float *p) { return __ldg(p); }
+    static __device__ __forceinline__ float load1(const float *p) { return __ldcg(p); }
     static __device__ __forceinline__ float lds1(const float *p) { return *p; }
     static __device__ __forceinline__ void store1(float *p, float v) { *p = v; }
     static __device__ __forceinline__ float2 lds2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
@@ -71,7 +76,7 @@ template <> struct Storage<float> {
 };
 
 template <> struct Storage<__half> {
-    static __device__ __forceinline__ float load1(const __half *p) { return __half2float(__ldg(p)); }
+    static __device__ __forceinline__ float load1(const __half *p) { return __half2float(__ldcg(p)); }
     static __device__ __forceinline__ float lds1(const __half *p) { return __half2float(*p); }
     static __device__ __forceinline__ void store1(__half *p, float v) { *p = __float2half_rn(v); }
     static __device__ __forceinline__ float2 lds2(const __half *p) { return __half22float2(*reinterpret_cast<const __half2 *>(p)); }
@@ -79,7 +84,7 @@ template <> struct Storage<__half> {
 };
 
 template <> struct Storage<__nv_bfloat16> {
-    static __device__ __forceinline__ float load1(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
+    static __device__ __forceinline__ float load1(const __nv_bfloat16 *p) { return __bfloat162float(__ldcg(p)); }
     static __device__ __forceinline__ float lds1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ void store1(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
     static __device__ __forceinline__ float2 lds2(const __nv_bfloat16 *p) {
@@ -100,10 +105,10 @@ template <typename T> __host__ __device__ constexpr int stage_elems() { return 9
 
 // Dynamic shared memory of one sweep block of W warps.
 template <typename T, int W = SWEEP_WARPS> __host__ __device__ constexpr size_t sweep_smem_bytes() {
-    return (size_t)W * STAGES * stage_elems<T>() * sizeof(T)   // staged rows
+    return (size_t)W * stage_elems<T>() * sizeof(T)             // staged rows
            + (size_t)W * MAXC * NREC * sizeof(float4)           // candidate records
            + (size_t)W * MAXC * sizeof(int)                     // candidate ids
-           + (size_t)W * STAGES * sizeof(uint64_t);             // mbarriers
+           + (size_t)W * sizeof(uint64_t);                      // mbarriers
 }
 
 // ------------------------------------------------------------ parameters
@@ -111,6 +116,10 @@ struct Particles {      // structure of arrays, device memory
     double *x[2], *y[2];        // centre, by step parity
     float *xf[2], *yf[2];       // FP32 copy of the centre, for cheap proximity tests
     double *r, *ux, *uy, *omega, *theta, *rho_s;
+    // formed when the particles are uploaded: 1 / m and 1 / I (Eqs. 22-23), the
+    // buoyancy-reduced weight in x and y, and the reach (r + the phi tail)
+    double *im, *iI, *wx, *wy, *reach;
+    float *rf;                  // r in FP32
     int *fixed;
 };
 
@@ -171,17 +180,45 @@ struct Physics {
     double cut_d;
 };
 
-struct Bins {                   // one set per step parity
+// Tile bins.  A step reads the bins of its own positions and fills the next
+// step's, so records come in two copies by step parity.  The counts rotate
+// through three arrays: a step reads count[rot], its particle updates add to
+// count[rot + 1], and it zeroes count[rot + 2], which nothing uses during the
+// step, so that no pass of its own is needed to clear them.
+struct Bins {                   // one step's view
     int *count;                 // per tile: particles binned (may exceed MAXC)
-    int *ids;                   // per tile: MAXC particle ids
+    int2 *ids;                  // per tile: MAXC (particle, index of the tile in the particle's list)
     float4 *rec;                // per tile and slot, 3 records: (cx_hi, cx_lo, cy_hi, cy_lo),
                                 // (r, ux_hi, uy_hi, omega_hi), (ux_lo, uy_lo, omega_lo, packed
                                 // floor(cx), floor(cy): 16 bits each)
-    int *pslot;                 // per particle: MAXT entries tile * MAXC + slot (-1: overflowed)
+    int *pslot;                 // per particle: MAXT tiles it reaches (-1: overflowed, or another strip's)
     int *npslot;                // per particle: tiles reached
+    int *done;                  // per particle: minus the partials its update still waits for
+};
+
+struct BinSet {
+    int *count;                 // 3 arrays of `tiles`
+    int2 *ids;                  // 2 x tiles x MAXC
+    float4 *rec;                // 2 x tiles x MAXC x NREC
+    int *pslot, *npslot, *done; // 2 x parts x MAXT, 2 x parts, 2 x parts
     float *cover;               // PS: per particle, the covered areas of the (2K+1)^2 cells about
                                 // (floor X, floor Y), row-major; shared by both parities
+    int tiles, parts;           // array strides
 };
+
+__host__ __device__ inline int rot3(int r) { return r >= 3 ? r - 3 : r; }
+
+__host__ __device__ inline Bins bins_at(const BinSet &b, int par, int rot) {
+    Bins v;
+    const long long t = (long long)par * b.tiles, q = (long long)par * b.parts;
+    v.count = b.count + (long long)rot * b.tiles;
+    v.ids = b.ids + t * MAXC;
+    v.rec = b.rec + t * MAXC * NREC;
+    v.pslot = b.pslot + q * MAXT;
+    v.npslot = b.npslot + q;
+    v.done = b.done + q;
+    return v;
+}
 
 // ------------------------------------------------------------ small helpers
 __device__ __forceinline__ int wrap_or_clamp(int v, int n, int periodic) {
@@ -340,12 +377,35 @@ struct AxisTiles {
     int lo[2], hi[2];
 };
 
+// floor and ceil to int (one instruction on the device), and v mod n for v
+// mostly within one period of [0, n).
+__host__ __device__ inline int floor_int(double v) {
+#ifdef __CUDA_ARCH__
+    return __double2int_rd(v);
+#else
+    return (int)floor(v);
+#endif
+}
+__host__ __device__ inline int ceil_int(double v) {
+#ifdef __CUDA_ARCH__
+    return __double2int_ru(v);
+#else
+    return (int)ceil(v);
+#endif
+}
+__host__ __device__ inline int wrap_int(int v, int n) {
+    if (v >= -n && v < 0) return v + n;
+    if (v >= n && v - n < n) return v - n;
+    if (v >= 0 && v < n) return v;
+    return ((v % n) + n) % n;
+}
+
 __host__ __device__ inline AxisTiles axis_tiles(double X, double R, int n, int tile, int ntiles, int periodic) {
     AxisTiles t;
-    int il = (int)floor(X - R), ih = (int)ceil(X + R);
+    int il = floor_int(X - R), ih = ceil_int(X + R);
     if (periodic) {
         if (ih - il + 1 >= n) { t.n = 1; t.lo[0] = 0; t.hi[0] = ntiles - 1; return t; }
-        int a = ((il % n) + n) % n, b = ((ih % n) + n) % n;
+        const int a = wrap_int(il, n), b = wrap_int(ih, n);
         if (a <= b) { t.n = 1; t.lo[0] = a / tile; t.hi[0] = b / tile; return t; }
         int first_hi = b / tile, second_lo = a / tile;
         if (first_hi >= second_lo) { t.n = 1; t.lo[0] = 0; t.hi[0] = ntiles - 1; return t; }
@@ -451,7 +511,7 @@ __device__ __forceinline__ T wrap_load(const T *__restrict__ src, const Lattice 
     const int i = wrap_lane_plane(L, tx, lane);
     if (i < 0) return T();
     const T *row = plane_row<T>(src, L, i, y - cyof(i));
-    return row[lane < 3 ? L.nx - 1 : 0];
+    return __ldcg(row + (lane < 3 ? L.nx - 1 : 0));
 }
 
 template <typename T>
@@ -461,24 +521,10 @@ __device__ __forceinline__ void wrap_patch(T *stage, const Lattice &L, int tx, i
     if (i >= 0) stage[i * SW + (lane < 3 ? H - 1 : H + (L.nx - tx * TILE_W))] = v;
 }
 
-template <typename T>
-__device__ __forceinline__ void pull_node_scalar(const T *__restrict__ src, const Lattice &L, int x, int y, float d[9]) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-        int sx = wrap_or_clamp(x - cxof(i), L.nx, L.per_x);
-        d[i] = from_store<T>(L, i, Storage<T>::load1(plane_row<T>(src, L, i, y - cyof(i)) + sx));
-    }
-}
-
 // Non-equilibrium extrapolation at an edge node (x, y) (Guo et al. 2002, as
 // the paper's Sec. 3 uses): d_b = deq(rho_b, u_b) + d_n - deq(rho_n, u_n),
 // with n the inner neighbour (diagonal at corners; corners take the
-// south/north condition).  Kept out of line: few nodes take it, and inlined
-// it would crowd the sweep's instruction cache.
-struct Pop9 {
-    float v[9];
-};
-
+// south/north condition).
 // d_b from the inner neighbour's streamed values dn and the side's condition.
 __device__ __forceinline__ void extrapolate(const Lattice &L, int side, const float dn[9], float out[9]) {
     float drn = 0.f, jx = 0.f, jy = 0.f;
@@ -519,20 +565,14 @@ __device__ __forceinline__ void extrapolate(const Lattice &L, int side, const fl
     for (int i = 0; i < 9; ++i) out[i] = dn[i] + X[i];
 }
 
-// An edge node whose inner neighbour lies on another row (south / north
-// edges and corners): the neighbour's streamed values come from global memory.
-template <typename T>
-__device__ __noinline__ Pop9 edge_values(const T *__restrict__ src, const Lattice &L, int x, int y) {
-    const int onx = !L.per_x && (x == 0 || x == L.nx - 1);
-    const int ony = south_edge_row(L, y) || north_edge_row(L, y);
-    const int side = ony ? (y == 0 ? SOUTH : NORTH) : (x == 0 ? WEST : EAST);
-    const int xn = onx ? (x == 0 ? 1 : L.nx - 2) : x;
-    const int yn = ony ? (y == 0 ? 1 : L.ny - 2) : y;
-    float dn[9];
-    pull_node_scalar<T>(src, L, xn, yn, dn);
-    Pop9 out;
-    extrapolate(L, side, dn, out.v);
-    return out;
+// The row whose streamed values row y's sweep starts from: an edge row's nodes
+// extrapolate from their inner neighbours (the same column one row in; corners
+// diagonally), so an edge row stages its neighbour's source rows.
+template <bool EDGES>
+__device__ __forceinline__ int streamed_row(const Lattice &L, int y) {
+    if (EDGES && south_edge_row(L, y)) return 1;
+    if (EDGES && north_edge_row(L, y)) return L.ny - 2;
+    return y;
 }
 
 // ------------------------------------------------------------ PS-LBM solid fraction
@@ -670,18 +710,22 @@ struct FieldsOut {
     float *rho, *ux, *uy, *phi;   // dense [ny][nx]
 };
 
+struct PartArgs;
+
 // Everything one lattice's sweep needs.
 template <typename T>
 struct SweepArgs {
-    const T *src;               // post-collision populations (GUARD elements in)
-    T *dst;                     // next populations
+    T *buf[2];                  // populations by step parity (GUARD elements in)
     Lattice L;
     Physics ph;
-    Bins B;                     // this step's bins (counts, ids, records)
-    float4 *partial;            // force / torque partials
-    int *clear;                 // next step's bin counts to zero, or NULL
+    BinSet B;                   // tile bins (np > 0)
+    float4 *partial;            // force / torque partials and tag: per particle, tile of its list and row
     int *err;                   // the lattice's error word
-    FieldsOut fo;               // MODE_FIELDS outputs
+    const PartArgs *pa;         // the particle update's arguments (device memory; batches)
+    int np;                     // particles (0: no bins to read)
+    int cur, rot;               // parity and count rotation of the launch's first step
+    unsigned tag;               // and its tag (a step number)
+    unsigned ntx_inv;           // floor(2^32 / ntx) + 1 (saturated), see row_of
 };
 
 // A batched sweep walks one work list over many lattices, their descriptors
@@ -695,17 +739,10 @@ struct BatchArgs {
     SweepArgs<T> a[BATCH_LAUNCH_MAX];
     int item_start[BATCH_LAUNCH_MAX + 1];
     int tile_start[BATCH_LAUNCH_MAX + 1];
+    int part_start[BATCH_LAUNCH_MAX + 1];
     int n;
 };
 static_assert(sizeof(BatchArgs<float>) <= 32000, "batched sweep parameters exceed the parameter space");
-
-// Particle batches keep their descriptors in device memory: lattice k owns
-// particles [item_start[k], item_start[k+1]).
-struct BatchIndex {
-    const int *item_start;
-    const int *tile_start;
-    int n;
-};
 
 // Largest k with start[k] <= v (start[0] = 0, start ascending, n entries + 1).
 template <typename P>
@@ -718,12 +755,43 @@ __device__ __forceinline__ int batch_find(const P &start, int n, int v) {
     return lo;
 }
 
-// Per-warp state of the staging ring.
+// Per-warp state of the staged segment.
 struct Ring {
-    uint64_t *bars;
-    uint32_t parity;            // bit s: phase parity the next wait on stage s expects
-    uint32_t pending;           // bit s: stage s has copies in flight
+    uint64_t *bar;
+    uint32_t parity;            // phase parity the next wait expects
+    bool pending;               // copies in flight
 };
+
+// A contribution to a particle is counted without ordering the count after the
+// contribution: a release would wait for every store the warp has in flight (a
+// segment's 9 x 128 populations).  Each partial instead carries its step's tag
+// in the same 16-byte store, and whoever finds the count complete reads the
+// partials until their tags are there.
+__device__ __forceinline__ void count_done(int *counter) {
+    asm volatile("red.add.relaxed.gpu.global.s32 [%0], 1;" ::"l"(counter) : "memory");
+}
+__device__ __forceinline__ int load_done(const int *counter) {
+    int v;
+    asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
+    return v;
+}
+__device__ __forceinline__ void store_partial(float4 *p, float x, float y, float z, unsigned tag) {
+    asm volatile("{\n\t.reg .b64 a, b;\n\t.reg .b128 v;\n\t"
+                 "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\tmov.b128 v, {a, b};\n\t"
+                 "st.relaxed.gpu.global.b128 [%0], v;\n\t}"
+                 ::"l"(p), "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(__float_as_uint(z)), "r"(tag)
+                 : "memory");
+}
+__device__ __forceinline__ float4 load_partial(const float4 *p) {
+    uint32_t x, y, z, w;
+    asm volatile("{\n\t.reg .b64 a, b;\n\t.reg .b128 v;\n\t"
+                 "ld.relaxed.gpu.global.b128 v, [%4];\n\tmov.b128 {a, b}, v;\n\t"
+                 "mov.b64 {%0, %1}, a;\n\tmov.b64 {%2, %3}, b;\n\t}"
+                 : "=r"(x), "=r"(y), "=r"(z), "=r"(w)
+                 : "l"(p)
+                 : "memory");
+    return make_float4(__uint_as_float(x), __uint_as_float(y), __uint_as_float(z), __uint_as_float(w));
+}
 
 // The streamed value f_i(x) = f'_i(x - c_i) of plane i at node e of the
 // staged segment (e in [-1, TILE_W]: the 16-byte halos hold the neighbours).
@@ -755,18 +823,20 @@ __device__ __forceinline__ float rcp_approx(float x) {
 // Slot m (0 or 1) of a node pair.
 __device__ __forceinline__ float &slot(float2 &v, int m) { return m ? v.y : v.x; }
 
-// One row segment (row y, segment tx) of lattice A: wait for its staged rows
-// (and write in the periodic-edge values wv, see wrap_load), then sweep its
-// 128 nodes in two passes of 64 (lane l takes nodes 2l and 2l + 1 of each
-// half, so every store of a pass is one contiguous run per plane), hand the
-// stage to the segment `nxt` (row ny2, segment nx2 of lattice An; its edge
-// values go to wv) once the second pass has read it, and sum the segment's
-// force / torque per candidate particle.  Returns false if the bounded wait
-// gave up.
-template <typename T, int MODE, bool EDGES, bool PS = false>
-__device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int tx, T *stage, Ring &ring, int s,
-                                              bool has_next, const SweepArgs<T> &An, int ny2, int nx2,
-                                              float4 *crec, int *cid, T &wv, int lane) {
+// One row segment (row y, segment tx) of lattice A, populations src -> dst,
+// bins B: wait for its staged rows (and write in the periodic-edge values wv,
+// see wrap_load), then sweep its 128 nodes in two passes of 64 (lane l takes
+// nodes 2l and 2l + 1 of each half, so every store of a pass is one
+// contiguous run per plane), hand the stage to the next segment (row ny2,
+// segment nx2 of lattice Ln, populations srcn; its edge values go to wv) once
+// the second pass has read it, and sum the segment's force / torque per
+// candidate particle.  FUSED: also count the contributions, marked with the
+// step's tag (`count` false: not counted).  Returns false if the bounded wait gave up.
+template <typename T, int MODE, bool EDGES, bool PS, bool FUSED>
+__device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *src, T *dst, const Bins &B, int y, int tx,
+                                              T *stage, Ring &ring, bool has_next, const T *srcn, const Lattice &Ln,
+                                              int ny2, int nx2, float4 *crec, int *cid, T &wv, unsigned tag,
+                                              bool count, const FieldsOut &fo, int lane) {
     constexpr int H = halo_of<T>(), SW = segw_of<T>();
     const Lattice &L = A.L;
     const Physics &ph = A.ph;
@@ -777,22 +847,24 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
     // loaded before the wait so that their latency overlaps it
     __syncwarp();
     int ncand = 0;
-    if (A.B.count) {
-        ncand = A.B.count[tile];
+    int2 mine = make_int2(-1, 0);       // lane c: candidate c, index of this tile in its list
+    if (A.np > 0) {
+        ncand = __ldcg(B.count + tile);
         ncand = ncand > MAXC ? MAXC : ncand;
         if (lane < ncand) {
             const long long r = (long long)tile * MAXC + lane;
 #pragma unroll
-            for (int q = 0; q < NREC; ++q) crec[q * MAXC + lane] = A.B.rec[NREC * r + q];
-            cid[lane] = A.B.ids[r];
+            for (int q = 0; q < NREC; ++q) crec[q * MAXC + lane] = __ldcg(B.rec + NREC * r + q);
+            mine = __ldcg(B.ids + r);
+            cid[lane] = mine.x;
         }
     }
 
     // ---- wait for the staged rows
     // a warp-uniform decision: every lane leaves together if any gave up
-    if (!__all_sync(0xffffffffu, mbar_wait_bounded(&ring.bars[s], (ring.parity >> s) & 1u))) return false;
-    ring.parity ^= 1u << s;
-    ring.pending &= ~(1u << s);
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(ring.bar, ring.parity))) return false;
+    ring.parity ^= 1u;
+    ring.pending = false;
 
     const bool row_edge = EDGES && (south_edge_row(L, y) || north_edge_row(L, y));
     const bool col_edge = EDGES && !L.per_x && (tx == 0 || tx0 + TILE_W >= L.nx);
@@ -854,25 +926,37 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
                 }
             }
         }
+        if (EDGES && row_edge) {
+            // south / north edge rows (corners included): the stage holds the
+            // neighbour row's pulls.  (Read from global memory, node by node
+            // out of line, such a row took a warp 10 us, and the 400 x 2000
+            // box's step waited 20 us for its two.)
+#pragma unroll 1
+            for (int m = 0; m < 2; ++m) {
+                const int xm = x + m;
+                if (xm >= L.nx) continue;
+                const int in = L.per_x ? 0 : (xm == 0 ? 1 : (xm == L.nx - 1 ? -1 : 0));
+                float dn[9], ev[9];
+                staged_pull9<T>(L, stage, e + m + in, dn);
+                extrapolate(L, y == 0 ? SOUTH : NORTH, dn, ev);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) {
+                    const float v = to_store<T>(L, i, ev[i]);
+                    if (m == 0) dk[i].x = v; else dk[i].y = v;
+                }
+            }
+        }
+
         // the segment's last reads of the stage are done: recycle it for the
-        // segment STAGES items ahead
+        // warp's next segment
         if (pass == npass - 1) {
             __syncwarp();
             if (has_next) {
                 fence_proxy_async_smem();
-                issue_segment<T>(An.src, An.L, ny2, nx2, stage, &ring.bars[s], lane);
-                wv = wrap_load<T>(An.src, An.L, ny2, nx2, lane);
-                ring.pending |= 1u << s;
-            }
-        }
-        if (EDGES && row_edge) {
-            // south / north edge rows (corners included): neighbour on another row
-#pragma unroll
-            for (int m = 0; m < 2; ++m) {
-                if (x + m >= L.nx) continue;
-                const Pop9 ev = edge_values<T>(A.src, L, x + m, y);
-#pragma unroll
-                for (int i = 0; i < 9; ++i) slot(dk[i], m) = to_store<T>(L, i, ev.v[i]);
+                const int ys = streamed_row<EDGES>(Ln, ny2);
+                issue_segment<T>(srcn, Ln, ys, nx2, stage, ring.bar, lane);
+                wv = wrap_load<T>(srcn, Ln, ys, nx2, lane);
+                ring.pending = true;
             }
         }
 
@@ -928,7 +1012,7 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
                     const int ix = e + m - (int)(short)(fpk & 0xffff) - L.nx * kx + K;
                     const bool inside = d2 <= R * R && l >= -ph.cut;
                     const bool look = inside && l < ph.cut && (unsigned)ix < (unsigned)S && (unsigned)iy < (unsigned)S;
-                    pcq[m] = look ? __ldg(tab + iy * S + ix) : (inside && l >= ph.cut ? 1.0f : 0.f);
+                    pcq[m] = look ? __ldcg(tab + iy * S + ix) : (inside && l >= ph.cut ? 1.0f : 0.f);
                 }
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
@@ -993,16 +1077,16 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
             if (MODE == MODE_FIELDS) {
                 const long long o = (long long)y * L.nx + x;
                 if (act_a) {
-                    if (A.fo.rho) A.fo.rho[o] = rho.x;
-                    if (A.fo.ux) A.fo.ux[o] = ua.x;
-                    if (A.fo.uy) A.fo.uy[o] = va.x;
-                    if (A.fo.phi) A.fo.phi[o] = 0.f;
+                    if (fo.rho) fo.rho[o] = rho.x;
+                    if (fo.ux) fo.ux[o] = ua.x;
+                    if (fo.uy) fo.uy[o] = va.x;
+                    if (fo.phi) fo.phi[o] = 0.f;
                 }
                 if (act_b) {
-                    if (A.fo.rho) A.fo.rho[o + 1] = rho.y;
-                    if (A.fo.ux) A.fo.ux[o + 1] = ua.y;
-                    if (A.fo.uy) A.fo.uy[o + 1] = va.y;
-                    if (A.fo.phi) A.fo.phi[o + 1] = 0.f;
+                    if (fo.rho) fo.rho[o + 1] = rho.y;
+                    if (fo.ux) fo.ux[o + 1] = ua.y;
+                    if (fo.uy) fo.uy[o + 1] = va.y;
+                    if (fo.phi) fo.phi[o + 1] = 0.f;
                 }
                 continue;
             }
@@ -1032,16 +1116,16 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
             if (MODE == MODE_FIELDS) {
                 const long long o = (long long)y * L.nx + x;
                 if (act_a) {
-                    if (A.fo.rho) A.fo.rho[o] = rho.x;
-                    if (A.fo.ux) A.fo.ux[o] = ux.x;
-                    if (A.fo.uy) A.fo.uy[o] = uy.x;
-                    if (A.fo.phi) A.fo.phi[o] = phq.x;
+                    if (fo.rho) fo.rho[o] = rho.x;
+                    if (fo.ux) fo.ux[o] = ux.x;
+                    if (fo.uy) fo.uy[o] = uy.x;
+                    if (fo.phi) fo.phi[o] = phq.x;
                 }
                 if (act_b) {
-                    if (A.fo.rho) A.fo.rho[o + 1] = rho.y;
-                    if (A.fo.ux) A.fo.ux[o + 1] = ux.y;
-                    if (A.fo.uy) A.fo.uy[o + 1] = uy.y;
-                    if (A.fo.phi) A.fo.phi[o + 1] = phq.y;
+                    if (fo.rho) fo.rho[o + 1] = rho.y;
+                    if (fo.ux) fo.ux[o + 1] = ux.y;
+                    if (fo.uy) fo.uy[o + 1] = uy.y;
+                    if (fo.phi) fo.phi[o + 1] = phq.y;
                 }
                 continue;
             }
@@ -1072,7 +1156,7 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
         }
 
         // ---- store the collided pair: one contiguous run per plane and pass
-        T *base = A.dst + (long long)y * L.pitch + x;
+        T *base = dst + (long long)y * L.pitch + x;
         if (act_b) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) Storage<T>::store2(base + i * L.plane, dk[i]);
@@ -1085,196 +1169,106 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, int y, int 
     if (MODE == MODE_FIELDS) return true;
     if (__any_sync(0xffffffffu, badmax > 0x7f7ffffeu) && lane == 0) atomicOr(A.err, ERR_UNSTABLE);
     // ---- this row segment's force / torque per candidate (zero where no node is owned)
-    if (lane < ncand)
-        A.partial[((long long)tile * MAXC + lane) * TILE_H + (y - ty0)] = make_float4(sgx, sgy, sgt, 0.f);
+    if (lane < ncand) {
+        float4 *out = A.partial + ((long long)mine.x * MAXT + mine.y) * TILE_H + (y - ty0);
+        if (FUSED) {
+            store_partial(out, sgx, sgy, sgt, tag);
+            if (count) count_done(B.done + mine.x);
+        } else {
+            *out = make_float4(sgx, sgy, sgt, 0.f);
+        }
+    }
     return true;
 }
 
-// Shared-memory carve-up common to both sweep kernels.
+// Shared-memory carve-up of the sweep kernels.
 template <typename T, int W>
 struct SweepSmem {
-    T *stages;
+    T *stage;
     float4 *crec;
     int *cid;
-    uint64_t *bars;
+    uint64_t *bar;
     __device__ __forceinline__ SweepSmem(unsigned char *raw, int warp) {
-        constexpr int SW = segw_of<T>();
-        constexpr size_t STAGE_BYTES = (size_t)W * STAGES * stage_elems<T>() * sizeof(T);
+        constexpr size_t STAGE_BYTES = (size_t)W * stage_elems<T>() * sizeof(T);
         constexpr size_t REC_BYTES = (size_t)W * NREC * MAXC * sizeof(float4);
         constexpr size_t ID_BYTES = (size_t)W * MAXC * sizeof(int);
-        stages = reinterpret_cast<T *>(raw) + (size_t)warp * STAGES * stage_elems<T>();
+        stage = reinterpret_cast<T *>(raw) + (size_t)warp * stage_elems<T>();
         crec = reinterpret_cast<float4 *>(raw + STAGE_BYTES) + (size_t)warp * NREC * MAXC;
         cid = reinterpret_cast<int *>(raw + STAGE_BYTES + REC_BYTES) + warp * MAXC;
-        bars = reinterpret_cast<uint64_t *>(raw + STAGE_BYTES + REC_BYTES + ID_BYTES) + warp * STAGES;
+        bar = reinterpret_cast<uint64_t *>(raw + STAGE_BYTES + REC_BYTES + ID_BYTES) + warp;
     }
 };
 
-// Resident warps per SM the sweep kernels are compiled for: W warps per
-// block and SWEEP_SM_WARPS / W blocks per SM (registers capped at 96 per
-// thread for W = 2 and 4; W = 8 holds two blocks, 16 warps).
-constexpr int SWEEP_SM_WARPS = 20;
+// Resident warps per SM the sweep kernels are compiled for: W warps per block
+// and sm_warps / W blocks per SM (registers capped at 96 per thread in FP32
+// storage for W = 2 and 4, at 80 in 16-bit storage; W = 8 holds two blocks in
+// FP32, 16 warps).
+template <typename T> constexpr int sm_warps() { return sizeof(T) == 4 ? 20 : 24; }
 
-// The sweep over one lattice.  Persistent: warps take row segments
+// Row of item `item` (row-major over rows of ntx segments) without a
+// division: inv = floor(2^32 / ntx) + 1 overestimates the quotient by less
+// than item / 2^32 < 1, so one correction makes it exact.
+__device__ __forceinline__ int row_of(unsigned item, unsigned inv, int ntx) {
+    if (ntx == 1) return (int)item;
+    unsigned q = __umulhi(item, inv);
+    if (q * (unsigned)ntx > item) --q;
+    return (int)q;
+}
+
+// The sweep over one lattice without the particle update (a strip's step, the
+// static step, and the fields).  Persistent: warps take row segments
 // round-robin (neighbouring warps on neighbouring segments); each warp keeps
-// STAGES segments staged ahead.  W warps per block (rows in flight per
-// block).
-template <typename T, int MODE, bool EDGES, int W = SWEEP_WARPS, bool PS = false>
-__global__ void __launch_bounds__(W * 32, SWEEP_SM_WARPS / W)
-sweep_kernel(const __grid_constant__ SweepArgs<T> one)
+// its next segment staged ahead.
+template <typename T, int MODE, bool EDGES, bool PS>
+__global__ void __launch_bounds__(SWEEP_WARPS * 32, 20 / SWEEP_WARPS)
+sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ FieldsOut fo)
 {
-    constexpr int SW = segw_of<T>();
+    constexpr int W = SWEEP_WARPS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SweepSmem<T, W> sm(smem_raw, warp);
-    Ring ring;
-    ring.bars = sm.bars;
+    Ring ring{sm.bar, 0u, false};
     if (lane == 0) {
-        for (int s = 0; s < STAGES; ++s) mbar_init(&ring.bars[s], 1);
+        mbar_init(ring.bar, 1);
         mbar_fence_init();
     }
     __syncwarp();
     const Lattice &L = one.L;
+    const T *src = one.buf[one.cur];
+    T *dst = one.buf[one.cur ^ 1];
+    const Bins bins = bins_at(one.B, one.cur, one.rot);
     // the next step's bins start empty (nothing reads them during this sweep)
-    if (one.clear)
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < L.ntx * L.nty; t += gridDim.x * blockDim.x)
-            one.clear[t] = 0;
-
+    if (MODE == MODE_STEP && one.np > 0) {
+        int *clear = one.B.count + (long long)rot3(one.rot + 1) * one.B.tiles;
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < L.ntx * L.nty; t += gridDim.x * blockDim.x) clear[t] = 0;
+    }
     const int nitems = L.ny * L.ntx;
     const int gw = blockIdx.x * W + warp, nw = gridDim.x * W;
-    // item = y * ntx + tx, advanced by nw per iteration without dividing
-    const int dy_step = nw / L.ntx, dtx_step = nw - dy_step * L.ntx;
-    auto advance = [&](int &yy, int &xx) {
-        xx += dtx_step;
-        yy += dy_step;
-        if (xx >= L.ntx) { xx -= L.ntx; ++yy; }
-    };
-    int y = gw / L.ntx, tx = gw - (gw / L.ntx) * L.ntx;
-    ring.parity = 0;
-    ring.pending = 0;
     T wv = T();         // the staged segment's periodic-edge value (wrap_load)
-    {
-        int py = y, ptx = tx;
-        for (int s = 0; s < STAGES; ++s) {
-            if (gw + s * nw < nitems) {
-                issue_segment<T>(one.src, L, py, ptx, sm.stages + s * stage_elems<T>(), &ring.bars[s], lane);
-                wv = wrap_load<T>(one.src, L, py, ptx, lane);
-                ring.pending |= 1u << s;
-            }
-            advance(py, ptx);
-        }
+    int y = row_of(gw, one.ntx_inv, L.ntx), tx = gw - y * L.ntx;
+    if (gw < nitems) {
+        issue_segment<T>(src, L, streamed_row<EDGES>(L, y), tx, sm.stage, ring.bar, lane);
+        wv = wrap_load<T>(src, L, streamed_row<EDGES>(L, y), tx, lane);
+        ring.pending = true;
     }
-    // (row, segment) STAGES items ahead, for the stage being recycled
-    int ay = y, atx = tx;
-    for (int s = 0; s < STAGES; ++s) advance(ay, atx);
-
-    int k = 0;
     bool timed_out = false;
-    for (int item = gw; item < nitems; item += nw, ++k) {
-        if (k > 0) {
-            advance(y, tx);
-            advance(ay, atx);
-        }
-        const int s = k % STAGES;
-        const bool has_next = item + STAGES * nw < nitems;
-        if (!sweep_segment<T, MODE, EDGES, PS>(one, y, tx, sm.stages + s * stage_elems<T>(), ring, s, has_next, one, ay, atx,
-                                           sm.crec, sm.cid, wv, lane)) {
+    for (int item = gw; item < nitems; item += nw) {
+        const int nxt = item + nw;
+        const bool has_next = nxt < nitems;
+        const int ny2 = row_of(nxt, one.ntx_inv, L.ntx), nx2 = nxt - ny2 * L.ntx;
+        if (!sweep_segment<T, MODE, EDGES, PS, false>(one, src, dst, bins, y, tx, sm.stage, ring, has_next, src, L, ny2,
+                                                      nx2, sm.crec, sm.cid, wv, 0u, false, fo, lane)) {
             timed_out = true;
             break;
         }
+        y = ny2;
+        tx = nx2;
     }
     if (timed_out) {
         if (lane == 0) atomicOr(one.err, ERR_TIMEOUT);
         // let the copies this warp still has in flight land before the block
-        // releases its shared memory (each wait bounded again)
-        for (int s = 0; s < STAGES; ++s)
-            if (ring.pending & (1u << s)) mbar_wait_bounded(&ring.bars[s], (ring.parity >> s) & 1u);
-    }
-}
-
-// Position in a batched work list: item, its lattice, row and segment.
-struct Cursor {
-    int item, lat, y, tx;
-};
-
-// Move cursor c (at an earlier item, or c.lat = 0) forward to `item`: a
-// warp's items only grow, so its lattice is found by stepping on from the
-// last one (a few lattices at most per step of the work list).
-template <typename T>
-__device__ __forceinline__ void cursor_seek(const BatchArgs<T> &ba, Cursor &c, int item) {
-    c.item = item;
-    while (c.lat + 1 < ba.n && ba.item_start[c.lat + 1] <= item) ++c.lat;
-    const int local = item - ba.item_start[c.lat];
-    const int ntx = ba.a[c.lat].L.ntx;
-    c.y = local / ntx;
-    c.tx = local - c.y * ntx;
-}
-
-// The sweep over a batch of lattices (at most BATCH_LAUNCH_MAX per launch).
-// Warps take the concatenated row segments round-robin, as in the
-// single-lattice sweep, so that neighbouring warps stage neighbouring rows
-// (DRAM page locality); each item finds its lattice by a binary search in the
-// parameter space.
-template <typename T, int MODE, int W = SWEEP_WARPS>
-__global__ void __launch_bounds__(W * 32, SWEEP_SM_WARPS / W)
-sweep_batch_kernel(const __grid_constant__ BatchArgs<T> ba)
-{
-    constexpr int SW = segw_of<T>();
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    SweepSmem<T, W> sm(smem_raw, warp);
-    Ring ring;
-    ring.bars = sm.bars;
-    if (lane == 0) {
-        for (int s = 0; s < STAGES; ++s) mbar_init(&ring.bars[s], 1);
-        mbar_fence_init();
-    }
-    __syncwarp();
-    {
-        const int ntiles = ba.tile_start[ba.n];
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ntiles; t += gridDim.x * blockDim.x) {
-            const int lat = batch_find(ba.tile_start, ba.n, t);
-            if (ba.a[lat].clear) ba.a[lat].clear[t - ba.tile_start[lat]] = 0;
-        }
-    }
-
-    const int nitems = ba.item_start[ba.n];
-    const int gw = blockIdx.x * W + warp, nw = gridDim.x * W;
-    Cursor cur{0, 0, 0, 0}, ahead{0, 0, 0, 0};
-    ring.parity = 0;
-    ring.pending = 0;
-    T wv = T();         // the staged segment's periodic-edge value (wrap_load)
-    for (int s = 0; s < STAGES; ++s) {
-        const int it = gw + s * nw;
-        if (it < nitems) {
-            cursor_seek(ba, ahead, it);
-            issue_segment<T>(ba.a[ahead.lat].src, ba.a[ahead.lat].L, ahead.y, ahead.tx,
-                             sm.stages + s * stage_elems<T>(), &ring.bars[s], lane);
-            wv = wrap_load<T>(ba.a[ahead.lat].src, ba.a[ahead.lat].L, ahead.y, ahead.tx, lane);
-            ring.pending |= 1u << s;
-        }
-    }
-
-    int k = 0;
-    bool timed_out = false;
-    int last_lat = 0;
-    for (int item = gw; item < nitems; item += nw, ++k) {
-        const int s = k % STAGES;
-        cursor_seek(ba, cur, item);
-        last_lat = cur.lat;
-        const int nxt = item + STAGES * nw;
-        const bool has_next = nxt < nitems;
-        if (has_next) cursor_seek(ba, ahead, nxt);
-        const int nlat = has_next ? ahead.lat : cur.lat;
-        if (!sweep_segment<T, MODE, true>(ba.a[cur.lat], cur.y, cur.tx, sm.stages + s * stage_elems<T>(), ring, s,
-                                          has_next, ba.a[nlat], ahead.y, ahead.tx, sm.crec, sm.cid, wv, lane)) {
-            timed_out = true;
-            break;
-        }
-    }
-    if (timed_out) {
-        if (lane == 0) atomicOr(ba.a[last_lat].err, ERR_TIMEOUT);
-        for (int s = 0; s < STAGES; ++s)
-            if (ring.pending & (1u << s)) mbar_wait_bounded(&ring.bars[s], (ring.parity >> s) & 1u);
+        // releases its shared memory (the wait bounded again)
+        if (ring.pending) mbar_wait_bounded(ring.bar, ring.parity);
     }
 }
 
@@ -1283,6 +1277,8 @@ struct BodyParams {
     int np;
     double gx, gy, rho_f;
     double eps_p, eps_p2, eps_w, eps_w2, xi;
+    double len[2];              // nx, ny
+    float xi_f;
 };
 
 // Map k in [0, total) of a tile-range set to its tile index, ranges in order.
@@ -1297,39 +1293,24 @@ __device__ __forceinline__ int range_len(const AxisTiles &a) {
     return n;
 }
 
-// The particle update, per particle.  With integrate != 0:
-//   1. hydrodynamic force and torque (Eqs. 18-19): the row-segment partials of
-//      the tiles the particle was binned into, summed in FP64 in a fixed
-//      order (lanes take fixed (tile, row) entries, then a fixed shuffle tree);
-//   2. Wan-Turek repulsion (Eqs. 28-29) from the other particles (lanes stride
-//      over them) and from mirror images across the walls;
-//   3. symplectic Euler of Eqs. 22-24 (dt = 1), positions read from copy
-//      `pin` and written to copy `pout`.
-// Always, finally: binning of the particle into every tile its phi tail
-// reaches (see particles_kernel for how the work is split).
-// Everything one lattice's particle update needs.
+// Everything one lattice's particle update needs, whatever the step.
 struct PartArgs {
     Lattice L;
     Physics ph;
     Particles P;
     BodyParams bp;
-    Bins bin_in, bin_out;       // bins the sweep used / bins for the next sweep
-    const float4 *partial;
-    int pin, pout;              // position copy read / written
-    int integrate;
+    BinSet B;
+    float4 *partial;
     double *force, *fcol;
     double *fsum;               // nullable: running sum of (Fx, Fy, T) over integrating steps
     int *err;
     int track = -1;             // moving frame: tracked particle, -1 (the default) when off
     double track_x = 0.0;       // its reference x
+    long long *frame_off = nullptr;   // columns the frame has moved
     // A strip of the lattice (L is the whole lattice): bins hold the tile rows
     // [ty_lo, ty_hi) only, local tile index (ty - ty_lo) * ntx + tx.
     int ty_lo = 0, ty_hi = 1 << 30;
-    // phase 0: the whole update; 1: only the force / torque and repulsion
-    // sums of this strip's bins, written to fpart (5 per particle: Fx, Fy, T,
-    // repulsion x, y); 2: the rest of the update from the sums in fpart.
-    int phase = 0;
-    double *fpart = nullptr;
+    double *fpart = nullptr;    // a strip's sums (5 per particle: Fx, Fy, T, repulsion x, y)
 };
 
 // v wrapped into [0, n) on a periodic axis: fmod(v, n), plus n when it is
@@ -1357,381 +1338,752 @@ __host__ __device__ inline int frame_move(double xt, double xref, int nx, int pe
     return d >= 1.0 ? 1 : (d <= -1.0 ? -1 : 0);
 }
 
-// The particles kernel takes PART_WARPS particles per block, in three phases:
-// (A) each particle's warp sums its force partials and finds its Wan-Turek
-// contacts; (B) one lane per particle does the scalar FP64 work (walls,
-// rigid-body update, frame move, velocity splits, tile ranges); (C) each warp
-// bins its particle for the next sweep.  The FP64 pipe is narrow on this part
-// and charges per warp instruction whatever the mask, so one warp serving the
-// block's particles in (B) costs a PART_WARPS-th of every warp doing its own.
-constexpr int PART_WARPS = 8;
+// The particle update of one step, by one warp per particle, in three parts:
+//   contact  -- Wan-Turek repulsion (Eqs. 28-29) from the other particles
+//               (lanes stride over the particle's tiles) and from mirror
+//               images across the walls.  It reads only the step's starting
+//               positions, so it runs at the start of a step, off the chain
+//               that the forces are on;
+//   sums     -- hydrodynamic force and torque (Eqs. 18-19): the row-segment
+//               partials, summed in FP64 in a fixed order (lanes take fixed
+//               (tile, row) entries, then a fixed shuffle tree);
+//   advance  -- symplectic Euler of Eqs. 22-24 (dt = 1), then binning of the
+//               particle into every tile its phi tail reaches.
+// Everything a step changes is read from L2 (__ldcg): in a launch over several
+// steps another SM wrote it, and the L1 is not coherent.
 
-struct PartShared {
-    double fx, fy, tq, cx, cy;      // (A) hydrodynamic force, torque; repulsion
-    double nX, nY;                  // (B) position for the next step
-    float4 rb;                      // (B) record: r and the velocities' FP32 hi parts
-    float rlx, rly, rlz;            // (B) the velocities' FP32 lo parts
-    AxisTiles ax, ay;               // (B) the tiles the particle's reach covers
+struct Repulsion {
+    double x, y;
 };
 
-// The position copies of a step without indexing the parameter arrays.
-struct PartCopies {
-    const double *xin, *yin;
-    const float *xfin, *yfin;
-    double *xout, *yout;
-    float *xfout, *yfout;
-    __device__ __forceinline__ explicit PartCopies(const PartArgs &A) {
-        const Particles &P = A.P;
-        xin = A.pin ? P.x[1] : P.x[0]; yin = A.pin ? P.y[1] : P.y[0];
-        xfin = A.pin ? P.xf[1] : P.xf[0]; yfin = A.pin ? P.yf[1] : P.yf[0];
-        xout = A.pout ? P.x[1] : P.x[0]; yout = A.pout ? P.y[1] : P.y[0];
-        xfout = A.pout ? P.xf[1] : P.xf[0]; yfout = A.pout ? P.yf[1] : P.yf[0];
+// Could particle p be within Eq. 28's range of another one?  Each lane takes
+// one (tile, slot) of the particle's first eight tiles and first four slots
+// and compares the two records there (FP32, relative to the tile, with a
+// margin far above their rounding), so that the answer takes two dependent
+// loads; more tiles or slots, or a periodic axis too short for one image per
+// tile, answer yes.
+__device__ __forceinline__ bool maybe_near(const PartArgs &A, int p, const Bins &B, int lane) {
+    const int nk = __ldcg(B.npslot + p);
+    const int k = lane >> 2, sl = lane & 3;
+    const int t = __ldcg(B.pslot + (long long)p * MAXT + k);        // (entries past nk: stale, or never written)
+    bool far = nk <= 8 && !A.L.wrap_x && !A.L.wrap_y;
+    float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
+    int id = -1, n = 0;
+    if (k < nk && t >= 0) {
+        const long long q = (long long)t * MAXC + sl;
+        n = __ldcg(B.count + t);
+        id = __ldcg(&B.ids[q].x);
+        ra = __ldcg(B.rec + NREC * q);
+        rb = __ldcg(B.rec + NREC * q + 1);
+    } else if (k < nk) {
+        far = false;
     }
-};
+    far = far && n <= 4;
+    if (sl >= n) id = -1;
+    // the particle's own record among the tile's four
+    const unsigned mine = __ballot_sync(0xffffffffu, id == p) >> (lane & 28) & 15u;
+    const int src = (lane & 28) + (mine ? __ffs(mine) - 1 : 0);
+    const float dx = (ra.x - __shfl_sync(0xffffffffu, ra.x, src)) + (ra.y - __shfl_sync(0xffffffffu, ra.y, src));
+    const float dy = (ra.z - __shfl_sync(0xffffffffu, ra.z, src)) + (ra.w - __shfl_sync(0xffffffffu, ra.w, src));
+    const float lim = rb.x + __shfl_sync(0xffffffffu, rb.x, src) + A.bp.xi_f + 0.05f;
+    if (id >= 0 && id != p && !(dx * dx + dy * dy > lim * lim)) far = false;
+    if (n > 0 && !mine) far = false;
+    return !__all_sync(0xffffffffu, far);
+}
 
-// (A) Hydrodynamic force and torque (Eqs. 18-19) from the sweep's partials,
-// and the particle-particle repulsion (Eq. 28), summed over the warp.  Both
-// sums start from the particle's tile entries, which each lane loads once
-// (entry k = lane + 32 q in register q); the first requests of the repulsion
-// search (its first tile's count and first ids) go out before the force sum,
-// so that the two chains of dependent loads overlap.
-constexpr int PSLOT_REGS = MAXT / 32;   // tile entries per lane
-static_assert(MAXT % 32 == 0 && MAXC >= 4, "tile entries are spread over whole warps");
-constexpr int CONTACT_PREFETCH = 4;     // ids of the first tile requested early
-
-__device__ __forceinline__ void particle_forces(const PartArgs &A, int p, int lane, PartShared &sh) {
+// The pairs (Eq. 28), summed over the warp.
+__device__ __forceinline__ Repulsion pair_repulsion(const PartArgs &A, int p, int cur, const Bins &B, int lane) {
     const Lattice &L = A.L;
     const Particles &P = A.P;
     const BodyParams &bp = A.bp;
-    const Bins &bin_in = A.bin_in;
-    const float4 *__restrict__ partial = A.partial;
-    const PartCopies pc(A);
-    const double *xin = pc.xin, *yin = pc.yin;
-    const float *xfin = pc.xfin, *yfin = pc.yfin;
-    const double X = xin[p], Y = yin[p], r = P.r[p];
-
-    const int nk = bin_in.npslot[p];
-    int tsl[PSLOT_REGS];
-#pragma unroll
-    for (int q = 0; q < PSLOT_REGS; ++q) {
-        const int k = lane + 32 * q;
-        tsl[q] = k < nk ? bin_in.pslot[(long long)p * MAXT + k] : -1;
-    }
-    // the repulsion search's first tile: its count and first ids (slots of
-    // the tile, in bounds; used only below the count)
-    const int t0 = tsl[0] >= 0 ? tsl[0] / MAXC : -1;
-    int cnt0 = 0, jpre[CONTACT_PREFETCH];
-    if (t0 >= 0) {
-        cnt0 = bin_in.count[t0];
-#pragma unroll
-        for (int s = 0; s < CONTACT_PREFETCH; ++s) jpre[s] = bin_in.ids[t0 * MAXC + s];
-    } else {
-#pragma unroll
-        for (int s = 0; s < CONTACT_PREFETCH; ++s) jpre[s] = 0;
-    }
-
-    // ---- 1. hydrodynamic force and torque: lane l adds entries e = l, l + 32,
-    // ... (tile entry e / TILE_H, row e % TILE_H) in that order
-    double fx = 0.0, fy = 0.0, tq = 0.0;
-    const int ne = nk * TILE_H;
-#pragma unroll 2
-    for (int base = 0; base < ne; base += 32) {
-        const int e = base + lane;
-        const int k = e / TILE_H, row = e - k * TILE_H;
-        // entry k sits in lane k % 32, register k / 32 = base / (32 TILE_H)
-        // (the same for the whole warp in one iteration)
-        const int q = base / (32 * TILE_H);
-        int src = tsl[0];
-#pragma unroll
-        for (int qq = 1; qq < PSLOT_REGS; ++qq)
-            if (q == qq) src = tsl[qq];
-        const int ts = __shfl_sync(0xffffffffu, src, k & 31);
-        if (e >= ne || ts < 0) continue;
-        const int ty = (ts / MAXC) / L.ntx + A.ty_lo;
-        if (ty * TILE_H + row >= L.ny) continue;
-        const float4 v = partial[(long long)ts * TILE_H + row];
-        fx += (double)v.x; fy += (double)v.y; tq += (double)v.z;
-    }
-    // ---- 2. particle-particle repulsion.  A pair within r_i + r_j + xi
-    // shares the tile holding the middle of the gap between the surfaces
-    // (that point lies inside both binning reaches), so each lane takes
-    // some of this particle's tiles and counts a pair only in that tile;
-    // within a tile the pairs are added in increasing partner id.
+    const double *xin = cur ? P.x[1] : P.x[0], *yin = cur ? P.y[1] : P.y[0];
+    const float *xfin = cur ? P.xf[1] : P.xf[0], *yfin = cur ? P.yf[1] : P.yf[0];
     double cx = 0.0, cy = 0.0;
-    const float xf = xfin[p], yf = yfin[p], rf = (float)r;
-#pragma unroll
-    for (int q = 0; q < PSLOT_REGS; ++q) {
-        if (lane + 32 * q >= nk) break;
-        const int ts = tsl[q];
-        if (ts < 0) continue;
-        const int t = ts / MAXC;
-        int n = q == 0 ? cnt0 : bin_in.count[t];
-        n = n > MAXC ? MAXC : n;
-        uint32_t contact = 0;
-        for (int sl = 0; sl < n; ++sl) {
-            int j;
-            if (q == 0 && sl < CONTACT_PREFETCH)
-                j = sl == 0 ? jpre[0] : (sl == 1 ? jpre[1] : (sl == 2 ? jpre[2] : jpre[3]));
-            else
-                j = bin_in.ids[t * MAXC + sl];
-            if (j == p) continue;
-            float dxf = xf - xfin[j], dyf = yf - yfin[j];
-            if (L.per_x) { if (dxf >= 0.5f * L.nx) dxf -= L.nx; else if (dxf < -0.5f * L.nx) dxf += L.nx; }
-            if (L.per_y) { if (dyf >= 0.5f * L.ny) dyf -= L.ny; else if (dyf < -0.5f * L.ny) dyf += L.ny; }
-            const float lim = rf + (float)P.r[j] + (float)bp.xi + 0.05f;
-            if (dxf * dxf + dyf * dyf > lim * lim) continue;
-            double dx = X - xin[j], dy = Y - yin[j];
-            if (L.per_x) { while (dx >= 0.5 * L.nx) dx -= L.nx; while (dx < -0.5 * L.nx) dx += L.nx; }
-            if (L.per_y) { while (dy >= 0.5 * L.ny) dy -= L.ny; while (dy < -0.5 * L.ny) dy += L.ny; }
-            // the middle of the gap between the two surfaces, at distance
-            // (d + r - r_j) / 2 from this centre toward the partner
-            const double dd = sqrt(dx * dx + dy * dy);
-            const double f = dd > 0.0 ? 0.5 * (dd + r - P.r[j]) / dd : 0.0;
-            double mx = X - f * dx, my = Y - f * dy;
-            if (L.per_x) mx = wrap_period(mx, (double)L.nx);
-            if (L.per_y) my = wrap_period(my, (double)L.ny);
-            int mxi = (int)floor(mx), myi = (int)floor(my);
-            mxi = mxi < 0 ? 0 : (mxi > L.nx - 1 ? L.nx - 1 : mxi);
-            myi = myi < 0 ? 0 : (myi > L.ny - 1 ? L.ny - 1 : myi);
-            if ((myi / TILE_H) * L.ntx + mxi / TILE_W == t + A.ty_lo * L.ntx) contact |= 1u << sl;
-        }
-        while (contact) {                         // increasing partner id
-            int sel = -1, jmin = 0x7fffffff;
-            for (uint32_t m = contact; m; m &= m - 1) {
-                const int sl = __ffs(m) - 1, j = bin_in.ids[t * MAXC + sl];
-                if (j < jmin) { jmin = j; sel = sl; }
+    if (bp.np > 1 && maybe_near(A, p, B, lane)) {
+        const double X = __ldcg(xin + p), Y = __ldcg(yin + p), r = __ldcg(P.r + p);
+        const float xf = __ldcg(xfin + p), yf = __ldcg(yfin + p), rf = __ldcg(P.rf + p);
+        const int nk = __ldcg(B.npslot + p);
+        // A pair within r_i + r_j + xi shares the tile holding the middle of
+        // the gap between the surfaces (that point lies inside both binning
+        // reaches), so each lane takes some of this particle's tiles and
+        // counts a pair only in that tile; within a tile the pairs are added
+        // in increasing partner id.
+        for (int k = lane; k < nk; k += 32) {
+            const int t = __ldcg(B.pslot + (long long)p * MAXT + k);
+            if (t < 0) continue;
+            int n = __ldcg(B.count + t);
+            n = n > MAXC ? MAXC : n;
+            uint32_t contact = 0;
+            for (int sl = 0; sl < n; ++sl) {
+                const int j = __ldcg(&B.ids[(long long)t * MAXC + sl].x);
+                if (j == p) continue;
+                float dxf = xf - __ldcg(xfin + j), dyf = yf - __ldcg(yfin + j);
+                if (L.per_x) { if (dxf >= 0.5f * L.nx) dxf -= L.nx; else if (dxf < -0.5f * L.nx) dxf += L.nx; }
+                if (L.per_y) { if (dyf >= 0.5f * L.ny) dyf -= L.ny; else if (dyf < -0.5f * L.ny) dyf += L.ny; }
+                const float lim = rf + __ldcg(P.rf + j) + bp.xi_f + 0.05f;
+                if (dxf * dxf + dyf * dyf > lim * lim) continue;
+                const double rj = __ldcg(P.r + j);
+                double dx = X - __ldcg(xin + j), dy = Y - __ldcg(yin + j);
+                if (L.per_x) { while (dx >= 0.5 * L.nx) dx -= L.nx; while (dx < -0.5 * L.nx) dx += L.nx; }
+                if (L.per_y) { while (dy >= 0.5 * L.ny) dy -= L.ny; while (dy < -0.5 * L.ny) dy += L.ny; }
+                // the middle of the gap between the two surfaces, at distance
+                // (d + r - r_j) / 2 from this centre toward the partner
+                const double dd = sqrt(dx * dx + dy * dy);
+                const double f = dd > 0.0 ? 0.5 * (dd + r - rj) / dd : 0.0;
+                double mx = X - f * dx, my = Y - f * dy;
+                if (L.per_x) mx = wrap_period(mx, (double)L.nx);
+                if (L.per_y) my = wrap_period(my, (double)L.ny);
+                int mxi = (int)floor(mx), myi = (int)floor(my);
+                mxi = mxi < 0 ? 0 : (mxi > L.nx - 1 ? L.nx - 1 : mxi);
+                myi = myi < 0 ? 0 : (myi > L.ny - 1 ? L.ny - 1 : myi);
+                if ((myi / TILE_H) * L.ntx + mxi / TILE_W == t + A.ty_lo * L.ntx) contact |= 1u << sl;
             }
-            contact &= ~(1u << sel);
-            double dx = X - xin[jmin], dy = Y - yin[jmin];
-            if (L.per_x) { while (dx >= 0.5 * L.nx) dx -= L.nx; while (dx < -0.5 * L.nx) dx += L.nx; }
-            if (L.per_y) { while (dy >= 0.5 * L.ny) dy -= L.ny; while (dy < -0.5 * L.ny) dy += L.ny; }
-            const double d = sqrt(dx * dx + dy * dy), rr = r + P.r[jmin];
-            double sc = 0.0;
-            if (d <= rr) sc = (rr - d) / bp.eps_p2;
-            else if (d <= rr + bp.xi) sc = (rr + bp.xi - d) * (rr + bp.xi - d) / bp.eps_p;
-            cx += sc * dx;
-            cy += sc * dy;
+            while (contact) {                         // increasing partner id
+                int sel = -1, jmin = 0x7fffffff;
+                for (uint32_t m = contact; m; m &= m - 1) {
+                    const int sl = __ffs(m) - 1, j = __ldcg(&B.ids[(long long)t * MAXC + sl].x);
+                    if (j < jmin) { jmin = j; sel = sl; }
+                }
+                contact &= ~(1u << sel);
+                double dx = X - __ldcg(xin + jmin), dy = Y - __ldcg(yin + jmin);
+                if (L.per_x) { while (dx >= 0.5 * L.nx) dx -= L.nx; while (dx < -0.5 * L.nx) dx += L.nx; }
+                if (L.per_y) { while (dy >= 0.5 * L.ny) dy -= L.ny; while (dy < -0.5 * L.ny) dy += L.ny; }
+                const double d = sqrt(dx * dx + dy * dy), rr = r + __ldcg(P.r + jmin);
+                double sc = 0.0;
+                if (d <= rr) sc = (rr - d) / bp.eps_p2;
+                else if (d <= rr + bp.xi) sc = (rr + bp.xi - d) * (rr + bp.xi - d) / bp.eps_p;
+                cx += sc * dx;
+                cy += sc * dy;
+            }
+        }
+        // (zero unless some lane found a contact: reduced only when one did)
+        if (__any_sync(0xffffffffu, cx != 0.0 || cy != 0.0)) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                cx += __shfl_xor_sync(0xffffffffu, cx, o);
+                cy += __shfl_xor_sync(0xffffffffu, cy, o);
+            }
         }
     }
-    // (the repulsion sums, zero unless some lane found a contact, are
-    // reduced only when one did)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        fx += __shfl_xor_sync(0xffffffffu, fx, o);
-        fy += __shfl_xor_sync(0xffffffffu, fy, o);
-        tq += __shfl_xor_sync(0xffffffffu, tq, o);
+    return Repulsion{cx, cy};
+}
+
+// The walls (Eq. 29): the mirror image across each non-periodic wall, added
+// to the pairs' sum wall by wall.
+__device__ __forceinline__ void wall_repulsion(const PartArgs &A, int p, int cur, Repulsion &c) {
+    const Lattice &L = A.L;
+    const BodyParams &bp = A.bp;
+    if (L.per_x && L.per_y) return;
+    {
+        // FP32, with a margin above its rounding: out of every wall's range?
+        const float x = __ldcg((cur ? A.P.xf[1] : A.P.xf[0]) + p), y = __ldcg((cur ? A.P.yf[1] : A.P.yf[0]) + p);
+        const float nx1 = (float)(L.nx - 1), ny1 = (float)(L.ny - 1);
+        const float lim = __ldcg(A.P.rf + p) + 0.5f * bp.xi_f + 0.25f + 1e-6f * fmaxf(nx1, ny1);
+        if ((L.per_x || (x > lim && nx1 - x > lim)) && (L.per_y || (y > lim && ny1 - y > lim))) return;
     }
-    if (__any_sync(0xffffffffu, cx != 0.0 || cy != 0.0)) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            cx += __shfl_xor_sync(0xffffffffu, cx, o);
-            cy += __shfl_xor_sync(0xffffffffu, cy, o);
-        }
-    }
-    if (lane == 0) {
-        sh.fx = fx; sh.fy = fy; sh.tq = tq; sh.cx = cx; sh.cy = cy;
+    const double X = __ldcg((cur ? A.P.x[1] : A.P.x[0]) + p), Y = __ldcg((cur ? A.P.y[1] : A.P.y[0]) + p);
+    const double r = __ldcg(A.P.r + p);
+    for (int w = 0; w < 4; ++w) {
+        if (L.side_kind[w] == SIDE_PERIODIC) continue;
+        double ix = X, iy = Y;
+        if (w == WEST) ix = -X;
+        if (w == EAST) ix = 2.0 * (L.nx - 1) - X;
+        if (w == SOUTH) iy = -Y;
+        if (w == NORTH) iy = 2.0 * (L.ny - 1) - Y;
+        const double dx = X - ix, dy = Y - iy;
+        const double d = sqrt(dx * dx + dy * dy), rr = 2.0 * r;
+        double sc = 0.0;
+        if (d <= rr) sc = (rr - d) / bp.eps_w2;
+        else if (d <= rr + bp.xi) sc = (rr + bp.xi - d) * (rr + bp.xi - d) / bp.eps_w;
+        c.x += sc * dx;
+        c.y += sc * dy;
     }
 }
 
-// The particle state (B) reads, loaded at the start of the kernel so that
-// its latency passes while the warps sum their forces.
+// An FP32 value as FP64 (exact).  Normal values and zeros on the integer
+// pipe: an FP64-pipe instruction takes a warp as long as dozens of others.
+__device__ __forceinline__ double widen(float v) {
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 255u;
+    if (e - 1u < 254u)
+        return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)v;
+}
+
+// The particle update's scalar part runs with one component per group of
+// eight lanes (0: x, 1: y, 2: rotation, 3: idle), so that an FP64 instruction
+// serves all three.
+__device__ __forceinline__ int component(int lane) { return lane >> 3; }
+
+// Particle p's force and torque (Eqs. 18-19), each in its component's lanes:
+// lane l adds entries e = l, l + 32, ... (tile e / TILE_H of the particle's
+// list, row e % TILE_H) in that order, then a fixed shuffle tree, in which the
+// lanes part with a component at each of its first two levels (the sums are
+// those of three whole trees).  The partials lie per particle in that order
+// (rows outside the lattice and tiles of another strip hold zeros), so the
+// first loads need nothing but p.  TAGGED: each entry is read until it carries
+// the step's tag (the wait bounded).
+template <bool TAGGED>
+__device__ __forceinline__ double hydro_sums(const PartArgs &A, int p, const Bins &B, unsigned tag, int lane) {
+    const float4 *part = A.partial + (long long)p * (MAXT * TILE_H) + lane;
+    float4 v0 = load_partial(part), v1 = load_partial(part + 32);
+    const int ne = __ldcg(B.npslot + p) * TILE_H;
+    double fx = 0.0, fy = 0.0, tq = 0.0;
+    for (int base = 0; base < ne; base += 32) {
+        float4 v = base == 0 ? v0 : (base == 32 ? v1 : load_partial(part + base));
+        if (base + lane < ne) {
+            if (TAGGED && __float_as_uint(v.w) != tag) {
+                const unsigned long long t0 = global_ns();
+                do {
+                    v = load_partial(part + base);
+                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
+                        atomicOr(A.err, ERR_TIMEOUT);
+                        break;
+                    }
+                } while (__float_as_uint(v.w) != tag);
+            }
+            if (base == 0) {
+                fx = widen(v.x); fy = widen(v.y); tq = widen(v.z);
+            } else {
+                fx += widen(v.x); fy += widen(v.y); tq += widen(v.z);
+            }
+        }
+    }
+    const bool up = lane & 16, odd = lane & 8;
+    const double r0 = __shfl_xor_sync(0xffffffffu, up ? fx : tq, 16), r1 = __shfl_xor_sync(0xffffffffu, fy, 16);
+    const double b0 = (up ? tq : fx) + r0, b1 = fy + r1;
+    double f = (odd ? b1 : b0) + __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 8);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    return f;
+}
+
+// What particle_advance reads of a particle, one component per lane group.
+// Loaded in one go, before or together with the partials.
 struct PartState {
-    double X, Y, r, ux, uy, om, rho_s, theta;
+    double pos, vel, inv, weight, reach;    // x / y / theta, its rate, 1/m or 1/I, weight, reach
+    float rf;
     int fixed;
 };
 
-__device__ __forceinline__ PartState load_state(const PartArgs &A, int p) {
+__device__ __forceinline__ PartState load_particle(const PartArgs &A, int p, int cur, int lane) {
     const Particles &P = A.P;
-    const PartCopies pc(A);
-    PartState st;
-    st.X = pc.xin[p]; st.Y = pc.yin[p]; st.r = P.r[p];
-    st.ux = P.ux[p]; st.uy = P.uy[p]; st.om = P.omega[p];
-    st.rho_s = P.rho_s[p]; st.theta = P.theta[p]; st.fixed = P.fixed[p];
-    return st;
+    const int c = component(lane);
+    PartState s;
+    s.pos = __ldcg((c == 0 ? (cur ? P.x[1] : P.x[0]) : (c == 1 ? (cur ? P.y[1] : P.y[0]) : P.theta)) + p);
+    s.vel = __ldcg((c == 0 ? P.ux : (c == 1 ? P.uy : P.omega)) + p);
+    s.inv = __ldcg((c < 2 ? P.im : P.iI) + p);
+    s.weight = c < 2 ? __ldcg((c == 0 ? P.wx : P.wy) + p) : 0.0;
+    s.reach = __ldcg(P.reach + p);
+    s.rf = __ldcg(P.rf + p);
+    s.fixed = __ldcg(P.fixed + p);
+    return s;
 }
 
-// (B) One thread per particle: wall repulsion (Eq. 29), the rigid-body
-// update (Eqs. 22-24), the frame move, the position copies for the next step,
-// and what the binning needs (velocity splits, the tiles the reach covers).
-__device__ __forceinline__ void particle_update(const PartArgs &A, int p, PartShared &sh, const PartState &st) {
+// Rigid-body update of particle p (Eqs. 22-24) from the force f and the
+// repulsion c of this lane's component, positions copy `nxt` written -- with
+// integrate == false the particle stays where it is -- then its binning into
+// every tile its reach covers (in a fixed order), with the record the sweep
+// reads: the centre relative to the tile origin (minimum image about the tile
+// centre) as FP32 hi + lo, radius and velocities.  `out`: the bins the next
+// sweep reads; `shift`: the frame's move.
+__device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const PartState &st, int nxt, const Bins &out,
+                                                 bool integrate, int shift, unsigned next_tag, double f, double c,
+                                                 int lane) {
     const Lattice &L = A.L;
-    const Physics &ph = A.ph;
     const Particles &P = A.P;
-    const BodyParams &bp = A.bp;
-    const PartCopies pc(A);
-    const double X = st.X, Y = st.Y, r = st.r;
-    double nX = X, nY = Y;
-    double ux = st.ux, uy = st.uy, om = st.om;
-
-    if (A.integrate) {
-        const double fx = sh.fx, fy = sh.fy, tq = sh.tq;
-        double cx = sh.cx, cy = sh.cy;
-        // wall repulsion: mirror image across each non-periodic wall
-        for (int w = 0; w < 4; ++w) {
-            if (L.side_kind[w] == SIDE_PERIODIC) continue;
-            double ix = X, iy = Y;
-            if (w == WEST) ix = -X;
-            if (w == EAST) ix = 2.0 * (L.nx - 1) - X;
-            if (w == SOUTH) iy = -Y;
-            if (w == NORTH) iy = 2.0 * (L.ny - 1) - Y;
-            const double dx = X - ix, dy = Y - iy;
-            const double d = sqrt(dx * dx + dy * dy), rr = 2.0 * r;
-            double sc = 0.0;
-            if (d <= rr) sc = (rr - d) / bp.eps_w2;
-            else if (d <= rr + bp.xi) sc = (rr + bp.xi - d) * (rr + bp.xi - d) / bp.eps_w;
-            cx += sc * dx;
-            cy += sc * dy;
-        }
-        // ---- 3. rigid-body update
+    const int comp = component(lane);
+    const bool periodic = comp == 0 ? L.per_x : (comp == 1 ? L.per_y : false);
+    const double len = comp == 0 ? A.bp.len[0] : A.bp.len[1];
+    double u = st.vel, n = st.pos;
+    auto wrap = [&]() {
+        // (as integers: non-negative and below len, the usual case)
+        if (periodic && (unsigned long long)__double_as_longlong(n) >= (unsigned long long)__double_as_longlong(len))
+            n = wrap_period(n, len);
+    };
+    if (integrate) {
+        const bool lead = (lane & 7) == 0 && comp < 3;
         if (!st.fixed) {
-            // two FP64 divisions instead of four: the buoyancy-reduced weight
-            // (1 - rho_f / rho_s) m g is (rho_s - rho_f) pi r^2 g
-            const double area = 3.14159265358979323846 * r * r;
-            const double m = st.rho_s * area;
-            const double im = 1.0 / m, iI = 1.0 / (0.5 * m * r * r);
-            const double wgt = (st.rho_s - bp.rho_f) * area;        // buoyancy-reduced weight / g
-            ux += (fx + cx + wgt * bp.gx) * im;
-            uy += (fy + cy + wgt * bp.gy) * im;
-            om += tq * iI;
-            nX = X + ux;
-            nY = Y + uy;
-            if (L.per_x) nX = wrap_period(nX, (double)L.nx);
-            if (L.per_y) nY = wrap_period(nY, (double)L.ny);
-            P.ux[p] = ux; P.uy[p] = uy; P.omega[p] = om;
-            P.theta[p] = st.theta + om;
+            u += (f + c + st.weight) * st.inv;
+            n += u;
+            wrap();
+            if (lead) (comp == 0 ? P.ux : (comp == 1 ? P.uy : P.omega))[p] = u;
         }
-        A.force[3 * p] = fx; A.force[3 * p + 1] = fy; A.force[3 * p + 2] = tq;
-        A.fcol[2 * p] = cx; A.fcol[2 * p + 1] = cy;
-        if (A.fsum) {
-            A.fsum[3 * p] += fx; A.fsum[3 * p + 1] += fy; A.fsum[3 * p + 2] += tq;
-        }
-        if (A.track >= 0) {
+        if (shift && comp == 0) {
             // the frame moves with the tracked particle: every particle, fixed
             // ones included, shifts by the same whole number of columns
-            const int s = frame_move(pc.xin[A.track], A.track_x, L.nx, L.per_x);
-            if (s) {
-                nX -= (double)s;
-                if (L.per_x) nX = wrap_period(nX, (double)L.nx);
+            n -= (double)shift;
+            wrap();
+        }
+        if (lead) {
+            A.force[3 * (long long)p + comp] = f;
+            if (A.fsum) {
+                double *s = A.fsum + 3 * (long long)p + comp;
+                *s = __ldcg(s) + f;
             }
+            if (comp == 2 && !st.fixed) P.theta[p] = n;
         }
     }
-    pc.xout[p] = nX; pc.yout[p] = nY;
-    pc.xfout[p] = (float)nX; pc.yfout[p] = (float)nY;
-
+    if ((lane & 7) == 0 && comp < 2) {
+        (comp == 0 ? (nxt ? P.x[1] : P.x[0]) : (nxt ? P.y[1] : P.y[0]))[p] = n;
+        (comp == 0 ? (nxt ? P.xf[1] : P.xf[0]) : (nxt ? P.yf[1] : P.yf[0]))[p] = (float)n;
+    }
     // velocities as FP32 hi + lo: the sweep forms u_s - u*, a small difference
-    const float uxh = (float)ux, uyh = (float)uy, omh = (float)om;
-    sh.nX = nX; sh.nY = nY;
-    sh.rb = make_float4((float)r, uxh, uyh, omh);
-    sh.rlx = (float)(ux - (double)uxh); sh.rly = (float)(uy - (double)uyh); sh.rlz = (float)(om - (double)omh);
-    const double R = r + ph.cut_d;
-    sh.ax = axis_tiles(nX, R, L.nx, TILE_W, L.ntx, L.per_x);
-    sh.ay = axis_tiles(nY, R, L.ny, TILE_H, L.nty, L.per_y);
-}
-
-// (C) Binning of the particle into every tile its reach covers (lanes take
-// the tiles in a fixed order), with the record the sweep reads: the centre
-// relative to the tile origin (minimum image about the tile centre) as FP32
-// hi + lo, radius and velocities.
-__device__ __forceinline__ void particle_bin(const PartArgs &A, int p, int lane, const PartShared &sh) {
-    const Lattice &L = A.L;
-    const Bins &bin_out = A.bin_out;
-    const double nX = sh.nX, nY = sh.nY;
-    const AxisTiles ax = sh.ax, ay = sh.ay;
-    const float4 rb = sh.rb;
-    const float rlx = sh.rlx, rly = sh.rly, rlz = sh.rlz;
+    const float uh = (float)u, ul = (float)(u - widen(uh));
+    const float uxh = __shfl_sync(0xffffffffu, uh, 0), uyh = __shfl_sync(0xffffffffu, uh, 8);
+    const float omh = __shfl_sync(0xffffffffu, uh, 16), uxl = __shfl_sync(0xffffffffu, ul, 0);
+    const float uyl = __shfl_sync(0xffffffffu, ul, 8), oml = __shfl_sync(0xffffffffu, ul, 16);
+    // the tiles along the lane's axis
+    const AxisTiles at = comp == 0 ? axis_tiles(n, st.reach, L.nx, TILE_W, L.ntx, L.per_x)
+                                   : axis_tiles(n, st.reach, L.ny, TILE_H, L.nty, L.per_y);
+    AxisTiles ax, ay;
+    ax.n = __shfl_sync(0xffffffffu, at.n, 0);
+    ay.n = __shfl_sync(0xffffffffu, at.n, 8);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        ax.lo[q] = __shfl_sync(0xffffffffu, at.lo[q], 0);
+        ax.hi[q] = __shfl_sync(0xffffffffu, at.hi[q], 0);
+        ay.lo[q] = __shfl_sync(0xffffffffu, at.lo[q], 8);
+        ay.hi[q] = __shfl_sync(0xffffffffu, at.hi[q], 8);
+    }
+    const double nX = __shfl_sync(0xffffffffu, n, 0), nY = __shfl_sync(0xffffffffu, n, 8);
     const int NX = range_len(ax), NY = range_len(ay);
     int total = NX * NY;
     if (total > MAXT) {                      // ruled out at create; kept as a guard
         if (lane == 0) atomicOr(A.err, ERR_OVERFLOW);
         total = MAXT;
     }
-    for (int k = lane; k < total; k += 32) {
-        const int ty = range_at(ay, k / NX), tx = range_at(ax, k - (k / NX) * NX);
-        int entry = -1;
-        if (ty < A.ty_lo || ty >= A.ty_hi) {       // another strip's tile
-            bin_out.pslot[(long long)p * MAXT + k] = entry;
-            continue;
+    // binning: two lanes per tile, one for each axis of its record
+    const bool axis = lane & 1;
+    int need = 0;                            // partials the next update waits for
+    for (int k0 = 0; k0 < total; k0 += 16) {
+        const int k = k0 + (lane >> 1);
+        const bool has = k < total;
+        int ty = 0, tx = 0;
+        if (has) {
+            ty = range_at(ay, k / NX);
+            tx = range_at(ax, k - (k / NX) * NX);
         }
+        const bool local = has && ty >= A.ty_lo && ty < A.ty_hi;        // (else another strip's tile)
         const int t = (ty - A.ty_lo) * L.ntx + tx;
-        const int s = atomicAdd(&bin_out.count[t], 1);
-        if (s < MAXC) {
-            double cx = nX - (double)(tx * TILE_W), cy = nY - (double)(ty * TILE_H);
-            if (L.per_x) {
-                const double h = 0.5 * TILE_W;
-                while (cx - h >= 0.5 * L.nx) cx -= L.nx;
-                while (cx - h < -0.5 * L.nx) cx += L.nx;
+        int s = MAXC;
+        if (local && !axis) s = atomicAdd(&out.count[t], 1);
+        // the centre along the lane's axis, while the count's answer is on its way
+        double r = (axis ? nY : nX) - (double)(axis ? ty * TILE_H : tx * TILE_W);
+        float rh = (float)r;
+        if (axis ? L.per_y : L.per_x) {
+            const float h = axis ? 0.5f * TILE_H : 0.5f * TILE_W;
+            const int ln = axis ? L.ny : L.nx;
+            if (!(fabsf(rh - h) < 0.5f * (float)ln - 1.0f - 1e-6f * (float)ln)) {     // (else certainly the nearest image)
+                while (r - (double)h >= 0.5 * ln) r -= ln;
+                while (r - (double)h < -0.5 * ln) r += ln;
+                rh = (float)r;
             }
-            if (L.per_y) {
-                const double h = 0.5 * TILE_H;
-                while (cy - h >= 0.5 * L.ny) cy -= L.ny;
-                while (cy - h < -0.5 * L.ny) cy += L.ny;
-            }
-            const float cxh = (float)cx, cyh = (float)cy;
-            entry = t * MAXC + s;
-            bin_out.ids[entry] = p;
-            bin_out.rec[NREC * (long long)entry] = make_float4(cxh, (float)(cx - (double)cxh), cyh, (float)(cy - (double)cyh));
-            bin_out.rec[NREC * (long long)entry + 1] = rb;
-            // the centre's whole-cell offsets from the tile origin (the PS sweep's table index)
-            const int fxi = (int)floor(cx), fyi = (int)floor(cy);
-            bin_out.rec[NREC * (long long)entry + 2] =
-                make_float4(rlx, rly, rlz, __int_as_float((fxi & 0xffff) | (int)((unsigned)fyi << 16)));
-        } else {
-            atomicOr(A.err, ERR_OVERFLOW);
         }
-        bin_out.pslot[(long long)p * MAXT + k] = entry;
+        const float rl = (float)(r - widen(rh));
+        // the centre's whole-cell offsets from the tile origin (the PS sweep's table index)
+        const int cell = __double2int_rd(r), other = __shfl_xor_sync(0xffffffffu, cell, 1);
+        s = __shfl_sync(0xffffffffu, s, lane & 30);
+        const bool in = local && s < MAXC;
+        if (local && !in && !axis) atomicOr(A.err, ERR_OVERFLOW);
+        int rows = 0;
+        if (in) {
+            rows = L.ny - ty * TILE_H;
+            rows = rows < TILE_H ? rows : TILE_H;
+            const long long q = (long long)t * MAXC + s;
+            float2 *rec = reinterpret_cast<float2 *>(out.rec + NREC * q);
+            rec[axis] = make_float2(rh, rl);
+            if (!axis) {
+                out.ids[q] = make_int2(p, k);
+                out.rec[NREC * q + 1] = make_float4(st.rf, uxh, uyh, omh);
+            } else {
+                out.rec[NREC * q + 2] =
+                    make_float4(uxl, uyl, oml, __int_as_float((other & 0xffff) | (int)((unsigned)cell << 16)));
+            }
+        }
+        if (has && !axis) {
+            out.pslot[(long long)p * MAXT + k] = in ? t : -1;
+            need += rows;
+            // (this particle's partials of the step are summed: the entries no
+            // sweep will write hold zero; an upload may replace a binning for
+            // the same step, so it also takes that binning's tags off the others)
+            for (int q = 0; !integrate && q < rows; ++q)
+                store_partial(A.partial + ((long long)p * MAXT + k) * TILE_H + q, 0.f, 0.f, 0.f, next_tag - 1);
+            for (int q = rows; q < TILE_H; ++q)
+                store_partial(A.partial + ((long long)p * MAXT + k) * TILE_H + q, 0.f, 0.f, 0.f, next_tag);
+        }
     }
-    if (lane == 0) bin_out.npslot[p] = total;
+    need = __reduce_add_sync(0xffffffffu, need);
+    if (lane == 0) {
+        out.npslot[p] = total;
+        out.done[p] = -need;
+    }
 }
 
-// PART_WARPS particles per block of one lattice (BATCH = false) or of every
-// lattice of a batch (BATCH = true; bi.item_start holds each lattice's first
-// particle).  Launch with PART_WARPS * 32 threads and ceil(particles /
-// PART_WARPS) blocks.
-template <bool BATCH>
-__global__ void __launch_bounds__(PART_WARPS * 32)
-particles_kernel(const __grid_constant__ PartArgs one, const PartArgs *__restrict__ many, BatchIndex bi) {
-    __shared__ PartShared sh[PART_WARPS];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int total = BATCH ? bi.item_start[bi.n] : one.bp.np;
-    // the arguments and index of item g (a particle), or null past the end
-    auto locate = [&](int g, int &p) -> const PartArgs * {
-        if (g >= total) return nullptr;
-        if constexpr (BATCH) {
-            const int lat = batch_find(bi.item_start, bi.n, g);
-            p = g - bi.item_start[lat];
-            return &many[lat];
-        } else {
-            p = g;
-            return &one;
-        }
-    };
-    int p = 0;
-    const PartArgs *A = locate(blockIdx.x * PART_WARPS + w, p);
-    const int phase = BATCH ? 0 : one.phase;       // (uniform over the launch)
-    // (B)'s lanes: their particle and its state, requested now
-    int q = 0;
-    const PartArgs *B = nullptr;
-    PartState st{};
-    if (phase != 1 && w == 0 && lane < PART_WARPS) {
-        B = locate(blockIdx.x * PART_WARPS + lane, q);
-        if (B) st = load_state(*B, q);
+// The particle update as a launch of its own, one warp per particle:
+//   integrate == 0: forms 1/m, 1/I, weight and reach and bins the particles
+//                   where they are (an upload);
+//   phase 0: the whole update after a sweep_kernel; 1: only the sums of a
+//   strip's bins, to fpart; 2: the rest from the sums in fpart.
+constexpr int PART_WARPS = 8;
+
+static __global__ void __launch_bounds__(PART_WARPS * 32)
+particles_kernel(const __grid_constant__ PartArgs A, int cur, int rot, unsigned next_tag, int integrate, int phase) {
+    const int lane = threadIdx.x & 31, p = blockIdx.x * PART_WARPS + (threadIdx.x >> 5);
+    if (p >= A.bp.np) return;
+    const int nxt = integrate ? cur ^ 1 : cur;
+    const Bins in = bins_at(A.B, cur, rot), out = integrate ? bins_at(A.B, nxt, rot3(rot + 1)) : in;
+    if (!integrate && lane == 0) {
+        const Particles &P = A.P;
+        const double r = P.r[p], rho_s = P.rho_s[p];
+        const double area = 3.14159265358979323846 * r * r, m = rho_s * area, wgt = (rho_s - A.bp.rho_f) * area;
+        P.im[p] = 1.0 / m;
+        P.iI[p] = 1.0 / (0.5 * m * r * r);
+        // (1 - rho_f / rho_s) m g is (rho_s - rho_f) pi r^2 g
+        P.wx[p] = wgt * A.bp.gx;
+        P.wy[p] = wgt * A.bp.gy;
+        P.reach[p] = r + A.ph.cut_d;
+        P.rf[p] = (float)r;
     }
-    if (A && A->integrate && phase != 2) particle_forces(*A, p, lane, sh[w]);
+    __syncwarp();
+    const int comp = component(lane);
+    double f = 0.0;
+    Repulsion c{0.0, 0.0};
+    if (integrate && phase != 2) {
+        c = pair_repulsion(A, p, cur, in, lane);
+        f = hydro_sums<false>(A, p, in, 0u, lane);
+    }
+    double *o = A.fpart ? A.fpart + 5 * (long long)p : nullptr;
     if (phase == 1) {
-        if (A && A->integrate && lane == 0) {
-            double *o = A->fpart + 5 * (long long)p;
-            o[0] = sh[w].fx; o[1] = sh[w].fy; o[2] = sh[w].tq; o[3] = sh[w].cx; o[4] = sh[w].cy;
-        }
+        if (integrate && (lane & 7) == 0 && comp < 3) o[comp] = f;
+        if (integrate && lane == 0) { o[3] = c.x; o[4] = c.y; }
         return;
     }
-    if (phase == 2 && A && lane == 0) {
-        const double *o = A->fpart + 5 * (long long)p;
-        sh[w].fx = o[0]; sh[w].fy = o[1]; sh[w].tq = o[2]; sh[w].cx = o[3]; sh[w].cy = o[4];
+    if (phase == 2) { f = o[comp < 3 ? comp : 0]; c.x = o[3]; c.y = o[4]; }
+    if (integrate) {
+        wall_repulsion(A, p, cur, c);
+        if (lane == 0) { A.fcol[2 * (long long)p] = c.x; A.fcol[2 * (long long)p + 1] = c.y; }
     }
+    particle_advance(A, p, load_particle(A, p, cur, lane), nxt, out, integrate != 0, 0, next_tag, f,
+                     comp == 0 ? c.x : (comp == 1 ? c.y : 0.0), lane);
+}
+
+// ------------------------------------------------------------ fused steps
+// One launch advances a lattice, or every lattice of a batch, by nsteps whole
+// steps.  Most blocks sweep; the first few update the particles: each of their
+// warps owns some, finds their repulsion at the start of a step, then watches
+// their counters and updates each particle as soon as its last partial is
+// counted, while the other blocks sweep on.  (Two other splits were measured
+// on the 4096^2 suspension.  The warp that counts a particle's last partial
+// updates it: a warp held up by one update is then the last to count on its
+// next segment too, one SM ended up with a seventh of all updates, 630 us a
+// step.  Each sweeping warp owns some: the update's registers and calls sit in
+// the sweep's loop, 234 us.)  Between steps the blocks meet at a barrier in
+// device memory (the launch is then cooperative: all blocks are resident).
+//
+// Row segments are dealt by tickets: a warp's first segment is fixed, each
+// further one comes from a counter, taken one segment ahead.  (Dealt
+// round-robin, the warps of the 4096^2 suspension finished their segments
+// between 160 and 220 us into the step.)  The blocks form TICKET_GROUPS
+// groups with a counter each, so that no counter is asked more than once in
+// some ten nanoseconds; a group's segments lie interleaved with the others',
+// which keeps all warps near the same rows.
+constexpr int TICKET_GROUPS = 8;
+
+struct GridSync {               // all 0 between launches
+    unsigned arrived, left;
+    unsigned pad[30];
+    unsigned ticket[3][TICKET_GROUPS][32];      // by step in rotation and group, a cache line each
+};
+
+struct StepRun {
+    int nsteps;
+    int dry;                    // sweep only: no contribution is counted, no particle updated (autotuning)
+    GridSync *sync;
+    int pblocks;                // leading blocks that update particles
+};
+
+// Thread 0 of a block: arrive, then wait until `target` blocks have arrived.
+// Returns false when the bounded wait gave up.
+__device__ __forceinline__ bool sync_blocks(GridSync *g, unsigned target) {
+    asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(&g->arrived) : "memory");
+    unsigned long long t0 = 0;
+    for (;;) {
+        unsigned v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&g->arrived) : "memory");
+        if ((int)(v - target) >= 0) return true;
+        const unsigned long long t = global_ns();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > WAIT_LIMIT_NS) return false;
+    }
+}
+
+// The frame's move by s columns, in place: warps take rows of planes, 32
+// columns at a time in the direction of the move (each value is read before
+// its column is overwritten).
+template <typename T>
+__device__ __noinline__ void shift_rows(T *buf, const Lattice &L, int s, int gw, int nw, int lane) {
+    for (int r = gw; r < 9 * L.ny; r += nw) {
+        T *line = buf + (long long)(r / L.ny) * L.plane + (long long)(r % L.ny) * L.pitch;
+        // the column entering: the far end on a periodic axis, else its neighbour
+        const T enter = __ldcg(line + (s > 0 ? (L.per_x ? 0 : L.nx - 1) : (L.per_x ? L.nx - 1 : 0)));
+        for (int b = 0; b < L.nx; b += 32) {
+            const int x = s > 0 ? b + lane : L.nx - 1 - b - lane;
+            const bool in = x >= 0 && x < L.nx, edge = x + s < 0 || x + s >= L.nx;
+            const T v = in && !edge ? __ldcg(line + x + s) : enter;
+            __syncwarp();
+            if (in) line[x] = v;
+            __syncwarp();
+        }
+    }
+}
+
+// Position in a work list: lattice, row and segment.
+struct Cursor {
+    int lat, y, tx;
+};
+
+// One lattice's work list.
+template <typename T>
+struct OneWork {
+    const SweepArgs<T> &one;
+    const PartArgs &pa;
+    __device__ __forceinline__ const PartArgs &part(int) const { return pa; }
+    __device__ __forceinline__ int items() const { return one.L.ny * one.L.ntx; }
+    __device__ __forceinline__ int tiles() const { return one.L.ntx * one.L.nty; }
+    __device__ __forceinline__ int parts() const { return one.np; }
+    __device__ __forceinline__ const SweepArgs<T> &args(int) const { return one; }
+    __device__ __forceinline__ void seek(Cursor &c, int item) const {
+        c.y = row_of(item, one.ntx_inv, one.L.ntx);
+        c.tx = item - c.y * one.L.ntx;
+    }
+    __device__ __forceinline__ int find_tile(int t, int &lat) const { lat = 0; return t; }
+    __device__ __forceinline__ int find_part(int g, int &lat) const { lat = 0; return g; }
+    // populations and positions read in step st of the launch, and its tile counts
+    __device__ __forceinline__ int parity(int, int st) const { return one.cur ^ (st & 1); }
+    __device__ __forceinline__ int rotation(int, int st) const { return (one.rot + st) % 3; }
+};
+
+// A batch's: the members' segments, tiles and particles, one after another.
+// A warp's items only grow within a step, so its lattice is found by stepping
+// on from the last one (a few lattices at most).
+template <typename T>
+struct BatchWork {
+    const BatchArgs<T> &ba;
+    __device__ __forceinline__ const PartArgs &part(int lat) const { return *ba.a[lat].pa; }
+    __device__ __forceinline__ int items() const { return ba.item_start[ba.n]; }
+    __device__ __forceinline__ int tiles() const { return ba.tile_start[ba.n]; }
+    __device__ __forceinline__ int parts() const { return ba.part_start[ba.n]; }
+    __device__ __forceinline__ const SweepArgs<T> &args(int lat) const { return ba.a[lat]; }
+    __device__ __forceinline__ void seek(Cursor &c, int item) const {
+        while (c.lat + 1 < ba.n && ba.item_start[c.lat + 1] <= item) ++c.lat;
+        const int local = item - ba.item_start[c.lat], ntx = ba.a[c.lat].L.ntx;
+        c.y = row_of(local, ba.a[c.lat].ntx_inv, ntx);
+        c.tx = local - c.y * ntx;
+    }
+    __device__ __forceinline__ int find_tile(int t, int &lat) const {
+        lat = batch_find(ba.tile_start, ba.n, t);
+        return t - ba.tile_start[lat];
+    }
+    __device__ __forceinline__ int find_part(int g, int &lat) const {
+        lat = batch_find(ba.part_start, ba.n, g);
+        return g - ba.part_start[lat];
+    }
+    __device__ __forceinline__ int parity(int lat, int st) const { return ba.a[lat].cur ^ (st & 1); }
+    __device__ __forceinline__ int rotation(int lat, int st) const { return (ba.a[lat].rot + st) % 3; }
+};
+
+// The particle blocks' part of a step: warp pw of npw.
+template <typename WORK>
+__device__ __forceinline__ bool update_particles(const WORK &wk, int st, int shift, int pw, int npw, int lane) {
+    const int total = wk.parts();
+    for (int g = pw; g < total; g += npw) {
+        int lat;
+        const int p = wk.find_part(g, lat);
+        const PartArgs &A = wk.part(lat);
+        Repulsion c = pair_repulsion(A, p, wk.parity(lat, st), bins_at(A.B, wk.parity(lat, st), wk.rotation(lat, st)), lane);
+        wall_repulsion(A, p, wk.parity(lat, st), c);
+        if (lane == 0) {
+            A.fcol[2 * (long long)p] = c.x;
+            A.fcol[2 * (long long)p + 1] = c.y;
+        }
+    }
+    __syncwarp();        // (the same warp reads them below)
+    // up to 32 of the warp's particles at a time, one watched by each lane
+    for (int g0 = pw; g0 < total; g0 += 32 * npw) {
+        const int g = g0 + lane * npw;
+        int lat = 0, p = -1;
+        const int *done = nullptr;
+        if (g < total) {
+            p = wk.find_part(g, lat);
+            const PartArgs &A = wk.part(lat);
+            done = A.B.done + (long long)wk.parity(lat, st) * A.B.parts + p;
+        }
+        unsigned long long t0 = global_ns();
+        while (__any_sync(0xffffffffu, done != nullptr)) {
+            unsigned ready = __ballot_sync(0xffffffffu, done != nullptr && load_done(done) == 0);
+            if (ready == 0) {
+                if (__any_sync(0xffffffffu, global_ns() - t0 > WAIT_LIMIT_NS)) return false;
+                __nanosleep(100);
+                continue;
+            }
+            if (ready >> lane & 1u) done = nullptr;
+            for (; ready; ready &= ready - 1) {
+                const int l = __ffs(ready) - 1;
+                const int q = __shfl_sync(0xffffffffu, p, l), ql = __shfl_sync(0xffffffffu, lat, l);
+                const PartArgs &A = wk.part(ql);
+                const int cur = wk.parity(ql, st), rot = wk.rotation(ql, st);
+                const unsigned tag = wk.args(ql).tag + st;
+                const PartState ps = load_particle(A, q, cur, lane);
+                const int comp = component(lane);
+                const double c = comp < 2 ? __ldcg(A.fcol + 2 * (long long)q + comp) : 0.0;
+                const double f = hydro_sums<true>(A, q, bins_at(A.B, cur, rot), tag, lane);
+                particle_advance(A, q, ps, cur ^ 1, bins_at(A.B, cur ^ 1, rot3(rot + 1)), true, shift, tag + 1, f, c, lane);
+            }
+            t0 = global_ns();
+        }
+    }
+    return true;
+}
+
+template <typename T, bool EDGES, int W, bool PS, typename WORK>
+__device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame, const StepRun &run) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ int s_stop, s_halt;      // a warp gave up; the block leaves (set between barriers)
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    SweepSmem<T, W> sm(smem_raw, warp);
+    Ring ring{sm.bar, 0u, false};
+    if (lane == 0) {
+        mbar_init(ring.bar, 1);
+        mbar_fence_init();
+    }
+    if (threadIdx.x == 0) s_stop = s_halt = 0;
     __syncthreads();
-    if (B) particle_update(*B, q, sh[lane], st);
+    const bool sweeps = (int)blockIdx.x >= run.pblocks;
+    // this block among the sweeping ones, its group and the group's warps
+    const int sb = (int)blockIdx.x - run.pblocks, nsb = (int)gridDim.x - run.pblocks;
+    const int ngroups = nsb < TICKET_GROUPS ? nsb : TICKET_GROUPS;
+    const int group = sb % ngroups, gwarps = (nsb / ngroups + (group < nsb % ngroups)) * W;
+    auto item_of = [&](int k) { return ((k / W) * ngroups + group) * W + (k & (W - 1)); };
+    const int nitems = wk.items();
+    const FieldsOut fo{nullptr, nullptr, nullptr, nullptr};
+    unsigned target = 0;
+
+    for (int st = 0; st < run.nsteps; ++st) {
+        bool timed_out = false;
+        int shift = 0;
+        const int track = frame ? frame->track : -1;    // (a batch's frames stand still)
+        if (track >= 0) {
+            const PartArgs &f = *frame;
+            shift = frame_move(__ldcg((wk.parity(0, st) ? f.P.x[1] : f.P.x[0]) + f.track), f.track_x, f.L.nx, f.L.per_x);
+        }
+        if (!sweeps) {
+            if (!run.dry && !update_particles(wk, st, shift, (int)blockIdx.x * W + warp, run.pblocks * W, lane)) {
+                if (lane == 0) atomicOr(wk.args(0).err, ERR_TIMEOUT);
+                timed_out = true;
+            }
+        } else {
+            Cursor c{0, 0, 0};
+            T wv = T();         // the staged segment's periodic-edge value (wrap_load)
+            int item = item_of((sb / ngroups) * W + warp);
+            bool have = item < nitems;
+            if (have) {
+                wk.seek(c, item);
+                const SweepArgs<T> &a = wk.args(c.lat);
+                const T *src = a.buf[wk.parity(c.lat, st)];
+                const int ys = streamed_row<EDGES>(a.L, c.y);
+                issue_segment<T>(src, a.L, ys, c.tx, sm.stage, ring.bar, lane);
+                wv = wrap_load<T>(src, a.L, ys, c.tx, lane);
+                ring.pending = true;
+            }
+            unsigned *ticket = &run.sync->ticket[st % 3][group][0];
+            if (warp == 0 && lane == 0 && sb < ngroups) run.sync->ticket[(st + 2) % 3][group][0] = 0;
+            if (!run.dry && wk.parts() > 0) {
+                // the counts the step after next adds to
+                for (int t = sb * blockDim.x + threadIdx.x; t < wk.tiles(); t += nsb * blockDim.x) {
+                    int lat;
+                    const int tl = wk.find_tile(t, lat);
+                    const SweepArgs<T> &a = wk.args(lat);
+                    if (a.np > 0) a.B.count[(long long)rot3(wk.rotation(lat, st) + 2) * a.B.tiles + tl] = 0;
+                }
+            }
+            while (have) {
+                int k = 0;
+                if (lane == 0) k = gwarps + (int)atomicAdd(ticket, 1u);
+                item = item_of(__shfl_sync(0xffffffffu, k, 0));
+                have = item < nitems;
+                Cursor nx = c;
+                if (have) wk.seek(nx, item);
+                const SweepArgs<T> &a = wk.args(c.lat), &an = wk.args(nx.lat);
+                const int cur = wk.parity(c.lat, st);
+                if (!sweep_segment<T, MODE_STEP, EDGES, PS, true>(
+                        a, a.buf[cur], a.buf[cur ^ 1], bins_at(a.B, cur, wk.rotation(c.lat, st)), c.y, c.tx, sm.stage,
+                        ring, have, an.buf[wk.parity(nx.lat, st)], an.L, nx.y, nx.tx, sm.crec, sm.cid, wv,
+                        a.tag + st - run.dry, !run.dry, fo, lane)) {
+                    if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+                    timed_out = true;
+                    break;
+                }
+                c = nx;
+            }
+        }
+        if (timed_out) {
+            if (lane == 0) s_stop = 1;
+            // let the copies this warp still has in flight land before the
+            // block releases its shared memory (the wait bounded again)
+            if (ring.pending) mbar_wait_bounded(ring.bar, ring.parity);
+        }
+        const bool more = st + 1 < run.nsteps;
+        if (run.nsteps == 1) break;
+        // ---- every block's populations, bins and positions, before the next
+        // step reads them (its bulk copies in the async proxy)
+        const int meets = shift != 0 ? 2 : (more ? 1 : 0);
+        for (int m = 0; m < meets; ++m) {
+            if (m == 1) {
+                shift_rows<T>(wk.args(0).buf[wk.parity(0, st) ^ 1], wk.args(0).L, shift, (int)blockIdx.x * W + warp,
+                              (int)gridDim.x * W, lane);
+                if (blockIdx.x == 0 && threadIdx.x == 0) *frame->frame_off = __ldcg(frame->frame_off) + shift;
+                if (!more) break;
+            }
+            asm volatile("fence.proxy.async;" ::: "memory");
+            __syncthreads();
+            target += gridDim.x;
+            if (threadIdx.x == 0) {
+                s_halt = s_stop;
+                if (!s_halt && !sync_blocks(run.sync, target)) {
+                    atomicOr(wk.args(0).err, ERR_TIMEOUT);
+                    s_halt = 1;
+                }
+            }
+            __syncthreads();
+            if (s_halt) break;
+            asm volatile("fence.proxy.async;" ::: "memory");
+        }
+        if (s_halt) break;
+    }
+    // the last block out leaves the counters as it found them
     __syncthreads();
-    if (A) particle_bin(*A, p, lane, sh[w]);
+    if (threadIdx.x == 0 && atomicAdd(&run.sync->left, 1u) == gridDim.x - 1) {
+        run.sync->arrived = 0;
+        run.sync->left = 0;
+        for (int q = 0; q < 3; ++q)
+            for (int g = 0; g < TICKET_GROUPS; ++g) run.sync->ticket[q][g][0] = 0;
+    }
+}
+
+template <typename T, bool EDGES, int W, bool PS = false>
+__global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
+step_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ PartArgs pa,
+            const __grid_constant__ StepRun run) {
+    const OneWork<T> wk{one, pa};
+    run_steps<T, EDGES, W, PS>(wk, &pa, run);
+}
+
+template <typename T, int W>
+__global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
+step_batch_kernel(const __grid_constant__ BatchArgs<T> ba, const __grid_constant__ StepRun run) {
+    const BatchWork<T> wk{ba};
+    run_steps<T, true, W, false>(wk, nullptr, run);
 }
 
 // ------------------------------------------------------------ conversions

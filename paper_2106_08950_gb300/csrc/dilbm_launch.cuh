@@ -6,22 +6,32 @@
 // code in the same arithmetic whatever the shape, so the autotuner may pick
 // any shape without changing a single result bit.
 //
-// The launchers of the step sweep are compiled once per storage type, each
-// in its own translation unit (dilbm_launch_f32.cu, _f16.cu, _bf16.cu).
+// The launchers are compiled once per storage type, each in its own
+// translation unit (dilbm_launch_f32.cu, _f16.cu, _bf16.cu).
 #pragma once
 #include "dilbm_kernels.cuh"
+
+#include <algorithm>
 
 namespace dilbm {
 
 struct SweepShape {
-    int warps = SWEEP_WARPS;    // rows in flight per block: 2, 4 or 8
+    int warps = 4;              // rows in flight per block: 2, 4 or 8
     int blocks_per_sm = 0;      // persistent blocks per SM; 0: as many as fit
 };
+
+constexpr SweepShape PS_SHAPE{SWEEP_WARPS, 0};     // the shape a PS-LBM context reports
+constexpr int PS_WARPS = 4;                        // warps per block its fused steps are compiled for
 
 constexpr int SHAPE_WARPS[3] = {2, 4, 8};
 
 __host__ inline bool shape_valid(const SweepShape &s) {
     return (s.warps == 2 || s.warps == 4 || s.warps == 8) && s.blocks_per_sm >= 0;
+}
+
+// row_of's multiplier: floor(2^32 / ntx) + 1 (unused for ntx == 1).
+inline unsigned ntx_inverse(int ntx) {
+    return ntx > 1 ? (unsigned)((1ull << 32) / (unsigned long long)ntx) + 1u : 0u;
 }
 
 // Blocks of `kern` (W warps, `smem` bytes of dynamic shared memory) resident
@@ -45,7 +55,7 @@ cudaError_t occupancy_of(K kern, int warps, size_t smem, int *cache, int *per_sm
 }
 
 // Persistent grid: num_sms x blocks per SM (capped by the shape and by the
-// kernel's occupancy), but no more blocks than the row segments need.
+// kernel's occupancy), but no more blocks than the work list needs.
 inline long long persistent_grid(long long items, int warps, int per_sm, int num_sms, const SweepShape &sh) {
     const int bps = sh.blocks_per_sm > 0 && sh.blocks_per_sm < per_sm ? sh.blocks_per_sm : per_sm;
     long long blocks = (long long)num_sms * bps;
@@ -54,98 +64,89 @@ inline long long persistent_grid(long long items, int warps, int per_sm, int num
     return blocks > 0 ? blocks : 1;
 }
 
-template <typename T, bool EDGES, int W>
-cudaError_t step_variant(const SweepArgs<T> &a, const SweepShape &sh, int num_sms, cudaStream_t st, bool query,
-                         int *per_sm_out) {
+// The blocks of a fused launch: sweeping blocks, and particle blocks in front
+// of them -- a warp per particle, up to a tenth of the resident blocks (at
+// 2048 discs on 4096^2 each warp then has about seven updates of a few
+// microseconds in a step of 200).
+inline long long fused_grid(long long items, long long parts, int warps, int per_sm, int num_sms, const SweepShape &sh,
+                            int *pblocks) {
+    const long long most = persistent_grid(1LL << 40, warps, per_sm, num_sms, sh);
+    const long long pb = std::min((parts + warps - 1) / warps, std::max(most / 10, 1LL));
+    *pblocks = (int)pb;
+    const long long sweep = persistent_grid(items, warps, per_sm, num_sms, sh);
+    return std::max(std::min(sweep, most - pb), 1LL) + pb;
+}
+
+// Blocks of a fused launch wait for one another (particle blocks for the
+// sweeping ones, and all of them between steps), so it is launched
+// cooperatively: the driver starts it only with every block resident.
+inline cudaError_t launch_steps(const void *kern, void **args, long long blocks, int warps, size_t smem, cudaStream_t st) {
+    return cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, st);
+}
+
+template <typename T, bool EDGES, int W, bool PS>
+cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run, const SweepShape &sh, int num_sms,
+                         cudaStream_t st, int *per_sm_out) {
     static int cache[64] = {};
     constexpr size_t smem = sweep_smem_bytes<T, W>();
+    auto *kern = step_kernel<T, EDGES, W, PS>;
     int per_sm = 1;
-    cudaError_t e = occupancy_of(sweep_kernel<T, MODE_STEP, EDGES, W>, W, smem, cache, &per_sm);
-    if (e != cudaSuccess || query) {
+    cudaError_t e = occupancy_of(kern, W, smem, cache, &per_sm);
+    if (e != cudaSuccess || per_sm_out) {
         if (per_sm_out) *per_sm_out = per_sm;
         return e;
     }
-    const long long items = (long long)a.L.ny * a.L.ntx;
-    const long long blocks = persistent_grid(items, W, per_sm, num_sms, sh);
-    sweep_kernel<T, MODE_STEP, EDGES, W><<<(unsigned)blocks, W * 32, smem, st>>>(a);
-    return cudaGetLastError();
+    const long long blocks = fused_grid((long long)a.L.ny * a.L.ntx, a.np, W, per_sm, num_sms, sh, &run.pblocks);
+    void *p[3] = {const_cast<SweepArgs<T> *>(&a), const_cast<PartArgs *>(&pa), &run};
+    return launch_steps((const void *)kern, p, blocks, W, smem, st);
 }
 
 template <typename T, int W>
-cudaError_t batch_variant(const BatchArgs<T> &ba, const SweepShape &sh, int num_sms, cudaStream_t st, bool query,
+cudaError_t batch_variant(const BatchArgs<T> &ba, StepRun run, const SweepShape &sh, int num_sms, cudaStream_t st,
                           int *per_sm_out) {
     static int cache[64] = {};
     constexpr size_t smem = sweep_smem_bytes<T, W>();
+    auto *kern = step_batch_kernel<T, W>;
     int per_sm = 1;
-    cudaError_t e = occupancy_of(sweep_batch_kernel<T, MODE_STEP, W>, W, smem, cache, &per_sm);
-    if (e != cudaSuccess || query) {
+    cudaError_t e = occupancy_of(kern, W, smem, cache, &per_sm);
+    if (e != cudaSuccess || per_sm_out) {
         if (per_sm_out) *per_sm_out = per_sm;
         return e;
     }
-    const long long blocks = persistent_grid(ba.item_start[ba.n], W, per_sm, num_sms, sh);
-    sweep_batch_kernel<T, MODE_STEP, W><<<(unsigned)blocks, W * 32, smem, st>>>(ba);
-    return cudaGetLastError();
+    const long long blocks = fused_grid(ba.item_start[ba.n], ba.part_start[ba.n], W, per_sm, num_sms, sh, &run.pblocks);
+    void *p[2] = {const_cast<BatchArgs<T> *>(&ba), &run};
+    return launch_steps((const void *)kern, p, blocks, W, smem, st);
 }
 
-// The PS-LBM step sweep (the paper's comparison method), in the default shape.
-template <typename T, bool EDGES>
-cudaError_t ps_variant(const SweepArgs<T> &a, int num_sms, cudaStream_t st) {
+// The sweep without the particle update, in the default shape (a strip's
+// step; MODE_FIELDS: the macroscopic fields instead of a step).
+template <typename T, int MODE, bool EDGES, bool PS>
+cudaError_t sweep_variant(const SweepArgs<T> &a, const FieldsOut &fo, int num_sms, cudaStream_t st) {
     static int cache[64] = {};
     constexpr size_t smem = sweep_smem_bytes<T>();
     int per_sm = 1;
-    cudaError_t e = occupancy_of(sweep_kernel<T, MODE_STEP, EDGES, SWEEP_WARPS, true>, SWEEP_WARPS, smem, cache, &per_sm);
+    cudaError_t e = occupancy_of(sweep_kernel<T, MODE, EDGES, PS>, SWEEP_WARPS, smem, cache, &per_sm);
     if (e != cudaSuccess) return e;
-    const long long blocks = persistent_grid((long long)a.L.ny * a.L.ntx, SWEEP_WARPS, per_sm, num_sms, SweepShape{});
-    sweep_kernel<T, MODE_STEP, EDGES, SWEEP_WARPS, true><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, st>>>(a);
+    const long long blocks = persistent_grid((long long)a.L.ny * a.L.ntx, SWEEP_WARPS, per_sm, num_sms, PS_SHAPE);
+    sweep_kernel<T, MODE, EDGES, PS><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, st>>>(a, fo);
     return cudaGetLastError();
 }
 
-// Generic bodies of the per-storage launchers.
+// Per-storage launchers, instantiated in dilbm_launch_f32.cu, _f16.cu and
+// _bf16.cu.  per_sm != NULL: launch nothing, return the kernel's resident
+// blocks per SM there.
 template <typename T>
-cudaError_t step_sweep_impl(const SweepArgs<T> &a, bool edges, const SweepShape &sh, int num_sms, cudaStream_t st,
-                            bool query, int *per_sm) {
-    switch (sh.warps) {
-    case 2: return edges ? step_variant<T, true, 2>(a, sh, num_sms, st, query, per_sm)
-                         : step_variant<T, false, 2>(a, sh, num_sms, st, query, per_sm);
-    case 4: return edges ? step_variant<T, true, 4>(a, sh, num_sms, st, query, per_sm)
-                         : step_variant<T, false, 4>(a, sh, num_sms, st, query, per_sm);
-    case 8: return edges ? step_variant<T, true, 8>(a, sh, num_sms, st, query, per_sm)
-                         : step_variant<T, false, 8>(a, sh, num_sms, st, query, per_sm);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-template <typename T>
-cudaError_t batch_sweep_impl(const BatchArgs<T> &ba, const SweepShape &sh, int num_sms, cudaStream_t st, bool query,
-                             int *per_sm) {
-    switch (sh.warps) {
-    case 2: return batch_variant<T, 2>(ba, sh, num_sms, st, query, per_sm);
-    case 4: return batch_variant<T, 4>(ba, sh, num_sms, st, query, per_sm);
-    case 8: return batch_variant<T, 8>(ba, sh, num_sms, st, query, per_sm);
-    default: return cudaErrorInvalidValue;
-    }
-}
-
-// Per-storage launchers (defined in dilbm_launch_f32.cu, _f16.cu, _bf16.cu).
-// query != 0: launch nothing, return the kernel's resident blocks per SM in
-// *per_sm.
-template <typename T>
-cudaError_t launch_step_sweep(const SweepArgs<T> &a, bool edges, const SweepShape &sh, int num_sms, cudaStream_t st,
-                              bool query = false, int *per_sm = nullptr);
-template <typename T>
-cudaError_t launch_batch_sweep(const BatchArgs<T> &ba, const SweepShape &sh, int num_sms, cudaStream_t st,
-                               bool query = false, int *per_sm = nullptr);
-
-template <> cudaError_t launch_step_sweep<float>(const SweepArgs<float> &, bool, const SweepShape &, int, cudaStream_t, bool, int *);
-template <> cudaError_t launch_step_sweep<__half>(const SweepArgs<__half> &, bool, const SweepShape &, int, cudaStream_t, bool, int *);
-template <> cudaError_t launch_step_sweep<__nv_bfloat16>(const SweepArgs<__nv_bfloat16> &, bool, const SweepShape &, int, cudaStream_t, bool, int *);
-template <typename T>
-cudaError_t launch_step_sweep_ps(const SweepArgs<T> &a, bool edges, int num_sms, cudaStream_t st);
-template <> cudaError_t launch_step_sweep_ps<float>(const SweepArgs<float> &, bool, int, cudaStream_t);
-template <> cudaError_t launch_step_sweep_ps<__half>(const SweepArgs<__half> &, bool, int, cudaStream_t);
-template <> cudaError_t launch_step_sweep_ps<__nv_bfloat16>(const SweepArgs<__nv_bfloat16> &, bool, int, cudaStream_t);
-template <> cudaError_t launch_batch_sweep<float>(const BatchArgs<float> &, const SweepShape &, int, cudaStream_t, bool, int *);
-template <> cudaError_t launch_batch_sweep<__half>(const BatchArgs<__half> &, const SweepShape &, int, cudaStream_t, bool, int *);
-template <> cudaError_t launch_batch_sweep<__nv_bfloat16>(const BatchArgs<__nv_bfloat16> &, const SweepShape &, int, cudaStream_t, bool, int *);
+struct Launch {
+    // fused steps of one lattice (PS-LBM: in the default shape)
+    static cudaError_t steps(const SweepArgs<T> &a, const PartArgs &pa, const StepRun &run, bool edges, bool ps, const SweepShape &sh,
+                             int num_sms, cudaStream_t st, int *per_sm = nullptr);
+    // fused steps of a batch
+    static cudaError_t batch(const BatchArgs<T> &ba, const StepRun &run, const SweepShape &sh, int num_sms,
+                             cudaStream_t st, int *per_sm = nullptr);
+    // a strip's sweep
+    static cudaError_t sweep(const SweepArgs<T> &a, bool edges, bool ps, int num_sms, cudaStream_t st);
+    static cudaError_t fields(const SweepArgs<T> &a, const FieldsOut &fo, bool edges, bool ps, int num_sms,
+                              cudaStream_t st);
+};
 
 }  // namespace dilbm

@@ -1,25 +1,6 @@
-// Step-sweep and batched-sweep launchers for __half storage, every launch
-// shape (warps per block 2, 4, 8; with and without edge handling).  One
-// translation unit per storage type so that the library compiles in parallel.
-#include "dilbm_launch.cuh"
+// The launchers for __half storage: every launch shape (2, 4 or 8 warps per
+// block; with and without edge handling).  One translation unit per storage
+// type so that the library compiles in parallel.
+#include "dilbm_launch_impl.cuh"
 
-namespace dilbm {
-
-template <>
-cudaError_t launch_step_sweep<__half>(const SweepArgs<__half> &a, bool edges, const SweepShape &sh, int num_sms,
-                                   cudaStream_t st, bool query, int *per_sm) {
-    return step_sweep_impl<__half>(a, edges, sh, num_sms, st, query, per_sm);
-}
-
-template <>
-cudaError_t launch_batch_sweep<__half>(const BatchArgs<__half> &ba, const SweepShape &sh, int num_sms, cudaStream_t st,
-                                    bool query, int *per_sm) {
-    return batch_sweep_impl<__half>(ba, sh, num_sms, st, query, per_sm);
-}
-
-template <>
-cudaError_t launch_step_sweep_ps<__half>(const SweepArgs<__half> &a, bool edges, int num_sms, cudaStream_t st) {
-    return edges ? ps_variant<__half, true>(a, num_sms, st) : ps_variant<__half, false>(a, num_sms, st);
-}
-
-}  // namespace dilbm
+template struct dilbm::Launch<__half>;

@@ -12,7 +12,7 @@
 // file-scope static device array of fixed size, declared below.  The caller
 // passes the populations, the particles and the force output.
 #include "dilbm.h"
-#include "dilbm_kernels.cuh"
+#include "dilbm_launch.cuh"
 
 #include <cmath>
 #include <string>
@@ -31,15 +31,16 @@ static_assert(DILBM_STATIC_PITCH(1) == 32 && DILBM_STATIC_PITCH(33) == 64, "pitc
 
 // Byte offsets of the scratch regions (each 256-byte aligned).
 constexpr size_t align256(size_t n) { return (n + 255) / 256 * 256; }
-constexpr size_t OFF_COUNT = 0;                                                    // int [2][tiles]
-constexpr size_t OFF_IDS = OFF_COUNT + align256(2 * sizeof(int) * S_MAX_TILES);    // int [2][tiles*MAXC]
-constexpr size_t OFF_REC = OFF_IDS + align256(2 * sizeof(int) * S_MAX_TILES * MAXC);
+constexpr size_t OFF_COUNT = 0;                                                    // int [3][tiles]
+constexpr size_t OFF_IDS = OFF_COUNT + align256(3 * sizeof(int) * S_MAX_TILES);    // int2 [2][tiles*MAXC]
+constexpr size_t OFF_REC = OFF_IDS + align256(2 * sizeof(int2) * S_MAX_TILES * MAXC);
 constexpr size_t OFF_PSLOT = OFF_REC + align256(2 * sizeof(float4) * S_MAX_TILES * MAXC * NREC);
 constexpr size_t OFF_NPSLOT = OFF_PSLOT + align256(2 * sizeof(int) * S_MAX_PARTICLES * MAXT);
-constexpr size_t OFF_PARTIAL = OFF_NPSLOT + align256(2 * sizeof(int) * S_MAX_PARTICLES);
-constexpr size_t OFF_PD = OFF_PARTIAL + align256(sizeof(float4) * S_MAX_TILES * MAXC * TILE_H);
-constexpr size_t OFF_PF = OFF_PD + align256(10 * sizeof(double) * S_MAX_PARTICLES);
-constexpr size_t OFF_FIXED = OFF_PF + align256(4 * sizeof(float) * S_MAX_PARTICLES);
+constexpr size_t OFF_DONE = OFF_NPSLOT + align256(2 * sizeof(int) * S_MAX_PARTICLES);
+constexpr size_t OFF_PARTIAL = OFF_DONE + align256(2 * sizeof(int) * S_MAX_PARTICLES);
+constexpr size_t OFF_PD = OFF_PARTIAL + align256(sizeof(float4) * S_MAX_PARTICLES * MAXT * TILE_H);
+constexpr size_t OFF_PF = OFF_PD + align256(15 * sizeof(double) * S_MAX_PARTICLES);
+constexpr size_t OFF_FIXED = OFF_PF + align256(5 * sizeof(float) * S_MAX_PARTICLES);
 constexpr size_t OFF_FCOL = OFF_FIXED + align256(sizeof(int) * S_MAX_PARTICLES);
 constexpr size_t OFF_ERR = OFF_FCOL + align256(2 * sizeof(double) * S_MAX_PARTICLES);
 constexpr size_t SCRATCH_BYTES = OFF_ERR + 256;
@@ -192,19 +193,23 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
     bp.eps_w = g->wan_turek[2];
     bp.eps_w2 = g->wan_turek[3];
     bp.xi = g->wan_turek[4];
+    bp.xi_f = (float)bp.xi;
+    bp.len[0] = g->nx;
+    bp.len[1] = g->ny;
 
     // ---- the scratch regions
     unsigned char *s = nullptr;
     int rc = scratch_address(&s);
     if (rc) return rc;
-    Bins bins[2]{};
-    for (int b = 0; b < 2; ++b) {
-        bins[b].count = reinterpret_cast<int *>(s + OFF_COUNT) + b * S_MAX_TILES;
-        bins[b].ids = reinterpret_cast<int *>(s + OFF_IDS) + (size_t)b * S_MAX_TILES * MAXC;
-        bins[b].rec = reinterpret_cast<float4 *>(s + OFF_REC) + (size_t)b * S_MAX_TILES * MAXC * NREC;
-        bins[b].pslot = reinterpret_cast<int *>(s + OFF_PSLOT) + (size_t)b * S_MAX_PARTICLES * MAXT;
-        bins[b].npslot = reinterpret_cast<int *>(s + OFF_NPSLOT) + b * S_MAX_PARTICLES;
-    }
+    BinSet B{};
+    B.tiles = S_MAX_TILES;
+    B.parts = S_MAX_PARTICLES;
+    B.count = reinterpret_cast<int *>(s + OFF_COUNT);
+    B.ids = reinterpret_cast<int2 *>(s + OFF_IDS);
+    B.rec = reinterpret_cast<float4 *>(s + OFF_REC);
+    B.pslot = reinterpret_cast<int *>(s + OFF_PSLOT);
+    B.npslot = reinterpret_cast<int *>(s + OFF_NPSLOT);
+    B.done = reinterpret_cast<int *>(s + OFF_DONE);
     float4 *partial = reinterpret_cast<float4 *>(s + OFF_PARTIAL);
     double *pd = reinterpret_cast<double *>(s + OFF_PD);
     float *pf = reinterpret_cast<float *>(s + OFF_PF);
@@ -212,34 +217,29 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
     Particles P{};
     P.x[0] = pd; P.x[1] = pd + M; P.y[0] = pd + 2 * M; P.y[1] = pd + 3 * M;
     P.r = pd + 4 * M; P.ux = pd + 5 * M; P.uy = pd + 6 * M; P.omega = pd + 7 * M;
-    P.theta = pd + 8 * M; P.rho_s = pd + 9 * M;
+    P.theta = pd + 8 * M; P.rho_s = pd + 9 * M; P.im = pd + 10 * M; P.iI = pd + 11 * M;
+    P.wx = pd + 12 * M; P.wy = pd + 13 * M; P.reach = pd + 14 * M; P.rf = pf + 4 * M;
     P.xf[0] = pf; P.xf[1] = pf + M; P.yf[0] = pf + 2 * M; P.yf[1] = pf + 3 * M;
     P.fixed = reinterpret_cast<int *>(s + OFF_FIXED);
     double *fcol = reinterpret_cast<double *>(s + OFF_FCOL);
     int *err = reinterpret_cast<int *>(s + OFF_ERR);
 
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    // what must start at zero: both bin counts and the error word
-    S_CUDA(cudaMemsetAsync(bins[0].count, 0, sizeof(int) * 2 * S_MAX_TILES, st));
+    // what must start at zero: the bin counts and the error word
+    S_CUDA(cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * S_MAX_TILES, st));
     S_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
 
-    auto part_args = [&](int pin, int pout, int integrate, const Bins &bin_in, const Bins &bin_out) {
-        PartArgs a{};
-        a.L = L;
-        a.ph = ph;
-        a.P = P;
-        a.bp = bp;
-        a.bin_in = bin_in;
-        a.bin_out = bin_out;
-        a.partial = partial;
-        a.pin = pin;
-        a.pout = pout;
-        a.integrate = integrate;
-        a.force = force;
-        a.fcol = fcol;
-        a.err = err;
-        return a;
-    };
+    PartArgs pa{};
+    pa.L = L;
+    pa.ph = ph;
+    pa.P = P;
+    pa.bp = bp;
+    pa.B = B;
+    pa.partial = partial;
+    pa.force = force;
+    pa.fcol = fcol;
+    pa.err = err;
+    const int pblocks = (np + PART_WARPS - 1) / PART_WARPS;
     if (np > 0) {
         particles_in_kernel<<<(np + 127) / 128, 128, 0, st>>>(particles, P, np, L.nx, L.ny, L.per_x, L.per_y,
                                                               ph.cut_d, err);
@@ -255,8 +255,7 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
                                                 "velocities, or a phi tail reaching more than " +
                                                     std::to_string(MAXT) + " tiles; nothing was changed");
         // bin the particles where they are (positions copy 0, bins 0)
-        particles_kernel<false><<<(np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, st>>>(part_args(0, 0, 0, bins[0], bins[0]),
-                                                                       nullptr, BatchIndex{});
+        particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, 0, 0u, 0, 0);
         S_CUDA(cudaGetLastError());
     }
 
@@ -264,35 +263,21 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
     int dev = 0, sms = 1;
     S_CUDA(cudaGetDevice(&dev));
     S_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t smem = sweep_smem_bytes<float>();
-    const long long items = (long long)L.ny * L.ntx;
-    long long blocks = 2LL * sms;
-    const long long need = (items + SWEEP_WARPS - 1) / SWEEP_WARPS;
-    if (blocks > need) blocks = need;
     SweepArgs<float> sa{};
-    sa.src = f_in + GUARD;
-    sa.dst = f_out + GUARD;
+    sa.buf[0] = const_cast<float *>(f_in) + GUARD;     // (parity 0: read only)
+    sa.buf[1] = f_out + GUARD;
     sa.L = L;
     sa.ph = ph;
-    sa.B = bins[0];
+    sa.B = B;
     sa.partial = partial;
-    sa.clear = np > 0 ? bins[1].count : nullptr;
     sa.err = err;
-    if (L.per_x && L.per_y) {
-        S_CUDA(cudaFuncSetAttribute(sweep_kernel<float, MODE_STEP, false>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sweep_kernel<float, MODE_STEP, false><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, st>>>(sa);
-    } else {
-        S_CUDA(cudaFuncSetAttribute(sweep_kernel<float, MODE_STEP, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sweep_kernel<float, MODE_STEP, true><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, st>>>(sa);
-    }
-    S_CUDA(cudaGetLastError());
+    sa.np = np;
+    sa.ntx_inv = ntx_inverse(L.ntx);
+    S_CUDA(Launch<float>::sweep(sa, !(L.per_x && L.per_y), false, sms, st));
 
     if (np > 0) {
         // force reduction, Wan-Turek, Newton-Euler (positions copy 0 -> 1)
-        particles_kernel<false><<<(np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, st>>>(part_args(0, 1, 1, bins[0], bins[1]),
-                                                                       nullptr, BatchIndex{});
+        particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, 0, 0u, 1, 0);
         S_CUDA(cudaGetLastError());
         particles_out_kernel<<<(np + 127) / 128, 128, 0, st>>>(particles, P, np);
         S_CUDA(cudaGetLastError());
