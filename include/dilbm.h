@@ -139,8 +139,9 @@ int dilbm_create(const dilbm_grid *grid, dilbm_lattice lattice, double tau,
  * a per-particle FP64 force/torque reduction and a rigid-body update.
  * Asynchronous: returns once the work is queued; errors raised on the device
  * (UNSTABLE, OVERFLOW) surface at the next dilbm_sync().  One cooperative
- * launch runs many steps (about 2^27 node updates); with PS-LBM, while timing,
- * and while the caller is capturing the context's stream, one step.
+ * launch runs many steps (about 2^27 node updates); with PS-LBM and while
+ * timing, one step.  Launches may be recorded into a graph by the caller: an
+ * even number of steps may be replayed any number of times.
  */
 int dilbm_step(dilbm_ctx *ctx, long long nsteps);
 

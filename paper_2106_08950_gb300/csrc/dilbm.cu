@@ -49,12 +49,10 @@ struct dilbm_ctx {
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;
     Particles P{};
-    unsigned tag = 0;                 // step number, marks the step's force partials
-    int rot = 0;                      // which of the three tile-count arrays the next step reads
     BinSet B{};                       // tile bins
     float4 *partial = nullptr;        // per particle, tile of its list and row: force / torque partials
     PartArgs *pa = nullptr;           // device: the particle update's arguments (push_part_args)
-    GridSync *sync = nullptr;         // device: the barrier of launches over several steps
+    GridSync *sync = nullptr;         // device: the barrier of launches over several steps, and the step clock
     double *force = nullptr, *fcol = nullptr;
     double *fsum = nullptr;           // per particle: sum of (Fx, Fy, T) since the last reset
     long long fsum_steps = 0;
@@ -220,6 +218,7 @@ PartArgs particle_args(const dilbm_ctx *c) {
     a.fcol = c->fcol;
     a.fsum = c->fsum;
     a.err = c->err;
+    a.clock = c->strip ? nullptr : &c->sync->clock;
     a.track = c->track;
     a.track_x = c->track_x;
     a.frame_off = c->frame_off;
@@ -246,7 +245,6 @@ int launch_cover(dilbm_ctx *c, int pos) {
 // (integrate == 0), or a phase of a strip's step.
 int launch_particles(dilbm_ctx *c, int integrate, int phase = 0) {
     particles_kernel<<<(c->np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, c->stream>>>(particle_args(c), c->cur,
-                                                                                              c->rot, integrate ? c->tag + 1 : c->tag,
                                                                                               integrate, phase);
     DILBM_CUDA(cudaGetLastError());
     c->launches += 1;
@@ -339,7 +337,9 @@ int upload_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
     DILBM_CUDA(cudaMemcpyAsync(c->P.r, h + 2 * np, sizeof(double) * 6 * np, cudaMemcpyHostToDevice, c->stream));
     DILBM_CUDA(cudaMemcpyAsync(c->P.fixed, fx, sizeof(int) * np, cudaMemcpyHostToDevice, c->stream));
     DILBM_CUDA(cudaEventRecord(c->up_done, c->stream));
-    DILBM_CUDA(cudaMemsetAsync(c->B.count + (size_t)c->rot * c->ntiles, 0, sizeof(int) * c->ntiles, c->stream));
+    clear_counts_kernel<<<(c->ntiles + 255) / 256, 256, 0, c->stream>>>(c->B, c->strip ? nullptr : &c->sync->clock, c->cur);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
     return launch_particles(c, 0);
 }
 
@@ -353,11 +353,10 @@ SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     a.B = c->B;
     a.partial = c->partial;
     a.err = c->err;
+    a.clock = c->strip ? nullptr : &c->sync->clock;
     a.pa = c->np > 0 ? c->pa : nullptr;
     a.np = c->np;
     a.cur = c->cur;
-    a.rot = c->rot;
-    a.tag = c->tag;
     a.ntx_inv = ntx_inverse(c->L.ntx);
     return a;
 }
@@ -405,8 +404,6 @@ int launch_strip_sweep(dilbm_ctx *c) {
 // The state the next step starts from, k steps on.
 void advance(dilbm_ctx *c, int k) {
     c->cur ^= k & 1;
-    c->rot = (c->rot + k) % 3;
-    c->tag += (unsigned)k;
     c->fsum_steps += k;
 }
 
@@ -849,14 +846,9 @@ int dilbm_step(dilbm_ctx *c, long long nsteps) {
     if (!c || nsteps < 0) return fail(DILBM_ERR_INVALID_ARG, "bad context or step count");
     if (c->strip) return fail(DILBM_ERR_INVALID_ARG, "a strip steps through dilbm_strip_begin / dilbm_strip_end");
     // several steps per launch; one per launch where timing brackets each
-    // step, the PS tables follow each step (made by the particle warps, a
-    // table took 20 us and the step 283 us instead of 237), or the caller is
-    // capturing the stream
-    long long most = c->method == DILBM_METHOD_PS ? 1 : steps_per_launch((double)c->L.nx * c->L.ny);
-    if (most > 1 && nsteps > 1 && c->stream != nullptr && c->stream != cudaStreamLegacy) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) most = 1;
-    }
+    // step, or the PS tables follow each step (made by the particle warps, a
+    // table took 20 us and the step 283 us instead of 237)
+    const long long most = c->method == DILBM_METHOD_PS ? 1 : steps_per_launch((double)c->L.nx * c->L.ny);
     for (long long t = 0; t < nsteps;) {
         const int k = (int)std::min(most, nsteps - t);
         const int rc = c->timing ? timed_step(c) : launch_fused(c, k);

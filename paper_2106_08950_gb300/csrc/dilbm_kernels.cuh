@@ -196,6 +196,15 @@ struct Bins {                   // one step's view
     int *done;                  // per particle: minus the partials its update still waits for
 };
 
+// The step a lattice stands at, in device memory: fused steps advance it, so
+// that launches recorded into a graph find it whatever ran before them.
+// (Contexts without fused steps, a strip's and the static step's, have none:
+// their counts rotate by parity.)
+struct StepClock {
+    unsigned tag;               // step number, marks the step's force partials
+    int rot;                    // which of the three tile-count arrays the step reads
+};
+
 struct BinSet {
     int *count;                 // 3 arrays of `tiles`
     int2 *ids;                  // 2 x tiles x MAXC
@@ -722,9 +731,9 @@ struct SweepArgs {
     float4 *partial;            // force / torque partials and tag: per particle, tile of its list and row
     int *err;                   // the lattice's error word
     const PartArgs *pa;         // the particle update's arguments (device memory; batches)
+    StepClock *clock;           // (null: see StepClock)
     int np;                     // particles (0: no bins to read)
-    int cur, rot;               // parity and count rotation of the launch's first step
-    unsigned tag;               // and its tag (a step number)
+    int cur;                    // parity of the launch's first step
     unsigned ntx_inv;           // floor(2^32 / ntx) + 1 (saturated), see row_of
 };
 
@@ -1236,10 +1245,10 @@ sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ F
     const Lattice &L = one.L;
     const T *src = one.buf[one.cur];
     T *dst = one.buf[one.cur ^ 1];
-    const Bins bins = bins_at(one.B, one.cur, one.rot);
+    const Bins bins = bins_at(one.B, one.cur, one.clock ? __ldcg(&one.clock->rot) : one.cur);
     // the next step's bins start empty (nothing reads them during this sweep)
     if (MODE == MODE_STEP && one.np > 0) {
-        int *clear = one.B.count + (long long)rot3(one.rot + 1) * one.B.tiles;
+        int *clear = one.B.count + (long long)(one.cur ^ 1) * one.B.tiles;
         for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < L.ntx * L.nty; t += gridDim.x * blockDim.x) clear[t] = 0;
     }
     const int nitems = L.ny * L.ntx;
@@ -1304,6 +1313,7 @@ struct PartArgs {
     double *force, *fcol;
     double *fsum;               // nullable: running sum of (Fx, Fy, T) over integrating steps
     int *err;
+    StepClock *clock = nullptr;       // (null: see StepClock)
     int track = -1;             // moving frame: tracked particle, -1 (the default) when off
     double track_x = 0.0;       // its reference x
     long long *frame_off = nullptr;   // columns the frame has moved
@@ -1720,6 +1730,12 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
     }
 }
 
+// An upload's binning starts from empty tiles.
+static __global__ void clear_counts_kernel(BinSet B, const StepClock *clock, int cur) {
+    int *count = B.count + (long long)(clock ? __ldcg(&clock->rot) : cur) * B.tiles;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < B.tiles; t += gridDim.x * blockDim.x) count[t] = 0;
+}
+
 // The particle update as a launch of its own, one warp per particle:
 //   integrate == 0: forms 1/m, 1/I, weight and reach and bins the particles
 //                   where they are (an upload);
@@ -1728,11 +1744,12 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
 constexpr int PART_WARPS = 8;
 
 static __global__ void __launch_bounds__(PART_WARPS * 32)
-particles_kernel(const __grid_constant__ PartArgs A, int cur, int rot, unsigned next_tag, int integrate, int phase) {
+particles_kernel(const __grid_constant__ PartArgs A, int cur, int integrate, int phase) {
     const int lane = threadIdx.x & 31, p = blockIdx.x * PART_WARPS + (threadIdx.x >> 5);
     if (p >= A.bp.np) return;
     const int nxt = integrate ? cur ^ 1 : cur;
-    const Bins in = bins_at(A.B, cur, rot), out = integrate ? bins_at(A.B, nxt, rot3(rot + 1)) : in;
+    const Bins in = bins_at(A.B, cur, A.clock ? __ldcg(&A.clock->rot) : cur), out = integrate ? bins_at(A.B, nxt, nxt) : in;
+    const unsigned next_tag = A.clock ? __ldcg(&A.clock->tag) : 0u;
     if (!integrate && lane == 0) {
         const Particles &P = A.P;
         const double r = P.r[p], rho_s = P.rho_s[p];
@@ -1790,9 +1807,10 @@ particles_kernel(const __grid_constant__ PartArgs A, int cur, int rot, unsigned 
 // which keeps all warps near the same rows.
 constexpr int TICKET_GROUPS = 8;
 
-struct GridSync {               // all 0 between launches
+struct GridSync {               // all 0 between launches, but for the clock
     unsigned arrived, left;
-    unsigned pad[30];
+    StepClock clock;            // a context's own (a batch's launches advance its members' clocks)
+    unsigned pad[28];
     unsigned ticket[3][TICKET_GROUPS][32];      // by step in rotation and group, a cache line each
 };
 
@@ -1859,9 +1877,9 @@ struct OneWork {
     }
     __device__ __forceinline__ int find_tile(int t, int &lat) const { lat = 0; return t; }
     __device__ __forceinline__ int find_part(int g, int &lat) const { lat = 0; return g; }
-    // populations and positions read in step st of the launch, and its tile counts
+    // which populations and positions step st of the launch reads
     __device__ __forceinline__ int parity(int, int st) const { return one.cur ^ (st & 1); }
-    __device__ __forceinline__ int rotation(int, int st) const { return (one.rot + st) % 3; }
+    __device__ __forceinline__ int lattices() const { return 1; }
 };
 
 // A batch's: the members' segments, tiles and particles, one after another.
@@ -1890,18 +1908,20 @@ struct BatchWork {
         return g - ba.part_start[lat];
     }
     __device__ __forceinline__ int parity(int lat, int st) const { return ba.a[lat].cur ^ (st & 1); }
-    __device__ __forceinline__ int rotation(int lat, int st) const { return (ba.a[lat].rot + st) % 3; }
+    __device__ __forceinline__ int lattices() const { return ba.n; }
 };
 
 // The particle blocks' part of a step: warp pw of npw.
 template <typename WORK>
-__device__ __forceinline__ bool update_particles(const WORK &wk, int st, int shift, int pw, int npw, int lane) {
+__device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock *clk, int st, int shift, int pw, int npw,
+                                                 int lane) {
     const int total = wk.parts();
     for (int g = pw; g < total; g += npw) {
         int lat;
         const int p = wk.find_part(g, lat);
         const PartArgs &A = wk.part(lat);
-        Repulsion c = pair_repulsion(A, p, wk.parity(lat, st), bins_at(A.B, wk.parity(lat, st), wk.rotation(lat, st)), lane);
+        Repulsion c = pair_repulsion(A, p, wk.parity(lat, st),
+                                     bins_at(A.B, wk.parity(lat, st), (clk[lat].rot + st) % 3), lane);
         wall_repulsion(A, p, wk.parity(lat, st), c);
         if (lane == 0) {
             A.fcol[2 * (long long)p] = c.x;
@@ -1932,8 +1952,8 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, int st, int shi
                 const int l = __ffs(ready) - 1;
                 const int q = __shfl_sync(0xffffffffu, p, l), ql = __shfl_sync(0xffffffffu, lat, l);
                 const PartArgs &A = wk.part(ql);
-                const int cur = wk.parity(ql, st), rot = wk.rotation(ql, st);
-                const unsigned tag = wk.args(ql).tag + st;
+                const int cur = wk.parity(ql, st), rot = (clk[ql].rot + st) % 3;
+                const unsigned tag = clk[ql].tag + st;
                 const PartState ps = load_particle(A, q, cur, lane);
                 const int comp = component(lane);
                 const double c = comp < 2 ? __ldcg(A.fcol + 2 * (long long)q + comp) : 0.0;
@@ -1946,10 +1966,11 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, int st, int shi
     return true;
 }
 
-template <typename T, bool EDGES, int W, bool PS, typename WORK>
+template <typename T, bool EDGES, int W, bool PS, int LATTICES, typename WORK>
 __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame, const StepRun &run) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ int s_stop, s_halt;      // a warp gave up; the block leaves (set between barriers)
+    __shared__ StepClock clk[LATTICES]; // every lattice's clock as the launch starts
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SweepSmem<T, W> sm(smem_raw, warp);
     Ring ring{sm.bar, 0u, false};
@@ -1958,6 +1979,10 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         mbar_fence_init();
     }
     if (threadIdx.x == 0) s_stop = s_halt = 0;
+    for (int k = threadIdx.x; k < wk.lattices(); k += blockDim.x) {
+        clk[k].tag = __ldcg(&wk.args(k).clock->tag);
+        clk[k].rot = __ldcg(&wk.args(k).clock->rot);
+    }
     __syncthreads();
     const bool sweeps = (int)blockIdx.x >= run.pblocks;
     // this block among the sweeping ones, its group and the group's warps
@@ -1978,7 +2003,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
             shift = frame_move(__ldcg((wk.parity(0, st) ? f.P.x[1] : f.P.x[0]) + f.track), f.track_x, f.L.nx, f.L.per_x);
         }
         if (!sweeps) {
-            if (!run.dry && !update_particles(wk, st, shift, (int)blockIdx.x * W + warp, run.pblocks * W, lane)) {
+            if (!run.dry && !update_particles(wk, clk, st, shift, (int)blockIdx.x * W + warp, run.pblocks * W, lane)) {
                 if (lane == 0) atomicOr(wk.args(0).err, ERR_TIMEOUT);
                 timed_out = true;
             }
@@ -2004,7 +2029,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                     int lat;
                     const int tl = wk.find_tile(t, lat);
                     const SweepArgs<T> &a = wk.args(lat);
-                    if (a.np > 0) a.B.count[(long long)rot3(wk.rotation(lat, st) + 2) * a.B.tiles + tl] = 0;
+                    if (a.np > 0) a.B.count[(long long)((clk[lat].rot + st + 2) % 3) * a.B.tiles + tl] = 0;
                 }
             }
             while (have) {
@@ -2017,9 +2042,9 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 const SweepArgs<T> &a = wk.args(c.lat), &an = wk.args(nx.lat);
                 const int cur = wk.parity(c.lat, st);
                 if (!sweep_segment<T, MODE_STEP, EDGES, PS, true>(
-                        a, a.buf[cur], a.buf[cur ^ 1], bins_at(a.B, cur, wk.rotation(c.lat, st)), c.y, c.tx, sm.stage,
+                        a, a.buf[cur], a.buf[cur ^ 1], bins_at(a.B, cur, (clk[c.lat].rot + st) % 3), c.y, c.tx, sm.stage,
                         ring, have, an.buf[wk.parity(nx.lat, st)], an.L, nx.y, nx.tx, sm.crec, sm.cid, wv,
-                        a.tag + st - run.dry, !run.dry, fo, lane)) {
+                        clk[c.lat].tag + st - run.dry, !run.dry, fo, lane)) {
                     if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
                     timed_out = true;
                     break;
@@ -2061,13 +2086,18 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         }
         if (s_halt) break;
     }
-    // the last block out leaves the counters as it found them
+    // the last block out leaves the counters as it found them, and advances the clocks
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(&run.sync->left, 1u) == gridDim.x - 1) {
         run.sync->arrived = 0;
         run.sync->left = 0;
         for (int q = 0; q < 3; ++q)
             for (int g = 0; g < TICKET_GROUPS; ++g) run.sync->ticket[q][g][0] = 0;
+        for (int k = 0; k < wk.lattices() && !run.dry; ++k) {
+            StepClock *c = wk.args(k).clock;
+            c->tag = clk[k].tag + (unsigned)run.nsteps;
+            c->rot = (clk[k].rot + run.nsteps) % 3;
+        }
     }
 }
 
@@ -2076,14 +2106,14 @@ __global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
 step_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ PartArgs pa,
             const __grid_constant__ StepRun run) {
     const OneWork<T> wk{one, pa};
-    run_steps<T, EDGES, W, PS>(wk, &pa, run);
+    run_steps<T, EDGES, W, PS, 1>(wk, &pa, run);
 }
 
 template <typename T, int W>
 __global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
 step_batch_kernel(const __grid_constant__ BatchArgs<T> ba, const __grid_constant__ StepRun run) {
     const BatchWork<T> wk{ba};
-    run_steps<T, true, W, false>(wk, nullptr, run);
+    run_steps<T, true, W, false, BATCH_LAUNCH_MAX>(wk, nullptr, run);
 }
 
 // ------------------------------------------------------------ conversions

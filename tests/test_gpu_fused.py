@@ -138,3 +138,39 @@ def test_particle_that_leaves_the_lattice(stream):
     assert np.array_equal(a.populations(), b.populations())
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("steps,replays", [(2, 1), (2, 5), (4, 3), (8, 2)])
+@pytest.mark.parametrize("batched", [False, True])
+def test_captured_steps_replay_from_any_step(stream, steps, replays, batched):
+    """A recorded even number of steps goes on from wherever the lattice
+    stands: after steps taken outside the graph, and by an upload and more
+    steps after the replays."""
+    import torch
+    probs = [W.periodic_suspension(n=256, count=8, seed=5), W.periodic_suspension(n=192, count=4, seed=6)]
+    side = torch.cuda.Stream()
+    want, got = ([D.Simulation(p, stream=int(s.cuda_stream)) for p in probs[: 1 + batched]] for s in (stream, side))
+    advance = [(lambda k, b=D.Batch(g): b.step(k)) if batched else g[0].step for g in (want, got)]
+    advance[0](2 + steps * replays)
+    advance[1](2)
+    for s in got:
+        s.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=side, capture_error_mode="thread_local"):
+        advance[1](steps)
+    with torch.cuda.stream(side):
+        for _ in range(replays):
+            graph.replay()
+    side.synchronize()
+    for after in range(2):
+        for a, b in zip(want, got):
+            assert np.array_equal(a.populations(), b.populations())
+            for x, y in zip(a.forces(), b.forces()):
+                assert np.array_equal(x, y)
+        for a, b, p in zip(want, got, probs):
+            a.set_particles(p.particles)
+            b.set_particles(p.particles)
+        for f in advance:
+            f(5)
+    for s in want + got:
+        s.close()
