@@ -106,7 +106,7 @@ template <typename T> __host__ __device__ constexpr int stage_elems() { return 9
 // Dynamic shared memory of one sweep block of W warps.
 template <typename T, int W = SWEEP_WARPS> __host__ __device__ constexpr size_t sweep_smem_bytes() {
     return (size_t)W * stage_elems<T>() * sizeof(T)             // staged rows
-           + (size_t)W * MAXC * NREC * sizeof(float4)           // candidate records
+           + (size_t)W * MAXC * (NREC + 1) * sizeof(float4)     // candidate records and force sums
            + (size_t)W * MAXC * sizeof(int)                     // candidate ids
            + (size_t)W * sizeof(uint64_t);                      // mbarriers
 }
@@ -144,6 +144,7 @@ struct Lattice {
     // 16-bit sweep takes moments of the stored s_i and adds these, so no
     // per-direction offset enters its inner loop.
     float ref_m[6];
+    float ref_om[3];            // -(omega M) / q
     // A strip of a larger lattice (one rank's rows): the post-collision rows
     // just south (halo[0]) and north (halo[1]) of it, 9 plane rows of `pitch`
     // elements each, with GUARD readable elements before and after; NULL
@@ -294,9 +295,12 @@ __device__ __forceinline__ void eq_dev9(float drho, float rho, float ux, float u
 // of sm_100+ (each component rounds exactly as the scalar op).
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+// a - b in one paired instruction: b * -1 + a rounds once, as a - b does.  (The
+// paired add has no subtracting form: negating b first takes two more.)
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, f2(-1.0f), a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return mul2(a, f2(-1.0f)); }
 
 __device__ __forceinline__ void moment_form2(float2 m0, float2 Bx, float2 By, float2 Mxx, float2 Myy, float2 Mxy,
                                              float2 X[9]) {
@@ -336,10 +340,11 @@ __device__ __forceinline__ void relax_to2(float2 d[9], const Lattice &L, float o
                                           float2 Bys, float2 Mxx, float2 Myy, float2 Mxy) {
     const float2 om = f2(omega);
     if constexpr (!std::is_same<T, float>::value) {
+        // (scaling by 1 / q is exact, so one FMA rounds as the difference does)
         const float2 iq = f2(L.ref_iq);
-        Mxx = mul2(sub2(Mxx, f2(omega * L.ref_m[3])), iq);
-        Myy = mul2(sub2(Myy, f2(omega * L.ref_m[4])), iq);
-        Mxy = mul2(sub2(Mxy, f2(omega * L.ref_m[5])), iq);
+        Mxx = fma2(Mxx, iq, f2(L.ref_om[0]));
+        Myy = fma2(Myy, iq, f2(L.ref_om[1]));
+        Mxy = fma2(Mxy, iq, f2(L.ref_om[2]));
     }
     float2 X[9];
     moment_form2(mul2(om, ms), Bxs, Bys, Mxx, Myy, Mxy, X);
@@ -828,6 +833,32 @@ __device__ __forceinline__ float rcp_approx(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// 1 / v of a pair of densities: the hardware's approximation and one
+// Newton-Raphson correction with its residual formed exactly by an FMA, after
+// which the reciprocal is correctly rounded (Markstein, IBM J. Res. Dev. 34
+// (1990) 111).  Compared with __frcp_rn over every normal FP32 value whose
+// reciprocal is normal: the same bits.
+__device__ __forceinline__ float2 recip2(float2 v) {
+    const float2 r = make_float2(rcp_approx(v.x), rcp_approx(v.y));
+    const float2 e = fma2(neg2(v), r, f2(1.0f));
+    return fma2(r, e, r);
+}
+
+// Square roots of a pair of squared distances (0, or at least the square of
+// a distance's rounding), the same way: v rsqrt(v), then one Newton-Raphson
+// (Heron) correction by the exact residual.
+__device__ __forceinline__ float2 sqrt2(float2 v) {
+    const float2 q = make_float2(rsqrt_approx(fmaxf(v.x, 1e-30f)), rsqrt_approx(fmaxf(v.y, 1e-30f)));
+    const float2 s = mul2(v, q);
+    const float2 e = fma2(neg2(s), s, v);
+    return fma2(e, mul2(f2(0.5f), q), s);
+}
 
 // Slot m (0 or 1) of a node pair.
 __device__ __forceinline__ float &slot(float2 &v, int m) { return m ? v.y : v.x; }
@@ -864,6 +895,9 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
             const long long r = (long long)tile * MAXC + lane;
 #pragma unroll
             for (int q = 0; q < NREC; ++q) crec[q * MAXC + lane] = __ldcg(B.rec + NREC * r + q);
+            // the segment's force / torque on the candidate so far (first
+            // pass, then second pass added)
+            crec[NREC * MAXC + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
             mine = __ldcg(B.ids + r);
             cid[lane] = mine.x;
         }
@@ -900,9 +934,6 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
     }
     __syncwarp();   // candidate records and edge values visible to the whole warp
 
-    // lane c < ncand: the segment's force / torque on candidate c so far
-    // (first pass, then second pass added)
-    float sgx = 0.f, sgy = 0.f, sgt = 0.f;
     unsigned badmax = 0u;
 
     // a row's last segment may end within its first half: its second pass
@@ -972,7 +1003,7 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
         // ---- solid fraction (Eq. 14), owner and particle velocity per node:
         // max over the tile's candidates, lowest particle id on ties
         float phi[2] = {0.f, 0.f}, rxn[2] = {0.f, 0.f}, ryn[2] = {0.f, 0.f};
-        int best[2] = {-1, -1}, best_id[2] = {0x7fffffff, 0x7fffffff};
+        int best[2] = {-1, -1};
         // (ncand is warp-uniform; a segment no particle reaches skips all of it)
         for (int c = 0; c < ncand; ++c) {
             const float4 ra = crec[c], rb = crec[MAXC + c];
@@ -1005,19 +1036,22 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
                 const int K = ph.ck, S = 2 * K + 1;
                 const float *tab = A.B.cover + (long long)id * S * S;
                 const int iy = (y - ty0) - (int)(short)((unsigned)fpk >> 16) - L.ny * ky + K;
-                float pcq[2], dxq[2];
+                float pcq[2];
+                float2 dxq = make_float2(dx0, dx0 + 1.0f);
+                int kxq[2] = {0, 0};
+                if (L.wrap_x) {
+#pragma unroll
+                    for (int m = 0; m < 2; ++m) {
+                        const float k = rintf(slot(dxq, m) * __frcp_rn((float)L.nx));
+                        slot(dxq, m) = fmaf(-(float)L.nx, k, slot(dxq, m));
+                        kxq[m] = (int)k;
+                    }
+                }
+                float2 d2q = fma2(dxq, dxq, f2(dy * dy)), lq = sub2(f2(rb.x), sqrt2(d2q));
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
-                    float dx = dx0 + (float)m;
-                    int kx = 0;
-                    if (L.wrap_x) {
-                        const float k = rintf(dx * __frcp_rn((float)L.nx));
-                        dx = fmaf(-(float)L.nx, k, dx);
-                        kx = (int)k;
-                    }
-                    dxq[m] = dx;
-                    const float d2 = fmaf(dx, dx, dy * dy);
-                    const float l = rb.x - sqrtf(d2);
+                    const int kx = kxq[m];
+                    const float d2 = slot(d2q, m), l = slot(lq, m);
                     const int ix = e + m - (int)(short)(fpk & 0xffff) - L.nx * kx + K;
                     const bool inside = d2 <= R * R && l >= -ph.cut;
                     const bool look = inside && l < ph.cut && (unsigned)ix < (unsigned)S && (unsigned)iy < (unsigned)S;
@@ -1027,27 +1061,33 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
                 for (int m = 0; m < 2; ++m) {
                     const float pc = pcq[m];
                     if (!(pc > 0.f)) continue;
-                    if (pc > phi[m] || (pc == phi[m] && id < best_id[m])) {
-                        phi[m] = pc; best[m] = c; best_id[m] = id; rxn[m] = dxq[m]; ryn[m] = dy;
+                    if (pc > phi[m] || (pc == phi[m] && id < cid[best[m]])) {
+                        phi[m] = pc; best[m] = c; rxn[m] = slot(dxq, m); ryn[m] = dy;
                     }
                 }
             } else {
+float2 dx = make_float2(dx0, dx0 + 1.0f);
+                if (L.wrap_x) {
+                    dx.x = fmaf(-(float)L.nx, rintf(dx.x * __frcp_rn((float)L.nx)), dx.x);
+                    dx.y = fmaf(-(float)L.nx, rintf(dx.y * __frcp_rn((float)L.nx)), dx.y);
+                }
+                const float2 d2 = fma2(dx, dx, f2(dy * dy));
+                const float2 l = sub2(f2(rb.x), sqrt2(d2));
+                // (1 + tanh(2l/eps)) / 2 == 1 / (1 + exp(-4l/eps)) == 1 / (1 + 2^(phi_k2 l)),
+                // with the hardware's base-2 exponential and reciprocal: the
+                // rounding of the argument phi_k2 l (|.| <= 23 inside the tail,
+                // a relative error of at most 23 * 2^-24 in the power) bounds
+                // the error either way, and both instructions add about an ulp.
+                // (Beyond the tail the value is not used.)
+                const float2 a = mul2(f2(ph.phi_k2), l);
+                const float2 den = add2(f2(1.0f), make_float2(ex2_approx(a.x), ex2_approx(a.y)));
+                const float pcs[2] = {rcp_approx(den.x), rcp_approx(den.y)};
+                const bool in[2] = {d2.x <= R * R && l.x >= -ph.cut, d2.y <= R * R && l.y >= -ph.cut};
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
-                    float dx = dx0 + (float)m;
-                    if (L.wrap_x) dx = fmaf(-(float)L.nx, rintf(dx * __frcp_rn((float)L.nx)), dx);
-                    const float d2 = fmaf(dx, dx, dy * dy);
-                    if (d2 > R * R) continue;
-                    const float l = rb.x - sqrtf(d2);
-                    if (l < -ph.cut) continue;
-                    // (1 + tanh(2l/eps)) / 2 == 1 / (1 + exp(-4l/eps)) == 1 / (1 + 2^(phi_k2 l)),
-                    // with the hardware's base-2 exponential and reciprocal: the
-                    // rounding of the argument phi_k2 l (|.| <= 23 inside the tail,
-                    // a relative error of at most 23 * 2^-24 in the power) bounds
-                    // the error either way, and both instructions add about an ulp
-                    const float pc = rcp_approx(1.0f + ex2_approx(ph.phi_k2 * l));
-                    if (pc > phi[m] || (pc == phi[m] && pc > 0.f && id < best_id[m])) {
-                        phi[m] = pc; best[m] = c; best_id[m] = id; rxn[m] = dx; ryn[m] = dy;
+                    const float pc = in[m] ? pcs[m] : 0.f;
+                    if (pc > phi[m] || (pc == phi[m] && pc > 0.f && id < cid[best[m]])) {
+                        phi[m] = pc; best[m] = c; rxn[m] = slot(dx, m); ryn[m] = dy;
                     }
                 }
             }
@@ -1070,9 +1110,9 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
             jy = fma2(q, jys, f2(L.ref_m[2]));
         }
         const float2 rho = add2(f2(1.0f), drho);
-        // u* (Eq. 16); CUDA's correctly rounded reciprocal (a biased one would
+        // u* (Eq. 16); a correctly rounded reciprocal (a biased one would
         // bias u* the same way on every node and step)
-        const float2 inv = make_float2(__frcp_rn(rho.x), __frcp_rn(rho.y));
+        const float2 inv = recip2(rho);
         const float2 ua = mul2(jx, inv), va = mul2(jy, inv);
         if (MODE == MODE_STEP) {
             // unstable: rho <= 0 or not finite (a non-finite population makes
@@ -1150,17 +1190,21 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
             const float gax = sa * du[0], gay = sa * dv[0], gbx = sb * du[1], gby = sb * dv[1];
             const float ta = fmaf(rxn[0], gay, -(ryn[0] * gax)), tb = fmaf(rxn[1], gby, -(ryn[1] * gbx));
             for (int c = 0; c < ncand; ++c) {
+                if (!__any_sync(0xffffffffu, own_a == c || own_b == c)) continue;
                 float v0 = 0.f, v1 = 0.f, v2 = 0.f;
                 if (own_a == c) { v0 = gax; v1 = gay; v2 = ta; }
                 if (own_b == c) { v0 += gbx; v1 += gby; v2 += tb; }
-                if (!__any_sync(0xffffffffu, own_a == c || own_b == c)) continue;
+                // three sums over 32 lanes in 6 shuffles: at the tree's first
+                // two levels the lanes part with a component each (as in
+                // hydro_sums), so that lanes 0, 8 and 16 end with x, y and the
+                // torque.  (One tree per component took 15.)
+                const bool up = lane & 16, odd = lane & 8;
+                const float r0 = __shfl_xor_sync(0xffffffffu, up ? v0 : v2, 16), r1 = __shfl_xor_sync(0xffffffffu, v1, 16);
+                const float b0 = (up ? v2 : v0) + r0, b1 = v1 + r1;
+                float g = (odd ? b1 : b0) + __shfl_xor_sync(0xffffffffu, odd ? b0 : b1, 8);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-                    v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-                    v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-                }
-                if (lane == c) { sgx += v0; sgy += v1; sgt += v2; }
+                for (int o = 4; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+                if ((lane & 7) == 0 && lane < 24) reinterpret_cast<float *>(crec + NREC * MAXC + c)[lane >> 3] += g;
             }
         }
 
@@ -1178,13 +1222,15 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
     if (MODE == MODE_FIELDS) return true;
     if (__any_sync(0xffffffffu, badmax > 0x7f7ffffeu) && lane == 0) atomicOr(A.err, ERR_UNSTABLE);
     // ---- this row segment's force / torque per candidate (zero where no node is owned)
+    __syncwarp();
     if (lane < ncand) {
+        const float4 sg = crec[NREC * MAXC + lane];
         float4 *out = A.partial + ((long long)mine.x * MAXT + mine.y) * TILE_H + (y - ty0);
         if (FUSED) {
-            store_partial(out, sgx, sgy, sgt, tag);
+            store_partial(out, sg.x, sg.y, sg.z, tag);
             if (count) count_done(B.done + mine.x);
         } else {
-            *out = make_float4(sgx, sgy, sgt, 0.f);
+            *out = sg;
         }
     }
     return true;
@@ -1199,10 +1245,10 @@ struct SweepSmem {
     uint64_t *bar;
     __device__ __forceinline__ SweepSmem(unsigned char *raw, int warp) {
         constexpr size_t STAGE_BYTES = (size_t)W * stage_elems<T>() * sizeof(T);
-        constexpr size_t REC_BYTES = (size_t)W * NREC * MAXC * sizeof(float4);
+        constexpr size_t REC_BYTES = (size_t)W * (NREC + 1) * MAXC * sizeof(float4);
         constexpr size_t ID_BYTES = (size_t)W * MAXC * sizeof(int);
         stage = reinterpret_cast<T *>(raw) + (size_t)warp * stage_elems<T>();
-        crec = reinterpret_cast<float4 *>(raw + STAGE_BYTES) + (size_t)warp * NREC * MAXC;
+        crec = reinterpret_cast<float4 *>(raw + STAGE_BYTES) + (size_t)warp * (NREC + 1) * MAXC;
         cid = reinterpret_cast<int *>(raw + STAGE_BYTES + REC_BYTES) + warp * MAXC;
         bar = reinterpret_cast<uint64_t *>(raw + STAGE_BYTES + REC_BYTES + ID_BYTES) + warp;
     }
