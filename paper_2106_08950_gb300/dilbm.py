@@ -208,6 +208,8 @@ def make_particles(parts) -> "C.Array":
 
 def particles_to_array(arr, n) -> np.ndarray:
     """(n, 8) float64: x, y, r, ux, uy, omega, theta, rho_s."""
+    if isinstance(arr, C.Array):         # one strided copy (value by value, 2048 particles took 1.1 ms)
+        return np.ndarray((n, 8), dtype=np.float64, buffer=arr, strides=(C.sizeof(Particle), 8)).copy()
     out = np.zeros((n, 8))
     for k in range(n):
         q = arr[k]
