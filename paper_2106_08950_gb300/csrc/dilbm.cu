@@ -630,11 +630,6 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         // m0 = rho - 1, B = rho u0, M = rho u0 u0^T
         const double m[6] = {r0 - 1.0, r0 * ux, r0 * uy, r0 * ux * ux, r0 * uy * uy, r0 * ux * uy};
         for (int k = 0; k < 6; ++k) L.ref_m[k] = wide ? 0.0f : (float)m[k];
-        const float omega = (float)(1.0 / tau);
-        for (int k = 0; k < 3; ++k) {
-            const float om = omega * L.ref_m[3 + k];
-            L.ref_om[k] = -om * L.ref_iq;
-        }
     }
     const bool strip = y0 > 0 || y1 < g->ny;
     if (strip) {

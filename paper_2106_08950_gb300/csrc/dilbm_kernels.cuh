@@ -144,7 +144,6 @@ struct Lattice {
     // 16-bit sweep takes moments of the stored s_i and adds these, so no
     // per-direction offset enters its inner loop.
     float ref_m[6];
-    float ref_om[3];            // -(omega M) / q
     // A strip of a larger lattice (one rank's rows): the post-collision rows
     // just south (halo[0]) and north (halo[1]) of it, 9 plane rows of `pitch`
     // elements each, with GUARD readable elements before and after; NULL
@@ -340,11 +339,10 @@ __device__ __forceinline__ void relax_to2(float2 d[9], const Lattice &L, float o
                                           float2 Bys, float2 Mxx, float2 Myy, float2 Mxy) {
     const float2 om = f2(omega);
     if constexpr (!std::is_same<T, float>::value) {
-        // (scaling by 1 / q is exact, so one FMA rounds as the difference does)
         const float2 iq = f2(L.ref_iq);
-        Mxx = fma2(Mxx, iq, f2(L.ref_om[0]));
-        Myy = fma2(Myy, iq, f2(L.ref_om[1]));
-        Mxy = fma2(Mxy, iq, f2(L.ref_om[2]));
+        Mxx = mul2(add2(Mxx, f2(-(omega * L.ref_m[3]))), iq);
+        Myy = mul2(add2(Myy, f2(-(omega * L.ref_m[4]))), iq);
+        Mxy = mul2(add2(Mxy, f2(-(omega * L.ref_m[5]))), iq);
     }
     float2 X[9];
     moment_form2(mul2(om, ms), Bxs, Bys, Mxx, Myy, Mxy, X);
