@@ -356,6 +356,7 @@ SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     a.clock = c->strip ? nullptr : &c->sync->clock;
     a.pa = c->np > 0 ? c->pa : nullptr;
     a.np = c->np;
+    a.eager = c->np <= MAXC && (long long)c->np * c->L.ntx * c->L.ny <= 65536;
     a.cur = c->cur;
     a.ntx_inv = ntx_inverse(c->L.ntx);
     return a;
@@ -1145,6 +1146,7 @@ void fill_groups(dilbm_batch *b) {
         for (int k = 0; k < ba.n; ++k) {
             const dilbm_ctx *c = b->members[g0 + k];
             ba.a[k] = sweep_args<T>(c);
+            ba.a[k].eager = 0;      // (the records of 64 lattices are too many: 242 us a step became 264)
             ba.item_start[k + 1] = ba.item_start[k] + c->L.ny * c->L.ntx;
             ba.tile_start[k + 1] = ba.tile_start[k] + c->L.ntx * c->L.nty;
             ba.part_start[k + 1] = ba.part_start[k] + c->np;

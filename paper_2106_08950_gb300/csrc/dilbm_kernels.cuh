@@ -186,7 +186,7 @@ struct Physics {
 // count[rot + 1], and it zeroes count[rot + 2], which nothing uses during the
 // step, so that no pass of its own is needed to clear them.
 struct Bins {                   // one step's view
-    int *count;                 // per tile: particles binned (may exceed MAXC)
+    int *count;                 // per tile: particles binned (may exceed MAXC), or their mask (see slot_mask)
     int2 *ids;                  // per tile: MAXC (particle, index of the tile in the particle's list)
     float4 *rec;                // per tile and slot, 3 records: (cx_hi, cx_lo, cy_hi, cy_lo),
                                 // (r, ux_hi, uy_hi, omega_hi), (ux_lo, uy_lo, omega_lo, packed
@@ -227,6 +227,16 @@ __host__ __device__ inline Bins bins_at(const BinSet &b, int par, int rot) {
     v.npslot = b.npslot + q;
     v.done = b.done + q;
     return v;
+}
+
+// The slots a tile's count word `w` says are taken.  With at most MAXC
+// particles a particle's slot is its number and the word is the mask itself,
+// so binning sends an OR and waits for no answer; with more, slots are handed
+// out by a counter, whose value may exceed MAXC.
+__device__ __forceinline__ bool masked_bins(int np) { return np <= MAXC; }
+__device__ __forceinline__ unsigned slot_mask(int w, int np) {
+    if (masked_bins(np)) return (unsigned)w;
+    return w >= MAXC ? 0xffffffffu : (1u << w) - 1u;
 }
 
 // ------------------------------------------------------------ small helpers
@@ -713,6 +723,12 @@ static __device__ __noinline__ float cell_cover(float dx, float dy, float r) {
     return 0.5f * w.area2 + w.seg;
 }
 
+// 16 bytes from global to shared memory without a register in between.
+__device__ __forceinline__ void copy16_async(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_async_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // ------------------------------------------------------------ the sweep
 // Mode: STEP writes the collided populations and the force partials; FIELDS
 // writes rho, the corrected velocity and phi of the streamed state instead.
@@ -736,6 +752,11 @@ struct SweepArgs {
     const PartArgs *pa;         // the particle update's arguments (device memory; batches)
     StepClock *clock;           // (null: see StepClock)
     int np;                     // particles (0: no bins to read)
+    // A segment's candidate records are loaded beside the word that says which
+    // are there (not after it: a trip to the L2 less) where particles own their
+    // slots and the records of all segments come to no more than 4 MB a step
+    // (half a microsecond of the L2's bandwidth).
+    bool eager;
     int cur;                    // parity of the launch's first step
     unsigned ntx_inv;           // floor(2^32 / ntx) + 1 (saturated), see row_of
 };
@@ -884,21 +905,24 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
     // ---- the tile's candidate particles (records written by the binning),
     // loaded before the wait so that their latency overlaps it
     __syncwarp();
-    int ncand = 0;
-    int2 mine = make_int2(-1, 0);       // lane c: candidate c, index of this tile in its list
+    unsigned cands = 0u;                    // the slots taken
     if (A.np > 0) {
-        ncand = __ldcg(B.count + tile);
-        ncand = ncand > MAXC ? MAXC : ncand;
-        if (lane < ncand) {
-            const long long r = (long long)tile * MAXC + lane;
+        const long long r = (long long)tile * MAXC + lane;
+        int2 mine = make_int2(-1, 0);       // the slot's particle, index of this tile in that particle's list
+        auto fetch = [&]() {
 #pragma unroll
-            for (int q = 0; q < NREC; ++q) crec[q * MAXC + lane] = __ldcg(B.rec + NREC * r + q);
-            // the segment's force / torque on the candidate so far (first
-            // pass, then second pass added)
-            crec[NREC * MAXC + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int q = 0; q < NREC; ++q) copy16_async(crec + q * MAXC + lane, B.rec + NREC * r + q);
             mine = __ldcg(B.ids + r);
-            cid[lane] = mine.x;
-        }
+        };
+        const bool eager = A.eager && lane < A.np;
+        if (eager) fetch();                 // (a slot not taken: stale, not used)
+        cands = slot_mask(__ldcg(B.count + tile), A.np);
+        if (!eager && (cands >> lane & 1u)) fetch();
+        // beside the records: the particle, and the segment's force / torque on
+        // it so far (first pass, then second pass added) with the index
+        cid[lane] = mine.x;
+        crec[NREC * MAXC + lane] = make_float4(0.f, 0.f, 0.f, __int_as_float(mine.y));
+        copies_async_done();
     }
 
     // ---- wait for the staged rows
@@ -1002,8 +1026,9 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
         // max over the tile's candidates, lowest particle id on ties
         float phi[2] = {0.f, 0.f}, rxn[2] = {0.f, 0.f}, ryn[2] = {0.f, 0.f};
         int best[2] = {-1, -1};
-        // (ncand is warp-uniform; a segment no particle reaches skips all of it)
-        for (int c = 0; c < ncand; ++c) {
+        // (cands is warp-uniform; a segment no particle reaches skips all of it)
+        for (unsigned left = cands; left; left &= left - 1) {
+            const int c = __ffs(left) - 1;
             const float4 ra = crec[c], rb = crec[MAXC + c];
             const float R = rb.x + ph.cut;
             float dy = ((float)(y - ty0) - ra.z) - ra.w;
@@ -1092,7 +1117,7 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
         }
 
         // warps with no node inside any particle's phi tail collide without the force term
-        const bool coupled = ncand > 0 && __any_sync(0xffffffffu, max(best[0], best[1]) >= 0);
+        const bool coupled = cands && __any_sync(0xffffffffu, max(best[0], best[1]) >= 0);
         const bool act_a = x < L.nx, act_b = x + 1 < L.nx;
 
         // ---- moments (Eq. 5, Eq. 16): of the stored values, then physical
@@ -1187,7 +1212,8 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
             const float sa = -prho.x * ph.kforce, sb = -prho.y * ph.kforce;
             const float gax = sa * du[0], gay = sa * dv[0], gbx = sb * du[1], gby = sb * dv[1];
             const float ta = fmaf(rxn[0], gay, -(ryn[0] * gax)), tb = fmaf(rxn[1], gby, -(ryn[1] * gbx));
-            for (int c = 0; c < ncand; ++c) {
+            for (unsigned left = cands; left; left &= left - 1) {
+                const int c = __ffs(left) - 1;
                 if (!__any_sync(0xffffffffu, own_a == c || own_b == c)) continue;
                 float v0 = 0.f, v1 = 0.f, v2 = 0.f;
                 if (own_a == c) { v0 = gax; v1 = gay; v2 = ta; }
@@ -1221,14 +1247,15 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
     if (__any_sync(0xffffffffu, badmax > 0x7f7ffffeu) && lane == 0) atomicOr(A.err, ERR_UNSTABLE);
     // ---- this row segment's force / torque per candidate (zero where no node is owned)
     __syncwarp();
-    if (lane < ncand) {
+    if (cands >> lane & 1u) {
         const float4 sg = crec[NREC * MAXC + lane];
-        float4 *out = A.partial + ((long long)mine.x * MAXT + mine.y) * TILE_H + (y - ty0);
+        const int id = cid[lane];
+        float4 *out = A.partial + ((long long)id * MAXT + __float_as_int(sg.w)) * TILE_H + (y - ty0);
         if (FUSED) {
             store_partial(out, sg.x, sg.y, sg.z, tag);
-            if (count) count_done(B.done + mine.x);
+            if (count) count_done(B.done + id);
         } else {
-            *out = sg;
+            *out = make_float4(sg.x, sg.y, sg.z, 0.f);
         }
     }
     return true;
@@ -1411,7 +1438,7 @@ struct Repulsion {
 };
 
 // Could particle p be within Eq. 28's range of another one?  Each lane takes
-// one (tile, slot) of the particle's first eight tiles and first four slots
+// one (tile, slot) of the particle's first eight tiles and first four taken slots
 // and compares the two records there (FP32, relative to the tile, with a
 // margin far above their rounding), so that the answer takes two dependent
 // loads; more tiles or slots, or a periodic axis too short for one image per
@@ -1424,8 +1451,16 @@ __device__ __forceinline__ bool maybe_near(const PartArgs &A, int p, const Bins 
     float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
     int id = -1, n = 0;
     if (k < nk && t >= 0) {
-        const long long q = (long long)t * MAXC + sl;
-        n = __ldcg(B.count + t);
+        unsigned m = (unsigned)__ldcg(B.count + t);
+        int s = sl;
+        if (masked_bins(A.bp.np)) {
+            n = __popc(m);
+            for (int i = 0; i < sl; ++i) m &= m - 1;
+            s = m ? __ffs(m) - 1 : 0;
+        } else {
+            n = (int)m;
+        }
+        const long long q = (long long)t * MAXC + s;
         id = __ldcg(&B.ids[q].x);
         ra = __ldcg(B.rec + NREC * q);
         rb = __ldcg(B.rec + NREC * q + 1);
@@ -1465,10 +1500,9 @@ __device__ __forceinline__ Repulsion pair_repulsion(const PartArgs &A, int p, in
         for (int k = lane; k < nk; k += 32) {
             const int t = __ldcg(B.pslot + (long long)p * MAXT + k);
             if (t < 0) continue;
-            int n = __ldcg(B.count + t);
-            n = n > MAXC ? MAXC : n;
             uint32_t contact = 0;
-            for (int sl = 0; sl < n; ++sl) {
+            for (unsigned taken = slot_mask(__ldcg(B.count + t), bp.np); taken; taken &= taken - 1) {
+                const int sl = __ffs(taken) - 1;
                 const int j = __ldcg(&B.ids[(long long)t * MAXC + sl].x);
                 if (j == p) continue;
                 float dxf = xf - __ldcg(xfin + j), dyf = yf - __ldcg(yfin + j);
@@ -1576,30 +1610,45 @@ __device__ __forceinline__ int component(int lane) { return lane >> 3; }
 // those of three whole trees).  The partials lie per particle in that order
 // (rows outside the lattice and tiles of another strip hold zeros), so the
 // first loads need nothing but p.  TAGGED: each entry is read until it carries
-// the step's tag (the wait bounded).
+// the step's tag; the wait is bounded, and sets *late when it gives up.
 template <bool TAGGED>
-__device__ __forceinline__ double hydro_sums(const PartArgs &A, int p, const Bins &B, unsigned tag, int lane) {
+__device__ __forceinline__ double hydro_sums(const PartArgs &A, int p, const Bins &B, unsigned tag, int lane, bool *late) {
+    constexpr int Q = 3;        // entries per lane held at once (and waited for together)
     const float4 *part = A.partial + (long long)p * (MAXT * TILE_H) + lane;
-    float4 v0 = load_partial(part), v1 = load_partial(part + 32);
-    const int ne = __ldcg(B.npslot + p) * TILE_H;
+    float4 v[Q];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) v[q] = load_partial(part + 32 * q);
+    const int ne = __ldcg(B.npslot + p) * TILE_H - lane;        // entries from this lane's first on
     double fx = 0.0, fy = 0.0, tq = 0.0;
-    for (int base = 0; base < ne; base += 32) {
-        float4 v = base == 0 ? v0 : (base == 32 ? v1 : load_partial(part + base));
-        if (base + lane < ne) {
-            if (TAGGED && __float_as_uint(v.w) != tag) {
-                const unsigned long long t0 = global_ns();
-                do {
-                    v = load_partial(part + base);
-                    if (global_ns() - t0 > WAIT_LIMIT_NS) {
-                        atomicOr(A.err, ERR_TIMEOUT);
-                        break;
-                    }
-                } while (__float_as_uint(v.w) != tag);
-            }
-            if (base == 0) {
-                fx = widen(v.x); fy = widen(v.y); tq = widen(v.z);
+    for (int base = 0; base < ne + lane; base += 32 * Q) {
+        if (base > 0) {
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (base + 32 * q < ne) v[q] = load_partial(part + base + 32 * q);
+        }
+        unsigned long long t0 = 0;
+        while (TAGGED) {
+            bool miss = false;
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+                if (base + 32 * q < ne && __float_as_uint(v[q].w) != tag) {
+                    v[q] = load_partial(part + base + 32 * q);
+                    miss = true;
+                }
+            // (together: lanes that left on their own would sum on their own)
+            if (!__any_sync(0xffffffffu, miss)) break;
+            const unsigned long long t = global_ns();
+            if (t0 == 0) t0 = t;
+            *late = __any_sync(0xffffffffu, t - t0 > WAIT_LIMIT_NS);
+            if (*late) break;
+        }
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if (base + 32 * q >= ne) break;
+            if (base + q == 0) {
+                fx = widen(v[q].x); fy = widen(v[q].y); tq = widen(v[q].z);
             } else {
-                fx += widen(v.x); fy += widen(v.y); tq += widen(v.z);
+                fx += widen(v[q].x); fy += widen(v[q].y); tq += widen(v[q].z);
             }
         }
     }
@@ -1616,6 +1665,7 @@ __device__ __forceinline__ double hydro_sums(const PartArgs &A, int p, const Bin
 // Loaded in one go, before or together with the partials.
 struct PartState {
     double pos, vel, inv, weight, reach;    // x / y / theta, its rate, 1/m or 1/I, weight, reach
+    double sum;                             // running sum of the force (PartArgs::fsum)
     float rf;
     int fixed;
 };
@@ -1629,6 +1679,7 @@ __device__ __forceinline__ PartState load_particle(const PartArgs &A, int p, int
     s.inv = __ldcg((c < 2 ? P.im : P.iI) + p);
     s.weight = c < 2 ? __ldcg((c == 0 ? P.wx : P.wy) + p) : 0.0;
     s.reach = __ldcg(P.reach + p);
+    s.sum = A.fsum && c < 3 ? __ldcg(A.fsum + 3 * (long long)p + c) : 0.0;
     s.rf = __ldcg(P.rf + p);
     s.fixed = __ldcg(P.fixed + p);
     return s;
@@ -1671,10 +1722,7 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
         }
         if (lead) {
             A.force[3 * (long long)p + comp] = f;
-            if (A.fsum) {
-                double *s = A.fsum + 3 * (long long)p + comp;
-                *s = __ldcg(s) + f;
-            }
+            if (A.fsum) A.fsum[3 * (long long)p + comp] = st.sum + f;
             if (comp == 2 && !st.fixed) P.theta[p] = n;
         }
     }
@@ -1715,13 +1763,19 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
         const bool has = k < total;
         int ty = 0, tx = 0;
         if (has) {
-            ty = range_at(ay, k / NX);
-            tx = range_at(ax, k - (k / NX) * NX);
+            const int ky = NX == 1 ? k : (NX == 2 ? k >> 1 : k / NX);
+            ty = range_at(ay, ky);
+            tx = range_at(ax, k - ky * NX);
         }
         const bool local = has && ty >= A.ty_lo && ty < A.ty_hi;        // (else another strip's tile)
         const int t = (ty - A.ty_lo) * L.ntx + tx;
         int s = MAXC;
-        if (local && !axis) s = atomicAdd(&out.count[t], 1);
+        if (masked_bins(A.bp.np)) {
+            if (local && !axis) atomicOr(&out.count[t], (int)(1u << p));
+            s = p;
+        } else if (local && !axis) {
+            s = atomicAdd(&out.count[t], 1);
+        }
         // the centre along the lane's axis, while the count's answer is on its way
         double r = (axis ? nY : nX) - (double)(axis ? ty * TILE_H : tx * TILE_W);
         float rh = (float)r;
@@ -1812,7 +1866,7 @@ particles_kernel(const __grid_constant__ PartArgs A, int cur, int integrate, int
     Repulsion c{0.0, 0.0};
     if (integrate && phase != 2) {
         c = pair_repulsion(A, p, cur, in, lane);
-        f = hydro_sums<false>(A, p, in, 0u, lane);
+        f = hydro_sums<false>(A, p, in, 0u, lane, nullptr);
     }
     double *o = A.fpart ? A.fpart + 5 * (long long)p : nullptr;
     if (phase == 1) {
@@ -1852,9 +1906,10 @@ particles_kernel(const __grid_constant__ PartArgs A, int cur, int integrate, int
 constexpr int TICKET_GROUPS = 8;
 
 struct GridSync {               // all 0 between launches, but for the clock
-    unsigned arrived, left;
+    unsigned arrived[2][32];    // sweeping blocks, particle blocks (a cache line each)
+    unsigned left;
     StepClock clock;            // a context's own (a batch's launches advance its members' clocks)
-    unsigned pad[28];
+    unsigned pad[29];
     unsigned ticket[3][TICKET_GROUPS][32];      // by step in rotation and group, a cache line each
 };
 
@@ -1865,14 +1920,16 @@ struct StepRun {
     int pblocks;                // leading blocks that update particles
 };
 
-// Thread 0 of a block: arrive, then wait until `target` blocks have arrived.
-// Returns false when the bounded wait gave up.
-__device__ __forceinline__ bool sync_blocks(GridSync *g, unsigned target) {
-    asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(&g->arrived) : "memory");
+// Thread 0 of a block: count it as arrived, and wait until `target` blocks
+// have; false when the bounded wait gave up.
+__device__ __forceinline__ void arrive_block(unsigned *arrived) {
+    asm volatile("red.add.release.gpu.global.u32 [%0], 1;" ::"l"(arrived) : "memory");
+}
+__device__ __forceinline__ bool await_blocks(const unsigned *arrived, unsigned target) {
     unsigned long long t0 = 0;
     for (;;) {
         unsigned v;
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&g->arrived) : "memory");
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(arrived) : "memory");
         if ((int)(v - target) >= 0) return true;
         const unsigned long long t = global_ns();
         if (t0 == 0) t0 = t;
@@ -1955,17 +2012,26 @@ struct BatchWork {
     __device__ __forceinline__ int lattices() const { return ba.n; }
 };
 
+// May every particle have a warp of its own?  Then nothing is counted: the
+// warp reads its particle's partials until they carry the step's tag, and has
+// all else that the update needs at hand before.  (A count costs the chain of
+// a small lattice's step two more trips to the L2.)
+template <typename WORK>
+__device__ __forceinline__ bool own_warps(const WORK &wk, int npw) { return wk.parts() <= npw; }
+
 // The particle blocks' part of a step: warp pw of npw.
 template <typename WORK>
 __device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock *clk, int st, int shift, int pw, int npw,
                                                  int lane) {
     const int total = wk.parts();
+    const bool own = own_warps(wk, npw);
+    bool late = false;
+    Repulsion c{0.0, 0.0};
     for (int g = pw; g < total; g += npw) {
         int lat;
         const int p = wk.find_part(g, lat);
         const PartArgs &A = wk.part(lat);
-        Repulsion c = pair_repulsion(A, p, wk.parity(lat, st),
-                                     bins_at(A.B, wk.parity(lat, st), (clk[lat].rot + st) % 3), lane);
+        c = pair_repulsion(A, p, wk.parity(lat, st), bins_at(A.B, wk.parity(lat, st), (clk[lat].rot + st) % 3), lane);
         wall_repulsion(A, p, wk.parity(lat, st), c);
         if (lane == 0) {
             A.fcol[2 * (long long)p] = c.x;
@@ -1985,7 +2051,7 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock
         }
         unsigned long long t0 = global_ns();
         while (__any_sync(0xffffffffu, done != nullptr)) {
-            unsigned ready = __ballot_sync(0xffffffffu, done != nullptr && load_done(done) == 0);
+            unsigned ready = __ballot_sync(0xffffffffu, done != nullptr && (own || load_done(done) == 0));
             if (ready == 0) {
                 if (__any_sync(0xffffffffu, global_ns() - t0 > WAIT_LIMIT_NS)) return false;
                 __nanosleep(100);
@@ -2000,9 +2066,11 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock
                 const unsigned tag = clk[ql].tag + st;
                 const PartState ps = load_particle(A, q, cur, lane);
                 const int comp = component(lane);
-                const double c = comp < 2 ? __ldcg(A.fcol + 2 * (long long)q + comp) : 0.0;
-                const double f = hydro_sums<true>(A, q, bins_at(A.B, cur, rot), tag, lane);
-                particle_advance(A, q, ps, cur ^ 1, bins_at(A.B, cur ^ 1, rot3(rot + 1)), true, shift, tag + 1, f, c, lane);
+                double ca = comp == 0 ? c.x : (comp == 1 ? c.y : 0.0);
+                if (!own && comp < 2) ca = __ldcg(A.fcol + 2 * (long long)q + comp);
+                const double f = hydro_sums<true>(A, q, bins_at(A.B, cur, rot), tag, lane, &late);
+                if (late) return false;
+                particle_advance(A, q, ps, cur ^ 1, bins_at(A.B, cur ^ 1, rot3(rot + 1)), true, shift, tag + 1, f, ca, lane);
             }
             t0 = global_ns();
         }
@@ -2013,7 +2081,6 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock
 template <typename T, bool EDGES, int W, bool PS, int LATTICES, typename WORK>
 __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame, const StepRun &run) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ int s_stop, s_halt;      // a warp gave up; the block leaves (set between barriers)
     __shared__ StepClock clk[LATTICES]; // every lattice's clock as the launch starts
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SweepSmem<T, W> sm(smem_raw, warp);
@@ -2022,7 +2089,6 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         mbar_init(ring.bar, 1);
         mbar_fence_init();
     }
-    if (threadIdx.x == 0) s_stop = s_halt = 0;
     for (int k = threadIdx.x; k < wk.lattices(); k += blockDim.x) {
         clk[k].tag = __ldcg(&wk.args(k).clock->tag);
         clk[k].rot = __ldcg(&wk.args(k).clock->rot);
@@ -2035,9 +2101,50 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     const int group = sb % ngroups, gwarps = (nsb / ngroups + (group < nsb % ngroups)) * W;
     auto item_of = [&](int k) { return ((k / W) * ngroups + group) * W + (k & (W - 1)); };
     const int nitems = wk.items();
+    const bool counted = !run.dry && !own_warps(wk, run.pblocks * W);
     const FieldsOut fo{nullptr, nullptr, nullptr, nullptr};
-    unsigned target = 0;
+    unsigned target[2] = {0, 0};        // arrivals that end the present meeting
+    // Between steps the blocks meet: what they have written is then visible,
+    // also to the bulk copies (the async proxy).  A warp that gave up (`bad`)
+    // takes its block out; the others' bounded waits then end.
+    auto arrive = [&](bool bad) {
+        if (sweeps) asm volatile("fence.proxy.async;" ::: "memory");
+        if (__syncthreads_or(bad)) return false;
+        target[0] += (unsigned)nsb;
+        target[1] += (unsigned)run.pblocks;
+        if (threadIdx.x == 0) arrive_block(run.sync->arrived[sweeps ? 0 : 1]);
+        return true;
+    };
+    auto await = [&](int which) {
+        bool bad = false;
+        if (threadIdx.x == 0 && !await_blocks(run.sync->arrived[which], target[which])) {
+            atomicOr(wk.args(0).err, ERR_TIMEOUT);
+            bad = true;
+        }
+        if (__syncthreads_or(bad)) return false;
+        asm volatile("fence.proxy.async;" ::: "memory");
+        return true;
+    };
+    // the warp's first segment of a step, its copy issued
+    Cursor c{0, 0, 0};
+    T wv = T();             // the staged segment's periodic-edge value (wrap_load)
+    int item = 0;
+    bool have = false;
+    auto open_step = [&](int st) {
+        c = Cursor{0, 0, 0};
+        item = item_of((sb / ngroups) * W + warp);
+        have = item < nitems;
+        if (!have) return;
+        wk.seek(c, item);
+        const SweepArgs<T> &a = wk.args(c.lat);
+        const T *src = a.buf[wk.parity(c.lat, st)];
+        const int ys = streamed_row<EDGES>(a.L, c.y);
+        issue_segment<T>(src, a.L, ys, c.tx, sm.stage, ring.bar, lane);
+        wv = wrap_load<T>(src, a.L, ys, c.tx, lane);
+        ring.pending = true;
+    };
 
+    if (sweeps) open_step(0);
     for (int st = 0; st < run.nsteps; ++st) {
         bool timed_out = false;
         int shift = 0;
@@ -2052,19 +2159,6 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 timed_out = true;
             }
         } else {
-            Cursor c{0, 0, 0};
-            T wv = T();         // the staged segment's periodic-edge value (wrap_load)
-            int item = item_of((sb / ngroups) * W + warp);
-            bool have = item < nitems;
-            if (have) {
-                wk.seek(c, item);
-                const SweepArgs<T> &a = wk.args(c.lat);
-                const T *src = a.buf[wk.parity(c.lat, st)];
-                const int ys = streamed_row<EDGES>(a.L, c.y);
-                issue_segment<T>(src, a.L, ys, c.tx, sm.stage, ring.bar, lane);
-                wv = wrap_load<T>(src, a.L, ys, c.tx, lane);
-                ring.pending = true;
-            }
             unsigned *ticket = &run.sync->ticket[st % 3][group][0];
             if (warp == 0 && lane == 0 && sb < ngroups) run.sync->ticket[(st + 2) % 3][group][0] = 0;
             if (!run.dry && wk.parts() > 0) {
@@ -2081,14 +2175,14 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 if (lane == 0) k = gwarps + (int)atomicAdd(ticket, 1u);
                 item = item_of(__shfl_sync(0xffffffffu, k, 0));
                 have = item < nitems;
-                Cursor nx = c;
+                        Cursor nx = c;
                 if (have) wk.seek(nx, item);
                 const SweepArgs<T> &a = wk.args(c.lat), &an = wk.args(nx.lat);
                 const int cur = wk.parity(c.lat, st);
                 if (!sweep_segment<T, MODE_STEP, EDGES, PS, true>(
                         a, a.buf[cur], a.buf[cur ^ 1], bins_at(a.B, cur, (clk[c.lat].rot + st) % 3), c.y, c.tx, sm.stage,
                         ring, have, an.buf[wk.parity(nx.lat, st)], an.L, nx.y, nx.tx, sm.crec, sm.cid, wv,
-                        clk[c.lat].tag + st - run.dry, !run.dry, fo, lane)) {
+                        clk[c.lat].tag + st - run.dry, counted, fo, lane)) {
                     if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
                     timed_out = true;
                     break;
@@ -2096,44 +2190,31 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 c = nx;
             }
         }
-        if (timed_out) {
-            if (lane == 0) s_stop = 1;
-            // let the copies this warp still has in flight land before the
-            // block releases its shared memory (the wait bounded again)
-            if (ring.pending) mbar_wait_bounded(ring.bar, ring.parity);
-        }
-        const bool more = st + 1 < run.nsteps;
         if (run.nsteps == 1) break;
-        // ---- every block's populations, bins and positions, before the next
-        // step reads them (its bulk copies in the async proxy)
-        const int meets = shift != 0 ? 2 : (more ? 1 : 0);
-        for (int m = 0; m < meets; ++m) {
-            if (m == 1) {
-                shift_rows<T>(wk.args(0).buf[wk.parity(0, st) ^ 1], wk.args(0).L, shift, (int)blockIdx.x * W + warp,
-                              (int)gridDim.x * W, lane);
-                if (blockIdx.x == 0 && threadIdx.x == 0) *frame->frame_off = __ldcg(frame->frame_off) + shift;
-                if (!more) break;
-            }
-            asm volatile("fence.proxy.async;" ::: "memory");
-            __syncthreads();
-            target += gridDim.x;
-            if (threadIdx.x == 0) {
-                s_halt = s_stop;
-                if (!s_halt && !sync_blocks(run.sync, target)) {
-                    atomicOr(wk.args(0).err, ERR_TIMEOUT);
-                    s_halt = 1;
-                }
-            }
-            __syncthreads();
-            if (s_halt) break;
-            asm volatile("fence.proxy.async;" ::: "memory");
+        const bool more = st + 1 < run.nsteps;
+        if (shift != 0) {
+            if (!arrive(timed_out) || !await(0) || !await(1)) break;
+            shift_rows<T>(wk.args(0).buf[wk.parity(0, st) ^ 1], wk.args(0).L, shift, (int)blockIdx.x * W + warp,
+                          (int)gridDim.x * W, lane);
+            if (blockIdx.x == 0 && threadIdx.x == 0) *frame->frame_off = __ldcg(frame->frame_off) + shift;
+            asm volatile("fence.proxy.async;" ::: "memory");        // (the particle blocks moved rows too)
         }
-        if (s_halt) break;
+        if (more) {
+            // the populations are there once the sweeping blocks have met, and
+            // the next step's first copies start; the bins and positions follow
+            if (!arrive(timed_out) || !await(0)) break;
+            if (shift != 0 && !await(1)) break;         // (every block moved rows)
+            if (sweeps) open_step(st + 1);
+            if (shift == 0 && !await(1)) break;
+        }
     }
+    // let the copies this warp still has in flight (it gave up, or its block
+    // left) land before the block releases its shared memory (the wait bounded)
+    if (ring.pending) mbar_wait_bounded(ring.bar, ring.parity);
     // the last block out leaves the counters as it found them, and advances the clocks
     __syncthreads();
     if (threadIdx.x == 0 && atomicAdd(&run.sync->left, 1u) == gridDim.x - 1) {
-        run.sync->arrived = 0;
+        run.sync->arrived[0][0] = run.sync->arrived[1][0] = 0;
         run.sync->left = 0;
         for (int q = 0; q < 3; ++q)
             for (int g = 0; g < TICKET_GROUPS; ++g) run.sync->ticket[q][g][0] = 0;
