@@ -356,6 +356,8 @@ SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     a.clock = c->strip ? nullptr : &c->sync->clock;
     a.pa = c->np > 0 ? c->pa : nullptr;
     a.np = c->np;
+    // (two copies of 9 populations, past some 3/4 of the 129 MB L2)
+    a.turn = (size_t)c->L.plane * 18 * c->elem > 96u << 20;
     a.eager = c->np <= MAXC && (long long)c->np * c->L.ntx * c->L.ny <= 65536;
     a.cur = c->cur;
     a.ntx_inv = ntx_inverse(c->L.ntx);

@@ -757,6 +757,11 @@ struct SweepArgs {
     // slots and the records of all segments come to no more than 4 MB a step
     // (half a microsecond of the L2's bandwidth).
     bool eager;
+    // Every second step takes the segments from the end, where two buffers do
+    // not fit the L2: the rows a step wrote last are read first by the next one
+    // and are still there.  (4096^2, us per step: FP32 216 -> 214, PS 238 ->
+    // 235; the 400 x 2000 box, which fits, lost 0.2 of 16.)
+    bool turn;
     int cur;                    // parity of the launch's first step
     unsigned ntx_inv;           // floor(2^32 / ntx) + 1 (saturated), see row_of
 };
@@ -1325,7 +1330,14 @@ sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ F
     const int nitems = L.ny * L.ntx;
     const int gw = blockIdx.x * W + warp, nw = gridDim.x * W;
     T wv = T();         // the staged segment's periodic-edge value (wrap_load)
-    int y = row_of(gw, one.ntx_inv, L.ntx), tx = gw - y * L.ntx;
+    // (from the end where the next step would: see SweepArgs::turn)
+    auto seek = [&](int k, int &sy, int &sx) {
+        const int item = one.turn && one.cur && k < nitems ? nitems - 1 - k : k;
+        sy = row_of(item, one.ntx_inv, L.ntx);
+        sx = item - sy * L.ntx;
+    };
+    int y, tx;
+    seek(gw, y, tx);
     if (gw < nitems) {
         issue_segment<T>(src, L, streamed_row<EDGES>(L, y), tx, sm.stage, ring.bar, lane);
         wv = wrap_load<T>(src, L, streamed_row<EDGES>(L, y), tx, lane);
@@ -1335,7 +1347,8 @@ sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ F
     for (int item = gw; item < nitems; item += nw) {
         const int nxt = item + nw;
         const bool has_next = nxt < nitems;
-        const int ny2 = row_of(nxt, one.ntx_inv, L.ntx), nx2 = nxt - ny2 * L.ntx;
+        int ny2, nx2;
+        seek(nxt, ny2, nx2);
         if (!sweep_segment<T, MODE, EDGES, PS, false>(one, src, dst, bins, y, tx, sm.stage, ring, has_next, src, L, ny2,
                                                       nx2, sm.crec, sm.cid, wv, 0u, false, fo, lane)) {
             timed_out = true;
@@ -1980,6 +1993,7 @@ struct OneWork {
     __device__ __forceinline__ int find_part(int g, int &lat) const { lat = 0; return g; }
     // which populations and positions step st of the launch reads
     __device__ __forceinline__ int parity(int, int st) const { return one.cur ^ (st & 1); }
+    __device__ __forceinline__ bool reversed(int st) const { return one.turn && parity(0, st); }
     __device__ __forceinline__ int lattices() const { return 1; }
 };
 
@@ -2009,6 +2023,7 @@ struct BatchWork {
         return g - ba.part_start[lat];
     }
     __device__ __forceinline__ int parity(int lat, int st) const { return ba.a[lat].cur ^ (st & 1); }
+    __device__ __forceinline__ bool reversed(int) const { return false; }
     __device__ __forceinline__ int lattices() const { return ba.n; }
 };
 
@@ -2135,6 +2150,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         item = item_of((sb / ngroups) * W + warp);
         have = item < nitems;
         if (!have) return;
+        if (wk.reversed(st)) item = nitems - 1 - item;
         wk.seek(c, item);
         const SweepArgs<T> &a = wk.args(c.lat);
         const T *src = a.buf[wk.parity(c.lat, st)];
@@ -2175,7 +2191,8 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 if (lane == 0) k = gwarps + (int)atomicAdd(ticket, 1u);
                 item = item_of(__shfl_sync(0xffffffffu, k, 0));
                 have = item < nitems;
-                        Cursor nx = c;
+                if (wk.reversed(st)) item = nitems - 1 - item;
+                Cursor nx = c;
                 if (have) wk.seek(nx, item);
                 const SweepArgs<T> &a = wk.args(c.lat), &an = wk.args(nx.lat);
                 const int cur = wk.parity(c.lat, st);
