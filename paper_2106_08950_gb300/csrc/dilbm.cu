@@ -84,32 +84,31 @@ struct dilbm_ctx {
     bool strip_open = false;               // between dilbm_strip_begin and dilbm_strip_end
     void *owned[40] = {};
     int nowned = 0;
-    // dilbm_set_particles packs into pinned host memory, so its copies run
-    // asynchronously; up_done marks when the last upload's copies have read it
+    // dilbm_set_particles packs into pinned host memory, which the device reads
+    // in place; up_done marks when it has
     void *up_stage = nullptr;
     cudaEvent_t up_done = nullptr;
-    // dilbm_forces with the state: one device block in the staging layout
-    // (force 3 np, fcol 2 np, x, y, r, ux, uy, omega, theta, rho_s as doubles,
-    // then fixed and the error word as ints), read back by one copy
-    double *readback = nullptr;
 };
 
-// Gathers dilbm_forces' outputs into the readback block (layout above).
+// Gathers dilbm_forces' outputs into pinned host memory: force 3 np, fcol
+// 2 np and, with the state, x, y, r, ux, uy, omega, theta, rho_s as doubles
+// (13 np in all), then fixed and the error word as ints.
 __global__ void readback_kernel(double *__restrict__ out, const double *__restrict__ force,
                                 const double *__restrict__ fcol, const double *__restrict__ x,
                                 const double *__restrict__ y, const double *__restrict__ rest,
-                                const int *__restrict__ fixed, const int *__restrict__ err, int np) {
+                                const int *__restrict__ fixed, const int *__restrict__ err, int np, int state) {
     const long long nd = 13LL * np;
     int *oi = reinterpret_cast<int *>(out + nd);
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nd + np + 1;
          i += (long long)gridDim.x * blockDim.x) {
         if (i < 3LL * np) out[i] = force[i];
         else if (i < 5LL * np) out[i] = fcol[i - 3LL * np];
+        else if (i == nd + np) oi[np] = *err;
+        else if (!state) continue;
         else if (i < 6LL * np) out[i] = x[i - 5LL * np];
         else if (i < 7LL * np) out[i] = y[i - 6LL * np];
         else if (i < nd) out[i] = rest[i - 7LL * np];
-        else if (i < nd + np) oi[i - nd] = fixed[i - nd];
-        else oi[np] = *err;
+        else oi[i - nd] = fixed[i - nd];
     }
 }
 
@@ -241,14 +240,24 @@ int launch_cover(dilbm_ctx *c, int pos) {
     return DILBM_OK;
 }
 
-// The particle update as a launch of its own: an upload's binning
-// (integrate == 0), or a phase of a strip's step.
-int launch_particles(dilbm_ctx *c, int integrate, int phase = 0) {
-    particles_kernel<<<(c->np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, c->stream>>>(particle_args(c), c->cur,
-                                                                                              integrate, phase);
+// The particles' present state binned (`in`: uploaded values, see the kernel).
+int launch_bin(dilbm_ctx *c, const double *in) {
+    // (a block per 1024 counts to zero, at most 32, where there are fewer for the particles)
+    const int blocks = std::max((c->np + PART_WARPS - 1) / PART_WARPS, std::min(c->ntiles / 1024, 32));
+    if (c->strip) DILBM_CUDA(cudaMemsetAsync(c->B.count + (size_t)c->cur * c->ntiles, 0, sizeof(int) * c->ntiles, c->stream));
+    bin_particles_kernel<<<blocks, PART_WARPS * 32, 0, c->stream>>>(particle_args(c), c->cur, in, &c->sync->left);
     DILBM_CUDA(cudaGetLastError());
     c->launches += 1;
-    if (c->method == DILBM_METHOD_PS && phase != 1) return launch_cover(c, integrate ? c->cur ^ 1 : c->cur);
+    if (c->method == DILBM_METHOD_PS) return launch_cover(c, c->cur);
+    return DILBM_OK;
+}
+
+// A phase of a strip's particle update.
+int launch_particles(dilbm_ctx *c, int phase) {
+    particles_kernel<<<(c->np + PART_WARPS - 1) / PART_WARPS, PART_WARPS * 32, 0, c->stream>>>(particle_args(c), c->cur, phase);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
+    if (c->method == DILBM_METHOD_PS && phase != 1) return launch_cover(c, c->cur ^ 1);
     return DILBM_OK;
 }
 
@@ -310,9 +319,9 @@ int upload_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
     set_wrap_flags(c, p, np);
     if ((rc = size_cover_tables(c, p, np))) return rc;
     if ((c->L.wrap_x != wx || c->L.wrap_y != wy || c->ph.ck != ck) && (rc = push_part_args(c))) return rc;
-    // pinned staging: x, y, then r, ux, uy, omega, theta, rho_s (one device
-    // slice), as doubles, then fixed as ints; reused once the previous
-    // upload's copies have read it
+    // pinned staging: x, y, r, ux, uy, omega, theta, rho_s as doubles, then
+    // fixed as ints; the binning reads it in place, and it is reused once the
+    // previous upload's has
     if (!c->up_stage) {
         if (cudaHostAlloc(&c->up_stage, (sizeof(double) * 8 + sizeof(int)) * (size_t)np, cudaHostAllocDefault) != cudaSuccess) {
             c->up_stage = nullptr;
@@ -330,17 +339,9 @@ int upload_particles(dilbm_ctx *c, const dilbm_particle *p, int np) {
         h[6 * np + k] = p[k].theta; h[7 * np + k] = p[k].rho_s;
         fx[k] = p[k].fixed ? 1 : 0;
     }
-    const int cur = c->cur;
-    DILBM_CUDA(cudaMemcpyAsync(c->P.x[cur], h, sizeof(double) * np, cudaMemcpyHostToDevice, c->stream));
-    DILBM_CUDA(cudaMemcpyAsync(c->P.y[cur], h + np, sizeof(double) * np, cudaMemcpyHostToDevice, c->stream));
-    // r, ux, uy, omega, theta, rho_s are consecutive slices of one allocation
-    DILBM_CUDA(cudaMemcpyAsync(c->P.r, h + 2 * np, sizeof(double) * 6 * np, cudaMemcpyHostToDevice, c->stream));
-    DILBM_CUDA(cudaMemcpyAsync(c->P.fixed, fx, sizeof(int) * np, cudaMemcpyHostToDevice, c->stream));
+    if (int lrc = launch_bin(c, h)) return lrc;
     DILBM_CUDA(cudaEventRecord(c->up_done, c->stream));
-    clear_counts_kernel<<<(c->ntiles + 255) / 256, 256, 0, c->stream>>>(c->B, c->strip ? nullptr : &c->sync->clock, c->cur);
-    DILBM_CUDA(cudaGetLastError());
-    c->launches += 1;
-    return launch_particles(c, 0);
+    return DILBM_OK;
 }
 
 template <typename T>
@@ -811,7 +812,7 @@ int dilbm_strip_begin(dilbm_ctx *c) {
     if (!c || !c->strip || c->strip_open) return fail(DILBM_ERR_INVALID_ARG, "not a strip, or a step already begun");
     int rc = launch_strip_sweep(c);
     if (rc) return rc;
-    if (c->np > 0 && (rc = launch_particles(c, 1, 1))) return rc;
+    if (c->np > 0 && (rc = launch_particles(c, 1))) return rc;
     // this strip's first and last rows of every plane, for the neighbours
     const size_t pitch_b = (size_t)c->L.pitch * c->elem, plane_b = (size_t)c->L.plane * c->elem;
     const char *dst = static_cast<const char *>(c->buf[c->cur ^ 1]);
@@ -826,7 +827,7 @@ int dilbm_strip_end(dilbm_ctx *c) {
     const dilbm::TraceRange trace("dilbm_strip_end");
     if (!c || !c->strip || !c->strip_open) return fail(DILBM_ERR_INVALID_ARG, "not a strip, or no step begun");
     int rc;
-    if (c->np > 0 && (rc = launch_particles(c, 1, 2))) return rc;
+    if (c->np > 0 && (rc = launch_particles(c, 2))) return rc;
     advance(c, 1);
     c->strip_open = false;
     return DILBM_OK;
@@ -878,24 +879,13 @@ int dilbm_forces(dilbm_ctx *c, double *force, double *fcol, dilbm_particle *stat
     double *hf = h, *hc = h + 3 * np, *hs = h + 5 * np;
     int *fx = reinterpret_cast<int *>(h + 13 * np), *herr = fx + np;
     const size_t block_bytes = sizeof(double) * 13 * np + sizeof(int) * (np + 1);
-    if (state) {
-        // everything in one copy, gathered on the device
-        if (!c->readback) {
-            void *q = nullptr;
-            if (cudaMalloc(&q, block_bytes) != cudaSuccess) return fail(DILBM_ERR_OOM, "device readback block for dilbm_forces");
-            c->readback = static_cast<double *>(q);
-        }
-        const int threads = 256, blocks = (int)((block_bytes / sizeof(int) + threads - 1) / threads);
-        readback_kernel<<<blocks < 4 * c->num_sms ? blocks : 4 * c->num_sms, threads, 0, c->stream>>>(
-            c->readback, c->force, c->fcol, c->P.x[c->cur], c->P.y[c->cur], c->P.r, c->P.fixed, c->err, (int)np);
-        DILBM_CUDA(cudaGetLastError());
-        c->launches += 1;
-        DILBM_CUDA(cudaMemcpyAsync(h, c->readback, block_bytes, cudaMemcpyDeviceToHost, c->stream));
-    } else {
-        DILBM_CUDA(cudaMemcpyAsync(hf, c->force, sizeof(double) * 3 * np, cudaMemcpyDeviceToHost, c->stream));
-        if (fcol) DILBM_CUDA(cudaMemcpyAsync(hc, c->fcol, sizeof(double) * 2 * np, cudaMemcpyDeviceToHost, c->stream));
-        DILBM_CUDA(cudaMemcpyAsync(herr, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-    }
+    // one kernel writes everything in place (gathered on the device and copied
+    // over, the answer came some 5 us later)
+    const int threads = 256, blocks = (int)((block_bytes / sizeof(double) + threads - 1) / threads);
+    readback_kernel<<<blocks < 4 * c->num_sms ? blocks : 4 * c->num_sms, threads, 0, c->stream>>>(
+        h, c->force, c->fcol, c->P.x[c->cur], c->P.y[c->cur], c->P.r, c->P.fixed, c->err, (int)np, state != nullptr);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
     DILBM_CUDA(cudaStreamSynchronize(c->stream));
     c->sticky |= *herr;
     std::memcpy(force, hf, sizeof(double) * 3 * np);
@@ -1067,7 +1057,6 @@ void dilbm_destroy(dilbm_ctx *c) {
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     if (c->up_done) cudaEventDestroy(c->up_done);
     if (c->up_stage) cudaFreeHost(c->up_stage);
-    if (c->readback) cudaFree(c->readback);
     delete c;
 }
 

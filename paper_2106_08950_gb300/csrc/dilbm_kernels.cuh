@@ -1841,58 +1841,86 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
     }
 }
 
-// An upload's binning starts from empty tiles.
-static __global__ void clear_counts_kernel(BinSet B, const StepClock *clock, int cur) {
-    int *count = B.count + (long long)(clock ? __ldcg(&clock->rot) : cur) * B.tiles;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < B.tiles; t += gridDim.x * blockDim.x) count[t] = 0;
-}
-
-// The particle update as a launch of its own, one warp per particle:
-//   integrate == 0: forms 1/m, 1/I, weight and reach and bins the particles
-//                   where they are (an upload);
-//   phase 0: the whole update after a sweep_kernel; 1: only the sums of a
-//   strip's bins, to fpart; 2: the rest from the sums in fpart.
+// New particles (an upload, or where they stand as a context starts), one warp
+// per particle: forms 1/m, 1/I, weight and reach and bins the particle where it
+// is.  `in`: the uploaded values in pinned host memory (x, y, r, ux, uy, omega,
+// theta, rho_s, np doubles each, then np ints `fixed`), read in place; null:
+// they are in device memory already.
+// With a clock, one launch does it all: the particles go into the tile counts
+// that a step would have added to (zero by then), the counts after them are
+// zeroed in their place, and the last block out moves the clock on to the new
+// ones.  (Four copies, a pass that cleared the counts and the binning took the
+// coupled 512^2 step 65 us, this 50.)  Without a clock the caller has zeroed
+// the counts of parity `cur`.
 constexpr int PART_WARPS = 8;
 
 static __global__ void __launch_bounds__(PART_WARPS * 32)
-particles_kernel(const __grid_constant__ PartArgs A, int cur, int integrate, int phase) {
+bin_particles_kernel(const __grid_constant__ PartArgs A, int cur, const double *__restrict__ in, unsigned *left) {
+    const int lane = threadIdx.x & 31, p = blockIdx.x * PART_WARPS + (threadIdx.x >> 5), np = A.bp.np;
+    const int rot = A.clock ? rot3(__ldcg(&A.clock->rot) + 1) : cur;
+    if (A.clock) {
+        int *zero = A.B.count + (long long)rot3(rot + 1) * A.B.tiles;
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < A.B.tiles; t += gridDim.x * blockDim.x) zero[t] = 0;
+    }
+    if (p < np) {
+        const Particles &P = A.P;
+        if (in) {
+            // r .. rho_s lie one after another
+            if (lane < 8) (lane == 0 ? P.x[cur] : (lane == 1 ? P.y[cur] : P.r + (lane - 2) * (long long)np))[p] = in[lane * (long long)np + p];
+            if (lane == 8) P.fixed[p] = reinterpret_cast<const int *>(in + 8 * (long long)np)[p];
+            __syncwarp();
+        }
+        if (lane == 0) {
+            const double r = P.r[p], rho_s = P.rho_s[p];
+            const double area = 3.14159265358979323846 * r * r, m = rho_s * area, wgt = (rho_s - A.bp.rho_f) * area;
+            P.im[p] = 1.0 / m;
+            P.iI[p] = 1.0 / (0.5 * m * r * r);
+            // (1 - rho_f / rho_s) m g is (rho_s - rho_f) pi r^2 g
+            P.wx[p] = wgt * A.bp.gx;
+            P.wy[p] = wgt * A.bp.gy;
+            P.reach[p] = r + A.ph.cut_d;
+            P.rf[p] = (float)r;
+        }
+        __syncwarp();
+        particle_advance(A, p, load_particle(A, p, cur, lane), cur, bins_at(A.B, cur, rot), false, 0,
+                         A.clock ? __ldcg(&A.clock->tag) : 0u, 0.0, 0.0, lane);
+    }
+    if (A.clock) {
+        __syncthreads();
+        if (threadIdx.x == 0 && atomicAdd(left, 1u) == gridDim.x - 1) {
+            *left = 0;
+            A.clock->rot = rot;
+        }
+    }
+}
+
+// The particle update as a launch of its own (a strip's step, the static
+// step), one warp per particle: phase 0: the whole update after a
+// sweep_kernel; 1: only the sums of a strip's bins, to fpart; 2: the rest from
+// the sums in fpart.
+static __global__ void __launch_bounds__(PART_WARPS * 32)
+particles_kernel(const __grid_constant__ PartArgs A, int cur, int phase) {
     const int lane = threadIdx.x & 31, p = blockIdx.x * PART_WARPS + (threadIdx.x >> 5);
     if (p >= A.bp.np) return;
-    const int nxt = integrate ? cur ^ 1 : cur;
-    const Bins in = bins_at(A.B, cur, A.clock ? __ldcg(&A.clock->rot) : cur), out = integrate ? bins_at(A.B, nxt, nxt) : in;
-    const unsigned next_tag = A.clock ? __ldcg(&A.clock->tag) : 0u;
-    if (!integrate && lane == 0) {
-        const Particles &P = A.P;
-        const double r = P.r[p], rho_s = P.rho_s[p];
-        const double area = 3.14159265358979323846 * r * r, m = rho_s * area, wgt = (rho_s - A.bp.rho_f) * area;
-        P.im[p] = 1.0 / m;
-        P.iI[p] = 1.0 / (0.5 * m * r * r);
-        // (1 - rho_f / rho_s) m g is (rho_s - rho_f) pi r^2 g
-        P.wx[p] = wgt * A.bp.gx;
-        P.wy[p] = wgt * A.bp.gy;
-        P.reach[p] = r + A.ph.cut_d;
-        P.rf[p] = (float)r;
-    }
-    __syncwarp();
+    const int nxt = cur ^ 1;
+    const Bins in = bins_at(A.B, cur, cur), out = bins_at(A.B, nxt, nxt);
     const int comp = component(lane);
     double f = 0.0;
     Repulsion c{0.0, 0.0};
-    if (integrate && phase != 2) {
+    if (phase != 2) {
         c = pair_repulsion(A, p, cur, in, lane);
         f = hydro_sums<false>(A, p, in, 0u, lane, nullptr);
     }
     double *o = A.fpart ? A.fpart + 5 * (long long)p : nullptr;
     if (phase == 1) {
-        if (integrate && (lane & 7) == 0 && comp < 3) o[comp] = f;
-        if (integrate && lane == 0) { o[3] = c.x; o[4] = c.y; }
+        if ((lane & 7) == 0 && comp < 3) o[comp] = f;
+        if (lane == 0) { o[3] = c.x; o[4] = c.y; }
         return;
     }
     if (phase == 2) { f = o[comp < 3 ? comp : 0]; c.x = o[3]; c.y = o[4]; }
-    if (integrate) {
-        wall_repulsion(A, p, cur, c);
-        if (lane == 0) { A.fcol[2 * (long long)p] = c.x; A.fcol[2 * (long long)p + 1] = c.y; }
-    }
-    particle_advance(A, p, load_particle(A, p, cur, lane), nxt, out, integrate != 0, 0, next_tag, f,
+    wall_repulsion(A, p, cur, c);
+    if (lane == 0) { A.fcol[2 * (long long)p] = c.x; A.fcol[2 * (long long)p + 1] = c.y; }
+    particle_advance(A, p, load_particle(A, p, cur, lane), nxt, out, true, 0, 0u, f,
                      comp == 0 ? c.x : (comp == 1 ? c.y : 0.0), lane);
 }
 

@@ -255,7 +255,7 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
                                                 "velocities, or a phi tail reaching more than " +
                                                     std::to_string(MAXT) + " tiles; nothing was changed");
         // bin the particles where they are (positions copy 0, bins 0)
-        particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, 0, 0);
+        bin_particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, nullptr, nullptr);
         S_CUDA(cudaGetLastError());
     }
 
@@ -277,7 +277,7 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
 
     if (np > 0) {
         // force reduction, Wan-Turek, Newton-Euler (positions copy 0 -> 1)
-        particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, 1, 0);
+        particles_kernel<<<pblocks, PART_WARPS * 32, 0, st>>>(pa, 0, 0);
         S_CUDA(cudaGetLastError());
         particles_out_kernel<<<(np + 127) / 128, 128, 0, st>>>(particles, P, np);
         S_CUDA(cudaGetLastError());
