@@ -358,7 +358,7 @@ SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     a.pa = c->np > 0 ? c->pa : nullptr;
     a.np = c->np;
     // (two copies of 9 populations, past some 3/4 of the 129 MB L2)
-    a.turn = (size_t)c->L.plane * 18 * c->elem > 96u << 20;
+    a.turn = (size_t)c->L.row * c->L.ny * 2 * c->elem > 96u << 20;
     a.eager = c->np <= MAXC && (long long)c->np * c->L.ntx * c->L.ny <= 65536;
     a.cur = c->cur;
     a.ntx_inv = ntx_inverse(c->L.ntx);
@@ -604,7 +604,8 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     L.nx = g->nx;
     L.ny = g->ny;
     L.pitch = (g->nx + 31) / 32 * 32;
-    L.plane = (long long)L.pitch * L.ny;
+    L.plane = L.pitch;
+    L.row = 9LL * L.pitch;
     L.ntx = (L.nx + TILE_W - 1) / TILE_W;
     L.nty = (L.ny + TILE_H - 1) / TILE_H;
     L.per_x = g->west.kind == DILBM_SIDE_PERIODIC;
@@ -645,7 +646,6 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         c->ty_lo = y0 / TILE_H;
         const bool cut_s = y0 > 0 || L.per_y, cut_n = y1 < g->ny || L.per_y;
         L.ny = y1 - y0;
-        L.plane = (long long)L.pitch * L.ny;
         L.nty = (L.ny + TILE_H - 1) / TILE_H;
         L.per_y = 0;
         if (cut_s) L.side_kind[SOUTH] = SIDE_HALO;
@@ -688,7 +688,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     }
     // each population buffer carries GUARD readable elements on both sides:
     // the sweep stages whole 16-byte-aligned row segments with their halos
-    const size_t pop_elems = 9 * (size_t)L.plane + 2 * (size_t)GUARD;
+    const size_t pop_elems = (size_t)L.row * L.ny + 2 * (size_t)GUARD;
     for (int b = 0; b < 2; ++b) {
         void *q = nullptr;
         cudaError_t e = cudaMalloc(&q, pop_elems * c->elem);
@@ -761,7 +761,6 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         // the neighbours' rows start in the same uniform state
         Lattice Lh = L;
         Lh.ny = 1;
-        Lh.plane = L.pitch;
         switch (c->storage) {
         case DILBM_FP32: init_kernel<float><<<64, 256, 0, c->stream>>>((float *)c->xrecv[k], Lh, drho, u0x, u0y); break;
         case DILBM_FP16_DEV: init_kernel<__half><<<64, 256, 0, c->stream>>>((__half *)c->xrecv[k], Lh, drho, u0x, u0y); break;
@@ -814,11 +813,10 @@ int dilbm_strip_begin(dilbm_ctx *c) {
     if (rc) return rc;
     if (c->np > 0 && (rc = launch_particles(c, 1))) return rc;
     // this strip's first and last rows of every plane, for the neighbours
-    const size_t pitch_b = (size_t)c->L.pitch * c->elem, plane_b = (size_t)c->L.plane * c->elem;
+    const size_t row_b = (size_t)c->L.row * c->elem;
     const char *dst = static_cast<const char *>(c->buf[c->cur ^ 1]);
-    DILBM_CUDA(cudaMemcpy2DAsync(c->xsend[0], pitch_b, dst, plane_b, pitch_b, 9, cudaMemcpyDeviceToDevice, c->stream));
-    DILBM_CUDA(cudaMemcpy2DAsync(c->xsend[1], pitch_b, dst + (size_t)(c->L.ny - 1) * pitch_b, plane_b, pitch_b, 9,
-                                 cudaMemcpyDeviceToDevice, c->stream));
+    DILBM_CUDA(cudaMemcpyAsync(c->xsend[0], dst, row_b, cudaMemcpyDeviceToDevice, c->stream));
+    DILBM_CUDA(cudaMemcpyAsync(c->xsend[1], dst + (size_t)(c->L.ny - 1) * row_b, row_b, cudaMemcpyDeviceToDevice, c->stream));
     c->strip_open = true;
     return DILBM_OK;
 }

@@ -155,6 +155,7 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
     L.ny = g->ny;
     L.pitch = DILBM_STATIC_PITCH(g->nx);
     L.plane = (long long)L.pitch * L.ny;
+    L.row = L.pitch;
     L.ntx = (L.nx + TILE_W - 1) / TILE_W;
     L.nty = (L.ny + TILE_H - 1) / TILE_H;
     const long long ntiles = (long long)L.ntx * L.nty;
