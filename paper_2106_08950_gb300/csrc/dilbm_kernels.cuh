@@ -893,6 +893,11 @@ __device__ __forceinline__ float2 sqrt2(float2 v) {
 // Slot m (0 or 1) of a node pair.
 __device__ __forceinline__ float &slot(float2 &v, int m) { return m ? v.y : v.x; }
 
+// Two neighbouring warps that share a segment (run_steps, HALVES) meet.
+__device__ __forceinline__ void meet_partner() {
+    asm volatile("bar.sync %0, 64;" ::"r"(1 + (int)(threadIdx.x >> 6)) : "memory");
+}
+
 // One row segment (row y, segment tx) of lattice A, populations src -> dst,
 // bins B: wait for its staged rows (and write in the periodic-edge values wv,
 // see wrap_load), then sweep its 128 nodes in two passes of 64 (lane l takes
@@ -901,12 +906,13 @@ __device__ __forceinline__ float &slot(float2 &v, int m) { return m ? v.y : v.x;
 // segment nx2 of lattice Ln, populations srcn; its edge values go to wv) once
 // the second pass has read it, and sum the segment's force / torque per
 // candidate particle.  FUSED: also count the contributions, marked with the
-// step's tag (`count` false: not counted).  Returns false if the bounded wait gave up.
-template <typename T, int MODE, bool EDGES, bool PS, bool FUSED>
+// step's tag (`count` false: not counted); HALVES: this warp runs the pass
+// `half`, its neighbour the other.  Returns false if the bounded wait gave up.
+template <typename T, int MODE, bool EDGES, bool PS, bool FUSED, bool HALVES = false>
 __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *src, T *dst, const Bins &B, int y, int tx,
                                               T *stage, Ring &ring, bool has_next, const T *srcn, const Lattice &Ln,
                                               int ny2, int nx2, float4 *crec, int *cid, T &wv, unsigned tag,
-                                              bool count, const FieldsOut &fo, int lane) {
+                                              bool count, const FieldsOut &fo, int lane, int half = 0) {
     constexpr int H = halo_of<T>(), SW = segw_of<T>();
     const Lattice &L = A.L;
     const Physics &ph = A.ph;
@@ -938,7 +944,10 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
 
     // ---- wait for the staged rows
     // a warp-uniform decision: every lane leaves together if any gave up
-    if (!__all_sync(0xffffffffu, mbar_wait_bounded(ring.bar, ring.parity))) return false;
+    if (!__all_sync(0xffffffffu, mbar_wait_bounded(ring.bar, ring.parity))) {
+        if (HALVES) meet_partner();
+        return false;
+    }
     ring.parity ^= 1u;
     ring.pending = false;
 
@@ -971,9 +980,9 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
 
     // a row's last segment may end within its first half: its second pass
     // would hold no node (no store, no force share), so it is not run
-    const int npass = tx0 + TILE_W / 2 < L.nx ? 2 : 1;
+    const int npass = tx0 + TILE_W / 2 < L.nx && !(HALVES && half == 0) ? 2 : 1;
 #pragma unroll 1
-    for (int pass = 0; pass < npass; ++pass) {
+    for (int pass = HALVES ? half : 0; pass < npass; ++pass) {
         const int e = pass * (TILE_W / 2) + 2 * lane;    // the pair's first node within the segment
         const int x = tx0 + e;
 
@@ -1257,9 +1266,16 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
     if (MODE == MODE_FIELDS) return true;
     if (__any_sync(0xffffffffu, badmax > 0x7f7ffffeu) && lane == 0) atomicOr(A.err, ERR_UNSTABLE);
     // ---- this row segment's force / torque per candidate (zero where no node is owned)
-    __syncwarp();
+    if (HALVES) meet_partner();
+    else __syncwarp();
+    if (HALVES && half == 1) return true;
     if (cands >> lane & 1u) {
-        const float4 sg = crec[NREC * MAXC + lane];
+        float4 sg = crec[NREC * MAXC + lane];
+        if (HALVES) {
+            // the partner's, the second pass's, added as one warp adds them
+            const float4 s2 = crec[(NREC + 1) * MAXC + NREC * MAXC + lane];
+            sg.x += s2.x; sg.y += s2.y; sg.z += s2.z;
+        }
         const int id = cid[lane];
         float4 *out = A.partial + ((long long)id * MAXT + __float_as_int(sg.w)) * TILE_H + (y - ty0);
         if (FUSED) {
@@ -2127,7 +2143,12 @@ __device__ __forceinline__ bool update_particles(const WORK &wk, const StepClock
     return true;
 }
 
-template <typename T, bool EDGES, int W, bool PS, int LATTICES, typename WORK>
+// HALVES: two warps share each row segment, one pass each, where that still
+// leaves every warp at most one: a step of such a lattice is as long as a
+// warp's chain through its segment.  (us per step: 200 x 100 cylinder 9.3 ->
+// 8.3, 501 x 101 channel with a moving frame 10.9 -> 9.9.  A kernel of its own:
+// decided at run time, it took 15 % from every other lattice.)
+template <typename T, bool EDGES, int W, bool PS, int LATTICES, bool HALVES, typename WORK>
 __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame, const StepRun &run) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ StepClock clk[LATTICES]; // every lattice's clock as the launch starts
@@ -2149,7 +2170,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     const int ngroups = nsb < TICKET_GROUPS ? nsb : TICKET_GROUPS;
     const int group = sb % ngroups, gwarps = (nsb / ngroups + (group < nsb % ngroups)) * W;
     auto item_of = [&](int k) { return ((k / W) * ngroups + group) * W + (k & (W - 1)); };
-    const int nitems = wk.items();
+    const int nitems = wk.items() << (int)HALVES;
     const bool counted = !run.dry && !own_warps(wk, run.pblocks * W);
     const FieldsOut fo{nullptr, nullptr, nullptr, nullptr};
     unsigned target[2] = {0, 0};        // arrivals that end the present meeting
@@ -2185,7 +2206,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         have = item < nitems;
         if (!have) return;
         if (wk.reversed(st)) item = nitems - 1 - item;
-        wk.seek(c, item);
+        wk.seek(c, item >> (int)HALVES);
         const SweepArgs<T> &a = wk.args(c.lat);
         const T *src = a.buf[wk.parity(c.lat, st)];
         const int ys = streamed_row<EDGES>(a.L, c.y);
@@ -2230,10 +2251,11 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                 if (have) wk.seek(nx, item);
                 const SweepArgs<T> &a = wk.args(c.lat), &an = wk.args(nx.lat);
                 const int cur = wk.parity(c.lat, st);
-                if (!sweep_segment<T, MODE_STEP, EDGES, PS, true>(
+                if (!sweep_segment<T, MODE_STEP, EDGES, PS, true, HALVES>(
                         a, a.buf[cur], a.buf[cur ^ 1], bins_at(a.B, cur, (clk[c.lat].rot + st) % 3), c.y, c.tx, sm.stage,
                         ring, have, an.buf[wk.parity(nx.lat, st)], an.L, nx.y, nx.tx, sm.crec, sm.cid, wv,
-                        clk[c.lat].tag + st - run.dry, counted, fo, lane)) {
+                        clk[c.lat].tag + st - run.dry, counted, fo, lane,
+                        warp & 1)) {
                     if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
                     timed_out = true;
                     break;
@@ -2277,19 +2299,19 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     }
 }
 
-template <typename T, bool EDGES, int W, bool PS = false>
+template <typename T, bool EDGES, int W, bool PS = false, bool HALVES = false>
 __global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
 step_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ PartArgs pa,
             const __grid_constant__ StepRun run) {
     const OneWork<T> wk{one, pa};
-    run_steps<T, EDGES, W, PS, 1>(wk, &pa, run);
+    run_steps<T, EDGES, W, PS, 1, HALVES>(wk, &pa, run);
 }
 
 template <typename T, int W>
 __global__ void __launch_bounds__(W * 32, sm_warps<T>() / W)
 step_batch_kernel(const __grid_constant__ BatchArgs<T> ba, const __grid_constant__ StepRun run) {
     const BatchWork<T> wk{ba};
-    run_steps<T, true, W, false, BATCH_LAUNCH_MAX>(wk, nullptr, run);
+    run_steps<T, true, W, false, BATCH_LAUNCH_MAX, false>(wk, nullptr, run);
 }
 
 // ------------------------------------------------------------ conversions

@@ -84,19 +84,32 @@ inline cudaError_t launch_steps(const void *kern, void **args, long long blocks,
     return cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, st);
 }
 
-template <typename T, bool EDGES, int W, bool PS>
+template <typename T, bool EDGES, int W, bool PS, bool HALVES = false>
 cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run, const SweepShape &sh, int num_sms,
                          cudaStream_t st, int *per_sm_out) {
     static int cache[64] = {};
     constexpr size_t smem = sweep_smem_bytes<T, W>();
-    auto *kern = step_kernel<T, EDGES, W, PS>;
+    auto *kern = step_kernel<T, EDGES, W, PS, HALVES>;
     int per_sm = 1;
     cudaError_t e = occupancy_of(kern, W, smem, cache, &per_sm);
     if (e != cudaSuccess || per_sm_out) {
         if (per_sm_out) *per_sm_out = per_sm;
         return e;
     }
-    const long long blocks = fused_grid((long long)a.L.ny * a.L.ntx, a.np, W, per_sm, num_sms, sh, &run.pblocks);
+    const long long items = (long long)a.L.ny * a.L.ntx;
+    long long blocks = fused_grid(items, a.np, W, per_sm, num_sms, sh, &run.pblocks);
+    if constexpr (W == 4 && !PS && !HALVES) {
+        // two warps to a segment, where every warp still has at most one (in
+        // the default shape)
+        static int halves_cache[64] = {};
+        int fit = 1;
+        e = occupancy_of(step_kernel<T, EDGES, W, PS, true>, W, smem, halves_cache, &fit);
+        if (e != cudaSuccess) return e;
+        fit = std::min(fit, per_sm);
+        if (fused_grid(1LL << 40, a.np, W, fit, num_sms, sh, &run.pblocks) - run.pblocks >= (2 * items + W - 1) / W)
+            return step_variant<T, EDGES, W, PS, true>(a, pa, run, sh, num_sms, st, per_sm_out);
+    }
+    if constexpr (HALVES) blocks = fused_grid(2 * items, a.np, W, per_sm, num_sms, sh, &run.pblocks);
     void *p[3] = {const_cast<SweepArgs<T> *>(&a), const_cast<PartArgs *>(&pa), &run};
     return launch_steps((const void *)kern, p, blocks, W, smem, st);
 }
