@@ -48,6 +48,8 @@ namespace dilbm {
 
 constexpr int TILE_W = 128;   // nodes per row segment (32 lanes x 4 nodes) and per tile row
 constexpr int TILE_H = 8;     // rows per binning tile
+constexpr int TILE_W_LOG2 = 7, TILE_H_LOG2 = 3;
+static_assert(TILE_W == 1 << TILE_W_LOG2 && TILE_H == 1 << TILE_H_LOG2, "tiles of a power of two");
 constexpr int MAXC = 32;      // candidate particles per tile
 constexpr int MAXT = 128;     // tiles one particle's phi tail may reach
 constexpr int NREC = 3;       // float4 records per binned particle
@@ -428,14 +430,15 @@ __host__ __device__ inline int wrap_int(int v, int n) {
     return ((v % n) + n) % n;
 }
 
-__host__ __device__ inline AxisTiles axis_tiles(double X, double R, int n, int tile, int ntiles, int periodic) {
+// (tiles of 2^shift nodes)
+__host__ __device__ inline AxisTiles axis_tiles(double X, double R, int n, int shift, int ntiles, int periodic) {
     AxisTiles t;
     int il = floor_int(X - R), ih = ceil_int(X + R);
     if (periodic) {
         if (ih - il + 1 >= n) { t.n = 1; t.lo[0] = 0; t.hi[0] = ntiles - 1; return t; }
         const int a = wrap_int(il, n), b = wrap_int(ih, n);
-        if (a <= b) { t.n = 1; t.lo[0] = a / tile; t.hi[0] = b / tile; return t; }
-        int first_hi = b / tile, second_lo = a / tile;
+        if (a <= b) { t.n = 1; t.lo[0] = a >> shift; t.hi[0] = b >> shift; return t; }
+        int first_hi = b >> shift, second_lo = a >> shift;
         if (first_hi >= second_lo) { t.n = 1; t.lo[0] = 0; t.hi[0] = ntiles - 1; return t; }
         t.n = 2; t.lo[0] = 0; t.hi[0] = first_hi; t.lo[1] = second_lo; t.hi[1] = ntiles - 1;
         return t;
@@ -443,7 +446,7 @@ __host__ __device__ inline AxisTiles axis_tiles(double X, double R, int n, int t
     il = il < 0 ? 0 : il;
     ih = ih > n - 1 ? n - 1 : ih;
     if (il > ih) { t.n = 0; return t; }
-    t.n = 1; t.lo[0] = il / tile; t.hi[0] = ih / tile;
+    t.n = 1; t.lo[0] = il >> shift; t.hi[0] = ih >> shift;
     return t;
 }
 
@@ -1771,13 +1774,14 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
     const float omh = __shfl_sync(0xffffffffu, uh, 16), uxl = __shfl_sync(0xffffffffu, ul, 0);
     const float uyl = __shfl_sync(0xffffffffu, ul, 8), oml = __shfl_sync(0xffffffffu, ul, 16);
     // the tiles along the lane's axis
-    const AxisTiles at = comp == 0 ? axis_tiles(n, st.reach, L.nx, TILE_W, L.ntx, L.per_x)
-                                   : axis_tiles(n, st.reach, L.ny, TILE_H, L.nty, L.per_y);
+    const AxisTiles at = axis_tiles(n, st.reach, comp == 0 ? L.nx : L.ny, comp == 0 ? TILE_W_LOG2 : TILE_H_LOG2,
+                                    comp == 0 ? L.ntx : L.nty, comp == 0 ? L.per_x : L.per_y);
     AxisTiles ax, ay;
     ax.n = __shfl_sync(0xffffffffu, at.n, 0);
     ay.n = __shfl_sync(0xffffffffu, at.n, 8);
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
+        if (q == 1 && ax.n < 2 && ay.n < 2) break;
         ax.lo[q] = __shfl_sync(0xffffffffu, at.lo[q], 0);
         ax.hi[q] = __shfl_sync(0xffffffffu, at.hi[q], 0);
         ay.lo[q] = __shfl_sync(0xffffffffu, at.lo[q], 8);
