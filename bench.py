@@ -401,8 +401,8 @@ def gpu_arm(args):
     sim.step(2)
     sim.sync()
 
-    # ---- device-resident throughput: steps replayed from CUDA graphs,
-    # bracketed by CUDA events on the launching stream
+    # ---- device-resident throughput: steps in fused launches, bracketed by
+    # CUDA events on the launching stream
     clocks = ClockSampler(local)
     clocks.start()
     time.sleep(0.3)
@@ -419,7 +419,8 @@ def gpu_arm(args):
     barrier(dist)
     launches = sim.launches - l0
     ms = ev0.elapsed_time(ev1)
-    # ---- the sweep kernel alone: events around each launch (direct launches)
+    # ---- the step kernel (sweep and particle update) one step per launch,
+    # events around each launch
     sim.set_timing(True)
     sim.step(min(args.steps, 400))
     sweep_ms, sweep_n = sim.sweep_time()
@@ -456,7 +457,8 @@ def gpu_arm(args):
                "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                "loop": "per step: dilbm_set_particles(host) + dilbm_step(1) + dilbm_forces(host)"}
 
-    # ---- roofline of the dominant kernel (the lattice sweep)
+    # ---- roofline of the dominant kernel (the fused step: the lattice sweep
+    # with the particle update beside it)
     peak, peak_kind = measured_peak_hbm()
     per_launch_ms = sweep_ms / max(sweep_n, 1)
     alg_bytes = BYTES_PER_NODE[args.storage] * nodes
@@ -464,7 +466,7 @@ def gpu_arm(args):
     traffic = measured_traffic(f"{args.workload}:{args.storage}:{prob.nx}x{prob.ny}" + (":ps" if prob.method == W.METHOD_PS else ""))
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic, "peak_kind": peak_kind,
-            "kernel": "sweep_kernel", "sweep_ms_per_launch": per_launch_ms,
+            "kernel": "step_kernel", "sweep_ms_per_launch": per_launch_ms,
             "sweep_share_of_step": per_launch_ms / (ms / args.steps) if ms > 0 else None,
             "algorithmic_bytes_per_launch": alg_bytes}
 
@@ -580,7 +582,7 @@ def batch_arm(args):
                        "storage": args.storage, "nodes": nodes, "nodes_all_ranks": total_nodes, "lattices": len(jobs),
                        "force_model": ", ".join(sorted({force_model_name(j.force_model) for j in jobs})),
                        "particles": sum(len(j.particles) for j in jobs),
-                       "launch": "one batched sweep + one batched particle launch per step, CUDA-graph replay",
+                       "launch": "one cooperative launch per several steps over all lattices' segments and particles",
                        "launch_shape": {"warps_per_block": shape[0], "blocks_per_sm": shape[1],
                                         "by": "--shape" if args.shape else "autotuner"},
                        "l2": f"{nodes * BYTES_PER_NODE[args.storage] / 1e6:.0f} MB of populations per step"},
@@ -588,7 +590,7 @@ def batch_arm(args):
                               "speedup_of_batch": value / alone_value},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                          "traffic": measured_traffic(f"batch:{args.storage}:{len(jobs)}x{nodes}"),
-                         "peak_kind": peak_kind, "kernel": "sweep_kernel (batched)",
+                         "peak_kind": peak_kind, "kernel": "step_batch_kernel",
                          "sweep_ms_per_launch": per_launch, "algorithmic_bytes_per_launch": alg},
             "gpu_launches": int(sum_over_ranks(dist, launches, dev)), "e2e": None, "clocks": clk}
     if rank == 0:
@@ -720,7 +722,7 @@ def serve_arm(args):
     total_work = sum_over_ranks(dist, work, dev)        # node updates of all ranks' requests
     stream = torch.cuda.Stream(device=dev)
     sh = int(stream.cuda_stream)
-    # warm-up: one small job through each path (module load, graph capture)
+    # warm-up: one small job through each path (module load)
     warm = [W.Request(0.0, 10, W.cylinder_drag())]
     replay_served(warm, "fp16", args, D)
     replay_single(warm, "fp32", D, sh)

@@ -419,8 +419,8 @@ class Strip(Simulation):
 
 
 class Batch:
-    """Several Simulations advanced together (``dilbm_batch_*``): one sweep and
-    one particle launch per step for all members, replayed from CUDA graphs.
+    """Several Simulations advanced together (``dilbm_batch_*``): one launch
+    runs several steps of all members.
     The members stay usable on their own; they must outlive the batch."""
 
     def __init__(self, sims):

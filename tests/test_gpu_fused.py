@@ -174,3 +174,62 @@ def test_captured_steps_replay_from_any_step(stream, steps, replays, batched):
             f(5)
     for s in want + got:
         s.close()
+
+
+def _grid_of_discs(nx, ny, count, walls):
+    """`count` small moving discs on a grid, some across tile edges."""
+    rows = max(1, int(np.sqrt(count * ny / nx)))
+    cols = -(-count // rows)
+    rng = np.random.default_rng(7)
+    parts = [W.Particle((k % cols + 0.5) * nx / cols, (k // cols + 0.5) * ny / rows, 5.0, ux=rng.uniform(-0.02, 0.02),
+                        uy=rng.uniform(-0.02, 0.02), omega=rng.uniform(-1e-3, 1e-3), rho_s=1.3) for k in range(count)]
+    sides = dict(west=W.Side(W.VELOCITY, 0.01, 0.0), east=W.Side(W.PRESSURE), south=W.wall(), north=W.wall(0.002)) if walls else {}
+    return W.Problem(nx=nx, ny=ny, tau=0.8, eps=1.5, gravity=(0.0, -1e-6), u0=(0.01, 0.0),
+                     wan_turek=W.wan_turek_defaults(5.0, 1.3, 1.0, 1e-5), particles=parts, **sides)
+
+
+# Where a lattice stepped alone takes another way than in a batch: two warps to
+# a segment (up to 1518 segments in FP32, 1822 in FP16, on 152 SMs), records
+# loaded beside the mask (discs times segments up to 65536), slots by number (up
+# to 32 discs), and steps from the end (two buffers over 96 MB).
+ALONE = [(256, 759, 2, True, "fp32"), (256, 760, 2, True, "fp32"), (200, 759, 3, False, "fp32"),
+         (190, 911, 2, True, "fp16"), (190, 912, 2, True, "fp16"), (3, 5, 0, True, "fp32"), (129, 8, 1, False, "bf16"),
+         (512, 512, 32, False, "fp32"), (512, 513, 32, False, "fp32"), (384, 300, 33, True, "fp32"),
+         (1184, 1184, 40, False, "fp32"), (1184, 1180, 40, False, "fp32"), (1700, 1700, 8, True, "fp16")]
+
+
+@pytest.mark.parametrize("nx,ny,count,walls,storage", ALONE)
+def test_alone_as_in_a_batch(stream, nx, ny, count, walls, storage):
+    prob = _grid_of_discs(nx, ny, count, walls)
+    a, b = (D.Simulation(prob, storage=storage, stream=int(stream.cuda_stream)) for _ in range(2))
+    batch = D.Batch([b])
+    for n in (1, 12, 7):
+        a.step(n)
+        batch.step(n)
+        assert np.array_equal(a.populations(), b.populations())
+        assert all(np.array_equal(x, y) for x, y in zip(a.fields(), b.fields()))
+        assert all(np.array_equal(x, y) for x, y in zip(a.forces(), b.forces()))
+    batch.sync()
+    batch.close()
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("count", [1, 32, 33])
+def test_uploads_in_a_row(stream, count):
+    """Uploads between steps, one or several in a row, leave the same state."""
+    prob = _grid_of_discs(400, 300, count, True)
+    a, b = (D.Simulation(prob, stream=int(stream.cuda_stream)) for _ in range(2))
+    moved = [W.Particle(q.x + 1.25, q.y - 0.5, q.r, ux=-q.ux, uy=q.uy, rho_s=1.2, fixed=k % 5 == 0)
+             for k, q in enumerate(prob.particles)]
+    for times in (1, 3, 2):
+        for s, m in ((a, 1), (b, times)):
+            s.step(2)
+            for k in range(m):
+                s.set_particles(prob.particles if k + 1 < m else moved)
+            s.step(4)
+        assert np.array_equal(a.populations(), b.populations())
+        assert all(np.array_equal(x, y) for x, y in zip(a.forces(), b.forces()))
+        assert all(np.array_equal(x, y) for x, y in zip(a.fields(), b.fields()))
+    a.close()
+    b.close()
