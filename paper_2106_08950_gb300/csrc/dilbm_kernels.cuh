@@ -31,11 +31,12 @@
 // few registers live; writes go straight from registers, one contiguous run
 // per plane and pair.
 //
-// One launch per step pair of kernels against one launch over many steps, us
-// per step (FP32 unless said): 200 x 100 cylinder 18.5 -> 11.5, 400 x 2000 box
-// 36.9 -> 17.3, 1793 x 179 channel in FP16 21.6 -> 13.3, 512^2 suspension
-// 22.6 -> 14.4, 501 x 101 channel with a moving frame 30.8 -> 11.7, 64 uneven
-// lattices 264 -> 242, 4096^2 suspension 225.6 -> 219.1 (FP16 221.4 -> 207.3).
+// Two launches a step (sweep, particles) against this, us per step (FP32 unless
+// said, default shapes): 200 x 100 cylinder 18.5 -> 8.3, 400 x 2000 box
+// 36.9 -> 16.0, 1793 x 179 channel in FP16 21.6 -> 11.6, 512^2 suspension
+// 22.6 -> 12.3, 501 x 101 channel with a moving frame 30.8 -> 9.7, 64 uneven
+// lattices 264 -> 237, 4096^2 suspension 225.6 -> 210 (FP16 221.4 -> 202, PS
+// 247 -> 230).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -131,8 +132,8 @@ struct Lattice {
     int nx, ny, pitch;          // nodes; row pitch in elements (multiple of 32)
     // Elements from a direction's row to the next direction's and from a row to
     // the next: pitch and 9 * pitch in a context, ny * pitch and pitch in the
-    // static step's planes (its caller's layout).  Rows against planes, 4096^2,
-    // us per step: FP32 214 -> 212, FP16 199 -> 197, PS 235 -> 233.
+    // static step's planes (its caller's layout).  Rows against planes on 4096^2,
+    // us per step less: FP32 1.3, FP16 2.1, PS 2.2.
     long long plane, row;
     int ntx, nty;               // tiles along x and y
     bool per_x, per_y;          // periodic axes
@@ -1876,7 +1877,7 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
 // that a step would have added to (zero by then), the counts after them are
 // zeroed in their place, and the last block out moves the clock on to the new
 // ones.  (Four copies, a pass that cleared the counts and the binning took the
-// coupled 512^2 step 65 us, this 50.)  Without a clock the caller has zeroed
+// coupled 512^2 step 64 us, this 48.)  Without a clock the caller has zeroed
 // the counts of parity `cur`.
 constexpr int PART_WARPS = 8;
 

@@ -65,13 +65,16 @@ inline long long persistent_grid(long long items, int warps, int per_sm, int num
 }
 
 // The blocks of a fused launch: sweeping blocks, and particle blocks in front
-// of them -- a warp per particle, up to a tenth of the resident blocks (at
-// 2048 discs on 4096^2 each warp then has about seven updates of a few
-// microseconds in a step of 200).
+// of them, up to a tenth of the resident ones.  A particle has a warp of its
+// own where a warp sweeps few segments; with more, a warp updates up to eight
+// particles while the others sweep (an update under load takes some 5 us, a
+// segment 4).  (Blocks for 2048 discs on 4096^2: 76 or 47 of 760, 223 us a step
+// with outputs; 31, 280.  For 1056 discs in 64 lattices: 76, 335 us; 31, 324.)
 inline long long fused_grid(long long items, long long parts, int warps, int per_sm, int num_sms, const SweepShape &sh,
                             int *pblocks) {
     const long long most = persistent_grid(1LL << 40, warps, per_sm, num_sms, sh);
-    const long long pb = std::min((parts + warps - 1) / warps, std::max(most / 10, 1LL));
+    const long long each = std::min(std::max(items / (6 * most * warps), 1LL), 8LL);
+    const long long pb = std::min((parts + warps * each - 1) / (warps * each), std::max(most / 10, 1LL));
     *pblocks = (int)pb;
     const long long sweep = persistent_grid(items, warps, per_sm, num_sms, sh);
     return std::max(std::min(sweep, most - pb), 1LL) + pb;
@@ -106,7 +109,7 @@ cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run,
         e = occupancy_of(step_kernel<T, EDGES, W, PS, true>, W, smem, halves_cache, &fit);
         if (e != cudaSuccess) return e;
         fit = std::min(fit, per_sm);
-        if (fused_grid(1LL << 40, a.np, W, fit, num_sms, sh, &run.pblocks) - run.pblocks >= (2 * items + W - 1) / W)
+        if (fused_grid(2 * items, a.np, W, fit, num_sms, sh, &run.pblocks) - run.pblocks >= (2 * items + W - 1) / W)
             return step_variant<T, EDGES, W, PS, true>(a, pa, run, sh, num_sms, st, per_sm_out);
     }
     if constexpr (HALVES) blocks = fused_grid(2 * items, a.np, W, per_sm, num_sms, sh, &run.pblocks);
