@@ -398,7 +398,7 @@ int launch_fields(dilbm_ctx *c, const FieldsOut &fo) {
 int launch_strip_sweep(dilbm_ctx *c) {
     const cudaError_t e = by_storage(c->storage, [&](auto t) {
         using T = decltype(t);
-        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, c->num_sms, c->stream);
+        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, c->shape, c->num_sms, c->stream);
     });
     if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
     c->launches += 1;
@@ -638,6 +638,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     }
     const bool strip = y0 > 0 || y1 < g->ny;
     if (strip) {
+        c->shape = SWEEP_SHAPE;
         // the particles keep the whole lattice's geometry; the sweep sees
         // rows [y0, y1) with halo rows beyond each cut
         c->strip = true;

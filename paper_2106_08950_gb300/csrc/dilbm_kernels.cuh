@@ -1329,12 +1329,11 @@ __device__ __forceinline__ int row_of(unsigned item, unsigned inv, int ntx) {
 // The sweep over one lattice without the particle update (a strip's step, the
 // static step, and the fields).  Persistent: warps take row segments
 // round-robin (neighbouring warps on neighbouring segments); each warp keeps
-// its next segment staged ahead.
-template <typename T, int MODE, bool EDGES, bool PS>
-__global__ void __launch_bounds__(SWEEP_WARPS * 32, 20 / SWEEP_WARPS)
+// its next segment staged ahead.  W warps per block.
+template <typename T, int MODE, bool EDGES, bool PS, int W>
+__global__ void __launch_bounds__(W * 32, 20 / W)
 sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ FieldsOut fo)
 {
-    constexpr int W = SWEEP_WARPS;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     SweepSmem<T, W> sm(smem_raw, warp);

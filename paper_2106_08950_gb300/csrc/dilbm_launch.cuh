@@ -20,7 +20,8 @@ struct SweepShape {
     int blocks_per_sm = 0;      // persistent blocks per SM; 0: as many as fit
 };
 
-constexpr SweepShape PS_SHAPE{SWEEP_WARPS, 0};     // the shape a PS-LBM context reports
+constexpr SweepShape SWEEP_SHAPE{SWEEP_WARPS, 0};  // sweep_kernel's: a strip's until another is set, and the fields'
+constexpr SweepShape PS_SHAPE = SWEEP_SHAPE;       // the one shape a PS-LBM context takes and reports
 constexpr int PS_WARPS = 4;                        // warps per block its fused steps are compiled for
 
 constexpr int SHAPE_WARPS[3] = {2, 4, 8};
@@ -134,17 +135,21 @@ cudaError_t batch_variant(const BatchArgs<T> &ba, StepRun run, const SweepShape 
     return launch_steps((const void *)kern, p, blocks, W, smem, st);
 }
 
-// The sweep without the particle update, in the default shape (a strip's
-// step; MODE_FIELDS: the macroscopic fields instead of a step).
-template <typename T, int MODE, bool EDGES, bool PS>
-cudaError_t sweep_variant(const SweepArgs<T> &a, const FieldsOut &fo, int num_sms, cudaStream_t st) {
+// The sweep without the particle update (a strip's step, in the strip's shape;
+// MODE_FIELDS: the macroscopic fields instead of a step).
+template <typename T, int MODE, bool EDGES, bool PS, int W = SWEEP_WARPS>
+cudaError_t sweep_variant(const SweepArgs<T> &a, const FieldsOut &fo, int num_sms, cudaStream_t st,
+                          const SweepShape &sh = SWEEP_SHAPE, int *per_sm_out = nullptr) {
     static int cache[64] = {};
-    constexpr size_t smem = sweep_smem_bytes<T>();
+    constexpr size_t smem = sweep_smem_bytes<T, W>();
     int per_sm = 1;
-    cudaError_t e = occupancy_of(sweep_kernel<T, MODE, EDGES, PS>, SWEEP_WARPS, smem, cache, &per_sm);
-    if (e != cudaSuccess) return e;
-    const long long blocks = persistent_grid((long long)a.L.ny * a.L.ntx, SWEEP_WARPS, per_sm, num_sms, PS_SHAPE);
-    sweep_kernel<T, MODE, EDGES, PS><<<(unsigned)blocks, SWEEP_WARPS * 32, smem, st>>>(a, fo);
+    cudaError_t e = occupancy_of(sweep_kernel<T, MODE, EDGES, PS, W>, W, smem, cache, &per_sm);
+    if (e != cudaSuccess || per_sm_out) {
+        if (per_sm_out) *per_sm_out = per_sm;
+        return e;
+    }
+    const long long blocks = persistent_grid((long long)a.L.ny * a.L.ntx, W, per_sm, num_sms, sh);
+    sweep_kernel<T, MODE, EDGES, PS, W><<<(unsigned)blocks, W * 32, smem, st>>>(a, fo);
     return cudaGetLastError();
 }
 
@@ -159,8 +164,9 @@ struct Launch {
     // fused steps of a batch
     static cudaError_t batch(const BatchArgs<T> &ba, const StepRun &run, const SweepShape &sh, int num_sms,
                              cudaStream_t st, int *per_sm = nullptr);
-    // a strip's sweep
-    static cudaError_t sweep(const SweepArgs<T> &a, bool edges, bool ps, int num_sms, cudaStream_t st);
+    // a strip's sweep (PS-LBM: in the default shape)
+    static cudaError_t sweep(const SweepArgs<T> &a, bool edges, bool ps, const SweepShape &sh, int num_sms,
+                             cudaStream_t st, int *per_sm = nullptr);
     static cudaError_t fields(const SweepArgs<T> &a, const FieldsOut &fo, bool edges, bool ps, int num_sms,
                               cudaStream_t st);
 };

@@ -274,7 +274,7 @@ extern "C" int dilbm_step_static(const dilbm_grid *g, double tau, double interfa
     sa.err = err;
     sa.np = np;
     sa.ntx_inv = ntx_inverse(L.ntx);
-    S_CUDA(Launch<float>::sweep(sa, !(L.per_x && L.per_y), false, sms, st));
+    S_CUDA(Launch<float>::sweep(sa, !(L.per_x && L.per_y), false, SWEEP_SHAPE, sms, st));
 
     if (np > 0) {
         // force reduction, Wan-Turek, Newton-Euler (positions copy 0 -> 1)
