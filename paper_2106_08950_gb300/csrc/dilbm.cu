@@ -395,11 +395,17 @@ int launch_fields(dilbm_ctx *c, const FieldsOut &fo) {
     return DILBM_OK;
 }
 
-int launch_strip_sweep(dilbm_ctx *c) {
-    const cudaError_t e = by_storage(c->storage, [&](auto t) {
+// A strip's sweep in shape `sh` (per_sm: occupancy only).
+cudaError_t strip_sweep(dilbm_ctx *c, const SweepShape &sh, int *per_sm = nullptr) {
+    return by_storage(c->storage, [&](auto t) {
         using T = decltype(t);
-        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, c->shape, c->num_sms, c->stream);
+        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, sh, c->num_sms, c->stream,
+                                per_sm);
     });
+}
+
+int launch_strip_sweep(dilbm_ctx *c) {
+    const cudaError_t e = strip_sweep(c, c->shape);
     if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
     c->launches += 1;
     return DILBM_OK;
@@ -1452,18 +1458,20 @@ int dilbm_autotune(dilbm_ctx *c, int reps, int *warps, int *blocks_per_sm) {
         report_shape(c->shape, warps, blocks_per_sm);
         return DILBM_OK;
     }
-    const auto key = std::make_tuple(0, c->storage, has_edges(c) ? 1 : 0, (long long)c->L.nx, (long long)c->L.ny);
+    // (a strip has no step clock: its sweep is a kernel of its own)
+    const auto key = std::make_tuple(c->strip ? 2 : 0, c->storage, has_edges(c) ? 1 : 0, (long long)c->L.nx, (long long)c->L.ny);
     SweepShape best = c->shape;
     if (!tuned(key, &best)) {
         std::vector<SweepShape> cands;
         std::vector<int> wps;
-        int rc = shape_candidates([&](const SweepShape &sh, int *per_sm) { return fused_steps(c, sh, StepRun{}, per_sm); },
-                                  &cands, &wps);
-        if (rc) return rc;
         // each launch sweeps the current state into the other buffer (what
         // the next step writes anyway) and updates no particle
-        rc = time_shapes(c->stream, reps, cands, wps,
-                         [&](const SweepShape &sh) { return fused_steps(c, sh, StepRun{1, 1, c->sync, 0}); }, &best);
+        auto sweep = [&](const SweepShape &sh, int *per_sm) {
+            return c->strip ? strip_sweep(c, sh, per_sm) : fused_steps(c, sh, StepRun{1, 1, c->sync, 0}, per_sm);
+        };
+        int rc = shape_candidates(sweep, &cands, &wps);
+        if (rc) return rc;
+        rc = time_shapes(c->stream, reps, cands, wps, [&](const SweepShape &sh) { return sweep(sh, nullptr); }, &best);
         c->launches += (long long)cands.size() * (reps + 1) * TUNE_ROUNDS;
         if (rc) return rc;
         remember(key, best);

@@ -1,4 +1,5 @@
-"""The calls a strip shares with a whole lattice: the launch shape.
+"""The calls a strip shares with a whole lattice: the launch shape, the
+autotuner.
 
 A strip steps through ``begin`` / ``end``; without an exchange between them
 its halo rows and force sums stay its own, which is enough here: the same
@@ -73,3 +74,21 @@ def test_a_strip_runs_in_the_shape_that_is_set(stream):
         ms[shape] = a.elapsed_time(b)
     s.close()
     assert ms[(2, 1)] > 1.5 * ms[(8, 0)], ms
+
+
+@pytest.mark.parametrize("storage", ["fp32", "fp16", "bf16"])
+def test_autotune_times_the_strips_own_sweep(stream, storage):
+    tuned, plain = (D.Strip(problem(nx=176, ny=104), 8, 104, storage, int(stream.cuda_stream)) for _ in range(2))
+    steps(tuned, 3)
+    before = tuned.launches
+    w, b = tuned.autotune(reps=2)
+    assert w in (2, 4, 8) and b >= 0
+    assert tuned.launches > before
+    before = tuned.launches
+    assert tuned.autotune(reps=2) == (w, b) and tuned.launches == before     # cached: nothing launched
+    steps(tuned, 6)
+    steps(plain, 9)
+    for x, y in zip(result(tuned), result(plain)):
+        assert np.array_equal(x, y)
+    tuned.close()
+    plain.close()
