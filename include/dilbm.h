@@ -293,8 +293,8 @@ const char *dilbm_last_error(void);
 
 /*
  * Measurement: with timing on, each step is a launch of its own (the sweep,
- * with the particle update running beside it), bracketed by CUDA events on
- * the context's stream; dilbm_sweep_time() returns their summed duration in
+ * with the particle update running beside it; on a strip the sweep alone),
+ * bracketed by CUDA events on the context's stream; dilbm_sweep_time() returns their summed duration in
  * milliseconds and the number of launches since timing was (re)enabled.
  * dilbm_launch_count() is the number of kernels this context has launched.
  */

@@ -404,9 +404,30 @@ cudaError_t strip_sweep(dilbm_ctx *c, const SweepShape &sh, int *per_sm = nullpt
     });
 }
 
+// A pair of events around a launch, for dilbm_sweep_time.
+int timing_pair(std::vector<cudaEvent_t> &ev, size_t &used, cudaEvent_t *e0, cudaEvent_t *e1) {
+    if (used + 2 > ev.size()) {
+        for (int k = 0; k < 64; ++k) {
+            cudaEvent_t e;
+            DILBM_CUDA(cudaEventCreate(&e));
+            ev.push_back(e);
+        }
+    }
+    *e0 = ev[used];
+    *e1 = ev[used + 1];
+    used += 2;
+    return DILBM_OK;
+}
+
 int launch_strip_sweep(dilbm_ctx *c) {
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    if (c->timing) {
+        if (int rc = timing_pair(c->ev, c->ev_used, &e0, &e1)) return rc;
+        DILBM_CUDA(cudaEventRecord(e0, c->stream));
+    }
     const cudaError_t e = strip_sweep(c, c->shape);
     if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
+    if (c->timing) DILBM_CUDA(cudaEventRecord(e1, c->stream));
     c->launches += 1;
     return DILBM_OK;
 }
@@ -437,21 +458,6 @@ int launch_fused(dilbm_ctx *c, int k) {
 int steps_per_launch(double nodes) {
     const double k = 134217728.0 / nodes;
     return k < 1.0 ? 1 : (k > 1024.0 ? 1024 : (int)k);
-}
-
-// A pair of events around a launch, for dilbm_sweep_time.
-int timing_pair(std::vector<cudaEvent_t> &ev, size_t &used, cudaEvent_t *e0, cudaEvent_t *e1) {
-    if (used + 2 > ev.size()) {
-        for (int k = 0; k < 64; ++k) {
-            cudaEvent_t e;
-            DILBM_CUDA(cudaEventCreate(&e));
-            ev.push_back(e);
-        }
-    }
-    *e0 = ev[used];
-    *e1 = ev[used + 1];
-    used += 2;
-    return DILBM_OK;
 }
 
 // One step, its launch bracketed by events.

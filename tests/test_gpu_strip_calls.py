@@ -1,5 +1,5 @@
 """The calls a strip shares with a whole lattice: the launch shape, the
-autotuner.
+autotuner, the sweep's timing.
 
 A strip steps through ``begin`` / ``end``; without an exchange between them
 its halo rows and force sums stay its own, which is enough here: the same
@@ -92,3 +92,19 @@ def test_autotune_times_the_strips_own_sweep(stream, storage):
         assert np.array_equal(x, y)
     tuned.close()
     plain.close()
+
+
+@pytest.mark.parametrize("method", [W.METHOD_DI, W.METHOD_PS])
+def test_timing_records_every_sweep_of_a_strip(stream, method):
+    prob = problem()
+    prob.method = method
+    s = D.Strip(prob, 0, 48, "fp32", int(stream.cuda_stream))
+    s.set_timing(True)
+    assert s.sweep_time() == (0.0, 0)
+    steps(s, 70)                            # past one allotment of events
+    ms, n = s.sweep_time()
+    assert n == 70 and ms > 0.0
+    s.set_timing(False)
+    steps(s, 2)
+    assert s.sweep_time()[1] == 0
+    s.close()
