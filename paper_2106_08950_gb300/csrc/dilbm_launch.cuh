@@ -9,26 +9,14 @@
 // The launchers are compiled once per storage type, each in its own
 // translation unit (dilbm_launch_f32.cu, _f16.cu, _bf16.cu).
 #pragma once
+#include "dilbm_grid.h"
 #include "dilbm_kernels.cuh"
 
-#include <algorithm>
-
 namespace dilbm {
-
-struct SweepShape {
-    int warps = 4;              // rows in flight per block: 2, 4 or 8
-    int blocks_per_sm = 0;      // persistent blocks per SM; 0: as many as fit
-};
 
 constexpr SweepShape SWEEP_SHAPE{SWEEP_WARPS, 0};  // sweep_kernel's: a strip's until another is set, and the fields'
 constexpr SweepShape PS_SHAPE = SWEEP_SHAPE;       // the one shape a PS-LBM context takes and reports
 constexpr int PS_WARPS = 4;                        // warps per block its fused steps are compiled for
-
-constexpr int SHAPE_WARPS[3] = {2, 4, 8};
-
-__host__ inline bool shape_valid(const SweepShape &s) {
-    return (s.warps == 2 || s.warps == 4 || s.warps == 8) && s.blocks_per_sm >= 0;
-}
 
 // row_of's multiplier: floor(2^32 / ntx) + 1 (unused for ntx == 1).
 inline unsigned ntx_inverse(int ntx) {
@@ -55,32 +43,6 @@ cudaError_t occupancy_of(K kern, int warps, size_t smem, int *cache, int *per_sm
     return cudaSuccess;
 }
 
-// Persistent grid: num_sms x blocks per SM (capped by the shape and by the
-// kernel's occupancy), but no more blocks than the work list needs.
-inline long long persistent_grid(long long items, int warps, int per_sm, int num_sms, const SweepShape &sh) {
-    const int bps = sh.blocks_per_sm > 0 && sh.blocks_per_sm < per_sm ? sh.blocks_per_sm : per_sm;
-    long long blocks = (long long)num_sms * bps;
-    const long long need = (items + warps - 1) / warps;
-    if (blocks > need) blocks = need;
-    return blocks > 0 ? blocks : 1;
-}
-
-// The blocks of a fused launch: sweeping blocks, and particle blocks in front
-// of them, up to a tenth of the resident ones.  A particle has a warp of its
-// own where a warp sweeps few segments; with more, a warp updates up to eight
-// particles while the others sweep (an update under load takes some 5 us, a
-// segment 4).  (Blocks for 2048 discs on 4096^2: 76 or 47 of 760, 223 us a step
-// with outputs; 31, 280.  For 1056 discs in 64 lattices: 76, 335 us; 31, 324.)
-inline long long fused_grid(long long items, long long parts, int warps, int per_sm, int num_sms, const SweepShape &sh,
-                            int *pblocks) {
-    const long long most = persistent_grid(1LL << 40, warps, per_sm, num_sms, sh);
-    const long long each = std::min(std::max(items / (6 * most * warps), 1LL), 8LL);
-    const long long pb = std::min((parts + warps * each - 1) / (warps * each), std::max(most / 10, 1LL));
-    *pblocks = (int)pb;
-    const long long sweep = persistent_grid(items, warps, per_sm, num_sms, sh);
-    return std::max(std::min(sweep, most - pb), 1LL) + pb;
-}
-
 // Blocks of a fused launch wait for one another (particle blocks for the
 // sweeping ones, and all of them between steps), so it is launched
 // cooperatively: the driver starts it only with every block resident.
@@ -101,7 +63,6 @@ cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run,
         return e;
     }
     const long long items = (long long)a.L.ny * a.L.ntx;
-    long long blocks = fused_grid(items, a.np, W, per_sm, num_sms, sh, &run.pblocks);
     if constexpr (W == 4 && !PS && !HALVES) {
         // two warps to a segment, where every warp still has at most one (in
         // the default shape)
@@ -109,13 +70,13 @@ cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run,
         int fit = 1;
         e = occupancy_of(step_kernel<T, EDGES, W, PS, true>, W, smem, halves_cache, &fit);
         if (e != cudaSuccess) return e;
-        fit = std::min(fit, per_sm);
-        if (fused_grid(2 * items, a.np, W, fit, num_sms, sh, &run.pblocks) - run.pblocks >= (2 * items + W - 1) / W)
+        if (one_item_per_warp(2 * items, a.np, W, fit, num_sms, sh))
             return step_variant<T, EDGES, W, PS, true>(a, pa, run, sh, num_sms, st, per_sm_out);
     }
-    if constexpr (HALVES) blocks = fused_grid(2 * items, a.np, W, per_sm, num_sms, sh, &run.pblocks);
+    const FusedGrid g = fused_grid(HALVES ? 2 * items : items, a.np, W, per_sm, num_sms, sh);
+    run.pblocks = g.pblocks;
     void *p[3] = {const_cast<SweepArgs<T> *>(&a), const_cast<PartArgs *>(&pa), &run};
-    return launch_steps((const void *)kern, p, blocks, W, smem, st);
+    return launch_steps((const void *)kern, p, g.blocks, W, smem, st);
 }
 
 template <typename T, int W>
@@ -130,9 +91,10 @@ cudaError_t batch_variant(const BatchArgs<T> &ba, StepRun run, const SweepShape 
         if (per_sm_out) *per_sm_out = per_sm;
         return e;
     }
-    const long long blocks = fused_grid(ba.item_start[ba.n], ba.part_start[ba.n], W, per_sm, num_sms, sh, &run.pblocks);
+    const FusedGrid g = fused_grid(ba.item_start[ba.n], ba.part_start[ba.n], W, per_sm, num_sms, sh);
+    run.pblocks = g.pblocks;
     void *p[2] = {const_cast<BatchArgs<T> *>(&ba), &run};
-    return launch_steps((const void *)kern, p, blocks, W, smem, st);
+    return launch_steps((const void *)kern, p, g.blocks, W, smem, st);
 }
 
 // The sweep without the particle update (a strip's step, in the strip's shape;
