@@ -359,7 +359,7 @@ SweepArgs<T> sweep_args(const dilbm_ctx *c) {
     a.np = c->np;
     // (two copies of 9 populations, past some 3/4 of the 129 MB L2)
     a.turn = (size_t)c->L.row * c->L.ny * 2 * c->elem > 96u << 20;
-    a.eager = c->np <= MAXC && (long long)c->np * c->L.ntx * c->L.ny <= 65536;
+    a.eager = c->np <= MAXC && (long long)c->np * c->L.ntx * c->L.ny <= 4096;
     a.cur = c->cur;
     a.ntx_inv = ntx_inverse(c->L.ntx);
     return a;
