@@ -1277,15 +1277,15 @@ int dilbm_batch_sync(dilbm_batch *b, int *first_failed) {
     DILBM_CUDA(cudaMemcpyAsync(b->err_host.data(), b->err_out, sizeof(int) * n, cudaMemcpyDeviceToHost, b->stream));
     DILBM_CUDA(cudaStreamSynchronize(b->stream));
     if (first_failed) *first_failed = -1;
+    int first = -1;
     for (int k = 0; k < n; ++k) {
         dilbm_ctx *c = b->members[k];
         c->sticky |= b->err_host[k];
-        if (c->sticky) {
-            if (first_failed) *first_failed = k;
-            return sticky_error(c->sticky);
-        }
+        if (c->sticky && first < 0) first = k;
     }
-    return DILBM_OK;
+    if (first < 0) return DILBM_OK;
+    if (first_failed) *first_failed = first;
+    return sticky_error(b->members[first]->sticky);
 }
 
 int dilbm_batch_errors(dilbm_batch *b, int *codes) {
