@@ -247,6 +247,21 @@ int dilbm_set_moving_frame(dilbm_ctx *ctx, int particle, double x_ref);
 int dilbm_wait_probe(void *cuda_stream, double *waited_seconds);
 
 /*
+ * The same check for the waits of a step, with no fault.  dilbm_stall_probe
+ * with a particle's index: that particle's next update waits for force
+ * partials that no sweep writes.  With -1 (dilbm_batch_stall_probe: of a
+ * batch's first launch): the blocks of the next launch over several steps wait
+ * for one block more than there is.  A wait gives up after 1 s and its launch
+ * ends (its other blocks' waits run out in their turn); every lattice in the
+ * launch has missed steps and reports TIMEOUT, at dilbm_sync and the like.  A
+ * lattice that has reported it takes no further steps: later launches return
+ * at once, and a batch leaves it out once the host has read its error.  The
+ * device stays usable.  Queued on the context's (the batch's) stream.
+ * Errors: INVALID_ARG (NULL, a strip, index), CUDA.
+ */
+int dilbm_stall_probe(dilbm_ctx *ctx, int particle);
+
+/*
  * Columns the frame has moved since create (0 if it never moved).  offset:
  * host.  Synchronises the stream.  Errors: INVALID_ARG, CUDA.
  */
@@ -330,6 +345,7 @@ int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilb
 int dilbm_batch_step(dilbm_batch *batch, long long nsteps);
 int dilbm_batch_sync(dilbm_batch *batch, int *first_failed);
 int dilbm_batch_errors(dilbm_batch *batch, int *codes);
+int dilbm_batch_stall_probe(dilbm_batch *batch);
 int dilbm_batch_set_timing(dilbm_batch *batch, int enable);
 int dilbm_batch_sweep_time(dilbm_batch *batch, double *ms_total, long long *launches);
 long long dilbm_batch_launch_count(const dilbm_batch *batch);

@@ -593,6 +593,24 @@ __global__ void wait_probe_kernel(int *err, unsigned long long *waited_ns) {
     }
 }
 
+// The same for a fused step's waits: particle p waits for the partials of one
+// tile more than it reaches (p < 0: the launch's blocks for one block more than
+// there is).
+__global__ void stall_kernel(const __grid_constant__ PartArgs A, GridSync *sync, int cur, int p) {
+    if (p < 0) {
+        atomicSub(&sync->arrived[0][0], 1u);
+        return;
+    }
+    const Bins B = bins_at(A.B, cur, A.clock->rot);
+    const int nk = B.npslot[p];
+    if (nk >= MAXT) return;
+    B.pslot[(long long)p * MAXT + nk] = -1;
+    for (int q = 0; q < TILE_H; ++q)
+        store_partial(A.partial + ((long long)p * MAXT + nk) * TILE_H + q, 0.f, 0.f, 0.f, A.clock->tag - 1);
+    B.npslot[p] = nk + 1;
+    B.done[p] -= TILE_H;
+}
+
 extern "C" {
 
 const char *dilbm_last_error(void) { return g_err.c_str(); }
@@ -758,7 +776,11 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         (e = cudaMemsetAsync(c->sync, 0, sizeof(GridSync), c->stream)) != cudaSuccess ||
         // (no partial carries the tag of a step to come)
         (e = cudaMemsetAsync(c->partial, 0xff, sizeof(float4) * MAXT * TILE_H * npa, c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * c->ntiles, c->stream)) != cudaSuccess)
+        (e = cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * c->ntiles, c->stream)) != cudaSuccess ||
+        // (where steps were given up: a count may stand beside ids never written,
+        // and the positions of the other parity be the ones that are read)
+        (e = cudaMemsetAsync(pd, 0, sizeof(double) * 4 * npa, c->stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(B.ids, 0, sizeof(int2) * 2 * c->ntiles * MAXC, c->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMemsetAsync"));
     // uniform initial state f^eq(rho_init, u0)
     const int blocks = 152 * 8;
@@ -974,6 +996,15 @@ int dilbm_wait_probe(void *cuda_stream, double *waited_seconds) {
     return DILBM_OK;
 }
 
+int dilbm_stall_probe(dilbm_ctx *c, int particle) {
+    if (!c || c->strip || particle < -1 || particle >= c->np)
+        return fail(DILBM_ERR_INVALID_ARG, "stall probe: NULL context, a strip, or a particle index out of range");
+    stall_kernel<<<1, 1, 0, c->stream>>>(particle_args(c), c->sync, c->cur, particle);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
+    return DILBM_OK;
+}
+
 int dilbm_force_mean_reset(dilbm_ctx *c) {
     if (!c) return fail(DILBM_ERR_INVALID_ARG, "NULL context");
     if (c->np > 0) DILBM_CUDA(cudaMemsetAsync(c->fsum, 0, sizeof(double) * 3 * c->np, c->stream));
@@ -1138,15 +1169,18 @@ __global__ void gather_errors_kernel(int *const *__restrict__ err, int n, int *_
 }
 
 // The launch arguments from the members' present state: members in groups of
-// at most BATCH_LAUNCH_MAX.
+// at most BATCH_LAUNCH_MAX.  A member known to have given up steps takes no
+// more of them, and a launch with it in would leave the others' out too.
 template <typename T>
 void fill_groups(dilbm_batch *b) {
     const int n = (int)b->members.size();
     for (int g0 = 0, g = 0; g0 < n; g0 += BATCH_LAUNCH_MAX, ++g) {
         BatchArgs<T> &ba = *static_cast<BatchArgs<T> *>(b->groups[g]);
-        ba.n = n - g0 < BATCH_LAUNCH_MAX ? n - g0 : BATCH_LAUNCH_MAX;
-        for (int k = 0; k < ba.n; ++k) {
-            const dilbm_ctx *c = b->members[g0 + k];
+        ba.n = 0;
+        for (int m = g0; m < n && m < g0 + BATCH_LAUNCH_MAX; ++m) {
+            const dilbm_ctx *c = b->members[m];
+            if (c->sticky & ERR_TIMEOUT) continue;
+            const int k = ba.n++;
             ba.a[k] = sweep_args<T>(c);
             ba.a[k].eager = 0;      // (the records of 64 lattices are too many: 242 us a step became 264)
             ba.item_start[k + 1] = ba.item_start[k] + c->L.ny * c->L.ntx;
@@ -1162,8 +1196,9 @@ cudaError_t batch_groups(dilbm_batch *b, const SweepShape &sh, int nsteps, int d
         using T = decltype(t);
         fill_groups<T>(b);
         for (size_t g = 0; g < b->groups.size(); ++g) {
-            const cudaError_t e = Launch<T>::batch(*static_cast<const BatchArgs<T> *>(b->groups[g]),
-                                                   StepRun{nsteps, dry, b->sync[g], 0}, sh, b->members[0]->num_sms, b->stream);
+            const BatchArgs<T> &ba = *static_cast<const BatchArgs<T> *>(b->groups[g]);
+            if (ba.n == 0) continue;
+            const cudaError_t e = Launch<T>::batch(ba, StepRun{nsteps, dry, b->sync[g], 0}, sh, b->members[0]->num_sms, b->stream);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
@@ -1294,6 +1329,14 @@ int dilbm_batch_errors(dilbm_batch *b, int *codes) {
     int rc = dilbm_batch_sync(b, &first);
     if (rc != DILBM_OK && first < 0) return rc;      // a CUDA error, not a member's
     for (size_t k = 0; k < b->members.size(); ++k) codes[k] = sticky_code(b->members[k]->sticky);
+    return DILBM_OK;
+}
+
+int dilbm_batch_stall_probe(dilbm_batch *b) {
+    if (!b) return fail(DILBM_ERR_INVALID_ARG, "NULL batch");
+    stall_kernel<<<1, 1, 0, b->stream>>>(PartArgs{}, b->sync[0], 0, -1);
+    DILBM_CUDA(cudaGetLastError());
+    b->launches += 1;
     return DILBM_OK;
 }
 

@@ -1977,8 +1977,9 @@ constexpr int TICKET_GROUPS = 8;
 struct GridSync {               // all 0 between launches, but for the clock
     unsigned arrived[2][32];    // sweeping blocks, particle blocks (a cache line each)
     unsigned left;
+    unsigned abandoned;         // a wait ran out, or had before the launch: not all steps were done
     StepClock clock;            // a context's own (a batch's launches advance its members' clocks)
-    unsigned pad[29];
+    unsigned pad[28];
     unsigned ticket[3][TICKET_GROUPS][32];      // by step in rotation and group, a cache line each
 };
 
@@ -2004,6 +2005,13 @@ __device__ __forceinline__ bool await_blocks(const unsigned *arrived, unsigned t
         if (t0 == 0) t0 = t;
         else if (t - t0 > WAIT_LIMIT_NS) return false;
     }
+}
+
+// A wait ran out: the launch ends early, and the last block out tells every
+// lattice in it.  (Before this block is counted out.)
+__device__ __forceinline__ void abandon(GridSync *sync) {
+    atomicExch(&sync->abandoned, 1u);
+    __threadfence();
 }
 
 // The frame's move by s columns, in place: warps take rows of planes, 32
@@ -2165,11 +2173,15 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         mbar_init(ring.bar, 1);
         mbar_fence_init();
     }
+    // A lattice whose steps were given up once takes no more of them: what its
+    // particles would wait for is not there.
+    bool dead = false;
     for (int k = threadIdx.x; k < wk.lattices(); k += blockDim.x) {
         clk[k].tag = __ldcg(&wk.args(k).clock->tag);
         clk[k].rot = __ldcg(&wk.args(k).clock->rot);
+        dead |= __ldcg(wk.args(k).err) & ERR_TIMEOUT;
     }
-    __syncthreads();
+    int st = __syncthreads_or(dead) ? run.nsteps + 1 : 0;
     const bool sweeps = (int)blockIdx.x >= run.pblocks;
     // this block among the sweeping ones, its group and the group's warps
     const int sb = (int)blockIdx.x - run.pblocks, nsb = (int)gridDim.x - run.pblocks;
@@ -2182,7 +2194,8 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     unsigned target[2] = {0, 0};        // arrivals that end the present meeting
     // Between steps the blocks meet: what they have written is then visible,
     // also to the bulk copies (the async proxy).  A warp that gave up (`bad`)
-    // takes its block out; the others' bounded waits then end.
+    // takes its block out; the others' bounded waits then end, and the launch:
+    // every lattice in it misses steps, and its error word says so.
     auto arrive = [&](bool bad) {
         if (sweeps) asm volatile("fence.proxy.async;" ::: "memory");
         if (__syncthreads_or(bad)) return false;
@@ -2193,10 +2206,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     };
     auto await = [&](int which) {
         bool bad = false;
-        if (threadIdx.x == 0 && !await_blocks(run.sync->arrived[which], target[which])) {
-            atomicOr(wk.args(0).err, ERR_TIMEOUT);
-            bad = true;
-        }
+        if (threadIdx.x == 0) bad = !await_blocks(run.sync->arrived[which], target[which]);
         if (__syncthreads_or(bad)) return false;
         asm volatile("fence.proxy.async;" ::: "memory");
         return true;
@@ -2221,8 +2231,8 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         ring.pending = true;
     };
 
-    if (sweeps) open_step(0);
-    for (int st = 0; st < run.nsteps; ++st) {
+    if (sweeps && st == 0) open_step(0);
+    for (; st < run.nsteps; ++st) {
         bool timed_out = false;
         int shift = 0;
         const int track = frame ? frame->track : -1;    // (a batch's frames stand still)
@@ -2232,7 +2242,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         }
         if (!sweeps) {
             if (!run.dry && !update_particles(wk, clk, st, shift, (int)blockIdx.x * W + warp, run.pblocks * W, lane)) {
-                if (lane == 0) atomicOr(wk.args(0).err, ERR_TIMEOUT);
+                if (lane == 0) abandon(run.sync);
                 timed_out = true;
             }
         } else {
@@ -2262,14 +2272,14 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
                         ring, have, an.buf[wk.parity(nx.lat, st)], an.L, nx.y, nx.tx, sm.crec, sm.cid, wv,
                         clk[c.lat].tag + st - run.dry, counted, fo, lane,
                         warp & 1)) {
-                    if (lane == 0) atomicOr(a.err, ERR_TIMEOUT);
+                    if (lane == 0) abandon(run.sync);
                     timed_out = true;
                     break;
                 }
                 c = nx;
             }
         }
-        if (run.nsteps == 1) break;
+        if (run.nsteps == 1) continue;
         const bool more = st + 1 < run.nsteps;
         if (shift != 0) {
             if (!arrive(timed_out) || !await(0) || !await(1)) break;
@@ -2292,9 +2302,12 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     if (ring.pending) mbar_wait_bounded(ring.bar, ring.parity);
     // the last block out leaves the counters as it found them, and advances the clocks
     __syncthreads();
+    if (threadIdx.x == 0 && st != run.nsteps) abandon(run.sync);        // (left before its end)
     if (threadIdx.x == 0 && atomicAdd(&run.sync->left, 1u) == gridDim.x - 1) {
         run.sync->arrived[0][0] = run.sync->arrived[1][0] = 0;
         run.sync->left = 0;
+        if (atomicExch(&run.sync->abandoned, 0u))
+            for (int k = 0; k < wk.lattices(); ++k) atomicOr(wk.args(k).err, ERR_TIMEOUT);
         for (int q = 0; q < 3; ++q)
             for (int g = 0; g < TICKET_GROUPS; ++g) run.sync->ticket[q][g][0] = 0;
         for (int k = 0; k < wk.lattices() && !run.dry; ++k) {

@@ -144,6 +144,8 @@ def load_library(path: Optional[str] = None):
     L.dilbm_force_mean_reset.argtypes = [vp]
     L.dilbm_set_moving_frame.argtypes = [vp, C.c_int, C.c_double]
     L.dilbm_wait_probe.argtypes = [vp, C.POINTER(C.c_double)]
+    L.dilbm_stall_probe.argtypes = [vp, C.c_int]
+    L.dilbm_batch_stall_probe.argtypes = [vp]
     L.dilbm_frame_offset.argtypes = [vp, C.POINTER(C.c_longlong)]
     L.dilbm_server_clock.argtypes = [vp]
     L.dilbm_server_clock.restype = C.c_double
@@ -161,7 +163,8 @@ def load_library(path: Optional[str] = None):
                  "dilbm_server_create", "dilbm_server_submit", "dilbm_server_progress", "dilbm_server_status",
                  "dilbm_server_result", "dilbm_force_mean", "dilbm_force_mean_reset", "dilbm_autotune",
                  "dilbm_set_shape", "dilbm_batch_autotune", "dilbm_batch_set_shape", "dilbm_set_moving_frame",
-                 "dilbm_frame_offset", "dilbm_wait_probe", "dilbm_create_strip", "dilbm_strip_begin",
+                 "dilbm_frame_offset", "dilbm_wait_probe", "dilbm_stall_probe", "dilbm_batch_stall_probe",
+                 "dilbm_create_strip", "dilbm_strip_begin",
                  "dilbm_strip_end", "dilbm_strip_buffers"):
         getattr(L, name).restype = C.c_int
     if path == LIB_PATH:
@@ -359,6 +362,11 @@ class Simulation:
         """``arr``: a ctypes array of Particle (e.g. in pinned memory)."""
         check(self.L.dilbm_set_particles(self.h, arr, self.np))
 
+    def stall_probe(self, particle: int) -> None:
+        """Failure-detection check (no fault): a wait of the next steps runs out
+        (``dilbm_stall_probe``)."""
+        check(self.L.dilbm_stall_probe(self.h, int(particle)))
+
     # -- launch shape
     def autotune(self, reps: int = 10):
         """Time the candidate sweep shapes on this lattice, keep the fastest;
@@ -450,6 +458,17 @@ class Batch:
         rc = self.L.dilbm_batch_sync(self.h, C.byref(bad))
         if rc != OK:
             raise DilbmError(rc, f"member {bad.value}: " + self.L.dilbm_last_error().decode(errors="replace"))
+
+    def errors(self):
+        """Every member's error code (``OK`` or its sticky error)."""
+        codes = (C.c_int * len(self.sims))()
+        check(self.L.dilbm_batch_errors(self.h, codes))
+        return list(codes)
+
+    def stall_probe(self) -> None:
+        """Failure-detection check (no fault): the blocks of the next launch over
+        several steps wait for one more than there is (``dilbm_batch_stall_probe``)."""
+        check(self.L.dilbm_batch_stall_probe(self.h))
 
     def autotune(self, reps: int = 10):
         w, b = C.c_int(), C.c_int()
