@@ -203,7 +203,8 @@ int dilbm_forces(dilbm_ctx *ctx, double *force, double *fcol, dilbm_particle *st
  * Time mean of the hydrodynamic force and torque (Eqs. 18-19) over the steps
  * since create or the last dilbm_force_mean_reset(): mean host np x 3
  * (Fx, Fy, T); *nsteps receives the number of steps averaged (the mean is 0
- * when it is 0).  Each step adds its force in FP64 on the device.
+ * when it is 0).  Each step adds its force in FP64 on the device, and counts
+ * where it runs: a recorded step once per replay.
  * dilbm_force_mean synchronises the stream; the reset is asynchronous.
  */
 int dilbm_force_mean(dilbm_ctx *ctx, double *mean, long long *nsteps);

@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -55,7 +56,7 @@ struct dilbm_ctx {
     GridSync *sync = nullptr;         // device: the barrier of launches over several steps, and the step clock
     double *force = nullptr, *fcol = nullptr;
     double *fsum = nullptr;           // per particle: sum of (Fx, Fy, T) since the last reset
-    long long fsum_steps = 0;
+    long long fsum_steps = 0;         // steps queued since then (see summed_steps)
     int *err = nullptr;
     int sticky = 0;
     float *fields = nullptr;          // 4 x nx x ny, allocated on first use
@@ -437,6 +438,11 @@ void advance(dilbm_ctx *c, int k) {
     c->cur ^= k & 1;
     c->fsum_steps += k;
 }
+
+// Steps whose forces the device has summed: `counted`, the steps its clock has
+// counted (modulo 2^32), which holds also where recorded launches were
+// replayed; `queued`, the host's count, tells the multiple of 2^32.
+long long summed_steps(long long queued, unsigned counted) { return queued + (int)(counted - (unsigned)queued); }
 
 // k steps in one launch (k == 1: no barrier, and the PS tables and the moving
 // frame's shift as launches of their own).
@@ -936,11 +942,13 @@ int dilbm_forces(dilbm_ctx *c, double *force, double *fcol, dilbm_particle *stat
 int dilbm_force_mean(dilbm_ctx *c, double *mean, long long *nsteps) {
     if (!c || !nsteps || (c->np > 0 && !mean)) return fail(DILBM_ERR_INVALID_ARG, "NULL argument");
     const int np = c->np;
-    *nsteps = c->fsum_steps;
-    if (np == 0) return read_sticky(c);
-    DILBM_CUDA(cudaMemcpyAsync(mean, c->fsum, sizeof(double) * 3 * np, cudaMemcpyDeviceToHost, c->stream));
+    unsigned tags[3] = {0, 0, 0};       // clock.tag, clock.rot, mean_tag
+    static_assert(offsetof(GridSync, mean_tag) == offsetof(GridSync, clock) + 2 * sizeof(unsigned), "read together below");
+    if (np > 0) DILBM_CUDA(cudaMemcpyAsync(mean, c->fsum, sizeof(double) * 3 * np, cudaMemcpyDeviceToHost, c->stream));
+    if (!c->strip) DILBM_CUDA(cudaMemcpyAsync(tags, &c->sync->clock, sizeof(tags), cudaMemcpyDeviceToHost, c->stream));
     const int rc = read_sticky(c);   // synchronises the stream
-    const double inv = c->fsum_steps > 0 ? 1.0 / (double)c->fsum_steps : 0.0;
+    *nsteps = c->strip ? c->fsum_steps : summed_steps(c->fsum_steps, tags[0] - tags[2]);
+    const double inv = *nsteps > 0 ? 1.0 / (double)*nsteps : 0.0;
     for (int k = 0; k < 3 * np; ++k) mean[k] *= inv;
     return rc;
 }
@@ -1008,6 +1016,7 @@ int dilbm_stall_probe(dilbm_ctx *c, int particle) {
 int dilbm_force_mean_reset(dilbm_ctx *c) {
     if (!c) return fail(DILBM_ERR_INVALID_ARG, "NULL context");
     if (c->np > 0) DILBM_CUDA(cudaMemsetAsync(c->fsum, 0, sizeof(double) * 3 * c->np, c->stream));
+    DILBM_CUDA(cudaMemcpyAsync(&c->sync->mean_tag, &c->sync->clock.tag, sizeof(unsigned), cudaMemcpyDeviceToDevice, c->stream));
     c->fsum_steps = 0;
     return DILBM_OK;
 }

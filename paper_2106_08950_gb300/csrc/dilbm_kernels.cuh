@@ -1974,12 +1974,13 @@ particles_kernel(const __grid_constant__ PartArgs A, int cur, int phase) {
 // which keeps all warps near the same rows.
 constexpr int TICKET_GROUPS = 8;
 
-struct GridSync {               // all 0 between launches, but for the clock
+struct GridSync {               // all 0 between launches, but for the clock and mean_tag
     unsigned arrived[2][32];    // sweeping blocks, particle blocks (a cache line each)
     unsigned left;
     unsigned abandoned;         // a wait ran out, or had before the launch: not all steps were done
     StepClock clock;            // a context's own (a batch's launches advance its members' clocks)
-    unsigned pad[28];
+    unsigned mean_tag;          // the clock's step number when the force sums were last zeroed
+    unsigned pad[27];
     unsigned ticket[3][TICKET_GROUPS][32];      // by step in rotation and group, a cache line each
 };
 
