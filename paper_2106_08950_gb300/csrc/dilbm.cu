@@ -225,10 +225,15 @@ PartArgs particle_args(const dilbm_ctx *c) {
     return a;
 }
 
-// The device copy that fused steps read, after anything in it has changed.
+__global__ void store_args_kernel(const __grid_constant__ PartArgs a, PartArgs *to) { *to = a; }
+
+// The device copy that a batch's steps read, after anything in it has changed.
+// (By a launch's parameters: a copy from this frame, recorded into a graph,
+// would read it when the frame is gone.)
 int push_part_args(dilbm_ctx *c) {
-    const PartArgs a = particle_args(c);
-    DILBM_CUDA(cudaMemcpyAsync(c->pa, &a, sizeof(a), cudaMemcpyHostToDevice, c->stream));
+    store_args_kernel<<<1, 1, 0, c->stream>>>(particle_args(c), c->pa);
+    DILBM_CUDA(cudaGetLastError());
+    c->launches += 1;
     return DILBM_OK;
 }
 
