@@ -51,7 +51,7 @@ struct dilbm_ctx {
     int cur = 0;
     Particles P{};
     BinSet B{};                       // tile bins
-    float4 *partial = nullptr;        // per particle, tile of its list and row: force / torque partials
+    float4 *partial = nullptr;        // force / torque partials (see partials_by_slot)
     PartArgs *pa = nullptr;           // device: the particle update's arguments (push_part_args)
     GridSync *sync = nullptr;         // device: the barrier of launches over several steps, and the step clock
     double *force = nullptr, *fcol = nullptr;
@@ -180,7 +180,7 @@ unsigned long long footprint_of(int nx, int ny, size_t elem, int np) {
     unsigned long long b = 2ull * (9ull * plane + 2ull * GUARD) * elem;           // populations A, B
     b += 15ull * npa * sizeof(double) + 5ull * npa * sizeof(float) + npa * sizeof(int);   // particle state
     b += 6ull * npa * sizeof(double) + 2ull * npa * sizeof(double) + sizeof(int);         // force, fsum, fcol, err
-    b += npa * MAXT * TILE_H * sizeof(float4);                                            // partials
+    b += (unsigned long long)partial_entries((long long)ntiles, (long long)npa) * sizeof(float4);   // partials
     b += 3ull * ntiles * sizeof(int) + 2ull * ntiles * MAXC * (sizeof(int2) + NREC * sizeof(float4)) +
          2ull * npa * (MAXT + 2) * sizeof(int);                                           // bins
     b += sizeof(PartArgs) + sizeof(GridSync);
@@ -614,10 +614,19 @@ __global__ void stall_kernel(const __grid_constant__ PartArgs A, GridSync *sync,
     }
     const Bins B = bins_at(A.B, cur, A.clock->rot);
     const int nk = B.npslot[p];
-    if (nk >= MAXT) return;
-    B.pslot[(long long)p * MAXT + nk] = -1;
-    for (int q = 0; q < TILE_H; ++q)
-        store_partial(A.partial + ((long long)p * MAXT + nk) * TILE_H + q, 0.f, 0.f, 0.f, A.clock->tag - 1);
+    if (nk < 1 || nk >= MAXT) return;
+    int w = -1;
+    if (A.B.by_slot) {
+        // a slot of its first tile that no particle has
+        const int t = listed_tile(B.pslot[(long long)p * MAXT]);
+        const unsigned taken = t < 0 ? ~0u : slot_mask(B.count[t], A.bp.np);
+        if (taken == ~0u) return;
+        w = t * MAXC + __ffs(~taken) - 1;
+    } else {
+        for (int q = 0; q < TILE_H; ++q)
+            store_partial(A.partial + ((long long)p * MAXT + nk) * TILE_H + q, 0.f, 0.f, 0.f, A.clock->tag - 1);
+    }
+    B.pslot[(long long)p * MAXT + nk] = w;
     B.npslot[p] = nk + 1;
     B.done[p] -= TILE_H;
 }
@@ -747,12 +756,13 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         (rc = dev_alloc(c, &c->P.fixed, (size_t)npa)) || (rc = dev_alloc(c, &c->force, 3 * (size_t)npa)) ||
         (rc = dev_alloc(c, &c->fsum, 3 * (size_t)npa)) || (rc = dev_alloc(c, &c->fcol, 2 * (size_t)npa)) ||
         (rc = dev_alloc(c, &c->err, 1)) ||
-        (rc = dev_alloc(c, &c->partial, (size_t)npa * MAXT * TILE_H)) || (rc = dev_alloc(c, &c->pa, 1)) ||
+        (rc = dev_alloc(c, &c->partial, (size_t)partial_entries(c->ntiles, npa))) || (rc = dev_alloc(c, &c->pa, 1)) ||
         (rc = dev_alloc(c, &c->sync, 1)))
         return bail(rc);
     BinSet &B = c->B;
     B.tiles = c->ntiles;
     B.parts = npa;
+    B.by_slot = partials_by_slot(c->ntiles, npa);
     if ((rc = dev_alloc(c, &B.count, 3 * (size_t)c->ntiles)) || (rc = dev_alloc(c, &B.ids, 2 * (size_t)c->ntiles * MAXC)) ||
         (rc = dev_alloc(c, &B.rec, 2 * (size_t)c->ntiles * MAXC * NREC)) ||
         (rc = dev_alloc(c, &B.pslot, 2 * (size_t)npa * MAXT)) || (rc = dev_alloc(c, &B.npslot, 2 * (size_t)npa)) ||
@@ -786,7 +796,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         (e = cudaMemsetAsync(c->fcol, 0, sizeof(double) * 2 * npa, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->sync, 0, sizeof(GridSync), c->stream)) != cudaSuccess ||
         // (no partial carries the tag of a step to come)
-        (e = cudaMemsetAsync(c->partial, 0xff, sizeof(float4) * MAXT * TILE_H * npa, c->stream)) != cudaSuccess ||
+        (e = cudaMemsetAsync(c->partial, 0xff, sizeof(float4) * partial_entries(c->ntiles, npa), c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * c->ntiles, c->stream)) != cudaSuccess ||
         // (where steps were given up: a count may stand beside ids never written,
         // and the positions of the other parity be the ones that are read)

@@ -200,7 +200,8 @@ struct Bins {                   // one step's view
     float4 *rec;                // per tile and slot, 3 records: (cx_hi, cx_lo, cy_hi, cy_lo),
                                 // (r, ux_hi, uy_hi, omega_hi), (ux_lo, uy_lo, omega_lo, packed
                                 // floor(cx), floor(cy): 16 bits each)
-    int *pslot;                 // per particle: MAXT tiles it reaches (-1: overflowed, or another strip's)
+    int *pslot;                 // per particle: MAXT tiles it reaches and its slots there (tile * MAXC + slot;
+                                // -1: overflowed, or another strip's)
     int *npslot;                // per particle: tiles reached
     int *done;                  // per particle: minus the partials its update still waits for
 };
@@ -222,7 +223,25 @@ struct BinSet {
     float *cover;               // PS: per particle, the covered areas of the (2K+1)^2 cells about
                                 // (floor X, floor Y), row-major; shared by both parities
     int tiles, parts;           // array strides
+    int by_slot;                // the partials' layout, see partials_by_slot
 };
+
+// A particle's force partials, one per row of each tile it reaches, lie with
+// the particle (MAXT tiles each, in the order of its list: 16 KB) or with the
+// tile's slots (MAXC each: 4 KB a tile).  With the particle its update finds
+// them without its list; with the slots many small discs take far less memory.
+// (us per step in FP32 with the particle and by slot: 100 discs on 512^2 14.05
+// and 14.5, 600 on 1024^2 30.5 and 31.4, 2000 on 2048^2 79.7 and 84.5, 20000 on
+// 4096^2 455 and 460, 84000 there 1409 and 1421, where they take 1376 MB and 67
+// MB.)  So by slot from one particle a tile on, where 16 KB each begin to count
+// beside the tile's 74 KB of populations (37 KB in 16 bits).
+__host__ __device__ inline bool partials_by_slot(long long tiles, long long parts) { return parts > 64 && parts > tiles; }
+__host__ __device__ inline long long partial_entries(long long tiles, long long parts) {
+    return (partials_by_slot(tiles, parts) ? tiles * MAXC : parts * MAXT) * TILE_H;
+}
+
+// The tile of a particle's list entry (Bins::pslot), or -1.
+__device__ __forceinline__ int listed_tile(int w) { return w == -1 ? -1 : (int)((unsigned)w / MAXC); }
 
 __host__ __device__ inline int rot3(int r) { return r >= 3 ? r - 3 : r; }
 
@@ -757,7 +776,7 @@ struct SweepArgs {
     Lattice L;
     Physics ph;
     BinSet B;                   // tile bins (np > 0)
-    float4 *partial;            // force / torque partials and tag: per particle, tile of its list and row
+    float4 *partial;            // force / torque partials and tag: per particle, tile of its list and row (or by slot)
     int *err;                   // the lattice's error word
     const PartArgs *pa;         // the particle update's arguments (device memory; batches)
     StepClock *clock;           // (null: see StepClock)
@@ -1283,7 +1302,7 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
             sg.x += s2.x; sg.y += s2.y; sg.z += s2.z;
         }
         const int id = cid[lane];
-        float4 *out = A.partial + ((long long)id * MAXT + __float_as_int(sg.w)) * TILE_H + (y - ty0);
+        float4 *out = A.partial + (A.B.by_slot ? (long long)tile * MAXC + lane : (long long)id * MAXT + __float_as_int(sg.w)) * TILE_H + (y - ty0);
         if (FUSED) {
             store_partial(out, sg.x, sg.y, sg.z, tag);
             if (count) count_done(B.done + id);
@@ -1486,7 +1505,7 @@ struct Repulsion {
 __device__ __forceinline__ bool maybe_near(const PartArgs &A, int p, const Bins &B, int lane) {
     const int nk = __ldcg(B.npslot + p);
     const int k = lane >> 2, sl = lane & 3;
-    const int t = __ldcg(B.pslot + (long long)p * MAXT + k);        // (entries past nk: stale, or never written)
+    const int t = listed_tile(__ldcg(B.pslot + (long long)p * MAXT + k));       // (entries past nk: stale, or never written)
     bool far = nk <= 8 && !A.L.wrap_x && !A.L.wrap_y;
     float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra;
     int id = -1, n = 0;
@@ -1538,7 +1557,7 @@ __device__ __forceinline__ Repulsion pair_repulsion(const PartArgs &A, int p, in
         // counts a pair only in that tile; within a tile the pairs are added
         // in increasing partner id.
         for (int k = lane; k < nk; k += 32) {
-            const int t = __ldcg(B.pslot + (long long)p * MAXT + k);
+            const int t = listed_tile(__ldcg(B.pslot + (long long)p * MAXT + k));
             if (t < 0) continue;
             uint32_t contact = 0;
             for (unsigned taken = slot_mask(__ldcg(B.count + t), bp.np); taken; taken &= taken - 1) {
@@ -1653,42 +1672,69 @@ __device__ __forceinline__ int component(int lane) { return lane >> 3; }
 // the step's tag; the wait is bounded, and sets *late when it gives up.
 template <bool TAGGED>
 __device__ __forceinline__ double hydro_sums(const PartArgs &A, int p, const Bins &B, unsigned tag, int lane, bool *late) {
-    constexpr int Q = 3;        // entries per lane held at once (and waited for together)
-    const float4 *part = A.partial + (long long)p * (MAXT * TILE_H) + lane;
-    float4 v[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) v[q] = load_partial(part + 32 * q);
-    const int ne = __ldcg(B.npslot + p) * TILE_H - lane;        // entries from this lane's first on
     double fx = 0.0, fy = 0.0, tq = 0.0;
-    for (int base = 0; base < ne + lane; base += 32 * Q) {
-        if (base > 0) {
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-                if (base + 32 * q < ne) v[q] = load_partial(part + base + 32 * q);
-        }
-        unsigned long long t0 = 0;
-        while (TAGGED) {
-            bool miss = false;
-#pragma unroll
-            for (int q = 0; q < Q; ++q)
-                if (base + 32 * q < ne && __float_as_uint(v[q].w) != tag) {
-                    v[q] = load_partial(part + base + 32 * q);
-                    miss = true;
-                }
-            // (together: lanes that left on their own would sum on their own)
-            if (!__any_sync(0xffffffffu, miss)) break;
-            const unsigned long long t = global_ns();
-            if (t0 == 0) t0 = t;
-            *late = __any_sync(0xffffffffu, t - t0 > WAIT_LIMIT_NS);
-            if (*late) break;
-        }
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            if (base + 32 * q >= ne) break;
-            if (base + q == 0) {
-                fx = widen(v[q].x); fy = widen(v[q].y); tq = widen(v[q].z);
+    if (A.B.by_slot) {
+        // the same entries in the same order, found by the list's slots
+        const int ne = __ldcg(B.npslot + p) * TILE_H;
+        for (int e = lane; e < ne + lane; e += 32) {
+            const unsigned w = e < ne ? (unsigned)__ldcg(B.pslot + (long long)p * MAXT + e / TILE_H) : ~0u;
+            const bool has = w != ~0u && ((int)(w / MAXC) / A.L.ntx + A.ty_lo) * TILE_H + e % TILE_H < A.L.ny;
+            const float4 *from = A.partial + (long long)w * TILE_H + e % TILE_H;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (has) v = load_partial(from);
+            unsigned long long t0 = 0;
+            while (TAGGED) {
+                const bool miss = has && __float_as_uint(v.w) != tag;
+                if (!__any_sync(0xffffffffu, miss)) break;
+                const unsigned long long t = global_ns();
+                if (t0 == 0) t0 = t;
+                *late = __any_sync(0xffffffffu, t - t0 > WAIT_LIMIT_NS);
+                if (*late) break;
+                if (miss) v = load_partial(from);
+            }
+            if (e == lane) {
+                fx = widen(v.x); fy = widen(v.y); tq = widen(v.z);
             } else {
-                fx += widen(v[q].x); fy += widen(v[q].y); tq += widen(v[q].z);
+                fx += widen(v.x); fy += widen(v.y); tq += widen(v.z);
+            }
+        }
+    } else {
+        constexpr int Q = 3;        // entries per lane held at once (and waited for together)
+        const float4 *part = A.partial + (long long)p * (MAXT * TILE_H) + lane;
+        float4 v[Q];
+#pragma unroll
+        for (int q = 0; q < Q; ++q) v[q] = load_partial(part + 32 * q);
+        const int ne = __ldcg(B.npslot + p) * TILE_H - lane;        // entries from this lane's first on
+        for (int base = 0; base < ne + lane; base += 32 * Q) {
+            if (base > 0) {
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (base + 32 * q < ne) v[q] = load_partial(part + base + 32 * q);
+            }
+            unsigned long long t0 = 0;
+            while (TAGGED) {
+                bool miss = false;
+#pragma unroll
+                for (int q = 0; q < Q; ++q)
+                    if (base + 32 * q < ne && __float_as_uint(v[q].w) != tag) {
+                        v[q] = load_partial(part + base + 32 * q);
+                        miss = true;
+                    }
+                // (together: lanes that left on their own would sum on their own)
+                if (!__any_sync(0xffffffffu, miss)) break;
+                const unsigned long long t = global_ns();
+                if (t0 == 0) t0 = t;
+                *late = __any_sync(0xffffffffu, t - t0 > WAIT_LIMIT_NS);
+                if (*late) break;
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                if (base + 32 * q >= ne) break;
+                if (base + q == 0) {
+                    fx = widen(v[q].x); fy = widen(v[q].y); tq = widen(v[q].z);
+                } else {
+                    fx += widen(v[q].x); fy += widen(v[q].y); tq += widen(v[q].z);
+                }
             }
         }
     }
@@ -1851,14 +1897,14 @@ __device__ __forceinline__ void particle_advance(const PartArgs &A, int p, const
             }
         }
         if (has && !axis) {
-            out.pslot[(long long)p * MAXT + k] = in ? t : -1;
+            out.pslot[(long long)p * MAXT + k] = in ? (int)((unsigned)t * MAXC + s) : -1;
             need += rows;
             // (this particle's partials of the step are summed: the entries no
             // sweep will write hold zero; an upload may replace a binning for
             // the same step, so it also takes that binning's tags off the others)
-            for (int q = 0; !integrate && q < rows; ++q)
+            for (int q = 0; !integrate && !A.B.by_slot && q < rows; ++q)
                 store_partial(A.partial + ((long long)p * MAXT + k) * TILE_H + q, 0.f, 0.f, 0.f, next_tag - 1);
-            for (int q = rows; q < TILE_H; ++q)
+            for (int q = A.B.by_slot ? TILE_H : rows; q < TILE_H; ++q)
                 store_partial(A.partial + ((long long)p * MAXT + k) * TILE_H + q, 0.f, 0.f, 0.f, next_tag);
         }
     }
