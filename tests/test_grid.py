@@ -47,7 +47,8 @@ def test_one_grid_holds_its_own_particle_blocks(grids):
     for items, parts, w, per_sm, bps, sms, blocks, pblocks, _ in grids:
         most = sms * (min(bps, per_sm) if bps else per_sm)
         each = min(max(items // (4 * most * w), 1), 8)              # particles of a warp
-        want = min(-(-parts // (w * each)), max(most // 10, 1))
+        share = most * 2 * parts // (2 * parts + items)             # a particle's update as two segments
+        want = min(-(-parts // (w * each)), max(most // 10, share, 1))
         assert pblocks == want
         assert blocks - pblocks >= 1
         assert blocks <= max(most, 2)                               # (one of each kind at least)
