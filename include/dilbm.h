@@ -140,8 +140,9 @@ int dilbm_create(const dilbm_grid *grid, dilbm_lattice lattice, double tau,
  * Asynchronous: returns once the work is queued; errors raised on the device
  * (UNSTABLE, OVERFLOW) surface at the next dilbm_sync().  One cooperative
  * launch runs many steps (about 2^27 node updates); with PS-LBM and while
- * timing, one step.  Launches may be recorded into a graph by the caller: an
- * even number of steps may be replayed any number of times.
+ * timing, and on small lattices without particles, one.  Launches may be
+ * recorded into a graph by the caller: an even number of steps may be replayed
+ * any number of times.
  */
 int dilbm_step(dilbm_ctx *ctx, long long nsteps);
 

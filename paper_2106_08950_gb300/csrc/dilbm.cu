@@ -401,11 +401,26 @@ int launch_fields(dilbm_ctx *c, const FieldsOut &fo) {
     return DILBM_OK;
 }
 
-// A strip's sweep in shape `sh` (per_sm: occupancy only).
-cudaError_t strip_sweep(dilbm_ctx *c, const SweepShape &sh, int *per_sm = nullptr) {
+// Does this context step by launches of the sweep alone?  A strip does, and a
+// lattice without particles up to some size: nothing waits for force sums there,
+// a launch that comes before the last one's end costs it less than the blocks'
+// meeting, and the sweep that counts no partials takes fewer registers.  (us per
+// step, fused and by sweeps: periodic FP32 384^2 6.7 and 3.8, 768^2 11.0 and 6.8,
+// 1400^2 23.6 and 21.7, 2048^2 46.8 and 46.4; FP16 768^2 13.0 and 6.9, 1400^2 23.1
+// and 19.1; between walls FP32 1800^2 38.3 and 37.7, 2048^2 47.6 and 48.6; FP16
+// 1800^2 33.7 and 31.6, 2048^2 40.1 and 43.9.)
+bool steps_by_sweeps(const dilbm_ctx *c) {
+    return c->strip || (c->np == 0 && (long long)c->L.ny * c->L.ntx <= 30000);
+}
+
+// Such a context's sweep in shape `sh` (chained: right behind another; dry: not
+// counted as a step; per_sm: occupancy only).
+cudaError_t lone_sweep(dilbm_ctx *c, const SweepShape &sh, bool chained, bool dry = false, int *per_sm = nullptr) {
     return by_storage(c->storage, [&](auto t) {
         using T = decltype(t);
-        return Launch<T>::sweep(sweep_args<T>(c), has_edges(c), c->method == DILBM_METHOD_PS, sh, c->num_sms, c->stream,
+        SweepArgs<T> a = sweep_args<T>(c);
+        if (dry) a.clock = nullptr;
+        return Launch<T>::sweep(a, has_edges(c), c->method == DILBM_METHOD_PS, sh, c->num_sms, c->stream, chained,
                                 per_sm);
     });
 }
@@ -425,13 +440,13 @@ int timing_pair(std::vector<cudaEvent_t> &ev, size_t &used, cudaEvent_t *e0, cud
     return DILBM_OK;
 }
 
-int launch_strip_sweep(dilbm_ctx *c) {
+int launch_sweep(dilbm_ctx *c, bool chained = false) {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (c->timing) {
         if (int rc = timing_pair(c->ev, c->ev_used, &e0, &e1)) return rc;
         DILBM_CUDA(cudaEventRecord(e0, c->stream));
     }
-    const cudaError_t e = strip_sweep(c, c->shape);
+    const cudaError_t e = lone_sweep(c, c->shape, chained && !c->timing);
     if (e != cudaSuccess) return cuda_fail(e, "sweep_kernel launch");
     if (c->timing) DILBM_CUDA(cudaEventRecord(e1, c->stream));
     c->launches += 1;
@@ -452,6 +467,13 @@ long long summed_steps(long long queued, unsigned counted) { return queued + (in
 // k steps in one launch (k == 1: no barrier, and the PS tables and the moving
 // frame's shift as launches of their own).
 int launch_fused(dilbm_ctx *c, int k) {
+    if (steps_by_sweeps(c)) {
+        for (int q = 0; q < k; ++q) {
+            if (const int rc = launch_sweep(c, q > 0)) return rc;
+            advance(c, 1);
+        }
+        return DILBM_OK;
+    }
     const cudaError_t e = fused_steps(c, c->shape, StepRun{k, 0, c->sync, 0});
     if (e != cudaSuccess) return cuda_fail(e, "step_kernel launch");
     c->launches += 1;
@@ -473,6 +495,7 @@ int steps_per_launch(double nodes) {
 
 // One step, its launch bracketed by events.
 int timed_step(dilbm_ctx *c) {
+    if (steps_by_sweeps(c)) return launch_fused(c, 1);          // (brackets its sweep itself)
     cudaEvent_t e0, e1;
     int rc = timing_pair(c->ev, c->ev_used, &e0, &e1);
     if (rc) return rc;
@@ -688,7 +711,6 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     }
     const bool strip = y0 > 0 || y1 < g->ny;
     if (strip) {
-        c->shape = SWEEP_SHAPE;
         // the particles keep the whole lattice's geometry; the sweep sees
         // rows [y0, y1) with halo rows beyond each cut
         c->strip = true;
@@ -703,6 +725,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
         if (cut_n) L.side_kind[NORTH] = SIDE_HALO;
     }
     c->ntiles = L.ntx * L.nty;
+    if (steps_by_sweeps(c)) c->shape = SWEEP_SHAPE;
     Physics &ph = c->ph;
     ph.omega = (float)(1.0 / tau);
     ph.kf = (float)(1.0 - 0.5 / tau);
@@ -865,7 +888,7 @@ int dilbm_create_strip(const dilbm_grid *g, dilbm_lattice lattice, double tau, d
 int dilbm_strip_begin(dilbm_ctx *c) {
     const dilbm::TraceRange trace("dilbm_strip_begin");
     if (!c || !c->strip || c->strip_open) return fail(DILBM_ERR_INVALID_ARG, "not a strip, or a step already begun");
-    int rc = launch_strip_sweep(c);
+    int rc = launch_sweep(c);
     if (rc) return rc;
     if (c->np > 0 && (rc = launch_particles(c, 1))) return rc;
     // this strip's first and last rows of every plane, for the neighbours
@@ -1531,8 +1554,9 @@ int dilbm_autotune(dilbm_ctx *c, int reps, int *warps, int *blocks_per_sm) {
         report_shape(c->shape, warps, blocks_per_sm);
         return DILBM_OK;
     }
-    // (a strip has no step clock: its sweep is a kernel of its own)
-    const auto key = std::make_tuple(c->strip ? 2 : 0, c->storage, has_edges(c) ? 1 : 0, (long long)c->L.nx, (long long)c->L.ny);
+    // (the sweep alone is a kernel of its own)
+    const bool lone = steps_by_sweeps(c);
+    const auto key = std::make_tuple(lone ? 2 : 0, c->storage, has_edges(c) ? 1 : 0, (long long)c->L.nx, (long long)c->L.ny);
     SweepShape best = c->shape;
     if (!tuned(key, &best)) {
         std::vector<SweepShape> cands;
@@ -1540,7 +1564,7 @@ int dilbm_autotune(dilbm_ctx *c, int reps, int *warps, int *blocks_per_sm) {
         // each launch sweeps the current state into the other buffer (what
         // the next step writes anyway) and updates no particle
         auto sweep = [&](const SweepShape &sh, int *per_sm) {
-            return c->strip ? strip_sweep(c, sh, per_sm) : fused_steps(c, sh, StepRun{1, 1, c->sync, 0}, per_sm);
+            return lone ? lone_sweep(c, sh, false, true, per_sm) : fused_steps(c, sh, StepRun{1, 1, c->sync, 0}, per_sm);
         };
         int rc = shape_candidates(sweep, &cands, &wps);
         if (rc) return rc;

@@ -1348,7 +1348,7 @@ __device__ __forceinline__ int row_of(unsigned item, unsigned inv, int ntx) {
 }
 
 // The sweep over one lattice without the particle update (a strip's step, the
-// static step, and the fields).  Persistent: warps take row segments
+// static step, a step of a small lattice without particles, and the fields).  Persistent: warps take row segments
 // round-robin (neighbouring warps on neighbouring segments); each warp keeps
 // its next segment staged ahead.  W warps per block.
 template <typename T, int MODE, bool EDGES, bool PS, int W>
@@ -1364,6 +1364,10 @@ sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ F
         mbar_fence_init();
     }
     __syncwarp();
+    // Launched while the step before still runs (sweep_variant, `chained`): wait
+    // for its end here, and let the step after come as this one's blocks leave.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const Lattice &L = one.L;
     const T *src = one.buf[one.cur];
     T *dst = one.buf[one.cur ^ 1];
@@ -1373,6 +1377,7 @@ sweep_kernel(const __grid_constant__ SweepArgs<T> one, const __grid_constant__ F
         int *clear = one.B.count + (long long)(one.cur ^ 1) * one.B.tiles;
         for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < L.ntx * L.nty; t += gridDim.x * blockDim.x) clear[t] = 0;
     }
+    if (MODE == MODE_STEP && one.clock && blockIdx.x == 0 && threadIdx.x == 0) one.clock->tag += 1;
     const int nitems = L.ny * L.ntx;
     const int gw = blockIdx.x * W + warp, nw = gridDim.x * W;
     T wv = T();         // the staged segment's periodic-edge value (wrap_load)

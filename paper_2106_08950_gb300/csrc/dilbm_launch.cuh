@@ -97,11 +97,14 @@ cudaError_t batch_variant(const BatchArgs<T> &ba, StepRun run, const SweepShape 
     return launch_steps((const void *)kern, p, g.blocks, W, smem, st);
 }
 
-// The sweep without the particle update (a strip's step, in the strip's shape;
-// MODE_FIELDS: the macroscopic fields instead of a step).
+// The sweep without the particle update (a step of a strip or of a small lattice
+// without particles, in its shape; MODE_FIELDS: the macroscopic fields instead
+// of a step).  `chained`: the launch before it on the stream is such a step too,
+// and this one may come before its end (it waits for it: a microsecond less
+// between steps).
 template <typename T, int MODE, bool EDGES, bool PS, int W = SWEEP_WARPS>
 cudaError_t sweep_variant(const SweepArgs<T> &a, const FieldsOut &fo, int num_sms, cudaStream_t st,
-                          const SweepShape &sh = SWEEP_SHAPE, int *per_sm_out = nullptr) {
+                          const SweepShape &sh = SWEEP_SHAPE, bool chained = false, int *per_sm_out = nullptr) {
     static int cache[64] = {};
     constexpr size_t smem = sweep_smem_bytes<T, W>();
     int per_sm = 1;
@@ -111,8 +114,17 @@ cudaError_t sweep_variant(const SweepArgs<T> &a, const FieldsOut &fo, int num_sm
         return e;
     }
     const long long blocks = persistent_grid((long long)a.L.ny * a.L.ntx, W, per_sm, num_sms, sh);
-    sweep_kernel<T, MODE, EDGES, PS, W><<<(unsigned)blocks, W * 32, smem, st>>>(a, fo);
-    return cudaGetLastError();
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(W * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &early;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, sweep_kernel<T, MODE, EDGES, PS, W>, a, fo);
 }
 
 // Per-storage launchers, instantiated in dilbm_launch_f32.cu, _f16.cu and
@@ -126,9 +138,9 @@ struct Launch {
     // fused steps of a batch
     static cudaError_t batch(const BatchArgs<T> &ba, const StepRun &run, const SweepShape &sh, int num_sms,
                              cudaStream_t st, int *per_sm = nullptr);
-    // a strip's sweep (PS-LBM: in the default shape)
+    // a sweep alone (PS-LBM: in the default shape)
     static cudaError_t sweep(const SweepArgs<T> &a, bool edges, bool ps, const SweepShape &sh, int num_sms,
-                             cudaStream_t st, int *per_sm = nullptr);
+                             cudaStream_t st, bool chained = false, int *per_sm = nullptr);
     static cudaError_t fields(const SweepArgs<T> &a, const FieldsOut &fo, bool edges, bool ps, int num_sms,
                               cudaStream_t st);
 };

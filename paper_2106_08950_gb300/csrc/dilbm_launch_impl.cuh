@@ -35,17 +35,17 @@ cudaError_t Launch<T>::batch(const BatchArgs<T> &ba, const StepRun &run, const S
 
 template <typename T>
 cudaError_t Launch<T>::sweep(const SweepArgs<T> &a, bool edges, bool ps, const SweepShape &sh, int num_sms,
-                             cudaStream_t st, int *per_sm) {
+                             cudaStream_t st, bool chained, int *per_sm) {
     const FieldsOut none{};
-    if (ps) return edges ? sweep_variant<T, MODE_STEP, true, true>(a, none, num_sms, st, SWEEP_SHAPE, per_sm)
-                         : sweep_variant<T, MODE_STEP, false, true>(a, none, num_sms, st, SWEEP_SHAPE, per_sm);
+    if (ps) return edges ? sweep_variant<T, MODE_STEP, true, true>(a, none, num_sms, st, SWEEP_SHAPE, chained, per_sm)
+                         : sweep_variant<T, MODE_STEP, false, true>(a, none, num_sms, st, SWEEP_SHAPE, chained, per_sm);
     switch (sh.warps) {
-    case 2: return edges ? sweep_variant<T, MODE_STEP, true, false, 2>(a, none, num_sms, st, sh, per_sm)
-                         : sweep_variant<T, MODE_STEP, false, false, 2>(a, none, num_sms, st, sh, per_sm);
-    case 4: return edges ? sweep_variant<T, MODE_STEP, true, false, 4>(a, none, num_sms, st, sh, per_sm)
-                         : sweep_variant<T, MODE_STEP, false, false, 4>(a, none, num_sms, st, sh, per_sm);
-    case 8: return edges ? sweep_variant<T, MODE_STEP, true, false, 8>(a, none, num_sms, st, sh, per_sm)
-                         : sweep_variant<T, MODE_STEP, false, false, 8>(a, none, num_sms, st, sh, per_sm);
+    case 2: return edges ? sweep_variant<T, MODE_STEP, true, false, 2>(a, none, num_sms, st, sh, chained, per_sm)
+                         : sweep_variant<T, MODE_STEP, false, false, 2>(a, none, num_sms, st, sh, chained, per_sm);
+    case 4: return edges ? sweep_variant<T, MODE_STEP, true, false, 4>(a, none, num_sms, st, sh, chained, per_sm)
+                         : sweep_variant<T, MODE_STEP, false, false, 4>(a, none, num_sms, st, sh, chained, per_sm);
+    case 8: return edges ? sweep_variant<T, MODE_STEP, true, false, 8>(a, none, num_sms, st, sh, chained, per_sm)
+                         : sweep_variant<T, MODE_STEP, false, false, 8>(a, none, num_sms, st, sh, chained, per_sm);
     default: return cudaErrorInvalidValue;
     }
 }
