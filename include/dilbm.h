@@ -142,7 +142,10 @@ int dilbm_create(const dilbm_grid *grid, dilbm_lattice lattice, double tau,
  * launch runs many steps (about 2^27 node updates); with PS-LBM and while
  * timing, and on small lattices without particles, one.  Launches may be
  * recorded into a graph by the caller: an even number of steps may be replayed
- * any number of times.
+ * any number of times.  A launch over several steps, and each PS-LBM step,
+ * starts only once all of its blocks (up to the whole device) are free of other
+ * kernels: beside a kernel that stays resident until this work is done, call
+ * dilbm_step with nsteps = 1 (DI-LBM), whose launch goes on with the SMs left.
  */
 int dilbm_step(dilbm_ctx *ctx, long long nsteps);
 

@@ -2039,7 +2039,8 @@ struct StepRun {
     int nsteps;
     int dry;                    // sweep only: no contribution is counted, no particle updated (autotuning)
     GridSync *sync;
-    int pblocks;                // leading blocks that update particles
+    int pblocks;                // blocks that update particles
+    int ahead;                  // of them, those first in the grid: all or none (see launch_steps)
 };
 
 // Thread 0 of a block: count it as arrived, and wait until `target` blocks
@@ -2234,9 +2235,11 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
         dead |= __ldcg(wk.args(k).err) & ERR_TIMEOUT;
     }
     int st = __syncthreads_or(dead) ? run.nsteps + 1 : 0;
-    const bool sweeps = (int)blockIdx.x >= run.pblocks;
-    // this block among the sweeping ones, its group and the group's warps
-    const int sb = (int)blockIdx.x - run.pblocks, nsb = (int)gridDim.x - run.pblocks;
+    // this block among the sweeping ones (from nsb on: a particle block), its group
+    // and the group's warps
+    const int nsb = (int)gridDim.x - run.pblocks;
+    const int sb = (int)blockIdx.x >= run.ahead ? (int)blockIdx.x - run.ahead : nsb + (int)blockIdx.x;
+    const bool sweeps = sb < nsb;
     const int ngroups = nsb < TICKET_GROUPS ? nsb : TICKET_GROUPS;
     const int group = sb % ngroups, gwarps = (nsb / ngroups + (group < nsb % ngroups)) * W;
     auto item_of = [&](int k) { return ((k / W) * ngroups + group) * W + (k & (W - 1)); };
@@ -2293,7 +2296,7 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
             shift = frame_move(__ldcg((wk.parity(0, st) ? f.P.x[1] : f.P.x[0]) + f.track), f.track_x, f.L.nx, f.L.per_x);
         }
         if (!sweeps) {
-            if (!run.dry && !update_particles(wk, clk, st, shift, (int)blockIdx.x * W + warp, run.pblocks * W, lane)) {
+            if (!run.dry && !update_particles(wk, clk, st, shift, (sb - nsb) * W + warp, run.pblocks * W, lane)) {
                 if (lane == 0) abandon(run.sync);
                 timed_out = true;
             }

@@ -43,11 +43,21 @@ cudaError_t occupancy_of(K kern, int warps, size_t smem, int *cache, int *per_sm
     return cudaSuccess;
 }
 
-// Blocks of a fused launch wait for one another (particle blocks for the
-// sweeping ones, and all of them between steps), so it is launched
-// cooperatively: the driver starts it only with every block resident.
-inline cudaError_t launch_steps(const void *kern, void **args, long long blocks, int warps, size_t smem, cudaStream_t st) {
-    return cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(warps * 32), args, smem, st);
+// Several steps: the blocks wait for one another (particle blocks for the
+// sweeping ones, and all of them between steps), so the launch is cooperative:
+// the driver starts it only with every block resident.  One step (`alone`):
+// particle blocks wait for the sweeping ones, which are then first in the grid
+// and wait for no block, so an ordinary launch makes progress on whatever SMs
+// are free.  (us per call of one step, cooperative and ordinary: 512^2 FP32 14.6
+// both, 1024^2 FP16 28.9 and 26.9, 200 small lattices 77.2 and 74.4; PS-LBM on
+// 512^2 20.9 and 22.6, so PS steps stay cooperative.)
+inline cudaError_t launch_steps(const void *kern, void **args, StepRun *run, const FusedGrid &g, bool alone, int warps,
+                                size_t smem, cudaStream_t st) {
+    const dim3 blocks((unsigned)g.blocks), threads(warps * 32);
+    run->pblocks = g.pblocks;
+    run->ahead = alone ? 0 : g.pblocks;
+    return alone ? cudaLaunchKernel(kern, blocks, threads, args, smem, st)
+                 : cudaLaunchCooperativeKernel(kern, blocks, threads, args, smem, st);
 }
 
 template <typename T, bool EDGES, int W, bool PS, bool HALVES = false>
@@ -74,9 +84,8 @@ cudaError_t step_variant(const SweepArgs<T> &a, const PartArgs &pa, StepRun run,
             return step_variant<T, EDGES, W, PS, true>(a, pa, run, sh, num_sms, st, per_sm_out);
     }
     const FusedGrid g = fused_grid(HALVES ? 2 * items : items, a.np, W, per_sm, num_sms, sh);
-    run.pblocks = g.pblocks;
     void *p[3] = {const_cast<SweepArgs<T> *>(&a), const_cast<PartArgs *>(&pa), &run};
-    return launch_steps((const void *)kern, p, g.blocks, W, smem, st);
+    return launch_steps((const void *)kern, p, &run, g, run.nsteps == 1 && !PS, W, smem, st);
 }
 
 template <typename T, int W>
@@ -92,9 +101,8 @@ cudaError_t batch_variant(const BatchArgs<T> &ba, StepRun run, const SweepShape 
         return e;
     }
     const FusedGrid g = fused_grid(ba.item_start[ba.n], ba.part_start[ba.n], W, per_sm, num_sms, sh);
-    run.pblocks = g.pblocks;
     void *p[2] = {const_cast<BatchArgs<T> *>(&ba), &run};
-    return launch_steps((const void *)kern, p, g.blocks, W, smem, st);
+    return launch_steps((const void *)kern, p, &run, g, run.nsteps == 1, W, smem, st);
 }
 
 // The sweep without the particle update (a step of a strip or of a small lattice

@@ -64,5 +64,6 @@ def test_a_launch_takes_both_counts_from_one_grid():
     """The launchers set the particle blocks from the grid that they launch,
     after any trial of another one."""
     src = open(os.path.join(B.CSRC, "dilbm_launch.cuh")).read()
-    assert src.count("const FusedGrid g = fused_grid(") == src.count("run.pblocks = g.pblocks;") == 2
-    assert src.count("pblocks") == 2 * 2 and src.count("g.blocks") == 2
+    assert src.count("const FusedGrid g = fused_grid(") == src.count("p, &run, g, ") == 2
+    assert src.count("run->pblocks = g.pblocks;") == 1 and src.count("dim3 blocks((unsigned)g.blocks)") == 1
+    assert "run.pblocks" not in src
