@@ -979,16 +979,22 @@ int dilbm_forces(dilbm_ctx *c, double *force, double *fcol, dilbm_particle *stat
 
 int dilbm_force_mean(dilbm_ctx *c, double *mean, long long *nsteps) {
     if (!c || !nsteps || (c->np > 0 && !mean)) return fail(DILBM_ERR_INVALID_ARG, "NULL argument");
-    const int np = c->np;
-    unsigned tags[3] = {0, 0, 0};       // clock.tag, clock.rot, mean_tag
-    static_assert(offsetof(GridSync, mean_tag) == offsetof(GridSync, clock) + 2 * sizeof(unsigned), "read together below");
-    if (np > 0) DILBM_CUDA(cudaMemcpyAsync(mean, c->fsum, sizeof(double) * 3 * np, cudaMemcpyDeviceToHost, c->stream));
-    if (!c->strip) DILBM_CUDA(cudaMemcpyAsync(tags, &c->sync->clock, sizeof(tags), cudaMemcpyDeviceToHost, c->stream));
-    const int rc = read_sticky(c);   // synchronises the stream
-    *nsteps = c->strip ? c->fsum_steps : summed_steps(c->fsum_steps, tags[0] - tags[2]);
+    // staged in pinned memory: the sums, then clock.tag, clock.rot, mean_tag and
+    // the error word
+    const size_t bytes = sizeof(double) * 3 * (size_t)c->np;
+    static_assert(offsetof(GridSync, mean_tag) == offsetof(GridSync, clock) + 2 * sizeof(unsigned), "copied together");
+    char *h = static_cast<char *>(t_stage.get(bytes + 4 * sizeof(unsigned)));
+    if (!h) return fail(DILBM_ERR_OOM, "pinned staging for dilbm_force_mean");
+    unsigned *words = reinterpret_cast<unsigned *>(h + bytes);
+    if (c->np > 0) DILBM_CUDA(cudaMemcpyAsync(h, c->fsum, bytes, cudaMemcpyDeviceToHost, c->stream));
+    DILBM_CUDA(cudaMemcpyAsync(words, &c->sync->clock, 3 * sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
+    DILBM_CUDA(cudaMemcpyAsync(words + 3, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    DILBM_CUDA(cudaStreamSynchronize(c->stream));
+    c->sticky |= (int)words[3];
+    *nsteps = c->strip ? c->fsum_steps : summed_steps(c->fsum_steps, words[0] - words[2]);
     const double inv = *nsteps > 0 ? 1.0 / (double)*nsteps : 0.0;
-    for (int k = 0; k < 3 * np; ++k) mean[k] *= inv;
-    return rc;
+    for (int k = 0; k < 3 * c->np; ++k) mean[k] = reinterpret_cast<double *>(h)[k] * inv;
+    return sticky_error(c->sticky);
 }
 
 int dilbm_set_moving_frame(dilbm_ctx *c, int particle, double x_ref) {
