@@ -178,8 +178,7 @@ unsigned long long footprint_of(int nx, int ny, size_t elem, int np) {
         (unsigned long long)((nx + TILE_W - 1) / TILE_W) * (unsigned long long)((ny + TILE_H - 1) / TILE_H);
     const unsigned long long npa = np > 0 ? (unsigned long long)np : 1ull;
     unsigned long long b = 2ull * (9ull * plane + 2ull * GUARD) * elem;           // populations A, B
-    b += 15ull * npa * sizeof(double) + 5ull * npa * sizeof(float) + npa * sizeof(int);   // particle state
-    b += 6ull * npa * sizeof(double) + 2ull * npa * sizeof(double) + sizeof(int);         // force, fsum, fcol, err
+    b += 23ull * npa * sizeof(double) + 5ull * npa * sizeof(float) + npa * sizeof(int) + sizeof(int);   // particle state, forces, err
     b += (unsigned long long)partial_entries((long long)ntiles, (long long)npa) * sizeof(float4);   // partials
     b += 3ull * ntiles * sizeof(int) + 2ull * ntiles * MAXC * (sizeof(int2) + NREC * sizeof(float4)) +
          2ull * npa * (MAXT + 2) * sizeof(int);                                           // bins
@@ -775,10 +774,8 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     const int npa = np > 0 ? np : 1;
     double *pd = nullptr;
     float *pf = nullptr;
-    if ((rc = dev_alloc(c, &pd, 15 * (size_t)npa)) || (rc = dev_alloc(c, &pf, 5 * (size_t)npa)) ||
-        (rc = dev_alloc(c, &c->P.fixed, (size_t)npa)) || (rc = dev_alloc(c, &c->force, 3 * (size_t)npa)) ||
-        (rc = dev_alloc(c, &c->fsum, 3 * (size_t)npa)) || (rc = dev_alloc(c, &c->fcol, 2 * (size_t)npa)) ||
-        (rc = dev_alloc(c, &c->err, 1)) ||
+    if ((rc = dev_alloc(c, &pd, 23 * (size_t)npa)) || (rc = dev_alloc(c, &pf, 5 * (size_t)npa)) ||
+        (rc = dev_alloc(c, &c->P.fixed, (size_t)npa)) || (rc = dev_alloc(c, &c->err, 1)) ||
         (rc = dev_alloc(c, &c->partial, (size_t)partial_entries(c->ntiles, npa))) || (rc = dev_alloc(c, &c->pa, 1)) ||
         (rc = dev_alloc(c, &c->sync, 1)))
         return bail(rc);
@@ -796,6 +793,7 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     c->P.theta = pd + 8 * npa; c->P.rho_s = pd + 9 * npa; c->P.im = pd + 10 * npa; c->P.iI = pd + 11 * npa;
     c->P.wx = pd + 12 * npa; c->P.wy = pd + 13 * npa; c->P.reach = pd + 14 * npa; c->P.rf = pf + 4 * npa;
     c->P.xf[0] = pf; c->P.xf[1] = pf + npa; c->P.yf[0] = pf + 2 * npa; c->P.yf[1] = pf + 3 * npa;
+    c->force = pd + 15 * (size_t)npa; c->fsum = pd + 18 * (size_t)npa; c->fcol = pd + 21 * (size_t)npa;
     if (c->strip) {
         // exchange buffers: 9 plane rows each, GUARD readable elements around
         const size_t row_elems = 9 * (size_t)L.pitch + 2 * (size_t)GUARD;
@@ -814,16 +812,13 @@ static int create_ctx(const dilbm_grid *g, dilbm_lattice lattice, double tau, do
     }
     cudaError_t e;
     if ((e = cudaMemsetAsync(c->err, 0, sizeof(int), c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->force, 0, sizeof(double) * 3 * npa, c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->fsum, 0, sizeof(double) * 3 * npa, c->stream)) != cudaSuccess ||
-        (e = cudaMemsetAsync(c->fcol, 0, sizeof(double) * 2 * npa, c->stream)) != cudaSuccess ||
+        // (the forces; the positions of the other parity, should the first steps be given up)
+        (e = cudaMemsetAsync(pd, 0, sizeof(double) * 23 * npa, c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(c->sync, 0, sizeof(GridSync), c->stream)) != cudaSuccess ||
         // (no partial carries the tag of a step to come)
         (e = cudaMemsetAsync(c->partial, 0xff, sizeof(float4) * partial_entries(c->ntiles, npa), c->stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(B.count, 0, sizeof(int) * 3 * c->ntiles, c->stream)) != cudaSuccess ||
-        // (where steps were given up: a count may stand beside ids never written,
-        // and the positions of the other parity be the ones that are read)
-        (e = cudaMemsetAsync(pd, 0, sizeof(double) * 4 * npa, c->stream)) != cudaSuccess ||
+        // (where steps were given up, a count may stand beside ids never written)
         (e = cudaMemsetAsync(B.ids, 0, sizeof(int2) * 2 * c->ntiles * MAXC, c->stream)) != cudaSuccess)
         return bail(cuda_fail(e, "cudaMemsetAsync"));
     // uniform initial state f^eq(rho_init, u0)
