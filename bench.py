@@ -534,18 +534,18 @@ def batch_arm(args):
     time.sleep(0.3)
     barrier(dist)
     torch.cuda.synchronize()
-    l0 = batch.launches
+    l0 = batch.kernels
     t0 = time.perf_counter()
     batch.step(args.steps)
     batch.sync()
     dt = time.perf_counter() - t0
-    launches = batch.launches - l0
+    launches = batch.kernels - l0
     clk = clocks.stop()
     dt = max_over_ranks(dist, dt, dev)
     total_nodes = sum_over_ranks(dist, nodes, dev)        # each rank has its own lattices
     value = total_nodes * args.steps / dt / 1e6
 
-    # the batched sweep alone, timed by CUDA events (direct launches)
+    # one step per launch, timed by CUDA events
     k_t = max(10, min(args.steps, 200))
     batch.set_timing(True)
     batch.step(k_t)

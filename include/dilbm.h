@@ -344,6 +344,7 @@ long long dilbm_launch_count(const dilbm_ctx *ctx);
  * dilbm_batch_launch_count: the passes the batch has run: a sweep pass per
  *   launch group and step, a particle pass per step, and the error gathers of
  *   dilbm_batch_sync (a launch covers both passes of several steps).
+ * dilbm_batch_kernel_count: the kernels the batch has launched.
  */
 typedef struct dilbm_batch dilbm_batch;
 int dilbm_batch_create(dilbm_ctx *const *members, int n, void *cuda_stream, dilbm_batch **out);
@@ -354,6 +355,7 @@ int dilbm_batch_stall_probe(dilbm_batch *batch);
 int dilbm_batch_set_timing(dilbm_batch *batch, int enable);
 int dilbm_batch_sweep_time(dilbm_batch *batch, double *ms_total, long long *launches);
 long long dilbm_batch_launch_count(const dilbm_batch *batch);
+long long dilbm_batch_kernel_count(const dilbm_batch *batch);
 void dilbm_batch_destroy(dilbm_batch *batch);
 int dilbm_batch_autotune(dilbm_batch *batch, int reps, int *warps, int *blocks_per_sm);
 int dilbm_batch_set_shape(dilbm_batch *batch, int warps, int blocks_per_sm);

@@ -1203,7 +1203,8 @@ struct dilbm_batch {
     bool timing = false;
     std::vector<cudaEvent_t> ev;
     size_t ev_used = 0;
-    long long launches = 0;
+    long long launches = 0;             // passes (dilbm_batch_launch_count)
+    long long kernels = 0;              // kernels launched
 };
 
 namespace {
@@ -1248,6 +1249,7 @@ cudaError_t batch_groups(dilbm_batch *b, const SweepShape &sh, int nsteps, int d
             if (ba.n == 0) continue;
             const cudaError_t e = Launch<T>::batch(ba, StepRun{nsteps, dry, b->sync[g], 0}, sh, b->members[0]->num_sms, b->stream);
             if (e != cudaSuccess) return e;
+            ++b->kernels;
         }
         return cudaSuccess;
     });
@@ -1357,6 +1359,7 @@ int dilbm_batch_sync(dilbm_batch *b, int *first_failed) {
     gather_errors_kernel<<<(n + 255) / 256, 256, 0, b->stream>>>(b->err_ptrs, n, b->err_out);
     DILBM_CUDA(cudaGetLastError());
     b->launches += 1;
+    b->kernels += 1;
     DILBM_CUDA(cudaMemcpyAsync(b->err_host.data(), b->err_out, sizeof(int) * n, cudaMemcpyDeviceToHost, b->stream));
     DILBM_CUDA(cudaStreamSynchronize(b->stream));
     if (first_failed) *first_failed = -1;
@@ -1385,6 +1388,7 @@ int dilbm_batch_stall_probe(dilbm_batch *b) {
     stall_kernel<<<1, 1, 0, b->stream>>>(PartArgs{}, b->sync[0], 0, -1);
     DILBM_CUDA(cudaGetLastError());
     b->launches += 1;
+    b->kernels += 1;
     return DILBM_OK;
 }
 
@@ -1411,6 +1415,8 @@ int dilbm_batch_sweep_time(dilbm_batch *b, double *ms_total, long long *launches
 }
 
 long long dilbm_batch_launch_count(const dilbm_batch *b) { return b ? b->launches : -1; }
+
+long long dilbm_batch_kernel_count(const dilbm_batch *b) { return b ? b->kernels : -1; }
 
 void dilbm_batch_destroy(dilbm_batch *b) {
     if (!b) return;

@@ -100,7 +100,7 @@ void release(dilbm_server *s, Job *j) {
 void drop_batch(dilbm_server *s) {
     for (int c = 0; c < NSTORE; ++c)
         if (s->batch[c]) {
-            s->launches_gone += dilbm_batch_launch_count(s->batch[c]);
+            s->launches_gone += dilbm_batch_kernel_count(s->batch[c]);
             dilbm_batch_destroy(s->batch[c]);
             s->batch[c] = nullptr;
         }
@@ -169,7 +169,7 @@ void fill_stats(const dilbm_server *s, dilbm_server_stats *st) {
     st->retire_seconds = s->t_retire;
     st->memory_in_use = s->in_use;
     long long l = s->launches_gone;
-    for (int c = 0; c < NSTORE; ++c) l += s->batch[c] ? dilbm_batch_launch_count(s->batch[c]) : 0;
+    for (int c = 0; c < NSTORE; ++c) l += s->batch[c] ? dilbm_batch_kernel_count(s->batch[c]) : 0;
     for (const Job *j : s->running) l += j->ctx ? dilbm_launch_count(j->ctx) : 0;
     st->launches = l;
 }

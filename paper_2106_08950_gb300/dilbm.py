@@ -126,6 +126,8 @@ def load_library(path: Optional[str] = None):
     L.dilbm_batch_sweep_time.argtypes = [vp, dp, C.POINTER(C.c_longlong)]
     L.dilbm_batch_launch_count.argtypes = [vp]
     L.dilbm_batch_launch_count.restype = C.c_longlong
+    L.dilbm_batch_kernel_count.argtypes = [vp]
+    L.dilbm_batch_kernel_count.restype = C.c_longlong
     L.dilbm_batch_destroy.argtypes = [vp]
     L.dilbm_batch_destroy.restype = None
     L.dilbm_batch_errors.argtypes = [vp, C.POINTER(C.c_int)]
@@ -489,7 +491,13 @@ class Batch:
 
     @property
     def launches(self) -> int:
+        """Passes run: a sweep and a particle pass per step (``dilbm_batch_launch_count``)."""
         return int(self.L.dilbm_batch_launch_count(self.h))
+
+    @property
+    def kernels(self) -> int:
+        """Kernels launched (``dilbm_batch_kernel_count``)."""
+        return int(self.L.dilbm_batch_kernel_count(self.h))
 
 
 class Server:
