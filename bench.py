@@ -467,7 +467,7 @@ def gpu_arm(args):
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": traffic, "peak_kind": peak_kind,
             "kernel": "step_kernel", "sweep_ms_per_launch": per_launch_ms,
-            "sweep_share_of_step": per_launch_ms / (ms / args.steps) if ms > 0 else None,
+            "one_step_launch_over_step": per_launch_ms / (ms / args.steps) if ms > 0 else None,
             "algorithmic_bytes_per_launch": alg_bytes}
 
     line = {"metric": METRIC, "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,

@@ -326,7 +326,8 @@ long long dilbm_launch_count(const dilbm_ctx *ctx);
  * Batches: many contexts advanced together (the same equations, Eqs. 13-19,
  * 22-24, 28-29, on every member).  One launch runs several steps over the
  * concatenated row segments and particles of all members (up to 84 members;
- * larger batches take a launch per 84); every member's result is bit for bit the one dilbm_step gives it alone.
+ * larger batches take a launch per 84); every member's result is bit for bit
+ * the one dilbm_step gives it alone.
  *
  * dilbm_batch_create: members[0..n-1] (1 <= n <= 1024 distinct contexts, all
  *   with the same storage; they stay owned by the caller and must outlive the
@@ -371,17 +372,19 @@ int dilbm_batch_set_shape(dilbm_batch *batch, int warps, int blocks_per_sm);
  *
  * dilbm_autotune / dilbm_batch_autotune time every candidate shape (each
  * warps-per-block value with as many blocks per SM as fit and with half as
- * many) in 3 interleaved rounds of reps
- * sweep launches of the current state
- * (reps <= 0: 10; the launches only write what the next step overwrites),
- * keep the one with the smallest median round time and report it in *warps
- * and *blocks_per_sm (nullable).  The choice is cached
- * per process, keyed by storage, edge handling and lattice size (for a
- * batch: storage, member count and total row segments), so tuning a second
- * context or batch of the same key launches nothing.  Both synchronise.
+ * many) in 7 interleaved rounds of reps one-step launches of the current state
+ * without particle updates (reps <= 0: 10; they only write what the next step
+ * overwrites).  Of those within 1 % of the smallest median round time they keep
+ * the one with the most resident warps, and report it in *warps and
+ * *blocks_per_sm (nullable).  The choice is cached
+ * per process, keyed by storage, edge handling and lattice size (apart for
+ * strips and other lattices that step by the sweep alone; for a batch: storage,
+ * member count and total row segments), so tuning a second context or batch of
+ * the same key launches nothing.  Both synchronise.
  * dilbm_set_shape / dilbm_batch_set_shape set a shape by hand.  A PS-LBM
- * context keeps the default shape (8 warps, blocks_per_sm 0): dilbm_autotune
- * reports it without timing and dilbm_set_shape rejects any other.
+ * context has one shape, reported as 8 warps and 0 (its fused steps run 4 warps
+ * per block): dilbm_autotune reports it without timing and dilbm_set_shape
+ * rejects any other.
  * Errors: INVALID_ARG, CUDA.
  */
 int dilbm_autotune(dilbm_ctx *ctx, int reps, int *warps, int *blocks_per_sm);

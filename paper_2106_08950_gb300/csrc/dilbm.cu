@@ -66,7 +66,7 @@ struct dilbm_ctx {
     int ntiles = 0;
     int num_sms = 1;
     bool timing = false;
-    std::vector<cudaEvent_t> ev;      // start/stop pairs around sweep launches
+    std::vector<cudaEvent_t> ev;      // start/stop pairs around timed launches
     size_t ev_used = 0;
     long long launches = 0;
     SweepShape shape{};               // launch shape of the step sweep (autotuned or default)
@@ -179,7 +179,7 @@ unsigned long long footprint_of(int nx, int ny, size_t elem, int np) {
     const unsigned long long npa = np > 0 ? (unsigned long long)np : 1ull;
     unsigned long long b = 2ull * (9ull * plane + 2ull * GUARD) * elem;           // populations A, B
     b += 23ull * npa * sizeof(double) + 5ull * npa * sizeof(float) + npa * sizeof(int) + sizeof(int);   // particle state, forces, err
-    b += (unsigned long long)partial_entries((long long)ntiles, (long long)npa) * sizeof(float4);   // partials
+    b += (unsigned long long)partial_entries((long long)ntiles, (long long)npa) * sizeof(float4);         // partials
     b += 3ull * ntiles * sizeof(int) + 2ull * ntiles * MAXC * (sizeof(int2) + NREC * sizeof(float4)) +
          2ull * npa * (MAXT + 2) * sizeof(int);                                           // bins
     b += sizeof(PartArgs) + sizeof(GridSync);
@@ -297,7 +297,7 @@ int launch_frame_shift(dilbm_ctx *c) {
 
 // PS-LBM: each particle's table of covered cell areas spans the cells within
 // K = ceil(r_max + reach) + 1 of its centre cell; grown when a larger radius
-// arrives (the particles kernel fills it, the sweep reads it).
+// arrives (cover_kernel fills it after each update, the sweep reads it).
 int size_cover_tables(dilbm_ctx *c, const dilbm_particle *p, int np) {
     if (c->method != DILBM_METHOD_PS || np == 0) return DILBM_OK;
     double rmax = 0.0;
@@ -463,8 +463,8 @@ void advance(dilbm_ctx *c, int k) {
 // replayed; `queued`, the host's count, tells the multiple of 2^32.
 long long summed_steps(long long queued, unsigned counted) { return queued + (int)(counted - (unsigned)queued); }
 
-// k steps in one launch (k == 1: no barrier, and the PS tables and the moving
-// frame's shift as launches of their own).
+// k steps: in one launch (k == 1: no barrier, and the PS tables and the moving
+// frame's shift as launches of their own), or by sweeps alone.
 int launch_fused(dilbm_ctx *c, int k) {
     if (steps_by_sweeps(c)) {
         for (int q = 0; q < k; ++q) {
@@ -483,10 +483,10 @@ int launch_fused(dilbm_ctx *c, int k) {
     return DILBM_OK;
 }
 
-// Steps one launch may run: about 2^27 node updates (two milliseconds at the
-// rates of large lattices), so that work on other streams never waits long
-// behind a launch that holds the SMs, and the gap between launches stays
-// below a thousandth of its time.
+// Steps one launch may run: about 2^27 node updates, at most 1024 (two
+// milliseconds at the rates of large lattices, eight on the smallest), so that
+// work on other streams never waits long behind a launch that holds the SMs,
+// and the gap between launches stays below a thousandth of its time.
 int steps_per_launch(double nodes) {
     const double k = 134217728.0 / nodes;
     return k < 1.0 ? 1 : (k > 1024.0 ? 1024 : (int)k);
@@ -1466,8 +1466,8 @@ int shape_candidates(Occ occupancy, std::vector<SweepShape> *out, std::vector<in
 // neighbour noise over all candidates alike).  The full-occupancy shapes of
 // the large sweeps differ by 1-2 %, so the median is taken over 7 rounds, and
 // candidates within TUNE_TIE of the fastest count as tied: the one keeping the
-// most warps resident per SM wins (a step runs the particle kernel between
-// sweeps, and there the shape with more warps measured faster).
+// most warps resident per SM wins (the timed launches update no particle, and
+// beside the updates the shape with more warps measured faster).
 constexpr int TUNE_ROUNDS = 7;
 constexpr float TUNE_TIE = 0.01f;
 
@@ -1548,7 +1548,7 @@ int dilbm_set_shape(dilbm_ctx *c, int warps, int blocks_per_sm) {
     const SweepShape sh{warps, blocks_per_sm};
     if (!c || !shape_valid(sh)) return fail(DILBM_ERR_INVALID_ARG, "warps must be 2, 4 or 8 and blocks_per_sm >= 0");
     if (c->method == DILBM_METHOD_PS && !same_shape(sh, PS_SHAPE))
-        return fail(DILBM_ERR_INVALID_ARG, "a PS-LBM context runs the sweep in the default shape (8 warps, 0)");
+        return fail(DILBM_ERR_INVALID_ARG, "a PS-LBM context has one launch shape, reported as (8 warps, 0)");
     c->shape = sh;
     return DILBM_OK;
 }

@@ -54,7 +54,7 @@ static_assert(TILE_W == 1 << TILE_W_LOG2 && TILE_H == 1 << TILE_H_LOG2, "tiles o
 constexpr int MAXC = 32;      // candidate particles per tile
 constexpr int MAXT = 128;     // tiles one particle's phi tail may reach
 constexpr int NREC = 3;       // float4 records per binned particle
-constexpr int SWEEP_WARPS = 8;   // default rows in flight per block (one row segment per warp)
+constexpr int SWEEP_WARPS = 8;   // default row segments in flight per block of the sweep alone (one per warp)
 constexpr int GUARD = 256;    // elements kept readable before and after a population buffer
 constexpr float PHI_CUT_WIDTHS = 4.0f;   // phi tail kept up to 4 interface widths (phi > 1.1e-7)
 constexpr unsigned long long WAIT_LIMIT_NS = 1000000000ull;   // bounded device waits: 1 s
@@ -1134,7 +1134,7 @@ __device__ __forceinline__ bool sweep_segment(const SweepArgs<T> &A, const T *sr
                     }
                 }
             } else {
-float2 dx = make_float2(dx0, dx0 + 1.0f);
+                float2 dx = make_float2(dx0, dx0 + 1.0f);
                 if (L.wrap_x) {
                     dx.x = fmaf(-(float)L.nx, rintf(dx.x * __frcp_rn((float)L.nx)), dx.x);
                     dx.y = fmaf(-(float)L.nx, rintf(dx.y * __frcp_rn((float)L.nx)), dx.y);
@@ -1302,7 +1302,8 @@ float2 dx = make_float2(dx0, dx0 + 1.0f);
             sg.x += s2.x; sg.y += s2.y; sg.z += s2.z;
         }
         const int id = cid[lane];
-        float4 *out = A.partial + (A.B.by_slot ? (long long)tile * MAXC + lane : (long long)id * MAXT + __float_as_int(sg.w)) * TILE_H + (y - ty0);
+        const long long entry = A.B.by_slot ? (long long)tile * MAXC + lane : (long long)id * MAXT + __float_as_int(sg.w);
+        float4 *out = A.partial + entry * TILE_H + (y - ty0);
         if (FUSED) {
             store_partial(out, sg.x, sg.y, sg.z, tag);
             if (count) count_done(B.done + id);

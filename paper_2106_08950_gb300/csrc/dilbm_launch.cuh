@@ -14,9 +14,9 @@
 
 namespace dilbm {
 
-constexpr SweepShape SWEEP_SHAPE{SWEEP_WARPS, 0};  // sweep_kernel's: a strip's until another is set, and the fields'
-constexpr SweepShape PS_SHAPE = SWEEP_SHAPE;       // the one shape a PS-LBM context takes and reports
-constexpr int PS_WARPS = 4;                        // warps per block its fused steps are compiled for
+constexpr SweepShape SWEEP_SHAPE{SWEEP_WARPS, 0};  // of the sweep alone until another is set, and of the fields
+constexpr SweepShape PS_SHAPE = SWEEP_SHAPE;       // the one shape that a PS-LBM context takes and reports; its
+constexpr int PS_WARPS = 4;                        // fused steps run with this many warps per block all the same
 
 // row_of's multiplier: floor(2^32 / ntx) + 1 (unused for ntx == 1).
 inline unsigned ntx_inverse(int ntx) {

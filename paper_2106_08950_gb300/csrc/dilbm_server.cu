@@ -3,9 +3,9 @@
 // Every admitted job is an ordinary context (dilbm_create) that stays
 // resident on the device until it has run its steps; all running jobs of one
 // storage type advance together as one batch (dilbm_batch_*), so that one
-// launch runs several steps of every lattice in the mix.  With per-job storage the batches of the storage types present run
-// side by side (each on its own stream), by the same macro-steps.  The server only
-// decides who runs: it admits queued jobs by free job slots and by a device
+// launch runs several steps of every lattice in the mix.  With per-job storage
+// the batches of the storage types present, each on its own stream, take the
+// same macro-steps.  The server only decides who runs: it admits queued jobs by free job slots and by a device
 // memory budget, cuts the run into macro-steps no longer than the shortest
 // remaining job, and re-forms the batch when jobs join or leave.  The method
 // itself (Eqs. 13-19, 22-24, 28-29) is untouched, so every job's result is
