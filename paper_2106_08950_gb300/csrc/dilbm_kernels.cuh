@@ -32,11 +32,11 @@
 // per plane and pair.
 //
 // Two launches a step (sweep, particles) against this, us per step (FP32 unless
-// said, default shapes): 200 x 100 cylinder 18.5 -> 8.3, 400 x 2000 box
-// 36.9 -> 16.0, 1793 x 179 channel in FP16 21.6 -> 11.6, 512^2 suspension
-// 22.6 -> 12.3, 501 x 101 channel with a moving frame 30.8 -> 9.7, 64 uneven
-// lattices 264 -> 237, 4096^2 suspension 225.6 -> 210 (FP16 221.4 -> 202, PS
-// 247 -> 230).
+// said, default shapes): 200 x 100 cylinder 18.5 -> 8.0, 400 x 2000 box
+// 36.9 -> 15.9, 1793 x 179 channel in FP16 21.6 -> 11.7, 512^2 suspension
+// 22.6 -> 11.5, 501 x 101 channel with a moving frame 30.8 -> 8.8, 64 uneven
+// lattices 264 -> 231, 4096^2 suspension 225.6 -> 210 (FP16 221.4 -> 202, PS
+// 247 -> 228).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -2028,8 +2028,7 @@ constexpr int TICKET_GROUPS = 8;
 
 struct GridSync {               // all 0 between launches, but for the clock and mean_tag
     unsigned arrived[2][32];    // sweeping blocks, particle blocks (a cache line each)
-    unsigned left;
-    unsigned abandoned;         // a wait ran out, or had before the launch: not all steps were done
+    unsigned left, pad0;        // blocks that have left; from bit 16 on, abandon()s
     StepClock clock;            // a context's own (a batch's launches advance its members' clocks)
     unsigned mean_tag;          // the clock's step number when the force sums were last zeroed
     unsigned pad[27];
@@ -2061,12 +2060,12 @@ __device__ __forceinline__ bool await_blocks(const unsigned *arrived, unsigned t
     }
 }
 
-// A wait ran out: the launch ends early, and the last block out tells every
-// lattice in it.  (Before this block is counted out.)
-__device__ __forceinline__ void abandon(GridSync *sync) {
-    atomicExch(&sync->abandoned, 1u);
-    __threadfence();
-}
+// A wait ran out (or had before the launch): not all steps were done, and the
+// last block out tells every lattice.  Before this block is counted out, in the
+// same word: a word of its own is a trip to the L2 more at the end of each
+// launch, 0.7 us of a PS step.
+constexpr unsigned ABANDONED = 1u << 16;
+__device__ __forceinline__ void abandon(GridSync *sync) { atomicAdd(&sync->left, ABANDONED); }
 
 // The frame's move by s columns, in place: warps take rows of planes, 32
 // columns at a time in the direction of the move (each value is read before
@@ -2359,10 +2358,11 @@ __device__ __forceinline__ void run_steps(const WORK &wk, const PartArgs *frame,
     // the last block out leaves the counters as it found them, and advances the clocks
     __syncthreads();
     if (threadIdx.x == 0 && st != run.nsteps) abandon(run.sync);        // (left before its end)
-    if (threadIdx.x == 0 && atomicAdd(&run.sync->left, 1u) == gridDim.x - 1) {
+    const unsigned left = threadIdx.x == 0 ? atomicAdd(&run.sync->left, 1u) : 0u;
+    if (threadIdx.x == 0 && left % ABANDONED == gridDim.x - 1) {
         run.sync->arrived[0][0] = run.sync->arrived[1][0] = 0;
         run.sync->left = 0;
-        if (atomicExch(&run.sync->abandoned, 0u))
+        if (left >= ABANDONED)
             for (int k = 0; k < wk.lattices(); ++k) atomicOr(wk.args(k).err, ERR_TIMEOUT);
         for (int q = 0; q < 3; ++q)
             for (int g = 0; g < TICKET_GROUPS; ++g) run.sync->ticket[q][g][0] = 0;
