@@ -924,7 +924,7 @@ int dilbm_step(dilbm_ctx *c, long long nsteps) {
     // several steps per launch; one per launch where timing brackets each
     // step, or the PS tables follow each step (made by the particle warps, a
     // table took 20 us and the step 283 us instead of 237)
-    const long long most = c->method == DILBM_METHOD_PS ? 1 : steps_per_launch((double)c->L.nx * c->L.ny);
+    const long long most = c->method == DILBM_METHOD_PS && c->np > 0 ? 1 : steps_per_launch((double)c->L.nx * c->L.ny);
     for (long long t = 0; t < nsteps;) {
         const int k = (int)std::min(most, nsteps - t);
         const int rc = c->timing ? timed_step(c) : launch_fused(c, k);

@@ -67,3 +67,21 @@ def test_same_bits_as_fused_steps(torch, nx, ny, walls, storage):
     batch.close()
     for s in (a, b, c):
         s.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(130, 70), (2100, 2100)])
+def test_ps_without_particles_is_the_plain_flow(torch, nx, ny):
+    """No covered cell: the same steps, several to a call (by sweeps, and fused)."""
+    side = torch.cuda.Stream()
+    prob = flow(nx, ny, True)
+    ps = flow(nx, ny, True)
+    ps.method = W.METHOD_PS
+    a, b = (stirred(D.Simulation(p, stream=int(side.cuda_stream))) for p in (prob, ps))
+    for n in (1, 6):
+        a.step(n)
+        b.step(n)
+    assert np.array_equal(a.populations(), b.populations())
+    assert all(np.array_equal(x, y) for x, y in zip(a.fields(), b.fields()))
+    for s in (a, b):
+        s.sync()
+        s.close()
