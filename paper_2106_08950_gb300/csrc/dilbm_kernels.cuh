@@ -35,7 +35,7 @@
 // said, default shapes): 200 x 100 cylinder 18.5 -> 8.0, 400 x 2000 box
 // 36.9 -> 15.9, 1793 x 179 channel in FP16 21.6 -> 11.7, 512^2 suspension
 // 22.6 -> 11.5, 501 x 101 channel with a moving frame 30.8 -> 8.8, 64 uneven
-// lattices 264 -> 231, 4096^2 suspension 225.6 -> 210 (FP16 221.4 -> 202, PS
+// lattices 264 -> 231, 4096^2 suspension 225.6 -> 211 (FP16 221.4 -> 198, PS
 // 247 -> 228).
 #pragma once
 
