@@ -85,3 +85,16 @@ def test_ps_without_particles_is_the_plain_flow(torch, nx, ny):
     for s in (a, b):
         s.sync()
         s.close()
+
+
+def test_on_the_default_streams(torch):
+    """The legacy and the per-thread default stream take the same steps."""
+    want = stirred(D.Simulation(flow(300, 120, True), stream=int(torch.cuda.Stream().cuda_stream)))
+    want.step(9)
+    for handle in (0, 1, 2):            # NULL, cudaStreamLegacy, cudaStreamPerThread
+        s = stirred(D.Simulation(flow(300, 120, True), stream=handle))
+        s.step(9)
+        assert np.array_equal(s.populations(), want.populations())
+        s.sync()
+        s.close()
+    want.close()
